@@ -141,9 +141,10 @@ gb_status gb_pool_seed(gb_pool* pool, int n_beams, int prompt_len, const void* k
  *   out_dev:    [max_beams][Hq][D] fp32 (rows of inactive slots are zero)
  *   flags:      GB_PATH_AUTO / GB_PATH_PER_BEAM / GB_PATH_GROUPED
  * Rows of inactive slots in the inputs are ignored.
- * Launches: the append, then one attention launch that also merges the
- * split and shared-prefix partial results into out_dev (bf16 pools; fp32
- * pools add a merge launch); layer 0 adds the step's planner first.  The
+ * Launches: one attention launch that also appends the new rows and merges
+ * the split and shared-prefix partial results into out_dev (bf16 pools; fp32
+ * pools append and merge in launches of their own); layer 0 adds the step's
+ * planner first.  The
  * attention launch's CTAs wait (bounded) on each other's partial results, so
  * they must all get an SM within the wait limit (2 s): nothing else should
  * hold the GPU's SMs for that long meanwhile.

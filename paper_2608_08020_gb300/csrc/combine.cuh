@@ -4,20 +4,20 @@
 // Each (beam b, KV head h) pair has R = nseg + npb records: on the grouped path, nseg records
 // of the beam's shared-prefix segments, and npb split-KV records of the per-beam warps whose
 // chunk range meets the pair's chunks (warp w's record of the pair is number w + b * Hkv + h).
-// A grouped CTA counts itself in ctl[kCtlGrpDone] once all of its records are written; a
-// per-beam warp counts each record it writes in pair_cnt[b * Hkv + h] (release: fence, then
+// A grouped CTA counts itself in the launch's kCntGrpDone once all of its records are written; a
+// per-beam warp counts each record it writes in pair[b * Hkv + h] (release: fence, then
 // the add).  After its own work, every warp of the merging CTAs takes pairs from the counter
-// ctl[kCtlPairNext] until none is left, so the warps that finish first take the pairs and the
+// kCntPairNext until none is left, so the warps that finish first take the pairs and the
 // last ones to finish find none.  Per pair it folds the segment records first (a bounded wait
 // until every grouped CTA has finished, long past on a large step), then waits (bounded) until
-// pair_cnt[p] == npb and folds the split-KV records, so what remains after the pair's last
+// pair[p] == npb and folds the split-KV records, so what remains after the pair's last
 // record is one batch of loads: running max M of the records' m, acc = sum o * 2^(m - M),
 // L = sum l * 2^(m - M), out[b][h * G + g][:] = acc / L.
 //
 // The waits end because every CTA they wait on gets an SM: the callers only let CTAs merge
 // that are resident together with the ones they wait on, or that wait only on CTAs which never
 // wait (k_attention).  Each wait is bounded and gives up as soon as the pool's status word is
-// set.  The counters are zeroed by k_append, the launch that precedes every attention launch.
+// set.  The counters are one of two sets; a launch zeroes the other one (Counters, internal.cuh).
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>
@@ -27,29 +27,29 @@
 namespace gb {
 
 // A per-beam warp has written the record of pair bh: make the writes visible, then count it.
-__device__ __forceinline__ void record_arrive(const PoolView& v, int bh, int lane) {
+__device__ __forceinline__ void record_arrive(const Counters& k, int bh, int lane) {
   fence_acq_rel_gpu();
   __syncwarp();
-  if (lane == 0) atomicAdd(&v.pair_cnt[bh], 1);
+  if (lane == 0) atomicAdd(&k.pair[bh], 1);
 }
 
 // A grouped CTA has written all of its records (called by every thread of the CTA).
-__device__ __forceinline__ void grouped_cta_done(const PoolView& v) {
+__device__ __forceinline__ void grouped_cta_done(const Counters& k) {
   __syncthreads();
   if (threadIdx.x == 0) {
     fence_acq_rel_gpu();
-    atomicAdd(&v.ctl[kCtlGrpDone], 1);
+    atomicAdd(&k.c[kCntGrpDone], 1);
   }
 }
 
 // Wait, with the whole warp polling, until pair p has npb split-KV records and ng grouped
 // CTAs have finished.  False on a timeout or when an error status is set.
-__device__ __forceinline__ bool wait_pair_records(const PoolView& v, int p, int npb, int ng) {
+__device__ __forceinline__ bool wait_pair_records(const PoolView& v, const Counters& k, int p, int npb, int ng) {
   const uint64_t t0 = globaltimer_ns();
   unsigned ns = 32;
   while (true) {
-    const int a = npb > 0 ? ld_acquire_gpu(&v.pair_cnt[p]) : 0;
-    const int g = ng > 0 ? ld_acquire_gpu(&v.ctl[kCtlGrpDone]) : 0;
+    const int a = npb > 0 ? ld_acquire_gpu(&k.pair[p]) : 0;
+    const int g = ng > 0 ? ld_acquire_gpu(&k.c[kCntGrpDone]) : 0;
     if (__all_sync(0xffffffffu, a >= npb && g >= ng)) return true;
     if (__any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&v.ctl[kCtlStatus]) != GB_OK ||
                                     globaltimer_ns() - t0 > kWaitLimitNs))
@@ -166,19 +166,26 @@ __device__ __forceinline__ void zero_pair(const PoolView& v, int b, int h, float
   for (int e = threadIdx.x & 31; e < G * 128; e += 32) ob[e] = 0.f;
 }
 
+// A step that was refused (no pages) has no attention: its outputs are zero.
+template <int G>
+__device__ __forceinline__ void zero_all_pairs(const PoolView& v, int cta, int nctas, float* __restrict__ out) {
+  const int nw = blockDim.x >> 5;
+  for (int p = cta * nw + (int)(threadIdx.x >> 5); p < v.max_beams * v.Hkv; p += nctas * nw)
+    zero_pair<G>(v, p / v.Hkv, p % v.Hkv, out);
+}
+
 // The merge phase of an attention launch, run by every warp of the merging CTAs after its own
 // work: `mode` selects the plan (0 per-beam, 1 with segments), W = warps of the per-beam
 // role, ng = CTAs of the grouped role (0 without one), out = [max_beams][Hq][128] fp32.
-// `claim`: the warps take pairs from the counter ctl[kCtlPairNext] as they finish (for CTAs
+// `claim`: the warps take pairs from the counter kCntPairNext as they finish (for CTAs
 // that start at different times) and fold a pair's segment records before they wait for its
 // split-KV records; otherwise merging CTA `cta` of `nctas` takes the pairs
 // p = cta + nctas * (warp + k * warps per CTA) and waits for all of a pair's records at once.
 template <int G>
-__device__ __forceinline__ void combine_pairs(const PoolView& v, int mode, int W, int ng, bool claim, int cta,
-                                              int nctas, float* __restrict__ out) {
+__device__ __forceinline__ void combine_pairs(const PoolView& v, const Counters& cnt, int mode, int W, int ng,
+                                              bool claim, int cta, int nctas, float* __restrict__ out) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int npairs = v.max_beams * v.Hkv;
-  const bool ok = v.ctl[kCtlStepOk] != 0;
   const int* off = plan_off(v, mode);
   const int* nn = plan_n(v, mode);
   const int Tot = off[v.max_beams];
@@ -187,12 +194,12 @@ __device__ __forceinline__ void combine_pairs(const PoolView& v, int mode, int W
   for (int k = 0;; ++k) {
     int p = cta + nctas * (warp + k * nw);
     if (claim) {
-      if (lane == 0) p = atomicAdd(&v.ctl[kCtlPairNext], 1);
+      if (lane == 0) p = atomicAdd(&cnt.c[kCntPairNext], 1);
       p = __shfl_sync(0xffffffffu, p, 0);
     }
     if (p >= npairs) break;
     const int b = p / v.Hkv, h = p - b * v.Hkv;
-    const bool act = ok && v.active[b] != 0;
+    const bool act = v.active[b] != 0;
     const int n = act ? nn[b] : 0;
     const int nseg = (act && mode == 1 && v.grouped) ? v.seg_nrec[b] : 0;
     const int o0 = off[b] + h * n;
@@ -208,12 +215,12 @@ __device__ __forceinline__ void combine_pairs(const PoolView& v, int mode, int W
     merge_init(st);
     bool good;
     if (claim) {
-      good = nseg == 0 || wait_pair_records(v, p, 0, ng);
+      good = nseg == 0 || wait_pair_records(v, cnt, p, 0, ng);
       if (good && nseg > 0) merge_fold(st, grec, (size_t)v.Hkv * rf, nseg);
-      good = good && (npb == 0 || wait_pair_records(v, p, npb, 0));
+      good = good && (npb == 0 || wait_pair_records(v, cnt, p, npb, 0));
       if (good && npb > 0) merge_fold(st, prec, rf, npb);
     } else {
-      good = wait_pair_records(v, p, npb, nseg > 0 ? ng : 0);
+      good = wait_pair_records(v, cnt, p, npb, nseg > 0 ? ng : 0);
       if (good) {
         merge_fold(st, prec, rf, npb);
         merge_fold(st, grec, (size_t)v.Hkv * rf, nseg);

@@ -416,11 +416,20 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
 template <int G>
 __global__ void __launch_bounds__(kMmaWarps * 32, 1)
     k_decode_mma(PoolView v, const __grid_constant__ CUtensorMap tm, const __grid_constant__ CUtensorMap tmh,
-                 int layer, const __nv_bfloat16* __restrict__ q, float qscale, int mode, float* __restrict__ out) {
+                 int layer, const __nv_bfloat16* __restrict__ q, NewRows nw, float qscale, int mode,
+                 float* __restrict__ out) {
   pdl_wait();
   pdl_launch_dependents();
-  decode_mma_body<G>(v, &tm, &tmh, layer, q, qscale, mode, (int)blockIdx.x, (int)gridDim.x);
-  combine_pairs<G>(v, mode, (int)gridDim.x * kMmaWarps, 0, false, (int)blockIdx.x, (int)gridDim.x, out);
+  const int c = (int)blockIdx.x, nctas = (int)gridDim.x;
+  if (v.ctl[kCtlStepOk] == 0) {
+    zero_all_pairs<G>(v, c, nctas, out);
+    return;
+  }
+  const int set = counter_set(v, layer);
+  const Counters cnt = counters(v, set);
+  zero_counters(v, set ^ 1, c, nctas);
+  decode_mma_body<G>(v, cnt, &tm, &tmh, layer, q, nw, qscale, mode, c, nctas);
+  combine_pairs<G>(v, cnt, mode, nctas * kMmaWarps, 0, false, c, nctas, out);
 }
 
 // Merge the partial records of each (beam, kv head) into out[b][h*G+g][:]: the split-KV
@@ -510,15 +519,15 @@ __global__ void __launch_bounds__(128) k_combine(PoolView v, int mode, int W, fl
 }
 
 template <int DT, int G>
-static cudaError_t launch_decode_t(gb_pool* pool, int layer, const void* q, float scale, float* out, int mode,
-                                   cudaStream_t s) {
+static cudaError_t launch_decode_t(gb_pool* pool, int layer, const void* q, const void* k_new, const void* v_new,
+                                   float scale, float* out, int mode, cudaStream_t s) {
   using S = DecodeSmem<DT, G>;
   const float qscale = scale * 1.4426950408889634f;  // log2(e): softmax in base 2
   cudaError_t e;
-  if (DT == GB_BF16 && pool->have_dtmap && pool->num_sms * kMmaWarps <= kMaxDecodeWarps) {
-    // One launch: the attention roles and the merge of their records.
+  if (fuses_append(pool)) {
+    // One launch: the new rows, the attention roles and the merge of their records.
     if (mode == 1) {
-      e = launch_attention(pool, layer, q, scale, out, s);  // grouped and per-beam roles (grouped.cu)
+      e = launch_attention(pool, layer, q, k_new, v_new, scale, out, s);  // grouped and per-beam roles (grouped.cu)
     } else {
       e = set_max_dynamic_smem(reinterpret_cast<const void*>(k_decode_mma<G>), DecodeMmaSmem::TOTAL);
       if (e != cudaSuccess) return e;
@@ -526,7 +535,8 @@ static cudaError_t launch_decode_t(gb_pool* pool, int layer, const void* q, floa
       e = launch_pdl(k_decode_mma<G>, pool->num_sms, kMmaWarps * 32, DecodeMmaSmem::TOTAL, s, pool->view,
                      *reinterpret_cast<const CUtensorMap*>(pool->dtmap),
                      *reinterpret_cast<const CUtensorMap*>(pool->dtmap_half), layer,
-                     static_cast<const __nv_bfloat16*>(q), qscale, mode, out);
+                     static_cast<const __nv_bfloat16*>(q),
+                     NewRows{static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new)}, qscale, mode, out);
       prof_end(pool, GB_PROF_DECODE, s);
       pool->launches += 1;
     }
@@ -554,8 +564,9 @@ static cudaError_t launch_decode_t(gb_pool* pool, int layer, const void* q, floa
 // One warp waits for the record count of pair 0 to reach one more than it holds; nothing
 // raises it, so the wait runs out (the same bounded wait as the attention launch's merge).
 __global__ void k_wait_selftest(PoolView v) {
-  const int have = v.pair_cnt[0];
-  if (!wait_pair_records(v, 0, have + 1, 0) && threadIdx.x == 0) set_status(v.ctl, GB_ERR_TIMEOUT);
+  const Counters cnt = counters(v, 0);
+  const int have = cnt.pair[0];
+  if (!wait_pair_records(v, cnt, 0, have + 1, 0) && threadIdx.x == 0) set_status(v.ctl, GB_ERR_TIMEOUT);
 }
 
 cudaError_t launch_wait_selftest(gb_pool* pool, cudaStream_t s) {
@@ -599,20 +610,25 @@ cudaError_t launch_decode_view(const PoolView& v, int W, int layer, const void* 
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_decode(gb_pool* pool, int layer, const void* q, float scale, float* out, int mode,
-                          cudaStream_t s) {
+// bf16 pools with the per-beam tensor maps: the warp-MMA kernels, which append as they go.
+bool fuses_append(const gb_pool* pool) {
+  return pool->view.dtype == GB_BF16 && pool->have_dtmap && pool->num_sms * kMmaWarps <= kMaxDecodeWarps;
+}
+
+cudaError_t launch_decode(gb_pool* pool, int layer, const void* q, const void* k_new, const void* v_new, float scale,
+                          float* out, int mode, cudaStream_t s) {
   const int G = pool->view.G;
   if (pool->view.dtype == GB_BF16) {
     switch (G) {
-      case 2: return launch_decode_t<GB_BF16, 2>(pool, layer, q, scale, out, mode, s);
-      case 4: return launch_decode_t<GB_BF16, 4>(pool, layer, q, scale, out, mode, s);
-      case 8: return launch_decode_t<GB_BF16, 8>(pool, layer, q, scale, out, mode, s);
+      case 2: return launch_decode_t<GB_BF16, 2>(pool, layer, q, k_new, v_new, scale, out, mode, s);
+      case 4: return launch_decode_t<GB_BF16, 4>(pool, layer, q, k_new, v_new, scale, out, mode, s);
+      case 8: return launch_decode_t<GB_BF16, 8>(pool, layer, q, k_new, v_new, scale, out, mode, s);
     }
   } else {
     switch (G) {
-      case 2: return launch_decode_t<GB_F32, 2>(pool, layer, q, scale, out, mode, s);
-      case 4: return launch_decode_t<GB_F32, 4>(pool, layer, q, scale, out, mode, s);
-      case 8: return launch_decode_t<GB_F32, 8>(pool, layer, q, scale, out, mode, s);
+      case 2: return launch_decode_t<GB_F32, 2>(pool, layer, q, k_new, v_new, scale, out, mode, s);
+      case 4: return launch_decode_t<GB_F32, 4>(pool, layer, q, k_new, v_new, scale, out, mode, s);
+      case 8: return launch_decode_t<GB_F32, 8>(pool, layer, q, k_new, v_new, scale, out, mode, s);
     }
   }
   return cudaErrorInvalidValue;

@@ -65,7 +65,7 @@ constexpr int kMmaStages = GB_MMA_STAGES, kMmaChains = GB_MMA_CHAINS;
 struct DecodeMmaSmem {
   static constexpr int STAGES = kMmaWarps * kMmaStages * kMmaStageBytes;
   static constexpr int BARS = kMmaWarps * kMmaStages * 8;
-  static constexpr int PLAN_BYTES = 3 * (kMaxBeams + 1) * 4;
+  static constexpr int PLAN_BYTES = 5 * (kMaxBeams + 1) * 4;  // offsets, chunk counts, start tokens, lengths, copied-from pages
   static constexpr int TOTAL = 1024 + STAGES + BARS + PLAN_BYTES;  // 1024: alignment slack
   static_assert(TOTAL <= 232448, "shared memory per block");
 };
@@ -114,13 +114,27 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   return *reinterpret_cast<const uint32_t*>(&t);
 }
 
+// The new K/V rows of the step, [max_beams][Hkv][128] bf16 each (16 uint4 per row).
+struct NewRows {
+  const uint4* k;
+  const uint4* v;
+};
+
 // The kernel's body, shared by the per-beam kernel (k_decode_mma, below in decode.cu) and the
 // attention kernel that also runs the grouped role (k_attention, grouped.cu): this CTA is
 // number `cta` of the `nctas` CTAs that take the per-beam work.  tm: 16-token boxes; tmh:
 // 8-token boxes (the last chunk of a range when it holds at most 8 valid tokens).
+//
+// The body also appends: the new token of (beam, head) is the last one of the pair's last chunk,
+// and the warp that holds that chunk puts the new row into the landed stage and into the pool.
+// After a fork a beam's partial tail page may have been copied on write by the planner (cow_old
+// names the page it was copied from): the tail page's chunks are then loaded from the old page
+// and written to the new one from the stage, new row and all.  This replaces a launch before
+// every attention launch (k_append, 2-3 us per layer even when overlapped).
 template <int G>
-__device__ __forceinline__ void decode_mma_body(const PoolView& v, const CUtensorMap* tm_p, const CUtensorMap* tmh_p,
-                                                int layer, const __nv_bfloat16* __restrict__ q, float qscale,
+__device__ __forceinline__ void decode_mma_body(const PoolView& v, const Counters& cnt, const CUtensorMap* tm_p,
+                                                const CUtensorMap* tmh_p, int layer,
+                                                const __nv_bfloat16* __restrict__ q, const NewRows& nw, float qscale,
                                                 int mode, int cta, int nctas) {
   using S = DecodeMmaSmem;
   constexpr int D = 128;
@@ -129,7 +143,8 @@ __device__ __forceinline__ void decode_mma_body(const PoolView& v, const CUtenso
   int* s_off = reinterpret_cast<int*>(smem + S::STAGES + S::BARS);
   int* s_n = s_off + (kMaxBeams + 1);
   int* s_start = s_n + (kMaxBeams + 1);
-  if (v.ctl[kCtlStepOk] == 0) return;
+  int* s_len = s_start + (kMaxBeams + 1);
+  int* s_cow = s_len + (kMaxBeams + 1);
   const int W = nctas * kMmaWarps;  // warps that share the per-beam work
   {
     const int* off = plan_off(v, mode);
@@ -139,6 +154,8 @@ __device__ __forceinline__ void decode_mma_body(const PoolView& v, const CUtenso
       s_off[i] = off[i];
       s_n[i] = i < v.max_beams ? nn[i] : 0;
       s_start[i] = i < v.max_beams ? st[i] : 0;
+      s_len[i] = i < v.max_beams ? v.seq_len[i] : 0;
+      s_cow[i] = i < v.max_beams ? v.cow_old[i] : -1;
     }
   }
   __syncthreads();
@@ -185,7 +202,11 @@ __device__ __forceinline__ void decode_mma_body(const PoolView& v, const CUtenso
       pw_b = qi.b;
       pw_i0 = qi.i;
       const int i = pw_i0 + lane;
-      pw_lane = i < qi.n ? v.tables[(size_t)qi.b * v.max_pages + (qi.tok0 + i * kChunk) / v.P] : 0;
+      const int pi = (qi.tok0 + i * kChunk) / v.P;
+      const int old = s_cow[qi.b];  // of the tail page, which holds the new token
+      pw_lane = i >= qi.n ? 0
+                : old >= 0 && pi == (s_len[qi.b] - 1) / v.P ? old
+                                                            : v.tables[(size_t)qi.b * v.max_pages + pi];
     }
     return __shfl_sync(0xffffffffu, pw_lane, qi.i - pw_i0);
   };
@@ -203,7 +224,7 @@ __device__ __forceinline__ void decode_mma_body(const PoolView& v, const CUtenso
       const uint32_t bar = bar0 + 8 * stage;
       // The last chunk of a (beam, head) with at most 8 valid tokens brings only its first
       // 8-token group (the consumer masks the rest of the stage, whatever it holds).
-      const bool half = qi.i == qi.n - 1 && v.seq_len[qi.b] - tok <= 8;
+      const bool half = qi.i == qi.n - 1 && s_len[qi.b] - tok <= 8;
       mbar_arrive_expect_tx(bar, half ? kMmaStageBytes / 2 : kMmaStageBytes);
       tma_chunk(stage0 + stage * kMmaStageBytes, half ? tmh_p : tm_p, wrow, bar, pol);
     }
@@ -242,12 +263,18 @@ __device__ __forceinline__ void decode_mma_body(const PoolView& v, const CUtenso
   float m0 = -INFINITY, m1 = -INFINITY, l0 = 0.f, l1 = 0.f;
   int L = 0;
   bool fresh = true;
+  uint4 nrow = make_uint4(0u, 0u, 0u, 0u);  // 16 bytes of the pair's new rows: lanes 0-15 K, 16-31 V
+  int npage = 0;                            // the page they go to
 
   int stage = 0;
   uint32_t parity = 0;
   for (int x = x_begin, k = 0; x < x_end; ++x, ++k) {
     if (fresh) {
-      L = v.seq_len[it.b];
+      L = s_len[it.b];
+      if (it.n - it.i <= x_end - x) {  // this warp holds the pair's last chunk
+        nrow = (lane < 16 ? nw.k : nw.v)[((size_t)it.b * v.Hkv + it.h) * 16 + (lane & 15)];
+        npage = v.tables[(size_t)it.b * v.max_pages + (L - 1) / v.P];
+      }
       const uint32_t* qrow = reinterpret_cast<const uint32_t*>(q + ((size_t)it.b * v.Hq + it.h * G + r) * D);
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
@@ -271,6 +298,40 @@ __device__ __forceinline__ void decode_mma_body(const PoolView& v, const CUtenso
     const uint32_t sb = stage0 + stage * kMmaStageBytes;
     const int tok0 = it.tok0 + it.i * kChunk;
     const int nvalid = min(kChunk, L - tok0);  // >= 1: a chunk starts before the beam's length
+    if (it.i == it.n - 1) {
+      // The new token, and zeros for the V rows past it (the page's rows there hold whatever the
+      // pool held), so that 0 * V stays 0 in the MMA.
+      unsigned char* vs = smem + (sb - smem_addr(smem));
+      const int t = nvalid - 1, kv = lane >> 4, piece = lane & 15;
+      const bool page_ok = npage >= 0 && npage < v.num_pages;
+      *reinterpret_cast<uint4*>(vs + (t >> 3) * 4096 + kv * 2048 + (piece >> 3) * 1024 + (t & 7) * 128 +
+                                (((piece & 7) ^ (t & 7)) << 4)) = nrow;
+      for (int idx = lane; idx < (kChunk - nvalid) * 16; idx += 32) {
+        const int tz = nvalid + (idx >> 4), pz = idx & 15;
+        *reinterpret_cast<uint4*>(vs + (tz >> 3) * 4096 + 2048 + (pz >> 3) * 1024 + (tz & 7) * 128 + (pz & 7) * 16) =
+            make_uint4(0u, 0u, 0u, 0u);
+      }
+      if (page_ok)
+        reinterpret_cast<uint4*>(v.kv + kv_elem_offset(v, layer, npage, kv, it.h, (L - 1) % v.P) * 2)[piece] = nrow;
+      else if (lane == 0)
+        set_status(v.ctl, GB_ERR_INVALID);
+      fence_proxy_async_smem();  // ordered before the TMA that later refills this stage
+      __syncwarp();
+    }
+    if (s_cow[it.b] >= 0 && tok0 / v.P == (L - 1) / v.P) {
+      // A chunk of a tail page copied on write: its rows before the new one go to the new page.
+      const int page = v.tables[(size_t)it.b * v.max_pages + (L - 1) / v.P];
+      if (page >= 0 && page < v.num_pages) {
+        const unsigned char* vs = smem + (sb - smem_addr(smem));
+        const int rows = min(kChunk, L - 1 - tok0);
+        for (int idx = lane; idx < rows * 32; idx += 32) {
+          const int t = idx >> 5, kv = lane >> 4, piece = lane & 15;
+          reinterpret_cast<uint4*>(v.kv + kv_elem_offset(v, layer, page, kv, it.h, (tok0 + t) % v.P) * 2)[piece] =
+              *reinterpret_cast<const uint4*>(vs + (t >> 3) * 4096 + kv * 2048 + (piece >> 3) * 1024 + (t & 7) * 128 +
+                                              (((piece & 7) ^ (t & 7)) << 4));
+        }
+      }
+    }
 
     // ---- S^T = K . Q^T (kMmaChains independent accumulator chains) -----------
     float sacc[kMmaChains][4];
@@ -291,18 +352,9 @@ __device__ __forceinline__ void decode_mma_body(const PoolView& v, const CUtenso
       sc[e] = t * qscale;
     }
     if (nvalid < kChunk) {
-      // Tokens past the beam's length: no score, and zero V rows (the page's rows there
-      // hold whatever the pool held), so that 0 * V stays 0 in the MMA.
+      // Tokens past the beam's length: no score.
       if (r >= nvalid) sc[0] = sc[1] = -INFINITY;
       if (r + 8 >= nvalid) sc[2] = sc[3] = -INFINITY;
-      unsigned char* vs = smem + (sb - smem_addr(smem));
-      for (int idx = lane; idx < (kChunk - nvalid) * 16; idx += 32) {
-        const int t = nvalid + (idx >> 4), piece = idx & 15;
-        *reinterpret_cast<uint4*>(vs + (t >> 3) * 4096 + 2048 + (piece >> 3) * 1024 + (t & 7) * 128 + (piece & 7) * 16) =
-            make_uint4(0u, 0u, 0u, 0u);
-      }
-      fence_proxy_async_smem();  // ordered before the TMA that later refills this stage
-      __syncwarp();
     }
     // ---- online softmax over the chunk's 16 tokens (per head column) ----------
     float mx0 = fmaxf(sc[0], sc[2]), mx1 = fmaxf(sc[1], sc[3]);
@@ -380,7 +432,7 @@ __device__ __forceinline__ void decode_mma_body(const PoolView& v, const CUtenso
           st_hint(rec + G * D + G + 2 * c + 1, l1, rpol);
         }
       }
-      record_arrive(v, it.b * v.Hkv + it.h, lane);
+      record_arrive(cnt, it.b * v.Hkv + it.h, lane);
       fresh = true;
     }
     if (x + 1 < x_end) iter_advance(it, s_n, s_start, v.Hkv, v.max_beams);

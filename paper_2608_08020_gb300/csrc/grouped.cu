@@ -32,7 +32,7 @@
 // Handshakes are mbarriers: full/empty per K stage and per V stage, sched_full/sched_empty
 // per unit slot, q_full/q_empty, s_full, p_full and pv_done per S/P tile (three in
 // tensor memory), max_full per tile parity, xch_full and o_free per unit.  The grid-wide
-// work counter is zeroed by k_append before each launch.  An S/P buffer is reused by
+// work counter belongs to the launch's counter set (internal.cuh).  An S/P buffer is reused by
 // S(n+3) only after P.V(n) has been issued: the tensor core runs a CTA's MMAs in issue
 // order, so P(n) has been read before S(n+3) overwrites it.  With three buffers S runs two
 // tiles ahead of the softmax.
@@ -159,7 +159,7 @@ __device__ __forceinline__ Unit load_unit(const PoolView& v, long long u) {
 // CTAs that take grouped work units; threads past kThreads only take part in the CTA's
 // barriers.
 template <int G>
-__device__ __forceinline__ void grouped_body(const PoolView& v, const CUtensorMap* tm_p, int layer,
+__device__ __forceinline__ void grouped_body(const PoolView& v, const Counters& cnt, const CUtensorMap* tm_p, int layer,
                                              const __nv_bfloat16* __restrict__ q, float qscale, int w_oob, int ng) {
   extern __shared__ __align__(1024) unsigned char sm[];
   const long long units = (long long)v.ctl[kCtlSegTiles] * v.Hkv;
@@ -224,7 +224,7 @@ __device__ __forceinline__ void grouped_body(const PoolView& v, const CUtensorMa
     // unit (or the end, -1) is published in slot uidx % kSchedSlots once every role has
     // read the unit that slot held before.
     int pending = 0;
-    if (lane == 0) pending = atomicAdd(&v.ctl[kCtlGrpNext], 1);
+    if (lane == 0) pending = atomicAdd(&cnt.c[kCntGrpNext], 1);
     // The next unit's description is loaded while this unit's second tile is issued, so at
     // the unit boundary only its page ids and member rows (loaded together) are waited for.
     Unit xn{};
@@ -232,7 +232,7 @@ __device__ __forceinline__ void grouped_body(const PoolView& v, const CUtensorMa
     for (;; ++uidx) {
       if (!ok || *abort_flag) break;
       const long long u = __shfl_sync(0xffffffffu, pending, 0);
-      if (lane == 0 && u < units) pending = atomicAdd(&v.ctl[kCtlGrpNext], 1);
+      if (lane == 0 && u < units) pending = atomicAdd(&cnt.c[kCntGrpNext], 1);
       const int k = uidx & (kSchedSlots - 1);
       if (lane == 0 && uidx >= kSchedSlots)
         ok = wait_or_abort(ctl + kBarSchedEmpty + 8 * k, ((uidx / kSchedSlots) - 1) & 1, abort_flag);
@@ -697,7 +697,7 @@ constexpr int kAttnSmem = kSmem > DecodeMmaSmem::TOTAL ? kSmem : DecodeMmaSmem::
 template <int G>
 __global__ void __launch_bounds__(kAttnThreads, 1)
     k_attention(PoolView v, const __grid_constant__ CUtensorMap tmg, const __grid_constant__ CUtensorMap tmd,
-                const __grid_constant__ CUtensorMap tmdh, int layer, const __nv_bfloat16* __restrict__ q,
+                const __grid_constant__ CUtensorMap tmdh, int layer, const __nv_bfloat16* __restrict__ q, NewRows nw,
                 float qscale, int w_oob, float* __restrict__ out) {
   pdl_wait();
   pdl_launch_dependents();
@@ -707,28 +707,28 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   // per-beam CTA gets an SM.  Small steps: [0, ng) grouped and [ng, S) per-beam side by side,
   // all S resident at once, all S merging; the rest leave at once.
   const int S = (int)gridDim.x / 2, c = (int)blockIdx.x;
-  const bool ok = v.ctl[kCtlStepOk] != 0;
-  int nd = S, ng = S;
-  if (ok) {
-    nd = decode_ctas(v, S);
-    if (nd < S) ng = S - nd;
+  if (v.ctl[kCtlStepOk] == 0) {
+    zero_all_pairs<G>(v, c, 2 * S, out);
+    return;
   }
+  const int set = counter_set(v, layer);
+  const Counters cnt = counters(v, set);
+  zero_counters(v, set ^ 1, c, 2 * S);
+  const int nd = decode_ctas(v, S), ng = nd < S ? S - nd : S;
   const bool split = nd < S;
   const int pb0 = split ? ng : S;  // first per-beam CTA
   if (c >= pb0 + nd) return;
   if (c < pb0) {
-    if (ok) {
-      grouped_body<G>(v, &tmg, layer, q, qscale, w_oob, ng);
-      grouped_cta_done(v);
-    }
+    grouped_body<G>(v, cnt, &tmg, layer, q, qscale, w_oob, ng);
+    grouped_cta_done(cnt);
     if (!split) return;
   } else {
-    decode_mma_body<G>(v, &tmd, &tmdh, layer, q, qscale, 1, c - pb0, nd);
+    decode_mma_body<G>(v, cnt, &tmd, &tmdh, layer, q, nw, qscale, 1, c - pb0, nd);
   }
   // A large step's per-beam CTAs start as grouped CTAs leave, so they take the pairs as they
   // finish; a small step's CTAs all start together and split the pairs evenly.
-  if (split) combine_pairs<G>(v, 1, nd * kMmaWarps, ng, false, c, S, out);
-  else combine_pairs<G>(v, 1, nd * kMmaWarps, ng, true, c - S, S, out);
+  if (split) combine_pairs<G>(v, cnt, 1, nd * kMmaWarps, ng, false, c, S, out);
+  else combine_pairs<G>(v, cnt, 1, nd * kMmaWarps, ng, true, c - S, S, out);
 }
 
 }  // namespace
@@ -781,8 +781,8 @@ void make_kv_tensor_maps(gb_pool* pool) {
 }
 
 template <int G>
-static cudaError_t launch_attention_t(gb_pool* pool, int layer, const void* q, float scale, float* out,
-                                      cudaStream_t s) {
+static cudaError_t launch_attention_t(gb_pool* pool, int layer, const void* q, const NewRows& nw, float scale,
+                                      float* out, cudaStream_t s) {
   {
     const cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(k_attention<G>), kAttnSmem);
     if (e != cudaSuccess) return e;
@@ -795,18 +795,20 @@ static cudaError_t launch_attention_t(gb_pool* pool, int layer, const void* q, f
                                    *reinterpret_cast<const CUtensorMap*>(pool->tmap),
                                    *reinterpret_cast<const CUtensorMap*>(pool->dtmap),
                                    *reinterpret_cast<const CUtensorMap*>(pool->dtmap_half), layer,
-                                   static_cast<const __nv_bfloat16*>(q), qscale, pool->tmap_oob, out);
+                                   static_cast<const __nv_bfloat16*>(q), nw, qscale, pool->tmap_oob, out);
   prof_end(pool, GB_PROF_DECODE, s);
   prof_end(pool, GB_PROF_GROUPED, s);
   pool->launches += 1;
   return e;
 }
 
-cudaError_t launch_attention(gb_pool* pool, int layer, const void* q, float scale, float* out, cudaStream_t s) {
+cudaError_t launch_attention(gb_pool* pool, int layer, const void* q, const void* k_new, const void* v_new, float scale,
+                             float* out, cudaStream_t s) {
+  const NewRows nw{static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new)};
   switch (pool->view.G) {
-    case 2: return launch_attention_t<2>(pool, layer, q, scale, out, s);
-    case 4: return launch_attention_t<4>(pool, layer, q, scale, out, s);
-    case 8: return launch_attention_t<8>(pool, layer, q, scale, out, s);
+    case 2: return launch_attention_t<2>(pool, layer, q, nw, scale, out, s);
+    case 4: return launch_attention_t<4>(pool, layer, q, nw, scale, out, s);
+    case 8: return launch_attention_t<8>(pool, layer, q, nw, scale, out, s);
   }
   return cudaErrorInvalidValue;
 }

@@ -44,21 +44,27 @@ enum Ctl : int {
   kCtlSegTileTok = 11, // sum over segments of (128-row tiles) x tokens
   kCtlSteps = 12,      // steps opened so far (index into the step-stats ring)
   kCtlSegSplit = 13,   // tokens per grouped work unit (segments are split along tokens)
-  kCtlGrpNext = 14,    // next grouped work unit to hand out (zeroed by k_append)
-  kCtlGrpDone = 15,    // grouped-role CTAs finished (zeroed by k_append)
   kCtlSegTok = 16,     // sum over segments of their tokens (the shared tokens the grouped path reads once)
   kCtlBarCount = 17,   // grid-barrier arrivals of the tournament kernel (only grows)
   kCtlSegGen = 19,     // segment rebuilds so far (stamps the per-page claim words)
   kCtlSegAlloc = 20,   // words 20-21: (segments << 32 | member slots) handed out by the running rebuild
   kCtlTailShared = 22, // 1 when a partial tail page may be shared (set by seed and forks, cleared by the planner)
-  kCtlPairNext = 23,   // next (beam, KV head) pair to merge in the attention launch (zeroed by k_append)
+  kCtlCounters = 24,   // words 24-26 and 28-30: the two counter sets of the attention launches (Counters)
   kCtlWords = 32
+};
+
+// Words of a counter set.
+enum CounterWord : int {
+  kCntGrpNext = 0,   // next grouped work unit to hand out
+  kCntGrpDone = 1,   // grouped-role CTAs finished
+  kCntPairNext = 2,  // next (beam, KV head) pair to merge
+  kCntWords = 4
 };
 
 // Byte offsets of the metadata regions.
 struct MetaLayout {
   size_t ctl, tables, seq_len, active, gen, nsteps, mean, lineage, refcnt, free_bits;
-  size_t plan, cow, partials, total, stats;
+  size_t plan, cow, cow_old, partials, total, stats;
   // shared-prefix segments
   size_t seg_cover, seg_nseg, seg_owner, seg_i0, seg_len, seg_rep, seg_g, seg_mem_off, seg_fill, seg_members,
       seg_tile_seg, seg_tile_t, grec, seg_bid, seg_rec_off, seg_nrec, seg_splits, seg_tile_split, seg_hist, pair_cnt;
@@ -88,6 +94,7 @@ struct PoolView {
   unsigned* free_bits;
   int* plan;            // [2 modes][3][max_beams + 1]: offsets, chunk counts, start tokens
   int* cow;             // [kMaxCowJobs][3] (old page, new page, rows) of the open step's copy-on-writes
+  int* cow_old;         // [max_beams] the page a beam's tail page was copied from by the open step, or -1
   // Shared-prefix segments (rebuilt after seed, prune/branch and release):
   int grouped;          // 1 when the grouped tensor-core path exists for this pool's dtype/shape
   int group_min;        // segments need at least this many sharing beams
@@ -113,8 +120,8 @@ struct PoolView {
   float* grec;          // [max_beams][kMaxSegDepth][Hkv] grouped partial records
   int* stats;           // [kStatsRing][kStatsWords] work of recent steps (see gb_pool_read_step_stats)
   float* partials;
-  int* pair_cnt;        // [max_beams * Hkv] per-beam records written for each (beam, KV head) by the
-                        // running attention launch (zeroed by k_append before it)
+  int* pair_cnt;        // [2][max_beams * Hkv] per-beam records written for each (beam, KV head) by the
+                        // running attention launch, one array per counter set (Counters)
   int record_floats;
   float* mlp_scratch;   // [kMlpScratchFloats] K-split partials of the MLP scorer
 };
@@ -128,6 +135,29 @@ __host__ __device__ inline int* plan_n(const PoolView& v, int mode) {
 }
 __host__ __device__ inline int* plan_start(const PoolView& v, int mode) {
   return plan_off(v, mode) + 2 * (v.max_beams + 1);
+}
+
+// The counters of one attention launch (work queue, finished CTAs, records per pair).  There are
+// two sets: launch n of a pool uses set n & 1 and zeroes the other one, which launch n - 1 used
+// and launch n + 1 will, so no launch has to come between two attention launches to reset them.
+// n counts layers: steps opened so far x layers + layer, so consecutive launches alternate; a
+// layer appended without attention (k_append) zeroes both sets, and so does k_init.
+struct Counters {
+  int* c;     // words kCntGrpNext, kCntGrpDone, kCntPairNext
+  int* pair;  // [max_beams * Hkv]
+};
+__device__ __forceinline__ Counters counters(const PoolView& v, int set) {
+  return {v.ctl + kCtlCounters + kCntWords * set, v.pair_cnt + (size_t)set * v.max_beams * v.Hkv};
+}
+__device__ __forceinline__ int counter_set(const PoolView& v, int layer) {
+  return (v.ctl[kCtlSteps] * v.layers + layer) & 1;
+}
+// Zero set `set`, spread over the grid (`cta` of CTAs of this size).
+__device__ __forceinline__ void zero_counters(const PoolView& v, int set, int cta, int nctas) {
+  const Counters k = counters(v, set);
+  for (int i = cta * (int)blockDim.x + (int)threadIdx.x; i < v.max_beams * v.Hkv; i += nctas * (int)blockDim.x)
+    k.pair[i] = 0;
+  if (cta == 0 && threadIdx.x < kCntWords) k.c[threadIdx.x] = 0;
 }
 
 #ifndef GB_DECODE_WEIGHT
@@ -303,12 +333,16 @@ cudaError_t set_max_dynamic_smem(const void* kernel, int bytes);
 // The attention of one layer-step on s, written to out: mode 0, the per-beam kernel; mode 1,
 // the attention kernel with the grouped and per-beam roles (launch_attention).  The bf16
 // kernels merge their records themselves; the fp32 kernel is followed by k_combine.
-cudaError_t launch_decode(gb_pool* pool, int layer, const void* q, float scale, float* out, int mode,
-                          cudaStream_t s);
+// With k_new/v_new the launch also writes the step's new rows into the pool (fuses_append(pool));
+// without them k_append has written them before.
+cudaError_t launch_decode(gb_pool* pool, int layer, const void* q, const void* k_new, const void* v_new, float scale,
+                          float* out, int mode, cudaStream_t s);
+bool fuses_append(const gb_pool* pool);
 cudaError_t launch_decode_view(const PoolView& v, int W, int layer, const void* q, float scale, float* out,
                                cudaStream_t s);
 cudaError_t rebuild_segments(gb_pool* pool, cudaStream_t s);
-cudaError_t launch_attention(gb_pool* pool, int layer, const void* q, float scale, float* out, cudaStream_t s);
+cudaError_t launch_attention(gb_pool* pool, int layer, const void* q, const void* k_new, const void* v_new, float scale,
+                             float* out, cudaStream_t s);
 cudaError_t launch_wait_selftest(gb_pool* pool, cudaStream_t s);
 void make_kv_tensor_maps(gb_pool* pool);
 cudaError_t launch_probe(gb_pool* pool, const void* hidden, int hidden_dtype, int H, const float* w,

@@ -38,6 +38,7 @@ MetaLayout meta_layout(const gb_pool_config& c) {
   m.free_bits = take((size_t)m.words * sizeof(unsigned));
   m.plan = take(2 * 3 * (B + 1) * sizeof(int));
   m.cow = take(kMaxCowJobs * 3 * sizeof(int));
+  m.cow_old = take(B * sizeof(int));
   m.record_floats = G * (c.head_dim + 2);
   m.partial_records = kMaxDecodeWarps + (int)B * c.num_kv_heads;  // record index: warp + b * Hkv + h
   m.partials = take((size_t)m.partial_records * m.record_floats * sizeof(float));
@@ -61,7 +62,7 @@ MetaLayout meta_layout(const gb_pool_config& c) {
   m.seg_splits = take(BD * sizeof(int));
   m.seg_tile_split = take(B * kMaxSegRecords * sizeof(int));
   m.seg_hist = take(2 * 256 * sizeof(int));
-  m.pair_cnt = take(B * c.num_kv_heads * sizeof(int));
+  m.pair_cnt = take(2 * B * c.num_kv_heads * sizeof(int));
   m.stats = take((size_t)kStatsRing * kStatsWords * sizeof(int));
   m.mlp_scratch = take((size_t)kMlpScratchFloats * sizeof(float));
   m.total = o;
@@ -159,6 +160,7 @@ __global__ void k_init(PoolView v) {
     v.free_bits[w] = bits;
   }
   for (long long i = tid; i < (long long)v.max_beams * v.max_pages; i += stride) v.tables[i] = -1;
+  for (long long i = tid; i < 2LL * v.max_beams * v.Hkv; i += stride) v.pair_cnt[i] = 0;
   if (tid == 0) {
     for (int i = 0; i < kCtlWords; ++i) v.ctl[i] = 0;
     v.ctl[kCtlNextLineage] = 1;
@@ -325,8 +327,10 @@ __global__ void __launch_bounds__(1024) k_step_begin(PoolView v, int n_tokens, c
     }
     __syncthreads();
   }
-  // The rows [0, L % P) of each copied page are copied layer by layer by the append kernel.
+  // The rows [0, L % P) of each copied page are copied layer by layer by the kernel that writes
+  // the layer's new rows: the append kernel from the job list, the attention launch from cow_old.
   if (b == 0) v.ctl[kCtlCowJobs] = min(s_ncow, kMaxCowJobs);
+  if (b < v.max_beams) v.cow_old[b] = cow ? tail : -1;
 
   const int Lnew = act ? L + n_tokens : 0;
   if (act) {
@@ -380,15 +384,11 @@ __global__ void __launch_bounds__(1024) k_step_begin(PoolView v, int n_tokens, c
 __global__ void k_append(PoolView v, int layer, int n_tokens, const char* kin, const char* vin) {
   pdl_wait();
   pdl_launch_dependents();
-  // The counters of the attention launch that follows (combine.cuh, the grouped role's
-  // work queue): the previous attention launch has completed (pdl_wait).
+  // Both counter sets of the attention launches (Counters): the previous attention launch has
+  // completed (pdl_wait), and this layer's own, which would alternate them, does not come.
   if (blockIdx.x == 0 && blockIdx.y == 0) {
-    for (int i = threadIdx.x; i < v.max_beams * v.Hkv; i += blockDim.x) v.pair_cnt[i] = 0;
-    if (threadIdx.x == 0) {
-      v.ctl[kCtlGrpNext] = 0;
-      v.ctl[kCtlGrpDone] = 0;
-      v.ctl[kCtlPairNext] = 0;
-    }
+    zero_counters(v, 0, 0, 1);
+    zero_counters(v, 1, 0, 1);
   }
   if (v.ctl[kCtlStepOk] == 0) return;
   const int vec_per_row = v.D * v.esize / 16;
@@ -554,6 +554,7 @@ extern "C" gb_status gb_pool_init(const gb_pool_config* cfg, void* kv_dev, void*
   v.free_bits = reinterpret_cast<unsigned*>(m + L.free_bits);
   v.plan = reinterpret_cast<int*>(m + L.plan);
   v.cow = reinterpret_cast<int*>(m + L.cow);
+  v.cow_old = reinterpret_cast<int*>(m + L.cow_old);
   v.partials = reinterpret_cast<float*>(m + L.partials);
   v.record_floats = L.record_floats;
   v.seg_cover = reinterpret_cast<int*>(m + L.seg_cover);
@@ -643,9 +644,9 @@ extern "C" gb_status gb_pool_seed(gb_pool* pool, int n_beams, int prompt_len, co
   return GB_OK;
 }
 
-// Shared by gb_decode_attention and gb_append_kv: open the step at layer 0
-// and write the new rows of `layer`.
-static gb_status append_layer(gb_pool* pool, int layer, int n_tokens, const void* k, const void* v,
+// Shared by gb_decode_attention and gb_append_kv: open the step at layer 0 and write the new
+// rows of `layer`, unless the attention launch that follows writes them itself (`fused`).
+static gb_status append_layer(gb_pool* pool, int layer, int n_tokens, const void* k, const void* v, bool fused,
                               cudaStream_t s) {
   if (!pool->seeded) return fail(pool, GB_ERR_STATE, "pool not seeded");
   if (layer < 0 || layer >= pool->cfg.num_layers || n_tokens < 1 || !k || !v)
@@ -666,11 +667,13 @@ static gb_status append_layer(gb_pool* pool, int layer, int n_tokens, const void
   }
   const int per_tok = pool->cfg.max_beams * pool->cfg.num_kv_heads * (pool->view.D * pool->view.esize / 16);
   const dim3 grid(std::max(1, std::min((per_tok + 255) / 256, pool->num_sms * 8)), std::min(2 * n_tokens, 65535));
-  prof_begin(pool, GB_PROF_APPEND, s);
-  launch_pdl(k_append, grid, 256, 0, s, pool->view, layer, n_tokens, static_cast<const char*>(k),
-             static_cast<const char*>(v));
+  prof_begin(pool, GB_PROF_APPEND, s);  // an empty interval when the attention launch appends
+  if (!fused) {
+    launch_pdl(k_append, grid, 256, 0, s, pool->view, layer, n_tokens, static_cast<const char*>(k),
+               static_cast<const char*>(v));
+    pool->launches += 1;
+  }
   prof_end(pool, GB_PROF_APPEND, s);
-  pool->launches += 1;
   gb_status st = check_launch(pool, "append");
   if (st != GB_OK) return st;
   pool->next_layer = (layer + 1) % pool->cfg.num_layers;
@@ -680,7 +683,7 @@ static gb_status append_layer(gb_pool* pool, int layer, int n_tokens, const void
 extern "C" gb_status gb_append_kv(gb_pool* pool, int layer, int n_tokens, const void* k_dev,
                                   const void* v_dev, gb_stream_t stream) {
   if (!pool) return GB_ERR_INVALID;
-  return append_layer(pool, layer, n_tokens, k_dev, v_dev, reinterpret_cast<cudaStream_t>(stream));
+  return append_layer(pool, layer, n_tokens, k_dev, v_dev, false, reinterpret_cast<cudaStream_t>(stream));
 }
 
 extern "C" gb_status gb_decode_attention(gb_pool* pool, int layer, const void* q_dev,
@@ -690,7 +693,8 @@ extern "C" gb_status gb_decode_attention(gb_pool* pool, int layer, const void* q
   if (!q_dev || !out_dev) return fail(pool, GB_ERR_INVALID, "decode: null pointer");
   if (flags < GB_PATH_AUTO || flags > GB_PATH_GROUPED) return fail(pool, GB_ERR_INVALID, "decode: bad flags");
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  gb_status st = append_layer(pool, layer, 1, k_new_dev, v_new_dev, s);
+  const bool fused = fuses_append(pool);
+  gb_status st = append_layer(pool, layer, 1, k_new_dev, v_new_dev, fused, s);
   if (st != GB_OK) return st;
   // Mode 1: shared-prefix segments go through the grouped tensor-core kernel and the
   // per-beam kernel reads only each beam's remainder; mode 0: every beam reads everything.
@@ -698,7 +702,9 @@ extern "C" gb_status gb_decode_attention(gb_pool* pool, int layer, const void* q
   // shares of the SMs (decode_ctas), or one after the other on every SM.
   const int mode = (flags == GB_PATH_PER_BEAM || !pool->view.grouped) ? 0 : 1;
   prof_begin(pool, GB_PROF_ATTENTION, s);
-  if (launch_decode(pool, layer, q_dev, scale, out_dev, mode, s) != cudaSuccess) return check_launch(pool, "decode");
+  if (launch_decode(pool, layer, q_dev, fused ? k_new_dev : nullptr, fused ? v_new_dev : nullptr, scale, out_dev, mode,
+                    s) != cudaSuccess)
+    return check_launch(pool, "decode");
   return check_launch(pool, "decode");
 }
 
