@@ -55,9 +55,9 @@ typedef int gb_status;
 #define GB_BF16 1
 
 /* Decode path selection for gb_decode_attention(). */
-#define GB_PATH_AUTO 0      /* grouped tensor-core path where a shared segment is dense enough */
+#define GB_PATH_AUTO 0      /* grouped tensor-core path where a shared segment is dense enough and the step is not tiny */
 #define GB_PATH_PER_BEAM 1  /* every beam reads its whole context itself */
-#define GB_PATH_GROUPED 2   /* like AUTO (kept for explicit requests) */
+#define GB_PATH_GROUPED 2   /* like AUTO, but tiny steps take the grouped path too */
 
 typedef struct CUstream_st* gb_stream_t; /* identical to cudaStream_t */
 typedef struct gb_pool gb_pool;          /* opaque host handle */

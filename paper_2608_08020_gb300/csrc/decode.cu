@@ -26,6 +26,7 @@
 
 #include "decode_mma.cuh"
 #include "internal.cuh"
+#include "local.cuh"
 #include "ptx.cuh"
 
 namespace gb {
@@ -428,6 +429,10 @@ __global__ void __launch_bounds__(kMmaWarps * 32, 1)
   const int set = counter_set(v, layer);
   const Counters cnt = counters(v, set);
   zero_counters(v, set ^ 1, c, nctas);
+  if (local_step_per_beam(v, nctas)) {
+    local_attention<G>(v, &tm, &tmh, layer, q, nw, qscale, c, nctas, out);
+    return;
+  }
   decode_mma_body<G>(v, cnt, &tm, &tmh, layer, q, nw, qscale, mode, c, nctas);
   combine_pairs<G>(v, cnt, mode, nctas * kMmaWarps, 0, false, c, nctas, out);
 }
@@ -520,14 +525,14 @@ __global__ void __launch_bounds__(128) k_combine(PoolView v, int mode, int W, fl
 
 template <int DT, int G>
 static cudaError_t launch_decode_t(gb_pool* pool, int layer, const void* q, const void* k_new, const void* v_new,
-                                   float scale, float* out, int mode, cudaStream_t s) {
+                                   float scale, float* out, int mode, bool allow_local, cudaStream_t s) {
   using S = DecodeSmem<DT, G>;
   const float qscale = scale * 1.4426950408889634f;  // log2(e): softmax in base 2
   cudaError_t e;
   if (fuses_append(pool)) {
     // One launch: the new rows, the attention roles and the merge of their records.
     if (mode == 1) {
-      e = launch_attention(pool, layer, q, k_new, v_new, scale, out, s);  // grouped and per-beam roles (grouped.cu)
+      e = launch_attention(pool, layer, q, k_new, v_new, scale, out, allow_local, s);  // grouped and per-beam roles (grouped.cu)
     } else {
       e = set_max_dynamic_smem(reinterpret_cast<const void*>(k_decode_mma<G>), DecodeMmaSmem::TOTAL);
       if (e != cudaSuccess) return e;
@@ -616,19 +621,19 @@ bool fuses_append(const gb_pool* pool) {
 }
 
 cudaError_t launch_decode(gb_pool* pool, int layer, const void* q, const void* k_new, const void* v_new, float scale,
-                          float* out, int mode, cudaStream_t s) {
+                          float* out, int mode, bool allow_local, cudaStream_t s) {
   const int G = pool->view.G;
   if (pool->view.dtype == GB_BF16) {
     switch (G) {
-      case 2: return launch_decode_t<GB_BF16, 2>(pool, layer, q, k_new, v_new, scale, out, mode, s);
-      case 4: return launch_decode_t<GB_BF16, 4>(pool, layer, q, k_new, v_new, scale, out, mode, s);
-      case 8: return launch_decode_t<GB_BF16, 8>(pool, layer, q, k_new, v_new, scale, out, mode, s);
+      case 2: return launch_decode_t<GB_BF16, 2>(pool, layer, q, k_new, v_new, scale, out, mode, allow_local, s);
+      case 4: return launch_decode_t<GB_BF16, 4>(pool, layer, q, k_new, v_new, scale, out, mode, allow_local, s);
+      case 8: return launch_decode_t<GB_BF16, 8>(pool, layer, q, k_new, v_new, scale, out, mode, allow_local, s);
     }
   } else {
     switch (G) {
-      case 2: return launch_decode_t<GB_F32, 2>(pool, layer, q, k_new, v_new, scale, out, mode, s);
-      case 4: return launch_decode_t<GB_F32, 4>(pool, layer, q, k_new, v_new, scale, out, mode, s);
-      case 8: return launch_decode_t<GB_F32, 8>(pool, layer, q, k_new, v_new, scale, out, mode, s);
+      case 2: return launch_decode_t<GB_F32, 2>(pool, layer, q, k_new, v_new, scale, out, mode, allow_local, s);
+      case 4: return launch_decode_t<GB_F32, 4>(pool, layer, q, k_new, v_new, scale, out, mode, allow_local, s);
+      case 8: return launch_decode_t<GB_F32, 8>(pool, layer, q, k_new, v_new, scale, out, mode, allow_local, s);
     }
   }
   return cudaErrorInvalidValue;

@@ -114,6 +114,141 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   return *reinterpret_cast<const uint32_t*>(&t);
 }
 
+// Softmax state of one (beam, head) pair in a warp: Q^T fragments (heads r < G, dims 16j + 2c (+1)
+// and 16j + 8 + 2c (+1)), O^T fragments (dims 16mt + r (+8), heads 2c, 2c + 1), and the running
+// max and this lane's share of the sum of heads 2c and 2c + 1.
+struct PairState {
+  uint32_t qf[8][2];
+  float o[8][4];
+  float m0, m1, l0, l1;
+};
+
+// Start pair (b, h): its query rows, an empty softmax.
+template <int G>
+__device__ __forceinline__ void pair_begin(PairState& st, const PoolView& v, const __nv_bfloat16* __restrict__ q, int b,
+                                           int h, int r, int c) {
+  const uint32_t* qrow = reinterpret_cast<const uint32_t*>(q + ((size_t)b * v.Hq + h * G + r) * 128);
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    st.qf[j][0] = r < G ? qrow[8 * j + c] : 0u;
+    st.qf[j][1] = r < G ? qrow[8 * j + 4 + c] : 0u;
+  }
+#pragma unroll
+  for (int mt = 0; mt < 8; ++mt) st.o[mt][0] = st.o[mt][1] = st.o[mt][2] = st.o[mt][3] = 0.f;
+  st.m0 = st.m1 = -INFINITY;
+  st.l0 = st.l1 = 0.f;
+}
+
+// ldmatrix row addresses of a lane (lane = 8 * matrix + row).  K, non-transposed, for
+// S^T's A operand: matrix bit 0 picks the token half, bit 1 the 8-dim half of the
+// k-step.  V, transposed, for O^T's A operand: bit 0 picks the 8-dim half of the m-tile,
+// bit 1 the token half.  The 16-byte piece x of row y of a 1 KiB block sits at x ^ y.
+__device__ __forceinline__ void ldsm_offsets(uint32_t (&koff)[4], uint32_t (&voff)[4], int lane) {
+  const int mi = lane >> 3, y = lane & 7;
+#pragma unroll
+  for (int jj = 0; jj < 4; ++jj) {
+    koff[jj] = (mi & 1) * 4096 + y * 128 + (((2 * jj + (mi >> 1)) ^ y) << 4);
+    voff[jj] = (mi >> 1) * 4096 + 2048 + y * 128 + (((2 * jj + (mi & 1)) ^ y) << 4);
+  }
+}
+
+// One landed 16-token chunk (stage address sb, its first nvalid >= 1 tokens) into the pair's state.
+__device__ __forceinline__ void chunk_attend(PairState& st, uint32_t sb, const uint32_t (&koff)[4],
+                                             const uint32_t (&voff)[4], int nvalid, float qscale, int r) {
+  // ---- S^T = K . Q^T (kMmaChains independent accumulator chains) -----------
+  float sacc[kMmaChains][4];
+#pragma unroll
+  for (int ch = 0; ch < kMmaChains; ++ch) sacc[ch][0] = sacc[ch][1] = sacc[ch][2] = sacc[ch][3] = 0.f;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    uint32_t a0, a1, a2, a3;
+    ldsm_x4(sb + koff[j & 3] + (j >> 2) * 1024, a0, a1, a2, a3);
+    mma_bf16(sacc[j % kMmaChains], a0, a1, a2, a3, st.qf[j][0], st.qf[j][1]);
+  }
+  float sc[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    float t = sacc[0][e];
+#pragma unroll
+    for (int ch = 1; ch < kMmaChains; ++ch) t += sacc[ch][e];
+    sc[e] = t * qscale;
+  }
+  if (nvalid < kChunk) {
+    // Tokens past the beam's length: no score.
+    if (r >= nvalid) sc[0] = sc[1] = -INFINITY;
+    if (r + 8 >= nvalid) sc[2] = sc[3] = -INFINITY;
+  }
+  // ---- online softmax over the chunk's 16 tokens (per head column) ----------
+  float mx0 = fmaxf(sc[0], sc[2]), mx1 = fmaxf(sc[1], sc[3]);
+#pragma unroll
+  for (int sh = 4; sh < 32; sh <<= 1) {
+    mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, sh));
+    mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, sh));
+  }
+  const bool up0 = mx0 > st.m0 + 8.f, up1 = mx1 > st.m1 + 8.f;
+  if (__any_sync(0xffffffffu, up0 || up1)) {
+    const float al0 = up0 ? ex2_approx(st.m0 - mx0) : 1.f;
+    const float al1 = up1 ? ex2_approx(st.m1 - mx1) : 1.f;
+    if (up0) st.m0 = mx0;
+    if (up1) st.m1 = mx1;
+#pragma unroll
+    for (int mt = 0; mt < 8; ++mt) {
+      st.o[mt][0] *= al0;
+      st.o[mt][1] *= al1;
+      st.o[mt][2] *= al0;
+      st.o[mt][3] *= al1;
+    }
+    st.l0 *= al0;
+    st.l1 *= al1;
+  }
+  const float p0 = ex2_approx(sc[0] - st.m0), p1 = ex2_approx(sc[1] - st.m1);
+  const float p2 = ex2_approx(sc[2] - st.m0), p3 = ex2_approx(sc[3] - st.m1);
+  st.l0 += p0 + p2;
+  st.l1 += p1 + p3;
+  const uint32_t pb0 = movmatrix_t(pack_bf16x2(p0, p1));  // P^T fragments: tokens 2c (+1), head r
+  const uint32_t pb1 = movmatrix_t(pack_bf16x2(p2, p3));  // tokens 8 + 2c (+1)
+  // ---- O^T += V^T . P^T ------------------------------------------------------
+#pragma unroll
+  for (int mt = 0; mt < 8; ++mt) {
+    uint32_t a0, a1, a2, a3;
+    ldsm_x4_t(sb + voff[mt & 3] + (mt >> 2) * 1024, a0, a1, a2, a3);
+    mma_bf16(st.o[mt], a0, a1, a2, a3, pb0, pb1);
+  }
+}
+
+// The last chunk of a pair holds the step's new token: put its row into the landed stage `vs` and
+// into the pool (page npage), and zero the V rows past it (the page's rows there hold whatever the
+// pool held), so that 0 * V stays 0 in the MMA.  nrow: 16 bytes of the row, lanes 0-15 K, 16-31 V.
+__device__ __forceinline__ void chunk_append(const PoolView& v, int layer, int h, int L, int nvalid, const uint4& nrow,
+                                             int npage, unsigned char* vs, int lane) {
+  const int t = nvalid - 1, kv = lane >> 4, piece = lane & 15;
+  *reinterpret_cast<uint4*>(vs + (t >> 3) * 4096 + kv * 2048 + (piece >> 3) * 1024 + (t & 7) * 128 +
+                            (((piece & 7) ^ (t & 7)) << 4)) = nrow;
+  for (int idx = lane; idx < (kChunk - nvalid) * 16; idx += 32) {
+    const int tz = nvalid + (idx >> 4), pz = idx & 15;
+    *reinterpret_cast<uint4*>(vs + (tz >> 3) * 4096 + 2048 + (pz >> 3) * 1024 + (tz & 7) * 128 + (pz & 7) * 16) =
+        make_uint4(0u, 0u, 0u, 0u);
+  }
+  if (npage >= 0 && npage < v.num_pages)
+    reinterpret_cast<uint4*>(v.kv + kv_elem_offset(v, layer, npage, kv, h, (L - 1) % v.P) * 2)[piece] = nrow;
+  else if (lane == 0)
+    set_status(v.ctl, GB_ERR_INVALID);
+  fence_proxy_async_smem();  // ordered before the TMA that later refills this stage
+  __syncwarp();
+}
+
+// A chunk of a tail page copied on write: its rows before the new one go to the new page.
+__device__ __forceinline__ void chunk_copied(const PoolView& v, int layer, int b, int h, int L, int tok0,
+                                             const unsigned char* vs, int lane) {
+  const int page = v.tables[(size_t)b * v.max_pages + (L - 1) / v.P];
+  if (page < 0 || page >= v.num_pages) return;
+  const int rows = min(kChunk, L - 1 - tok0), kv = lane >> 4, piece = lane & 15;
+  for (int t = 0; t < rows; ++t)
+    reinterpret_cast<uint4*>(v.kv + kv_elem_offset(v, layer, page, kv, h, (tok0 + t) % v.P) * 2)[piece] =
+        *reinterpret_cast<const uint4*>(vs + (t >> 3) * 4096 + kv * 2048 + (piece >> 3) * 1024 + (t & 7) * 128 +
+                                        (((piece & 7) ^ (t & 7)) << 4));
+}
+
 // The new K/V rows of the step, [max_beams][Hkv][128] bf16 each (16 uint4 per row).
 struct NewRows {
   const uint4* k;
@@ -244,23 +379,10 @@ __device__ __forceinline__ void decode_mma_body(const PoolView& v, const Counter
     }
   }
 
-  // ldmatrix row addresses of this lane (lane = 8 * matrix + row).  K, non-transposed, for
-  // S^T's A operand: matrix bit 0 picks the token half, bit 1 the 8-dim half of the
-  // k-step.  V, transposed, for O^T's A operand: bit 0 picks the 8-dim half of the m-tile,
-  // bit 1 the token half.  The 16-byte piece x of row y of a 1 KiB block sits at x ^ y.
   uint32_t koff[4], voff[4];
-  {
-    const int mi = lane >> 3, y = lane & 7;
-#pragma unroll
-    for (int jj = 0; jj < 4; ++jj) {
-      koff[jj] = (mi & 1) * 4096 + y * 128 + (((2 * jj + (mi >> 1)) ^ y) << 4);
-      voff[jj] = (mi >> 1) * 4096 + 2048 + y * 128 + (((2 * jj + (mi & 1)) ^ y) << 4);
-    }
-  }
+  ldsm_offsets(koff, voff, lane);
 
-  uint32_t qf[8][2];  // Q^T fragments: heads r < G, dims 16j + 2c (+1) and 16j + 8 + 2c (+1)
-  float o[8][4];      // O^T fragments: dims 16mt + r (+8), heads 2c, 2c + 1
-  float m0 = -INFINITY, m1 = -INFINITY, l0 = 0.f, l1 = 0.f;
+  PairState st;
   int L = 0;
   bool fresh = true;
   uint4 nrow = make_uint4(0u, 0u, 0u, 0u);  // 16 bytes of the pair's new rows: lanes 0-15 K, 16-31 V
@@ -275,16 +397,7 @@ __device__ __forceinline__ void decode_mma_body(const PoolView& v, const Counter
         nrow = (lane < 16 ? nw.k : nw.v)[((size_t)it.b * v.Hkv + it.h) * 16 + (lane & 15)];
         npage = v.tables[(size_t)it.b * v.max_pages + (L - 1) / v.P];
       }
-      const uint32_t* qrow = reinterpret_cast<const uint32_t*>(q + ((size_t)it.b * v.Hq + it.h * G + r) * D);
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        qf[j][0] = r < G ? qrow[8 * j + c] : 0u;
-        qf[j][1] = r < G ? qrow[8 * j + 4 + c] : 0u;
-      }
-#pragma unroll
-      for (int mt = 0; mt < 8; ++mt) o[mt][0] = o[mt][1] = o[mt][2] = o[mt][3] = 0.f;
-      m0 = m1 = -INFINITY;
-      l0 = l1 = 0.f;
+      pair_begin<G>(st, v, q, it.b, it.h, r, c);
       fresh = false;
     }
     if (!mbar_wait_bounded(bar0 + 8 * stage, parity, kWaitLimitNs)) {
@@ -298,100 +411,10 @@ __device__ __forceinline__ void decode_mma_body(const PoolView& v, const Counter
     const uint32_t sb = stage0 + stage * kMmaStageBytes;
     const int tok0 = it.tok0 + it.i * kChunk;
     const int nvalid = min(kChunk, L - tok0);  // >= 1: a chunk starts before the beam's length
-    if (it.i == it.n - 1) {
-      // The new token, and zeros for the V rows past it (the page's rows there hold whatever the
-      // pool held), so that 0 * V stays 0 in the MMA.
-      unsigned char* vs = smem + (sb - smem_addr(smem));
-      const int t = nvalid - 1, kv = lane >> 4, piece = lane & 15;
-      const bool page_ok = npage >= 0 && npage < v.num_pages;
-      *reinterpret_cast<uint4*>(vs + (t >> 3) * 4096 + kv * 2048 + (piece >> 3) * 1024 + (t & 7) * 128 +
-                                (((piece & 7) ^ (t & 7)) << 4)) = nrow;
-      for (int idx = lane; idx < (kChunk - nvalid) * 16; idx += 32) {
-        const int tz = nvalid + (idx >> 4), pz = idx & 15;
-        *reinterpret_cast<uint4*>(vs + (tz >> 3) * 4096 + 2048 + (pz >> 3) * 1024 + (tz & 7) * 128 + (pz & 7) * 16) =
-            make_uint4(0u, 0u, 0u, 0u);
-      }
-      if (page_ok)
-        reinterpret_cast<uint4*>(v.kv + kv_elem_offset(v, layer, npage, kv, it.h, (L - 1) % v.P) * 2)[piece] = nrow;
-      else if (lane == 0)
-        set_status(v.ctl, GB_ERR_INVALID);
-      fence_proxy_async_smem();  // ordered before the TMA that later refills this stage
-      __syncwarp();
-    }
-    if (s_cow[it.b] >= 0 && tok0 / v.P == (L - 1) / v.P) {
-      // A chunk of a tail page copied on write: its rows before the new one go to the new page.
-      const int page = v.tables[(size_t)it.b * v.max_pages + (L - 1) / v.P];
-      if (page >= 0 && page < v.num_pages) {
-        const unsigned char* vs = smem + (sb - smem_addr(smem));
-        const int rows = min(kChunk, L - 1 - tok0);
-        for (int idx = lane; idx < rows * 32; idx += 32) {
-          const int t = idx >> 5, kv = lane >> 4, piece = lane & 15;
-          reinterpret_cast<uint4*>(v.kv + kv_elem_offset(v, layer, page, kv, it.h, (tok0 + t) % v.P) * 2)[piece] =
-              *reinterpret_cast<const uint4*>(vs + (t >> 3) * 4096 + kv * 2048 + (piece >> 3) * 1024 + (t & 7) * 128 +
-                                              (((piece & 7) ^ (t & 7)) << 4));
-        }
-      }
-    }
-
-    // ---- S^T = K . Q^T (kMmaChains independent accumulator chains) -----------
-    float sacc[kMmaChains][4];
-#pragma unroll
-    for (int ch = 0; ch < kMmaChains; ++ch) sacc[ch][0] = sacc[ch][1] = sacc[ch][2] = sacc[ch][3] = 0.f;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      uint32_t a0, a1, a2, a3;
-      ldsm_x4(sb + koff[j & 3] + (j >> 2) * 1024, a0, a1, a2, a3);
-      mma_bf16(sacc[j % kMmaChains], a0, a1, a2, a3, qf[j][0], qf[j][1]);
-    }
-    float sc[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      float t = sacc[0][e];
-#pragma unroll
-      for (int ch = 1; ch < kMmaChains; ++ch) t += sacc[ch][e];
-      sc[e] = t * qscale;
-    }
-    if (nvalid < kChunk) {
-      // Tokens past the beam's length: no score.
-      if (r >= nvalid) sc[0] = sc[1] = -INFINITY;
-      if (r + 8 >= nvalid) sc[2] = sc[3] = -INFINITY;
-    }
-    // ---- online softmax over the chunk's 16 tokens (per head column) ----------
-    float mx0 = fmaxf(sc[0], sc[2]), mx1 = fmaxf(sc[1], sc[3]);
-#pragma unroll
-    for (int sh = 4; sh < 32; sh <<= 1) {
-      mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, sh));
-      mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, sh));
-    }
-    const bool up0 = mx0 > m0 + 8.f, up1 = mx1 > m1 + 8.f;
-    if (__any_sync(0xffffffffu, up0 || up1)) {
-      const float al0 = up0 ? ex2_approx(m0 - mx0) : 1.f;
-      const float al1 = up1 ? ex2_approx(m1 - mx1) : 1.f;
-      if (up0) m0 = mx0;
-      if (up1) m1 = mx1;
-#pragma unroll
-      for (int mt = 0; mt < 8; ++mt) {
-        o[mt][0] *= al0;
-        o[mt][1] *= al1;
-        o[mt][2] *= al0;
-        o[mt][3] *= al1;
-      }
-      l0 *= al0;
-      l1 *= al1;
-    }
-    const float p0 = ex2_approx(sc[0] - m0), p1 = ex2_approx(sc[1] - m1);
-    const float p2 = ex2_approx(sc[2] - m0), p3 = ex2_approx(sc[3] - m1);
-    l0 += p0 + p2;
-    l1 += p1 + p3;
-    const uint32_t pb0 = movmatrix_t(pack_bf16x2(p0, p1));  // P^T fragments: tokens 2c (+1), head r
-    const uint32_t pb1 = movmatrix_t(pack_bf16x2(p2, p3));  // tokens 8 + 2c (+1)
-    // ---- O^T += V^T . P^T ------------------------------------------------------
-#pragma unroll
-    for (int mt = 0; mt < 8; ++mt) {
-      uint32_t a0, a1, a2, a3;
-      ldsm_x4_t(sb + voff[mt & 3] + (mt >> 2) * 1024, a0, a1, a2, a3);
-      mma_bf16(o[mt], a0, a1, a2, a3, pb0, pb1);
-    }
+    unsigned char* vs = smem + (sb - smem_addr(smem));
+    if (it.i == it.n - 1) chunk_append(v, layer, it.h, L, nvalid, nrow, npage, vs, lane);
+    if (s_cow[it.b] >= 0 && tok0 / v.P == (L - 1) / v.P) chunk_copied(v, layer, it.b, it.h, L, tok0, vs, lane);
+    chunk_attend(st, sb, koff, voff, nvalid, qscale, r);
     __syncwarp();
     if (ip_x < x_end) {
       if (lane == 0) fence_proxy_async_smem();
@@ -410,8 +433,8 @@ __device__ __forceinline__ void decode_mma_body(const PoolView& v, const Counter
     if (last_of_bh) {
 #pragma unroll
       for (int sh = 4; sh < 32; sh <<= 1) {
-        l0 += __shfl_xor_sync(0xffffffffu, l0, sh);
-        l1 += __shfl_xor_sync(0xffffffffu, l1, sh);
+        st.l0 += __shfl_xor_sync(0xffffffffu, st.l0, sh);
+        st.l1 += __shfl_xor_sync(0xffffffffu, st.l1, sh);
       }
       float* rec = v.partials + (size_t)(w + it.b * v.Hkv + it.h) * v.record_floats;
       if (2 * c < G) {
@@ -420,16 +443,16 @@ __device__ __forceinline__ void decode_mma_body(const PoolView& v, const Counter
         const uint64_t rpol = policy_evict_last();  // the merge reads the record back from L2
 #pragma unroll
         for (int mt = 0; mt < 8; ++mt) {
-          st_hint(o0 + 16 * mt, o[mt][0], rpol);
-          st_hint(o1 + 16 * mt, o[mt][1], rpol);
-          st_hint(o0 + 16 * mt + 8, o[mt][2], rpol);
-          st_hint(o1 + 16 * mt + 8, o[mt][3], rpol);
+          st_hint(o0 + 16 * mt, st.o[mt][0], rpol);
+          st_hint(o1 + 16 * mt, st.o[mt][1], rpol);
+          st_hint(o0 + 16 * mt + 8, st.o[mt][2], rpol);
+          st_hint(o1 + 16 * mt + 8, st.o[mt][3], rpol);
         }
         if (r == 0) {
-          st_hint(rec + G * D + 2 * c, m0, rpol);
-          st_hint(rec + G * D + 2 * c + 1, m1, rpol);
-          st_hint(rec + G * D + G + 2 * c, l0, rpol);
-          st_hint(rec + G * D + G + 2 * c + 1, l1, rpol);
+          st_hint(rec + G * D + 2 * c, st.m0, rpol);
+          st_hint(rec + G * D + 2 * c + 1, st.m1, rpol);
+          st_hint(rec + G * D + G + 2 * c, st.l0, rpol);
+          st_hint(rec + G * D + G + 2 * c + 1, st.l1, rpol);
         }
       }
       record_arrive(cnt, it.b * v.Hkv + it.h, lane);

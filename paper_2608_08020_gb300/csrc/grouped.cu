@@ -58,6 +58,7 @@
 
 #include "decode_mma.cuh"
 #include "internal.cuh"
+#include "local.cuh"
 #include "ptx.cuh"
 #include "tc.cuh"
 
@@ -698,14 +699,15 @@ template <int G>
 __global__ void __launch_bounds__(kAttnThreads, 1)
     k_attention(PoolView v, const __grid_constant__ CUtensorMap tmg, const __grid_constant__ CUtensorMap tmd,
                 const __grid_constant__ CUtensorMap tmdh, int layer, const __nv_bfloat16* __restrict__ q, NewRows nw,
-                float qscale, int w_oob, float* __restrict__ out) {
+                float qscale, int w_oob, bool allow_local, float* __restrict__ out) {
   pdl_wait();
   pdl_launch_dependents();
   // Grid of 2 S CTAs (S = SM count).  Large steps: CTAs [0, S) take the grouped role and
   // leave, CTAs [S, 2S) the per-beam role, each on an SM as a grouped CTA leaves it (CTAs
   // start in index order), and merge the records; a grouped CTA never waits, so every
-  // per-beam CTA gets an SM.  Small steps: [0, ng) grouped and [ng, S) per-beam side by side,
-  // all S resident at once, all S merging; the rest leave at once.
+  // per-beam CTA gets an SM.  Smaller steps (decode_ctas): [0, ng) grouped and [ng, S) per-beam side by side,
+  // all S resident at once, all S merging; the rest leave at once.  The smallest steps run
+  // without either role (local.cuh).
   const int S = (int)gridDim.x / 2, c = (int)blockIdx.x;
   if (v.ctl[kCtlStepOk] == 0) {
     zero_all_pairs<G>(v, c, 2 * S, out);
@@ -714,6 +716,10 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   const int set = counter_set(v, layer);
   const Counters cnt = counters(v, set);
   zero_counters(v, set ^ 1, c, 2 * S);
+  if (allow_local && local_step(v, S)) {
+    if (c < S) local_attention<G>(v, &tmd, &tmdh, layer, q, nw, qscale, c, S, out);
+    return;
+  }
   const int nd = decode_ctas(v, S), ng = nd < S ? S - nd : S;
   const bool split = nd < S;
   const int pb0 = split ? ng : S;  // first per-beam CTA
@@ -782,7 +788,7 @@ void make_kv_tensor_maps(gb_pool* pool) {
 
 template <int G>
 static cudaError_t launch_attention_t(gb_pool* pool, int layer, const void* q, const NewRows& nw, float scale,
-                                      float* out, cudaStream_t s) {
+                                      float* out, bool allow_local, cudaStream_t s) {
   {
     const cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(k_attention<G>), kAttnSmem);
     if (e != cudaSuccess) return e;
@@ -795,7 +801,7 @@ static cudaError_t launch_attention_t(gb_pool* pool, int layer, const void* q, c
                                    *reinterpret_cast<const CUtensorMap*>(pool->tmap),
                                    *reinterpret_cast<const CUtensorMap*>(pool->dtmap),
                                    *reinterpret_cast<const CUtensorMap*>(pool->dtmap_half), layer,
-                                   static_cast<const __nv_bfloat16*>(q), nw, qscale, pool->tmap_oob, out);
+                                   static_cast<const __nv_bfloat16*>(q), nw, qscale, pool->tmap_oob, allow_local, out);
   prof_end(pool, GB_PROF_DECODE, s);
   prof_end(pool, GB_PROF_GROUPED, s);
   pool->launches += 1;
@@ -803,12 +809,12 @@ static cudaError_t launch_attention_t(gb_pool* pool, int layer, const void* q, c
 }
 
 cudaError_t launch_attention(gb_pool* pool, int layer, const void* q, const void* k_new, const void* v_new, float scale,
-                             float* out, cudaStream_t s) {
+                             float* out, bool allow_local, cudaStream_t s) {
   const NewRows nw{static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new)};
   switch (pool->view.G) {
-    case 2: return launch_attention_t<2>(pool, layer, q, nw, scale, out, s);
-    case 4: return launch_attention_t<4>(pool, layer, q, nw, scale, out, s);
-    case 8: return launch_attention_t<8>(pool, layer, q, nw, scale, out, s);
+    case 2: return launch_attention_t<2>(pool, layer, q, nw, scale, out, allow_local, s);
+    case 4: return launch_attention_t<4>(pool, layer, q, nw, scale, out, allow_local, s);
+    case 8: return launch_attention_t<8>(pool, layer, q, nw, scale, out, allow_local, s);
   }
   return cudaErrorInvalidValue;
 }

@@ -336,13 +336,13 @@ cudaError_t set_max_dynamic_smem(const void* kernel, int bytes);
 // With k_new/v_new the launch also writes the step's new rows into the pool (fuses_append(pool));
 // without them k_append has written them before.
 cudaError_t launch_decode(gb_pool* pool, int layer, const void* q, const void* k_new, const void* v_new, float scale,
-                          float* out, int mode, cudaStream_t s);
+                          float* out, int mode, bool allow_local, cudaStream_t s);
 bool fuses_append(const gb_pool* pool);
 cudaError_t launch_decode_view(const PoolView& v, int W, int layer, const void* q, float scale, float* out,
                                cudaStream_t s);
 cudaError_t rebuild_segments(gb_pool* pool, cudaStream_t s);
 cudaError_t launch_attention(gb_pool* pool, int layer, const void* q, const void* k_new, const void* v_new, float scale,
-                             float* out, cudaStream_t s);
+                             float* out, bool allow_local, cudaStream_t s);
 cudaError_t launch_wait_selftest(gb_pool* pool, cudaStream_t s);
 void make_kv_tensor_maps(gb_pool* pool);
 cudaError_t launch_probe(gb_pool* pool, const void* hidden, int hidden_dtype, int H, const float* w,

@@ -1,0 +1,239 @@
+// The attention of a small step, merged inside each CTA.
+//
+// When a step's whole per-beam work is a few chunks per warp of the GPU, reading it is not what
+// takes the time: the grouped role's set-up, the partial records in global memory and the waits of
+// their merge are (a layer-step of 13 beams x 340 tokens took 21 us for 10 MB).  Here a team of
+// w = 1, 2, 3, 4, 6 or 12 warps of one CTA takes a (beam, KV head) pair at a time, splits the beam's
+// whole context (shared pages included: they come from L2) into w runs of chunks, and merges the
+// warps' softmax states through shared memory: no records, no counters, no waits between CTAs.
+// The arithmetic of a chunk is the per-beam role's (decode_mma.cuh).
+#pragma once
+#include "decode_mma.cuh"
+
+namespace gb {
+
+#ifndef GB_LOCAL_SCALE
+#define GB_LOCAL_SCALE 1  // for sweeps of the rule below
+#endif
+
+// Whether local_attention on `nctas` CTAs beats the two roles.  It takes about 8 us + 1.0 us per
+// chunk and warp; the roles take 35-40 us at least with their merge, the time of their bytes above
+// that, and about 3 us per grouped unit and SM.  Measured per layer-step, local / roles (us):
+// 3.5 chunks per warp 11.5 / 28 (32 beams x 400), 17.7: 25.6 / 40 (64 x 1000), 26: 34 / 40
+// (64 x 1500), 28.5: 41 / 60 (13 x 8000, G = 8); from there on it depends on what sharing saves:
+// 35: 43 / 45.5 and 47 / 53.5 with 2-2.6 times the roles' reads, 40: 46 / 50 (2.9 times), 53: 68 / 64
+// (2.4 times), 56: 62 / 53 (4.8 times), 70: 72 / 45 (prompt of 3500 of 4000 tokens); and many small
+// segments cost the grouped role more: 56: 68 / 87 (9.5 units per SM), 74 / 158 (18 units).
+__device__ __forceinline__ bool local_step(const PoolView& v, int nctas) {
+  const long long all = plan_off(v, 0)[v.max_beams];  // (beam, head, chunk) units of the whole contexts
+  const long long roles = plan_off(v, 1)[v.max_beams] + (long long)v.ctl[kCtlSegTileTok] * v.Hkv / kChunk;
+  const long long units = (long long)v.ctl[kCtlSegTiles] * v.Hkv - 3 * nctas;  // grouped units above 3 per SM
+  const long long w = (long long)kMmaWarps * nctas;
+  return all <= GB_LOCAL_SCALE * (w * (all <= 3 * roles ? 44 : 28) + (units > 0 ? 4 * kMmaWarps * units : 0));
+}
+
+// The same for the per-beam path, whose other form splits the whole contexts evenly over all warps
+// of the GPU.
+__device__ __forceinline__ bool local_step_per_beam(const PoolView& v, int nctas) {
+  return plan_off(v, 0)[v.max_beams] <= GB_LOCAL_SCALE * 44ll * kMmaWarps * nctas;
+}
+
+// Warps per team: the number that minimises rounds of pairs x (chunks per warp + what a pair
+// costs beside its chunks: page ids, query rows and the first load, then the merge of a team).
+__device__ __forceinline__ int local_team(int npairs, int chunks_per_pair, int nctas) {
+  const int ws[6] = {1, 2, 3, 4, 6, 12};
+  int best = 1, best_cost = 0x7fffffff;
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    const int w = ws[i], teams = nctas * (kMmaWarps / w);
+    const int cost = (npairs + teams - 1) / teams * ((chunks_per_pair + w - 1) / w + 3 + (w > 1 ? 1 : 0));
+    if (cost < best_cost) {
+      best = w;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
+static_assert(kMmaWarps == 12, "team sizes divide the CTA's warps");
+
+__device__ __forceinline__ void team_sync(int team, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(threads) : "memory");
+}
+
+// All pairs of the pool, CTA `cta` of `nctas`; kMmaWarps * 32 threads.  Shared memory: the warps'
+// stages and barriers as in decode_mma_body; a warp's record for its team's merge lies over its
+// own stages, which are idle by then.
+template <int G>
+__device__ __forceinline__ void local_attention(const PoolView& v, const CUtensorMap* tm_p, const CUtensorMap* tmh_p,
+                                                int layer, const __nv_bfloat16* __restrict__ q, const NewRows& nw,
+                                                float qscale, int cta, int nctas, float* __restrict__ out) {
+  using S = DecodeMmaSmem;
+  constexpr int HS = 132;  // floats per head of a record: 128 and a pad, so that the stores below
+                           // (4 head pairs x 8 rows) fall on 32 banks
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* smem = smem_raw + ((1024 - (smem_addr(smem_raw) & 1023)) & 1023);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int r = lane >> 2, c = lane & 3;
+  const uint32_t stage0 = smem_addr(smem) + warp * kMmaStages * kMmaStageBytes;
+  const uint32_t bar0 = smem_addr(smem) + S::STAGES + warp * kMmaStages * 8;
+  static_assert((G * HS + 2 * G) * 4 <= kMmaStages * kMmaStageBytes, "a record fits the warp's stages");
+
+  const int npairs = v.max_beams * v.Hkv;
+  const int w = local_team(npairs, (plan_off(v, 0)[v.max_beams] + npairs - 1) / npairs, nctas);
+  const int tpc = kMmaWarps / w, team = warp / w, wi = warp - team * w;
+
+  if (lane == 0) {
+    for (int s = 0; s < kMmaStages; ++s) mbar_init(bar0 + 8 * s, 1);
+    fence_mbar_init();
+  }
+  __syncwarp();
+  uint32_t koff[4], voff[4];
+  ldsm_offsets(koff, voff, lane);
+  const uint64_t pol = policy_evict_normal();  // siblings read the shared pages again
+  const int pg8 = v.P >> 3, layer_pages = layer * v.num_pages;
+  int stage = 0;
+  uint32_t parity = 0;
+  bool alive = true;  // false once a wait ran out: no more loads, the pairs' outputs are zero
+
+  for (int p = cta + nctas * team; p < npairs; p += nctas * tpc) {
+    const int b = p / v.Hkv, h = p - b * v.Hkv;
+    const int n = plan_n(v, 0)[b], L = v.seq_len[b], old = v.cow_old[b];
+    float* ob = out + ((size_t)b * v.Hq + (size_t)h * G) * 128;
+    if (n == 0) {  // an inactive slot
+      if (wi == 0) zero_pair<G>(v, b, h, out);
+      continue;
+    }
+    const int i0 = wi * n / w, i1 = (wi + 1) * n / w;
+    const int* tb = v.tables + (size_t)b * v.max_pages;
+    const int tail = (L - 1) / v.P;
+    PairState st;
+    uint4 nrow = make_uint4(0u, 0u, 0u, 0u);
+    int npage = 0, pw = 0, pages = 0;
+    auto load_pages = [&](int i) {  // lane l: the page of chunk i + l
+      pw = i;
+      const int pi = (i + lane) * kChunk / v.P;
+      pages = i + lane >= i1 ? 0 : old >= 0 && pi == tail ? old : tb[pi];
+    };
+    auto issue = [&](int i, int s) {
+      if (i >= pw + 32) load_pages(i);
+      int page = __shfl_sync(0xffffffffu, pages, i - pw);
+      if (lane == 0) {
+        if (page < 0 || page >= v.num_pages) {
+          set_status(v.ctl, GB_ERR_INVALID);
+          page = 0;
+        }
+        const int tok = i * kChunk;
+        const int wrow = ((layer_pages + page) * 2 * v.Hkv + h) * pg8 + ((tok & (v.P - 1)) >> 3);
+        const bool half = i == n - 1 && L - tok <= 8;
+        mbar_arrive_expect_tx(bar0 + 8 * s, half ? kMmaStageBytes / 2 : kMmaStageBytes);
+        tma_chunk(stage0 + s * kMmaStageBytes, half ? tmh_p : tm_p, wrow, bar0 + 8 * s, pol);
+      }
+    };
+    load_pages(i0);
+    int ii = i0;  // next chunk to load
+    for (int s = 0; s < kMmaStages && ii < i1 && alive; ++s, ++ii) issue(ii, (stage + s) % kMmaStages);
+    pair_begin<G>(st, v, q, b, h, r, c);
+    if (i0 < i1 && i1 == n) {  // this warp holds the pair's last chunk
+      nrow = (lane < 16 ? nw.k : nw.v)[(size_t)p * 16 + (lane & 15)];
+      npage = tb[tail];
+    }
+    for (int i = i0; i < i1 && alive; ++i) {
+      if (!mbar_wait_bounded(bar0 + 8 * stage, parity, kWaitLimitNs)) {
+        if (lane == 0) set_status(v.ctl, GB_ERR_TIMEOUT);
+        for (int s = 1; s < kMmaStages; ++s) {  // a bounded chance for the copies in flight
+          const int k = stage + s;
+          if (i + s < ii)
+            mbar_wait_bounded(bar0 + 8 * (k % kMmaStages), parity ^ (k >= kMmaStages ? 1u : 0u), kWaitLimitNs / 4);
+        }
+        alive = false;
+        break;
+      }
+      unsigned char* vs = smem + (stage0 + stage * kMmaStageBytes - smem_addr(smem));
+      const int tok0 = i * kChunk, nvalid = min(kChunk, L - tok0);
+      if (i == n - 1) chunk_append(v, layer, h, L, nvalid, nrow, npage, vs, lane);
+      if (old >= 0 && tok0 / v.P == tail) chunk_copied(v, layer, b, h, L, tok0, vs, lane);
+      chunk_attend(st, stage0 + stage * kMmaStageBytes, koff, voff, nvalid, qscale, r);
+      __syncwarp();
+      if (ii < i1) {
+        if (lane == 0) fence_proxy_async_smem();
+        issue(ii++, stage);
+      }
+      if (++stage == kMmaStages) {
+        stage = 0;
+        parity ^= 1u;
+      }
+    }
+#pragma unroll
+    for (int sh = 4; sh < 32; sh <<= 1) {
+      st.l0 += __shfl_xor_sync(0xffffffffu, st.l0, sh);
+      st.l1 += __shfl_xor_sync(0xffffffffu, st.l1, sh);
+    }
+    if (w == 1) {
+      if (2 * c < G) {
+        float* o0 = ob + 2 * c * 128 + r;
+#pragma unroll
+        for (int mt = 0; mt < 8; ++mt) {
+          o0[16 * mt] = alive ? st.o[mt][0] / st.l0 : 0.f;
+          o0[16 * mt + 128] = alive ? st.o[mt][1] / st.l1 : 0.f;
+          o0[16 * mt + 8] = alive ? st.o[mt][2] / st.l0 : 0.f;
+          o0[16 * mt + 136] = alive ? st.o[mt][3] / st.l1 : 0.f;
+        }
+      }
+      continue;
+    }
+    // The warp's record, then the team's merge: out = sum o 2^(m - M) / sum l 2^(m - M).  A warp
+    // without chunks has m = -inf and l = 0; one whose wait ran out marks its record with l < 0.
+    __syncwarp();
+    float* rec = reinterpret_cast<float*>(smem + warp * kMmaStages * kMmaStageBytes);
+    if (2 * c < G) {
+      float* o0 = rec + 2 * c * HS + r;
+#pragma unroll
+      for (int mt = 0; mt < 8; ++mt) {
+        o0[16 * mt] = st.o[mt][0];
+        o0[16 * mt + HS] = st.o[mt][1];
+        o0[16 * mt + 8] = st.o[mt][2];
+        o0[16 * mt + HS + 8] = st.o[mt][3];
+      }
+      if (r == 0) {
+        rec[G * HS + 2 * c] = st.m0;
+        rec[G * HS + 2 * c + 1] = st.m1;
+        rec[G * HS + G + 2 * c] = alive ? st.l0 : -1.f;
+        rec[G * HS + G + 2 * c + 1] = alive ? st.l1 : -1.f;
+      }
+    }
+    team_sync(team, w * 32);
+    const float* recs = reinterpret_cast<const float*>(smem + team * w * kMmaStages * kMmaStageBytes);
+    constexpr int RS = kMmaStages * kMmaStageBytes / 4;  // floats from one warp's record to the next
+    for (int e = wi * 32 + lane; e < G * 32; e += w * 32) {
+      const int g = e >> 5, d = 4 * (e & 31);
+      float M = -INFINITY;
+      bool good = true;
+      for (int k = 0; k < w; ++k) {
+        M = fmaxf(M, recs[k * RS + G * HS + g]);
+        good = good && !(recs[k * RS + G * HS + G + g] < 0.f);
+      }
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+      float l = 0.f;
+      for (int k = 0; k < w; ++k) {
+        const float m = recs[k * RS + G * HS + g];
+        if (m == -INFINITY) continue;
+        const float sc = exp2f(m - M);
+        const float4 x = *reinterpret_cast<const float4*>(recs + k * RS + g * HS + d);
+        acc.x = fmaf(x.x, sc, acc.x);
+        acc.y = fmaf(x.y, sc, acc.y);
+        acc.z = fmaf(x.z, sc, acc.z);
+        acc.w = fmaf(x.w, sc, acc.w);
+        l = fmaf(recs[k * RS + G * HS + G + g], sc, l);
+      }
+      float* od = ob + g * 128 + d;
+      od[0] = good ? acc.x / l : 0.f;
+      od[1] = good ? acc.y / l : 0.f;
+      od[2] = good ? acc.z / l : 0.f;
+      od[3] = good ? acc.w / l : 0.f;
+    }
+    fence_proxy_async_smem();  // the records' memory is refilled by TMA for the next pair
+    team_sync(team, w * 32);
+  }
+}
+
+}  // namespace gb

@@ -703,7 +703,7 @@ extern "C" gb_status gb_decode_attention(gb_pool* pool, int layer, const void* q
   const int mode = (flags == GB_PATH_PER_BEAM || !pool->view.grouped) ? 0 : 1;
   prof_begin(pool, GB_PROF_ATTENTION, s);
   if (launch_decode(pool, layer, q_dev, fused ? k_new_dev : nullptr, fused ? v_new_dev : nullptr, scale, out_dev, mode,
-                    s) != cudaSuccess)
+                    flags != GB_PATH_GROUPED, s) != cudaSuccess)
     return check_launch(pool, "decode");
   return check_launch(pool, "decode");
 }
