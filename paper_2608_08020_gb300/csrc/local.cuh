@@ -32,15 +32,10 @@ __device__ __forceinline__ bool local_step(const PoolView& v, int nctas) {
   return all <= GB_LOCAL_SCALE * (w * (all <= 3 * roles ? 44 : 28) + (units > 0 ? 4 * kMmaWarps * units : 0));
 }
 
-// The same for the per-beam path, whose other form splits the whole contexts evenly over all warps
-// of the GPU.
-__device__ __forceinline__ bool local_step_per_beam(const PoolView& v, int nctas) {
-  return plan_off(v, 0)[v.max_beams] <= GB_LOCAL_SCALE * 44ll * kMmaWarps * nctas;
-}
-
 // Warps per team: the number that minimises rounds of pairs x (chunks per warp + what a pair
 // costs beside its chunks: page ids, query rows and the first load, then the merge of a team).
-__device__ __forceinline__ int local_team(int npairs, int chunks_per_pair, int nctas) {
+// *cost gets that, in the time of a chunk.
+__device__ __forceinline__ int local_team(int npairs, int chunks_per_pair, int nctas, int* cost_out) {
   const int ws[6] = {1, 2, 3, 4, 6, 12};
   int best = 1, best_cost = 0x7fffffff;
 #pragma unroll
@@ -52,9 +47,29 @@ __device__ __forceinline__ int local_team(int npairs, int chunks_per_pair, int n
       best_cost = cost;
     }
   }
+  *cost_out = best_cost;
   return best;
 }
 static_assert(kMmaWarps == 12, "team sizes divide the CTA's warps");
+
+// The same for the per-beam path, whose other form splits the whole contexts evenly over all warps
+// of the GPU.  Where beams share pages, siblings of neighbouring teams read them at about the same
+// time here, and from L2: 79 against 117 us per layer-step for 64 beams x 4000 tokens, 188 / 326
+// (193 x 2962), 101 / 160 (40 x 8000, whose pairs fill 73% of the teams' rounds), 370 / 448
+// (256 x 4000), 265 / 256-303 (152 x 4000).  So a tree whose beams share a third of their contexts
+// takes this form unless uneven rounds cost it more than 1.6 times; one that shares little has
+// nothing to gain but an even split.
+__device__ __forceinline__ bool local_step_per_beam(const PoolView& v, int nctas) {
+  const long long all = plan_off(v, 0)[v.max_beams], w = kMmaWarps * nctas;
+  if (all <= GB_LOCAL_SCALE * 44 * w) return true;
+  if (!v.grouped || v.ctl[kCtlSegCount] == 0) return false;
+  const long long unshared = plan_off(v, 1)[v.max_beams] + (long long)v.ctl[kCtlSegTok] * v.Hkv / kChunk;
+  if (2 * all < 3 * unshared) return false;
+  const int npairs = v.max_beams * v.Hkv;
+  int cost;
+  local_team(npairs, (int)((all + npairs - 1) / npairs), nctas, &cost);
+  return 5ll * cost <= 8 * ((all + w - 1) / w + 6);
+}
 
 __device__ __forceinline__ void team_sync(int team, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(threads) : "memory");
@@ -79,7 +94,8 @@ __device__ __forceinline__ void local_attention(const PoolView& v, const CUtenso
   static_assert((G * HS + 2 * G) * 4 <= kMmaStages * kMmaStageBytes, "a record fits the warp's stages");
 
   const int npairs = v.max_beams * v.Hkv;
-  const int w = local_team(npairs, (plan_off(v, 0)[v.max_beams] + npairs - 1) / npairs, nctas);
+  int cost;
+  const int w = local_team(npairs, (plan_off(v, 0)[v.max_beams] + npairs - 1) / npairs, nctas, &cost);
   const int tpc = kMmaWarps / w, team = warp / w, wi = warp - team * w;
 
   if (lane == 0) {
