@@ -239,7 +239,8 @@ __global__ void __launch_bounds__(1024) k_step_begin(PoolView v, int n_tokens, c
   __shared__ int tmp[33];
   __shared__ int s_alloc[kMaxBeams];
   __shared__ int s_tail[kMaxBeams];
-  __shared__ int s_ncow, s_nact;
+  __shared__ int s_act[kMaxBeams], s_cow[kMaxBeams];  // active slots, slots that copy their tail page
+  __shared__ int s_ncow, s_len;
   __shared__ int s_tok[2];
   __shared__ int s_ctl[8];  // free pages, steps, and the segment totals of the step record
   const int b = threadIdx.x;
@@ -249,6 +250,7 @@ __global__ void __launch_bounds__(1024) k_step_begin(PoolView v, int n_tokens, c
   const int cover = (seg_cover != nullptr && b < v.max_beams) ? seg_cover[b] : 0;
   if (b == 0) {
     s_ncow = 0;
+    s_len = 0;
     s_ctl[0] = v.ctl[kCtlFree];
     s_ctl[1] = v.ctl[kCtlSteps];
     s_ctl[2] = v.ctl[kCtlSegRowTok];
@@ -288,9 +290,9 @@ __global__ void __launch_bounds__(1024) k_step_begin(PoolView v, int n_tokens, c
     too_long = last_idx >= v.max_pages;
   }
   int total_need, nact;
+  if (act) s_len = L;  // any active slot's length
   block_exclusive_scan(need_total, tmp, &total_need);
-  block_exclusive_scan(act ? 1 : 0, tmp, &nact);
-  if (b == 0) s_nact = nact;
+  const int arank = block_exclusive_scan(act ? 1 : 0, tmp, &nact);
   const bool any_too_long = __syncthreads_or(too_long);
   if (any_too_long || total_need > s_ctl[0]) {
     if (b == 0) v.ctl[kCtlCowJobs] = 0;
@@ -298,34 +300,92 @@ __global__ void __launch_bounds__(1024) k_step_begin(PoolView v, int n_tokens, c
     return;
   }
 
-  for (int k = 0; k < n_tokens; ++k) {
-    const int pos = L + k;
-    const bool need_new = act && (pos % v.P) == 0;
-    const bool need = need_new || (k == 0 && cow);
-    if (!__syncthreads_or(need)) continue;
-    int n_need;
-    const int rank = block_exclusive_scan(need ? 1 : 0, tmp, &n_need);
-    const int got = find_lowest_free(v, n_need, s_alloc, tmp);
-    if (got < n_need) {  // cannot happen after the count check; keep the pool consistent
+  // The sequential rule takes the lowest free page at every need, token by token and slots
+  // ascending; nothing is freed in between, so the r-th need of the step gets the r-th lowest free
+  // page.  Beams of one length (every state the calls build: all advance together and a child takes
+  // its parent's length) need their pages at the same tokens, so need r is copy r of the first
+  // ncow, then page j = (r - ncow) / nact of active slot (r - ncow) % nact, and one pass over the
+  // bitmap places them all.  (A pass per token with its block barriers took 88 us for 256 beams x
+  // 199 tokens.)  Other states take the sequential form below.
+  const bool uniform = !__syncthreads_or(act && L != s_len);
+  if (uniform) {
+    int ncow;
+    const int cr = block_exclusive_scan(cow ? 1 : 0, tmp, &ncow);
+    if (cow) s_cow[cr] = b;
+    if (act) s_act[arank] = b;
+    if (cow) atomicSub(&v.refcnt[tail], 1);
+    __syncthreads();
+    const int len = s_len, first_new = (len + v.P - 1) / v.P;
+    int found = 0, w0 = max(v.ctl[kCtlCursor], 0);
+    while (found < total_need && w0 < v.words) {
+      const int w = w0 + b;
+      unsigned bits = w < v.words ? v.free_bits[w] : 0u;
+      if (w == v.words - 1 && (v.num_pages & 31)) bits &= (1u << (v.num_pages & 31)) - 1u;
+      int total;
+      int r = found + block_exclusive_scan(__popc(bits), tmp, &total);
+      const unsigned before = bits;
+      while (bits && r < total_need) {
+        const int page = w * 32 + __ffs(bits) - 1;
+        bits &= bits - 1u;
+        int slot, idx;
+        if (r < ncow) {  // copy-on-write of a shared tail page
+          slot = s_cow[r];
+          idx = len / v.P;
+          v.cow[3 * r] = s_tail[slot];
+          v.cow[3 * r + 1] = page;
+          v.cow[3 * r + 2] = len % v.P;
+        } else {
+          const int j = (r - ncow) / nact;
+          slot = s_act[r - ncow - j * nact];
+          idx = first_new + j;
+        }
+        v.refcnt[page] = 1;
+        v.tables[(size_t)slot * v.max_pages + idx] = page;
+        if (++r == total_need) v.ctl[kCtlCursor] = w;
+      }
+      if (bits != before) v.free_bits[w] = (v.free_bits[w] & ~before) | bits;
+      found += total;
+      w0 += blockDim.x;
+    }
+    if (b == 0) {
+      s_ncow = ncow;
+      if (total_need > 0) v.ctl[kCtlFree] = s_ctl[0] - total_need;
+    }
+    if (found < total_need) {  // cannot happen after the count check
       if (b == 0) { set_status(v.ctl, GB_ERR_OOM); v.ctl[kCtlStepOk] = 0; }
       return;
     }
-    take_pages(v, s_alloc, n_need);
-    if (need) {
-      const int page = s_alloc[rank];
-      v.refcnt[page] = 1;
-      v.tables[(size_t)b * v.max_pages + pos / v.P] = page;
-      if (!need_new) {  // copy-on-write of the shared tail page
-        atomicSub(&v.refcnt[tail], 1);
-        const int j = atomicAdd(&s_ncow, 1);
-        if (j < kMaxCowJobs) {
-          v.cow[3 * j] = tail;
-          v.cow[3 * j + 1] = page;
-          v.cow[3 * j + 2] = L % v.P;
+    __syncthreads();
+  } else {
+    for (int k = 0; k < n_tokens; ++k) {
+      const int pos = L + k;
+      const bool need_new = act && (pos % v.P) == 0;
+      const bool need = need_new || (k == 0 && cow);
+      if (!__syncthreads_or(need)) continue;
+      int n_need;
+      const int rank = block_exclusive_scan(need ? 1 : 0, tmp, &n_need);
+      const int got = find_lowest_free(v, n_need, s_alloc, tmp);
+      if (got < n_need) {  // cannot happen after the count check; keep the pool consistent
+        if (b == 0) { set_status(v.ctl, GB_ERR_OOM); v.ctl[kCtlStepOk] = 0; }
+        return;
+      }
+      take_pages(v, s_alloc, n_need);
+      if (need) {
+        const int page = s_alloc[rank];
+        v.refcnt[page] = 1;
+        v.tables[(size_t)b * v.max_pages + pos / v.P] = page;
+        if (!need_new) {  // copy-on-write of the shared tail page
+          atomicSub(&v.refcnt[tail], 1);
+          const int j = atomicAdd(&s_ncow, 1);
+          if (j < kMaxCowJobs) {
+            v.cow[3 * j] = tail;
+            v.cow[3 * j + 1] = page;
+            v.cow[3 * j + 2] = L % v.P;
+          }
         }
       }
+      __syncthreads();
     }
-    __syncthreads();
   }
   // The rows [0, L % P) of each copied page are copied layer by layer by the kernel that writes
   // the layer's new rows: the append kernel from the job list, the attention launch from cow_old.
@@ -370,7 +430,7 @@ __global__ void __launch_bounds__(1024) k_step_begin(PoolView v, int n_tokens, c
     e[6] = n_tokens;
     e[7] = step;
     e[8] = v.grouped ? s_ctl[6] : 0;
-    e[9] = s_nact;
+    e[9] = nact;
     v.ctl[kCtlSteps] = step + 1;
   }
   if (b == 0) {
@@ -410,50 +470,84 @@ __global__ void k_append(PoolView v, int layer, int n_tokens, const char* kin, c
     uint4* dst = reinterpret_cast<uint4*>(v.kv + kv_elem_offset(v, layer, v.cow[3 * j + 1], kv, head, row) * v.esize);
     dst[vec] = src[vec];
   }
-  // New rows: blockIdx.y walks (K|V, token), x covers (slot, head, 16-byte vector) with
-  // 32-bit index arithmetic (a row is 256 bytes, 16 vectors, for every supported shape).
-  const int per_tok = v.max_beams * v.Hkv * vec_per_row;
-  for (int y = blockIdx.y; y < 2 * n_tokens; y += gridDim.y) {
-    const int kv = y >= n_tokens ? 1 : 0;
-    const int k = y - kv * n_tokens;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < per_tok; i += gridDim.x * blockDim.x) {
-      const int vec = i & 15;
-      const int r = i >> 4;
-      const int b = r / v.Hkv, head = r - b * v.Hkv;
+  // New rows.  blockIdx.y walks (page of the new range, K|V), blockIdx.x the slots: one CTA writes
+  // the new tokens of one page of one beam, all heads, so the slot's state and its page id are read
+  // once for up to P tokens, the source is read in rows of Hkv * 256 contiguous bytes, and a
+  // thread's loads (four at a time) are independent.  A thread per 16-byte piece that looked its
+  // own page up ran at 3.8 TB/s of reads and writes (110 us for 256 beams x 199 tokens x 2 KiB).
+  const int runs = (n_tokens + v.P - 1) / v.P + 1;
+  for (int y = blockIdx.y; y < 2 * runs; y += gridDim.y) {
+    const int kv = y & 1;
+    for (int b = blockIdx.x; b < v.max_beams; b += gridDim.x) {
       if (!v.active[b]) continue;
-      const int pos = v.seq_len[b] - n_tokens + k;
-      if (pos < 0) continue;
-      const int page = v.tables[(size_t)b * v.max_pages + pos / v.P];
-      if (page < 0 || page >= v.num_pages) { set_status(v.ctl, GB_ERR_INVALID); continue; }
-      const char* src = (kv ? vin : kin) + ((((long long)k * v.max_beams + b) * v.Hkv + head) * v.D) * v.esize;
-      char* dst = v.kv + kv_elem_offset(v, layer, page, kv, head, pos % v.P) * v.esize;
-      reinterpret_cast<uint4*>(dst)[vec] = reinterpret_cast<const uint4*>(src)[vec];
+      const int L = v.seq_len[b], pos0 = L - n_tokens;
+      if (pos0 < 0) continue;
+      const int pi = pos0 / v.P + (y >> 1);
+      const int t0 = max(pos0, pi * v.P), t1 = min(L, (pi + 1) * v.P);
+      if (t0 >= t1) continue;
+      const int page = v.tables[(size_t)b * v.max_pages + pi];
+      if (page < 0 || page >= v.num_pages) {
+        if (threadIdx.x == 0) set_status(v.ctl, GB_ERR_INVALID);
+        continue;
+      }
+      const int row16 = v.Hkv * 16;  // 16-byte pieces of one token (a head's row is 256 bytes)
+      const uint4* src = reinterpret_cast<const uint4*>(kv ? vin : kin) + ((size_t)(t0 - pos0) * v.max_beams + b) * row16;
+      uint4* dst = reinterpret_cast<uint4*>(v.kv + kv_elem_offset(v, layer, page, kv, 0, t0 - pi * v.P) * v.esize);
+      const size_t tok_stride = (size_t)v.max_beams * row16;
+      const int count = (t1 - t0) * row16;
+      for (int i0 = threadIdx.x; i0 < count; i0 += 4 * blockDim.x) {
+        uint4 x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = i0 + u * blockDim.x;
+          if (i < count) x[u] = __ldcs(src + (size_t)(i / row16) * tok_stride + i % row16);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = i0 + u * blockDim.x;
+          const int t = i / row16, r = i - t * row16;
+          if (i < count) dst[((r >> 4) * v.P + t) * 16 + (r & 15)] = x[u];
+        }
+      }
     }
   }
 }
 
-// Release listed slots in order (one CTA).
+// Release listed slots (one CTA), 1024 entries of the list at a time.  An entry is taken when its
+// slot is in range, active, and not named by an earlier entry; the first entry that is not decides
+// the status, as if they were processed in order.  Each taken slot's references are dropped by a
+// warp of its own (one slot after another took 2 us each, most of it two dependent loads).
 __global__ void __launch_bounds__(1024) k_release(PoolView v, const int* slots, int n) {
   pdl_wait();
   pdl_launch_dependents();
-  for (int i = 0; i < n; ++i) {
-    const int s = slots[i];
-    if (s < 0 || s >= v.max_beams) {
-      if (threadIdx.x == 0) set_status(v.ctl, GB_ERR_INVALID);
-      continue;
-    }
-    if (!v.active[s]) {
-      if (threadIdx.x == 0) set_status(v.ctl, GB_ERR_STATE);
-      __syncthreads();
-      continue;
-    }
-    const int npg = (v.seq_len[s] + v.P - 1) / v.P;
-    for (int j = threadIdx.x; j < npg; j += blockDim.x) {
-      const int p = v.tables[(size_t)s * v.max_pages + j];
-      if (p >= 0 && p < v.num_pages) unref_page(v, p);
+  __shared__ int s_first[kMaxBeams];  // first entry of this part of the list that names the slot
+  __shared__ int s_take[1024];
+  __shared__ int s_bad;               // (entry << 3) | code of the first bad entry
+  const int tid = threadIdx.x;
+  for (int base = 0; base < n; base += 1024) {
+    s_first[tid] = 0x7fffffff;
+    if (tid == 0) s_bad = 0x7fffffff;
+    __syncthreads();
+    const int s = base + tid < n ? slots[base + tid] : -1;
+    const bool in = base + tid < n && s >= 0 && s < v.max_beams;
+    if (in) atomicMin(&s_first[s], tid);
+    __syncthreads();
+    const bool take = in && s_first[s] == tid && v.active[s];
+    if (base + tid < n && !take) atomicMin(&s_bad, (tid << 3) | (in ? GB_ERR_STATE : GB_ERR_INVALID));
+    s_take[tid] = take ? s : -1;
+    __syncthreads();
+    if (tid == 0 && s_bad != 0x7fffffff) set_status(v.ctl, s_bad & 7);
+    for (int i = tid >> 5; i < min(1024, n - base); i += 32) {
+      const int t = s_take[i];
+      if (t < 0) continue;
+      const int npg = (v.seq_len[t] + v.P - 1) / v.P;
+      for (int j = tid & 31; j < npg; j += 32) {
+        const int p = v.tables[(size_t)t * v.max_pages + j];
+        if (p >= 0 && p < v.num_pages) unref_page(v, p);
+      }
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (take) {
       v.active[s] = 0;
       v.seq_len[s] = 0;
       v.gen[s] = 0;
@@ -665,8 +759,8 @@ static gb_status append_layer(gb_pool* pool, int layer, int n_tokens, const void
   } else if (n_tokens != pool->step_tokens) {
     return fail(pool, GB_ERR_STATE, "token count differs from the one layer 0 reserved");
   }
-  const int per_tok = pool->cfg.max_beams * pool->cfg.num_kv_heads * (pool->view.D * pool->view.esize / 16);
-  const dim3 grid(std::max(1, std::min((per_tok + 255) / 256, pool->num_sms * 8)), std::min(2 * n_tokens, 65535));
+  const int runs = (n_tokens + pool->cfg.page_size - 1) / pool->cfg.page_size + 1;  // pages a beam's new tokens meet
+  const dim3 grid(pool->cfg.max_beams, std::min(2 * runs, 65535));
   prof_begin(pool, GB_PROF_APPEND, s);  // an empty interval when the attention launch appends
   if (!fused) {
     launch_pdl(k_append, grid, 256, 0, s, pool->view, layer, n_tokens, static_cast<const char*>(k),
