@@ -11,18 +11,20 @@
 //          (gb_decode_attention on the step pool: it appends k, v first)
 //   x   += W_o a;   u = LN2(x);   x += W_2 (SiLU(W_1 u) * W_3 u)  (Eq. 5)
 //   y_t  = sigmoid(w_out . LN(x) + b_out)                        (Eq. 6)
-// The matrix products are the split-K tcgen05 GEMM of gemm.cu (bf16 operands, fp32
-// partials); each product's epilogue is one kernel that sums the partials in a fixed
-// order and applies what follows it (GELU, residual add, the next LayerNorm, RoPE,
-// SwiGLU, the output head), one CTA per row.  The residual stream x is fp32; the
-// operands of the products (LayerNorm outputs, q/k/v, attention outputs, SwiGLU
-// outputs) are rounded to bf16.
+// Every product runs on tcgen05 (bf16 operands, fp32 accumulation).  W_in, whose K is the
+// generator's hidden size, is the split-K GEMM of gemm.cu; the others are k_fused_gemm, which
+// builds its A operand itself (LayerNorm of the residual stream, or the attention output rounded
+// to bf16) and finishes the product (RoPE, residual add, SwiGLU) in the same launch.  The residual
+// stream x is fp32; the operands of the products (LayerNorm outputs, q/k/v, attention outputs,
+// SwiGLU outputs) are rounded to bf16.
 //
 // Model shape: L = the step pool's layers, Hq query heads and Hkv key/value heads of
 // 128 dims (the step pool's head counts, bf16 K/V), d_model = Hq * 128.  LayerNorm
 // eps 1e-5; GELU the exact (erf) form; rotary pairs (i, i + 64) with angle
 // t * 10000^(-i/64); softmax scale 1/sqrt(128).
 #include "internal.cuh"
+#include "ptx.cuh"
+#include "tc.cuh"
 
 namespace gb {
 namespace {
@@ -142,28 +144,6 @@ __device__ __forceinline__ float block_sum(float v, float* red) {
   return t;
 }
 
-// LayerNorm of the row held in shared memory (n floats): gain and bias applied, bf16 out.
-__device__ void layer_norm_row(const float* row, int n, const float* __restrict__ g, const float* __restrict__ b,
-                               __nv_bfloat16* __restrict__ out, float* red) {
-  float s = 0.f;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) s += row[i];
-  const float mu = block_sum(s, red) / (float)n;
-  float v = 0.f;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const float c = row[i] - mu;
-    v = fmaf(c, c, v);
-  }
-  const float var = block_sum(v, red) / (float)n;
-  const float r = 1.0f / sqrtf(var + kLnEps);
-  for (int i = threadIdx.x; i < n; i += blockDim.x) out[i] = __float2bfloat16_rn((row[i] - mu) * r * g[i] + b[i]);
-}
-
-__device__ __forceinline__ float sum_partials(const float* __restrict__ P, int splits, int M, int N, int m, int n) {
-  float z = 0.f;
-  for (int k = 0; k < splits; ++k) z += P[((size_t)k * M + m) * N + n];
-  return z;
-}
-
 __device__ __forceinline__ bool row_live(const int* active, int m) { return active == nullptr || active[m] != 0; }
 
 // Input LayerNorm of Eq. 4: u[m] = LN_in(h[m]) (bf16 h, H wide, H % 64 == 0).  Inactive
@@ -214,132 +194,368 @@ __global__ void __launch_bounds__(kRowThreads) k_ln_in(const __nv_bfloat16* __re
   }
 }
 
-enum RowMode { kGeluLn = 0, kResidLn = 1, kResidHead = 2 };
-
-// Epilogue of a d-wide product, one CTA per row m:
-//   kGeluLn:    x[m] = GELU(z)            then u[m] = LN(x[m])           (Eq. 4, then LN1 of layer 0)
-//   kResidLn:   x[m] += z                 then u[m] = LN(x[m])           (residual, then the next LN)
-//   kResidHead: x[m] += z                 then score[m] = sigmoid(w_out . LN(x[m]) + b_out)   (Eq. 6)
-// z = the sum of the product's K-split partials.  Inactive rows: u = 0, score = 0.
-template <int Mode>
-__global__ void __launch_bounds__(kRowThreads) k_row_epilogue(const float* __restrict__ P, int splits, int M, int d,
-                                                              float* __restrict__ x, const float* __restrict__ g,
-                                                              const float* __restrict__ b, const int* __restrict__ active,
-                                                              __nv_bfloat16* __restrict__ u,
-                                                              const float* __restrict__ w_out,
-                                                              const float* __restrict__ b_out,
-                                                              float* __restrict__ score) {
+// x = GELU(z) of Eq. 4 (exact, erf), z = the sum of the product's K-split partials.
+__global__ void __launch_bounds__(kRowThreads) k_gelu_epilogue(const float* __restrict__ P, int splits, int n4,
+                                                               float* __restrict__ x) {
   pdl_wait();
   pdl_launch_dependents();
-  extern __shared__ float row[];
-  __shared__ float red[33];
-  const int m = blockIdx.x;
+  const int i = blockIdx.x * kRowThreads + threadIdx.x;
+  if (i >= n4) return;
+  float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int k = 0; k < splits; ++k) {
+    const float4 p = reinterpret_cast<const float4*>(P)[(size_t)k * n4 + i];
+    z = make_float4(z.x + p.x, z.y + p.y, z.z + p.z, z.w + p.w);
+  }
+  auto gelu = [](float t) { return 0.5f * t * (1.0f + erff(t * 0.70710678118654752f)); };
+  reinterpret_cast<float4*>(x)[i] = make_float4(gelu(z.x), gelu(z.y), gelu(z.z), gelu(z.w));
+}
+
+__device__ __forceinline__ float warp_sum(float v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Output head (Eq. 6), one warp per row: score = sigmoid(w_out . LN(x) + b_out); 0 for inactive rows.
+__global__ void __launch_bounds__(kRowThreads) k_head(const float* __restrict__ x, int M, int d,
+                                                      const float* __restrict__ g, const float* __restrict__ b,
+                                                      const float* __restrict__ w_out, const float* __restrict__ b_out,
+                                                      const int* __restrict__ active, float* __restrict__ score) {
+  pdl_wait();
+  pdl_launch_dependents();
+  const int m = blockIdx.x * (kRowThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (m >= M) return;
   if (!row_live(active, m)) {
-    if (Mode == kResidHead) {
-      if (score && threadIdx.x == 0) score[m] = 0.f;
+    if (lane == 0) score[m] = 0.f;
+    return;
+  }
+  const float4* row = reinterpret_cast<const float4*>(x + (size_t)m * d);
+  float s = 0.f, v = 0.f, dot = 0.f;
+  for (int i = lane; i < d / 4; i += 32) s += (row[i].x + row[i].y) + (row[i].z + row[i].w);
+  const float mu = warp_sum(s) / (float)d;
+  for (int i = lane; i < d / 4; i += 32) {
+    const float4 y = row[i];
+    v = fmaf(y.x - mu, y.x - mu, v);
+    v = fmaf(y.y - mu, y.y - mu, v);
+    v = fmaf(y.z - mu, y.z - mu, v);
+    v = fmaf(y.w - mu, y.w - mu, v);
+  }
+  const float r = 1.0f / sqrtf(warp_sum(v) / (float)d + kLnEps);
+  for (int i = lane; i < d / 4; i += 32) {
+    const float4 y = row[i], gg = reinterpret_cast<const float4*>(g)[i], bb = reinterpret_cast<const float4*>(b)[i],
+                 w = reinterpret_cast<const float4*>(w_out)[i];
+    dot = fmaf((y.x - mu) * r * gg.x + bb.x, w.x, dot);
+    dot = fmaf((y.y - mu) * r * gg.y + bb.y, w.y, dot);
+    dot = fmaf((y.z - mu) * r * gg.z + bb.z, w.z, dot);
+    dot = fmaf((y.w - mu) * r * gg.w + bb.w, w.w, dot);
+  }
+  const float y = warp_sum(dot) + b_out[0];
+  if (lane == 0) score[m] = 1.0f / (1.0f + expf(-y));
+}
+
+// ---- products with their operand and epilogue in one launch -------------------------------------
+//
+// Grid (row tiles of mt = 32, 64 or 128 slots) x (64-column tiles).  A CTA of 256 threads builds its
+// rows' A operand in shared memory (128-byte swizzle, 512 of K at a time), loads its 64 rows of the
+// weights, multiplies (128 x 64 x 16 tcgen05.mma into tensor memory; the rows past mt are never
+// read) and finishes its tile.  At these sizes (64 slots, d = 512: 32 MFLOP and 0.5-2 MiB of weights
+// a product) a product is latency: the chain of LayerNorm, GEMM with K-split partials in global
+// memory and epilogue was three launches of 6-9 us each.  So K is not split, the LayerNorm is
+// recomputed by every column tile (its rows come from L2), and the weights, which do not depend on
+// the previous launch, are loaded before waiting for it.  mt is the smallest that keeps the grid
+// within the SMs: fewer rows per CTA shorten its own chain.
+enum AMode { kALn, kAF32, kABf16 };              // LayerNorm of fp32 rows; fp32 rows; bf16 rows
+enum EMode { kEQkv, kEResid, kESwiglu };         // RoPE and q/k/v in bf16; x += z; SwiGLU in bf16
+
+constexpr int kFThreads = 256, kFN = 64, kFK = 512;
+constexpr int kFA = 0, kFABlock = 128 * 128;               // 64 of K: 128 rows x 128 bytes
+constexpr int kFB = kFA + kFK / 64 * kFABlock, kFBBlock = kFN * 128;
+constexpr int kFCtl = kFB + kFK / 64 * kFBBlock;            // mbarrier, tensor-memory address
+constexpr int kFStat = kFCtl + 16;                          // float [2][128]: mean and 1/std of the rows
+constexpr int kFSmem = kFStat + 1024;
+constexpr int kFTile = kFN + 1;                             // epilogue tile [128][65] over the A operand
+static_assert(128 * kFTile * 4 <= kFB && kFSmem <= 232448 - 1024, "shared memory per block");
+
+struct FusedArgs {
+  const void* a;            // [M][K]
+  const float *g, *b;       // LayerNorm gain and bias (kALn)
+  const __nv_bfloat16* w;   // weights, rows of K
+  int M, K, mt;
+  const int* active;
+  float* x;                 // kEResid: [M][d]
+  int d;
+  __nv_bfloat16 *q, *kn, *vn;  // kEQkv
+  int Hq, Hkv, pos_shift;
+  const int* pos_of;
+  __nv_bfloat16* u;         // kESwiglu: [M][F]
+  int F;
+  int* ctl;
+};
+
+// Weight row of column n of column tile t.  A rotary tile holds 32 (i, i + 64) pairs of one head, a
+// SwiGLU tile 32 columns of W_1 and the same of W_3, so each tile finishes on its own.
+template <int E>
+__device__ __forceinline__ int weight_row(const FusedArgs& p, int t, int n) {
+  if (E == kEQkv) {
+    const int rot = 2 * (p.Hq + p.Hkv);
+    if (t < rot) return (t >> 1) * kHd + (t & 1) * 32 + (n & 31) + (n >> 5) * (kHd / 2);
+    return (p.Hq + p.Hkv) * kHd + (t - rot) * kFN + n;
+  }
+  if (E == kESwiglu) return t * 32 + (n & 31) + (n >> 5) * p.F;
+  return t * kFN + n;
+}
+
+template <int A, int E>
+__global__ void __launch_bounds__(kFThreads, 1) k_fused_gemm(FusedArgs p) {
+  extern __shared__ __align__(1024) unsigned char sm[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int m0 = blockIdx.x * p.mt, t = blockIdx.y;
+  const uint32_t sbase = smem_addr(sm), bar = sbase + kFCtl;
+  float* s_mu = reinterpret_cast<float*>(sm + kFStat);
+  float* s_rs = s_mu + 128;
+  if (sbase & 1023) {
+    if (tid == 0) set_status(p.ctl, GB_ERR_UNSUPPORTED);
+    return;
+  }
+  if (tid == 0) {
+    mbar_init(bar, 1);
+    fence_mbar_init();
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(bar + 8), "r"(kFN));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  auto load_b = [&](int k0) {
+    const int pc = min(kFK, p.K - k0) / 8;  // 16-byte pieces per row
+    for (int i = tid; i < kFN * pc; i += kFThreads) {
+      const int n = i / pc, c = i - n * pc;
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sbase + kFB + (c >> 3) * kFBBlock + swz(n, (c & 7) * 8)),
+                   "l"(p.w + (size_t)weight_row<E>(p, t, n) * p.K + k0 + 8 * c)
+                   : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  load_b(0);
+  pdl_wait();
+  pdl_launch_dependents();
+
+  const float* af = static_cast<const float*>(p.a);
+  auto live_row = [&](int r) { return r < p.mt && m0 + r < p.M && row_live(p.active, m0 + r); };
+  // LayerNorm statistics of rows longer than one pass: the mean, then the centred squares.
+  if (A == kALn && p.K > kFK) {
+    for (int r = warp; r < p.mt; r += kFThreads / 32) {
+      if (!live_row(r)) continue;
+      const float4* row = reinterpret_cast<const float4*>(af + (size_t)(m0 + r) * p.K);
+      float s = 0.f, v = 0.f;
+#pragma unroll 4
+      for (int i = lane; i < p.K / 4; i += 32) {
+        const float4 y = row[i];
+        s += (y.x + y.y) + (y.z + y.w);
+      }
+      const float mu = warp_sum(s) / (float)p.K;
+#pragma unroll 4
+      for (int i = lane; i < p.K / 4; i += 32) {
+        const float4 y = row[i];
+        v = fmaf(y.x - mu, y.x - mu, v);
+        v = fmaf(y.y - mu, y.y - mu, v);
+        v = fmaf(y.z - mu, y.z - mu, v);
+        v = fmaf(y.w - mu, y.w - mu, v);
+      }
+      const float rs = 1.0f / sqrtf(warp_sum(v) / (float)p.K + kLnEps);
+      if (lane == 0) {
+        s_mu[r] = mu;
+        s_rs[r] = rs;
+      }
+    }
+    __syncwarp();  // a row's statistics are read by the warp that wrote them
+  }
+
+  bool ok = true;
+  int pass = 0;
+  uint32_t tmem = 0;
+  for (int k0 = 0; k0 < p.K; k0 += kFK, ++pass) {
+    const int kw = min(kFK, p.K - k0);
+    if (pass > 0) {  // the previous pass's operands have been read
+      ok = ok && mbar_wait_bounded(bar, (pass - 1) & 1, kWaitLimitNs);
+      load_b(k0);
+    }
+    // A: row r = warp + 8 j of the tile, four rows in flight per warp.
+    if (A == kABf16) {
+      const __nv_bfloat16* ab = static_cast<const __nv_bfloat16*>(p.a);
+      for (int r0 = warp; r0 < p.mt; r0 += kFThreads / 32 * 4) {
+        uint4 v[4][kFK / 256];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int r = r0 + kFThreads / 32 * u;
+          const bool live = live_row(r);
+#pragma unroll
+          for (int i = 0; i < kFK / 256; ++i) {
+            const int c = 8 * lane + 256 * i;
+            v[u][i] = live && c < kw ? *reinterpret_cast<const uint4*>(ab + (size_t)(m0 + r) * p.K + k0 + c)
+                                     : make_uint4(0u, 0u, 0u, 0u);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int r = r0 + kFThreads / 32 * u;
+#pragma unroll
+          for (int i = 0; i < kFK / 256; ++i) {
+            const int c = 8 * lane + 256 * i;
+            if (r < p.mt && c < kw) *reinterpret_cast<uint4*>(sm + kFA + (c >> 6) * kFABlock + swz(r, c & 63)) = v[u][i];
+          }
+        }
+      }
     } else {
-      for (int i = threadIdx.x; i < d; i += blockDim.x) u[(size_t)m * d + i] = __float2bfloat16_rn(0.f);
+      float4 gg[kFK / 128], bb[kFK / 128];
+      if (A == kALn) {
+#pragma unroll
+        for (int i = 0; i < kFK / 128; ++i) {
+          const int c = 4 * lane + 128 * i;
+          gg[i] = c < kw ? *reinterpret_cast<const float4*>(p.g + k0 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+          bb[i] = c < kw ? *reinterpret_cast<const float4*>(p.b + k0 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+      }
+      for (int r0 = warp; r0 < p.mt; r0 += kFThreads / 32 * 4) {
+        float4 v[4][kFK / 128];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int r = r0 + kFThreads / 32 * u;
+          const bool live = live_row(r);
+#pragma unroll
+          for (int i = 0; i < kFK / 128; ++i) {
+            const int c = 4 * lane + 128 * i;
+            v[u][i] = live && c < kw ? *reinterpret_cast<const float4*>(af + (size_t)(m0 + r) * p.K + k0 + c)
+                                     : make_float4(0.f, 0.f, 0.f, 0.f);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int r = r0 + kFThreads / 32 * u;
+          if (r >= p.mt) break;
+          float mu = 0.f, rs = 1.f;
+          if (A == kALn && p.K <= kFK) {
+            float s = 0.f, q = 0.f;
+#pragma unroll
+            for (int i = 0; i < kFK / 128; ++i) s += (v[u][i].x + v[u][i].y) + (v[u][i].z + v[u][i].w);
+            mu = warp_sum(s) / (float)p.K;
+#pragma unroll
+            for (int i = 0; i < kFK / 128; ++i)
+              if (4 * lane + 128 * i < kw) {
+                q = fmaf(v[u][i].x - mu, v[u][i].x - mu, q);
+                q = fmaf(v[u][i].y - mu, v[u][i].y - mu, q);
+                q = fmaf(v[u][i].z - mu, v[u][i].z - mu, q);
+                q = fmaf(v[u][i].w - mu, v[u][i].w - mu, q);
+              }
+            rs = 1.0f / sqrtf(warp_sum(q) / (float)p.K + kLnEps);
+          } else if (A == kALn && live_row(r)) {
+            mu = s_mu[r];
+            rs = s_rs[r];
+          }
+#pragma unroll
+          for (int i = 0; i < kFK / 128; ++i) {
+            const int c = 4 * lane + 128 * i;
+            if (c >= kw) continue;
+            float4 y = v[u][i];
+            if (A == kALn)
+              y = make_float4((y.x - mu) * rs * gg[i].x + bb[i].x, (y.y - mu) * rs * gg[i].y + bb[i].y,
+                              (y.z - mu) * rs * gg[i].z + bb[i].z, (y.w - mu) * rs * gg[i].w + bb[i].w);
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(y.x, y.y), hi = __floats2bfloat162_rn(y.z, y.w);
+            *reinterpret_cast<uint2*>(sm + kFA + (c >> 6) * kFABlock + swz(r, c & 63)) =
+                make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+          }
+        }
+      }
     }
-    return;
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    fence_proxy_async_smem();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    tmem = *reinterpret_cast<volatile uint32_t*>(sm + kFCtl + 8);
+    if (tid == 0 && ok) {
+      constexpr uint32_t ID = idesc(128, kFN, false);
+      for (int kb = 0; kb < kw / 64; ++kb)
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+          mma(tmem, sdesc(sbase + kFA + kb * kFABlock + kk * 32, 16, 1024),
+              sdesc(sbase + kFB + kb * kFBBlock + kk * 32, 16, 1024), ID, (pass > 0 || kb > 0 || kk > 0) ? 1u : 0u);
+      mma_commit(bar);
+    }
   }
-  float* xm = x + (size_t)m * d;
-  for (int i = threadIdx.x; i < d; i += blockDim.x) {
-    const float z = sum_partials(P, splits, M, d, m, i);
-    const float y = Mode == kGeluLn ? 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)) : xm[i] + z;
-    xm[i] = y;
-    row[i] = y;
+  ok = ok && mbar_wait_bounded(bar, (pass - 1) & 1, kWaitLimitNs);
+  ok = __syncthreads_and(ok) != 0;
+  tc_fence_after();
+  float* tile = reinterpret_cast<float*>(sm + kFA);  // [mt][65]
+  if (ok && warp < p.mt / 32) {
+#pragma unroll
+    for (int c0 = 0; c0 < kFN; c0 += 32) {
+      float z[32];
+      tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + c0, z);
+#pragma unroll
+      for (int i = 0; i < 32; ++i) tile[(warp * 32 + lane) * kFTile + c0 + i] = z[i];
+    }
   }
+  tc_fence_before();
   __syncthreads();
-  if (Mode != kResidHead) {
-    layer_norm_row(row, d, g, b, u + (size_t)m * d, red);
+  tc_fence_after();
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kFN));
+  if (!ok) {
+    if (tid == 0) set_status(p.ctl, GB_ERR_TIMEOUT);
     return;
   }
-  // Output head: LN, dot with w_out (fixed order), bias, sigmoid.
-  float s = 0.f;
-  for (int i = threadIdx.x; i < d; i += blockDim.x) s += row[i];
-  const float mu = block_sum(s, red) / (float)d;
-  float v = 0.f;
-  for (int i = threadIdx.x; i < d; i += blockDim.x) {
-    const float c = row[i] - mu;
-    v = fmaf(c, c, v);
-  }
-  const float r = 1.0f / sqrtf(block_sum(v, red) / (float)d + kLnEps);
-  float dot = 0.f;
-  for (int i = threadIdx.x; i < d; i += blockDim.x) dot = fmaf((row[i] - mu) * r * g[i] + b[i], w_out[i], dot);
-  const float y = block_sum(dot, red) + b_out[0];
-  if (threadIdx.x == 0 && score) score[m] = 1.0f / (1.0f + expf(-y));
-}
 
-// Epilogue of the q/k/v product, one CTA per row m: sums the partials, rotates the
-// (i, i + 64) pairs of every q and k head by pos * 10000^(-i/64) with pos = pos_of[m] +
-// pos_shift (0 without pos_of), and writes q [M][Hq][128], k and v [M][Hkv][128] in bf16.
-__global__ void __launch_bounds__(kRowThreads) k_qkv_epilogue(const float* __restrict__ P, int splits, int M, int Hq,
-                                                              int Hkv, const int* __restrict__ pos_of, int pos_shift,
-                                                              const int* __restrict__ active,
-                                                              __nv_bfloat16* __restrict__ q,
-                                                              __nv_bfloat16* __restrict__ kn,
-                                                              __nv_bfloat16* __restrict__ vn) {
-  pdl_wait();
-  pdl_launch_dependents();
-  const int m = blockIdx.x;
-  const int N = (Hq + 2 * Hkv) * kHd;
-  const bool live = row_live(active, m);
-  const float pos = pos_of && live ? (float)(pos_of[m] + pos_shift) : 0.f;
-  const int pairs = (Hq + Hkv) * (kHd / 2);
-  for (int j = threadIdx.x; j < pairs; j += blockDim.x) {
-    const int head = j / (kHd / 2), i = j % (kHd / 2);
-    const int col = head * kHd + i;
-    float a = 0.f, c = 0.f;
-    if (live) {
-      const float x1 = sum_partials(P, splits, M, N, m, col), x2 = sum_partials(P, splits, M, N, m, col + kHd / 2);
-      const float ang = pos * powf(10000.0f, -(float)i / (float)(kHd / 2));
-      float sn, cs;
-      sincosf(ang, &sn, &cs);
-      a = x1 * cs - x2 * sn;
-      c = x1 * sn + x2 * cs;
+  const int rows = min(p.mt, p.M - m0);
+  if (E == kEQkv) {
+    const int rot = 2 * (p.Hq + p.Hkv);
+    if (t < rot) {
+      // Rotate the pairs (i, i + 64) by pos * 10000^(-i/64); inactive rows give zeros.
+      const int head = t >> 1, i = (t & 1) * 32 + lane;
+      const float inv = powf(10000.0f, -(float)i / (float)(kHd / 2));
+      for (int r = warp; r < rows; r += kFThreads / 32) {
+        const int m = m0 + r;
+        float a = 0.f, c = 0.f;
+        if (row_live(p.active, m)) {
+          const float x1 = tile[r * kFTile + lane], x2 = tile[r * kFTile + 32 + lane];
+          const float pos = p.pos_of ? (float)(p.pos_of[m] + p.pos_shift) : 0.f;
+          float sn, cs;
+          sincosf(pos * inv, &sn, &cs);
+          a = x1 * cs - x2 * sn;
+          c = x1 * sn + x2 * cs;
+        }
+        __nv_bfloat16* dst =
+            head < p.Hq ? p.q + ((size_t)m * p.Hq + head) * kHd : p.kn + ((size_t)m * p.Hkv + head - p.Hq) * kHd;
+        dst[i] = __float2bfloat16_rn(a);
+        dst[i + kHd / 2] = __float2bfloat16_rn(c);
+      }
+    } else {
+      for (int i = tid; i < rows * kFN; i += kFThreads) {
+        const int r = i / kFN, c = i % kFN, m = m0 + r;
+        p.vn[(size_t)m * p.Hkv * kHd + (t - rot) * kFN + c] =
+            __float2bfloat16_rn(row_live(p.active, m) ? tile[r * kFTile + c] : 0.f);
+      }
     }
-    __nv_bfloat16* dst = head < Hq ? q + ((size_t)m * Hq + head) * kHd : kn + ((size_t)m * Hkv + head - Hq) * kHd;
-    dst[i] = __float2bfloat16_rn(a);
-    dst[i + kHd / 2] = __float2bfloat16_rn(c);
-  }
-  for (int j = threadIdx.x; j < Hkv * kHd; j += blockDim.x)
-    vn[(size_t)m * Hkv * kHd + j] =
-        __float2bfloat16_rn(live ? sum_partials(P, splits, M, N, m, (Hq + Hkv) * kHd + j) : 0.f);
-}
-
-// SwiGLU epilogue: u[m][n] = SiLU(z[m][n]) * z[m][F + n] in bf16 (z = W_13 u, F wide halves).
-__global__ void __launch_bounds__(kRowThreads) k_swiglu_epilogue(const float* __restrict__ P, int splits, int M, int F,
-                                                                 const int* __restrict__ active,
-                                                                 __nv_bfloat16* __restrict__ u) {
-  pdl_wait();
-  pdl_launch_dependents();
-  const int m = blockIdx.x;
-  const bool live = row_live(active, m);
-  for (int n = threadIdx.x; n < F; n += blockDim.x) {
-    float y = 0.f;
-    if (live) {
-      const float g1 = sum_partials(P, splits, M, 2 * F, m, n), g3 = sum_partials(P, splits, M, 2 * F, m, F + n);
-      y = g1 / (1.0f + expf(-g1)) * g3;
+  } else if (E == kEResid) {
+    for (int i = tid; i < rows * kFN; i += kFThreads) {
+      const int r = i / kFN, c = i % kFN, m = m0 + r;
+      if (row_live(p.active, m)) p.x[(size_t)m * p.d + t * kFN + c] += tile[r * kFTile + c];
     }
-    u[(size_t)m * F + n] = __float2bfloat16_rn(y);
+  } else {
+    for (int i = tid; i < rows * 32; i += kFThreads) {
+      const int r = i / 32, c = i % 32, m = m0 + r;
+      if (!row_live(p.active, m)) continue;
+      const float g1 = tile[r * kFTile + c], g3 = tile[r * kFTile + 32 + c];
+      p.u[(size_t)m * p.F + t * 32 + c] = __float2bfloat16_rn(g1 / (1.0f + expf(-g1)) * g3);
+    }
   }
-}
-
-// Attention outputs (fp32) to the bf16 operand of W_o.
-__global__ void k_to_bf16(const float* __restrict__ a, size_t n, __nv_bfloat16* __restrict__ u) {
-  pdl_wait();
-  pdl_launch_dependents();
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    u[i] = __float2bfloat16_rn(a[i]);
 }
 
 // Attention of the first position alone (the seed row): softmax over one key is 1, so
 // query head h returns the value of KV head h / G.
 __global__ void k_first_position_attention(const __nv_bfloat16* __restrict__ vn, int Hq, int G,
-                                           __nv_bfloat16* __restrict__ u) {
+                                           float* __restrict__ att) {
   pdl_wait();
   pdl_launch_dependents();
-  for (int j = threadIdx.x; j < Hq * kHd; j += blockDim.x) u[j] = vn[(j / kHd / G) * kHd + j % kHd];
+  for (int j = threadIdx.x; j < Hq * kHd; j += blockDim.x) att[j] = __bfloat162float(vn[(j / kHd / G) * kHd + j % kHd]);
 }
 
 struct Run {
@@ -369,12 +585,15 @@ struct Run {
     return splits;
   }
 
-  template <int Mode>
-  void rows(int splits, int M, const float* g, const float* b, const int* active, const float* w_out,
-            const float* b_out, float* score) {
-    launch_pdl(k_row_epilogue<Mode>, M, kRowThreads, s.d * sizeof(float), st, part(), splits, M, s.d, x(), g, b,
-               active, u(), w_out, b_out, score);
+  // One fused product of `tiles` 64-column tiles.
+  template <int A, int E>
+  bool fused(FusedArgs p, int tiles) {
+    p.ctl = pool->view.ctl;
+    p.mt = 32;
+    while (p.mt < 128 && (p.M + p.mt - 1) / p.mt * tiles > pool->num_sms) p.mt *= 2;
+    if (set_max_dynamic_smem(reinterpret_cast<const void*>(k_fused_gemm<A, E>), kFSmem) != cudaSuccess) return false;
     ++launches;
+    return launch_pdl(k_fused_gemm<A, E>, dim3((p.M + p.mt - 1) / p.mt, tiles), kFThreads, kFSmem, st, p) == cudaSuccess;
   }
 
   // The layer stack on M rows.  step = true: rows are the step pool's slots, attention
@@ -382,62 +601,84 @@ struct Run {
   // slots' sequence lengths.  step = false: one row at position 0 (the seed), whose
   // per-layer k and v go to the seed buffers.
   bool layers(int M, bool step, const int* active, float* score) {
-    const int* pos_of = step ? pool->view.seq_len : nullptr;
+    float* att = reinterpret_cast<float*>(ws + L.att);
+    __nv_bfloat16* q = reinterpret_cast<__nv_bfloat16*>(ws + L.q);
+    FusedArgs base{};
+    base.M = M;
+    base.active = active;
+    base.x = x();
+    base.d = s.d;
     for (int l = 0; l < s.L; ++l) {
-      int sp = gemm(u(), M, wt<__nv_bfloat16>(layer_tensor(l, kWqkv)), s.Nqkv, s.d);
-      if (!sp) return false;
-      __nv_bfloat16* q = reinterpret_cast<__nv_bfloat16*>(ws + L.q);
       __nv_bfloat16* kn = reinterpret_cast<__nv_bfloat16*>(ws + (step ? L.kn : L.seedk)) +
                           (step ? 0 : (size_t)l * s.Hkv * kHd);
       __nv_bfloat16* vn = reinterpret_cast<__nv_bfloat16*>(ws + (step ? L.vn : L.seedv)) +
                           (step ? 0 : (size_t)l * s.Hkv * kHd);
-      // Layer 0 opens the step pool's step, which advances every length by one: the new
-      // position is seq_len before layer 0 and seq_len - 1 after it.
-      launch_pdl(k_qkv_epilogue, M, kRowThreads, 0, st, part(), sp, M, s.Hq, s.Hkv, pos_of, l > 0 ? -1 : 0, active,
-                 q, kn, vn);
-      ++launches;
+      // q, k, v = RoPE(W_qkv LN1(x)).  Layer 0 opens the step pool's step, which advances every
+      // length by one: the new position is seq_len before layer 0 and seq_len - 1 after it.
+      FusedArgs p = base;
+      p.a = x();
+      p.g = wt<float>(layer_tensor(l, kLn1G));
+      p.b = wt<float>(layer_tensor(l, kLn1B));
+      p.w = wt<__nv_bfloat16>(layer_tensor(l, kWqkv));
+      p.K = s.d;
+      p.q = q;
+      p.kn = kn;
+      p.vn = vn;
+      p.Hq = s.Hq;
+      p.Hkv = s.Hkv;
+      p.pos_of = step ? pool->view.seq_len : nullptr;
+      p.pos_shift = l > 0 ? -1 : 0;
+      if (!fused<kALn, kEQkv>(p, s.Nqkv / kFN)) return false;
       if (!step && l + 1 == s.L) break;  // the seed needs only each layer's k and v
       if (step) {
-        float* att = reinterpret_cast<float*>(ws + L.att);
         if (gb_decode_attention(pool, l, q, kn, vn, 0.08838834764831845f, att, GB_PATH_AUTO,
                                 reinterpret_cast<gb_stream_t>(st)) != GB_OK)
           return false;
-        const size_t n = (size_t)M * s.d;
-        launch_pdl(k_to_bf16, (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096), 256, 0, st,
-                   static_cast<const float*>(att), n, u());
       } else {
-        k_first_position_attention<<<1, kRowThreads, 0, st>>>(vn, s.Hq, s.G, u());
+        launch_pdl(k_first_position_attention, 1, kRowThreads, 0, st, static_cast<const __nv_bfloat16*>(vn), s.Hq, s.G,
+                   att);
+        ++launches;
       }
+      p = base;  // x += W_o a
+      p.a = att;
+      p.w = wt<__nv_bfloat16>(layer_tensor(l, kWo));
+      p.K = s.d;
+      if (!fused<kAF32, kEResid>(p, s.d / kFN)) return false;
+      p = base;  // u = SiLU(W_1 LN2(x)) * W_3 LN2(x)
+      p.a = x();
+      p.g = wt<float>(layer_tensor(l, kLn2G));
+      p.b = wt<float>(layer_tensor(l, kLn2B));
+      p.w = wt<__nv_bfloat16>(layer_tensor(l, kW13));
+      p.K = s.d;
+      p.u = u();
+      p.F = s.F;
+      if (!fused<kALn, kESwiglu>(p, s.F / 32)) return false;
+      p = base;  // x += W_2 u
+      p.a = u();
+      p.w = wt<__nv_bfloat16>(layer_tensor(l, kW2));
+      p.K = s.F;
+      if (!fused<kABf16, kEResid>(p, s.d / kFN)) return false;
+    }
+    if (step) {
+      launch_pdl(k_head, (M + kRowThreads / 32 - 1) / (kRowThreads / 32), kRowThreads, 0, st,
+                 static_cast<const float*>(x()), M, s.d, wt<float>(tail(0)), wt<float>(tail(1)), wt<float>(tail(2)),
+                 wt<float>(tail(3)), active, score);
       ++launches;
-      sp = gemm(u(), M, wt<__nv_bfloat16>(layer_tensor(l, kWo)), s.d, s.d);
-      if (!sp) return false;
-      rows<kResidLn>(sp, M, wt<float>(layer_tensor(l, kLn2G)), wt<float>(layer_tensor(l, kLn2B)), active, nullptr,
-                     nullptr, nullptr);
-      sp = gemm(u(), M, wt<__nv_bfloat16>(layer_tensor(l, kW13)), 2 * s.F, s.d);
-      if (!sp) return false;
-      launch_pdl(k_swiglu_epilogue, M, kRowThreads, 0, st, part(), sp, M, s.F, active, u());
-      ++launches;
-      sp = gemm(u(), M, wt<__nv_bfloat16>(layer_tensor(l, kW2)), s.d, s.F);
-      if (!sp) return false;
-      if (l + 1 < s.L)
-        rows<kResidLn>(sp, M, wt<float>(layer_tensor(l + 1, kLn1G)), wt<float>(layer_tensor(l + 1, kLn1B)), active,
-                       nullptr, nullptr, nullptr);
-      else if (step)
-        rows<kResidHead>(sp, M, wt<float>(tail(0)), wt<float>(tail(1)), active, wt<float>(tail(2)),
-                         wt<float>(tail(3)), score);
     }
     return true;
   }
 
-  // Eq. 4 and LN1 of layer 0 on M rows of h.
+  // Eq. 4 on M rows of h.
   bool input(const void* h, int M, const int* active) {
     launch_pdl(k_ln_in, M, kRowThreads, s.H * sizeof(float), st, reinterpret_cast<const __nv_bfloat16*>(h), s.H,
                wt<float>(0), wt<float>(1), active, u());
     ++launches;
     const int sp = gemm(u(), M, wt<__nv_bfloat16>(2), s.d, s.H);
     if (!sp) return false;
-    rows<kGeluLn>(sp, M, wt<float>(layer_tensor(0, kLn1G)), wt<float>(layer_tensor(0, kLn1B)), active, nullptr,
-                  nullptr, nullptr);
+    const int n4 = M * (s.d / 4);
+    launch_pdl(k_gelu_epilogue, (n4 + kRowThreads - 1) / kRowThreads, kRowThreads, 0, st,
+               static_cast<const float*>(part()), sp, n4, x());
+    ++launches;
     return true;
   }
 };
