@@ -122,12 +122,31 @@ def ptr(x) -> int | None:
     return x.data_ptr()
 
 
+_torch = None         # the torch module once it has been imported
+_raw_stream = None    # () -> cudaStream_t of the current torch stream
+
+
+def _bind_torch(torch) -> None:
+    """Pick the cheapest way to the current stream: the raw-handle query where torch has it (0.3 us a
+    call; building a torch.cuda.Stream object costs 3 us, as much as the library call itself)."""
+    global _torch, _raw_stream
+    get_raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    get_device = getattr(torch._C, "_cuda_getDevice", None)
+    if get_raw is not None and get_device is not None:
+        _raw_stream = lambda: get_raw(get_device())  # noqa: E731
+    else:
+        _raw_stream = lambda: torch.cuda.current_stream().cuda_stream  # noqa: E731
+    _torch = torch
+
+
 def stream_handle(s) -> int | None:
     if s is None:
         try:
-            import torch
-            if torch.cuda.is_available() and torch.cuda.is_initialized():
-                return torch.cuda.current_stream().cuda_stream
+            if _torch is None:
+                import torch
+                _bind_torch(torch)
+            if _torch.cuda.is_initialized():
+                return _raw_stream()
         except Exception:
             pass
         return None
