@@ -142,9 +142,8 @@ gb_status gb_pool_seed(gb_pool* pool, int n_beams, int prompt_len, const void* k
  *   flags:      GB_PATH_AUTO / GB_PATH_PER_BEAM / GB_PATH_GROUPED
  * Rows of inactive slots in the inputs are ignored.
  * Launches: one attention launch that also appends the new rows and merges
- * the split and shared-prefix partial results into out_dev (bf16 pools; fp32
- * pools append and merge in launches of their own); layer 0 adds the step's
- * planner first.  The
+ * the split and shared-prefix partial results into out_dev; layer 0 adds the
+ * step's planner first.  The
  * attention launch's CTAs wait (bounded) on each other's partial results, so
  * they must all get an SM within the wait limit (2 s): nothing else should
  * hold the GPU's SMs for that long meanwhile.
@@ -294,10 +293,10 @@ gb_status gb_pool_read_state(gb_pool* pool, const gb_pool_state* state, gb_strea
  * (all of gb_prune_branch or gb_fork_slots, the shared-prefix segment rebuild included),
  * GB_PROF_GROUPED (the attention launch when it has the grouped shared-prefix role),
  * GB_PROF_PLAN (the step planner: page allocation and decode plans, layer 0),
- * GB_PROF_APPEND (the K/V append of a layer), GB_PROF_COMBINE (the separate merge of
- * partial results after the fp32 kernel; bf16 pools merge inside the attention launch) or
- * GB_PROF_ATTENTION (the attention of a layer, up to its merged output except for the fp32
- * kernel's separate merge).  Passing NULL events stops recording.  The events stay
+ * GB_PROF_APPEND (the K/V append launch of gb_append_kv; an empty interval in gb_decode_attention,
+ * whose attention launch appends), GB_PROF_COMBINE (an empty interval: every attention launch
+ * merges its partial results itself) or GB_PROF_ATTENTION (the attention of a layer, up to its
+ * merged output).  Passing NULL events stops recording.  The events stay
  * owned by the caller.  Under stream capture the records become external event
  * nodes of the graph.
  */

@@ -59,18 +59,19 @@ __device__ __forceinline__ bool wait_pair_records(const PoolView& v, const Count
   }
 }
 
-// The running state of one pair's merge (one warp; lane l owns the elements 4l .. 4l + 3 of
-// every head g of the pair).
-template <int G>
+// The running state of one pair's merge (one warp; lane l owns the float4 elements l + 32 j of the
+// pair's G heads of D dims, so with D = 128 element j belongs to head j).
+template <int G, int D>
 struct MergeState {
-  float M[G], L[G];
-  float4 acc[G];
+  static constexpr int N = G * D / 128;
+  float M[N], L[N];
+  float4 acc[N];
 };
 
-template <int G>
-__device__ __forceinline__ void merge_init(MergeState<G>& st) {
+template <int G, int D>
+__device__ __forceinline__ void merge_init(MergeState<G, D>& st) {
 #pragma unroll
-  for (int g = 0; g < G; ++g) {
+  for (int g = 0; g < MergeState<G, D>::N; ++g) {
     st.M[g] = -INFINITY;
     st.L[g] = 0.f;
     st.acc[g] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -79,28 +80,29 @@ __device__ __forceinline__ void merge_init(MergeState<G>& st) {
 
 // Fold the records rec0, rec0 + stride, ... (cnt of them) into the state.  The records exist:
 // the caller waited for them.
-template <int G>
-__device__ __forceinline__ void merge_fold(MergeState<G>& st, const float* rec0, size_t stride, int cnt) {
-  constexpr int D = 128, GD = G * D;
-  constexpr int RB = G >= 8 ? 1 : 16 / G;  // records per batch of loads: 8-16 float4 in flight per lane
+template <int G, int D>
+__device__ __forceinline__ void merge_fold(MergeState<G, D>& st, const float* rec0, size_t stride, int cnt) {
+  constexpr int GD = G * D, N = MergeState<G, D>::N;
+  constexpr int RB = N >= 8 ? 1 : 16 / N;  // records per batch of loads: 8-16 float4 in flight per lane
   const int lane = threadIdx.x & 31;
   for (int r0 = 0; r0 < cnt; r0 += RB) {
-    float4 x[RB][G];
-    float mk[RB][G], lk[RB][G];
+    float4 x[RB][N];
+    float mk[RB][N], lk[RB][N];
 #pragma unroll
     for (int k = 0; k < RB; ++k) {
       if (r0 + k < cnt) {
         // L2 loads: the records were written by other SMs during this launch.
         const float* rec = rec0 + (size_t)(r0 + k) * stride;
 #pragma unroll
-        for (int g = 0; g < G; ++g) {
-          x[k][g] = __ldcg(reinterpret_cast<const float4*>(rec + g * D) + lane);
-          mk[k][g] = __ldcg(rec + GD + g);
-          lk[k][g] = __ldcg(rec + GD + G + g);
+        for (int g = 0; g < N; ++g) {
+          const int head = 4 * (lane + 32 * g) / D;
+          x[k][g] = __ldcg(reinterpret_cast<const float4*>(rec) + lane + 32 * g);
+          mk[k][g] = __ldcg(rec + GD + head);
+          lk[k][g] = __ldcg(rec + GD + G + head);
         }
       } else {
 #pragma unroll
-        for (int g = 0; g < G; ++g) {
+        for (int g = 0; g < N; ++g) {
           x[k][g] = make_float4(0.f, 0.f, 0.f, 0.f);
           mk[k][g] = -INFINITY;  // a record that saw no token (or none at all) adds nothing
           lk[k][g] = 0.f;
@@ -108,7 +110,7 @@ __device__ __forceinline__ void merge_fold(MergeState<G>& st, const float* rec0,
       }
     }
 #pragma unroll
-    for (int g = 0; g < G; ++g) {
+    for (int g = 0; g < N; ++g) {
       float mnew = st.M[g];
 #pragma unroll
       for (int k = 0; k < RB; ++k) mnew = fmaxf(mnew, mk[k][g]);
@@ -136,18 +138,17 @@ __device__ __forceinline__ void merge_fold(MergeState<G>& st, const float* rec0,
 }
 
 // out[b][h * G + g][:] = acc / L.
-template <int G>
-__device__ __forceinline__ void merge_write(const PoolView& v, const MergeState<G>& st, int b, int h,
+template <int G, int D>
+__device__ __forceinline__ void merge_write(const PoolView& v, const MergeState<G, D>& st, int b, int h,
                                             float* __restrict__ out) {
-  constexpr int D = 128;
   const int lane = threadIdx.x & 31;
   float* ob = out + ((size_t)b * v.Hq + (size_t)h * G) * D;
   const bool vec_out = (reinterpret_cast<uintptr_t>(out) & 15) == 0;
 #pragma unroll
-  for (int g = 0; g < G; ++g) {
+  for (int g = 0; g < MergeState<G, D>::N; ++g) {
     const float4 res = make_float4(st.acc[g].x / st.L[g], st.acc[g].y / st.L[g], st.acc[g].z / st.L[g],
                                    st.acc[g].w / st.L[g]);
-    float* d = ob + g * D + 4 * lane;
+    float* d = ob + 4 * (lane + 32 * g);
     if (vec_out) {
       *reinterpret_cast<float4*>(d) = res;
     } else {
@@ -160,18 +161,18 @@ __device__ __forceinline__ void merge_write(const PoolView& v, const MergeState<
 }
 
 // Zero the output rows of pair (b, h) (an inactive beam, or a failed wait).
-template <int G>
+template <int G, int D = 128>
 __device__ __forceinline__ void zero_pair(const PoolView& v, int b, int h, float* __restrict__ out) {
-  float* ob = out + ((size_t)b * v.Hq + (size_t)h * G) * 128;
-  for (int e = threadIdx.x & 31; e < G * 128; e += 32) ob[e] = 0.f;
+  float* ob = out + ((size_t)b * v.Hq + (size_t)h * G) * D;
+  for (int e = threadIdx.x & 31; e < G * D; e += 32) ob[e] = 0.f;
 }
 
 // A step that was refused (no pages) has no attention: its outputs are zero.
-template <int G>
+template <int G, int D = 128>
 __device__ __forceinline__ void zero_all_pairs(const PoolView& v, int cta, int nctas, float* __restrict__ out) {
   const int nw = blockDim.x >> 5;
   for (int p = cta * nw + (int)(threadIdx.x >> 5); p < v.max_beams * v.Hkv; p += nctas * nw)
-    zero_pair<G>(v, p / v.Hkv, p % v.Hkv, out);
+    zero_pair<G, D>(v, p / v.Hkv, p % v.Hkv, out);
 }
 
 // The merge phase of an attention launch, run by every warp of the merging CTAs after its own
@@ -181,7 +182,7 @@ __device__ __forceinline__ void zero_all_pairs(const PoolView& v, int cta, int n
 // that start at different times) and fold a pair's segment records before they wait for its
 // split-KV records; otherwise merging CTA `cta` of `nctas` takes the pairs
 // p = cta + nctas * (warp + k * warps per CTA) and waits for all of a pair's records at once.
-template <int G>
+template <int G, int D = 128>
 __device__ __forceinline__ void combine_pairs(const PoolView& v, const Counters& cnt, int mode, int W, int ng,
                                               bool claim, int cta, int nctas, float* __restrict__ out) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -206,12 +207,12 @@ __device__ __forceinline__ void combine_pairs(const PoolView& v, const Counters&
     const int first = o0 / c;
     const int npb = n > 0 ? (o0 + n - 1) / c - first + 1 : 0;
     if (npb + nseg == 0) {
-      zero_pair<G>(v, b, h, out);
+      zero_pair<G, D>(v, b, h, out);
       continue;
     }
     const float* grec = v.grec + ((size_t)b * kMaxSegRecords * v.Hkv + h) * rf;  // [b][record][Hkv]
     const float* prec = v.partials + (size_t)(first + p) * rf;                     // first + p, ...
-    MergeState<G> st;
+    MergeState<G, D> st;
     merge_init(st);
     bool good;
     if (claim) {
@@ -230,7 +231,7 @@ __device__ __forceinline__ void combine_pairs(const PoolView& v, const Counters&
       merge_write(v, st, b, h, out);
     } else {
       if (lane == 0) set_status(v.ctl, GB_ERR_TIMEOUT);  // kept if already set
-      zero_pair<G>(v, b, h, out);
+      zero_pair<G, D>(v, b, h, out);
     }
   }
 }

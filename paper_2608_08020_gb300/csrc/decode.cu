@@ -68,7 +68,7 @@ struct DecodeSmem {
   // Rounded to 128 bytes so every warp's stages start 16-byte aligned (bulk-copy destinations).
   static constexpr int WARP_BYTES = (kDecodeStages * T::STAGE_BYTES + PBUF + 8 * kDecodeStages + 127) / 128 * 128;
   static_assert(WARP_BYTES % 128 == 0 && T::STAGE_BYTES % 16 == 0, "stage alignment");
-  static constexpr int PLAN_BYTES = 3 * (kMaxBeams + 1) * 4;
+  static constexpr int PLAN_BYTES = 5 * (kMaxBeams + 1) * 4;  // offsets, chunk counts, start tokens, lengths, copied-from pages
   static constexpr int TOTAL = kDecodeWarps * WARP_BYTES + PLAN_BYTES;
 };
 
@@ -85,11 +85,11 @@ __device__ __forceinline__ void unpack16x2(const uint4& u, float2* f) {
   }
 }
 
-template <int DT, int G>
-__global__ void __launch_bounds__(kDecodeWarps * 32, 1)
-    k_decode(PoolView v, int layer, const void* __restrict__ qptr, float qscale, int mode, int W) {
-  pdl_wait();
-  pdl_launch_dependents();
+// The kernels' body (plan 0, W warps).  Pool: the step's new rows are appended on the way, as in
+// decode_mma_body, and every record is counted for the merge.
+template <int DT, int G, bool Pool>
+__device__ __forceinline__ void decode_body(const PoolView& v, const Counters& cnt, int layer,
+                                            const void* __restrict__ qptr, const NewRows& nw, float qscale, int W) {
   using T = KvTraits<DT>;
   using S = DecodeSmem<DT, G>;
   constexpr int NS = G / 2;  // scores held per lane after the reduce-scatter
@@ -99,15 +99,20 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
   int* s_off = reinterpret_cast<int*>(smem + kDecodeWarps * S::WARP_BYTES);
   int* s_n = s_off + (kMaxBeams + 1);
   int* s_start = s_n + (kMaxBeams + 1);
-  if (v.ctl[kCtlStepOk] == 0) return;
+  int* s_len = s_start + (kMaxBeams + 1);
+  int* s_cow = s_len + (kMaxBeams + 1);
   {
-    const int* off = plan_off(v, mode);
-    const int* nn = plan_n(v, mode);
-    const int* st = plan_start(v, mode);
+    const int* off = plan_off(v, 0);
+    const int* nn = plan_n(v, 0);
+    const int* st = plan_start(v, 0);
     for (int i = threadIdx.x; i <= v.max_beams; i += blockDim.x) {
       s_off[i] = off[i];
       s_n[i] = i < v.max_beams ? nn[i] : 0;
       s_start[i] = i < v.max_beams ? st[i] : 0;
+      if (Pool) {
+        s_len[i] = i < v.max_beams ? v.seq_len[i] : 0;
+        s_cow[i] = i < v.max_beams ? v.cow_old[i] : -1;
+      }
     }
   }
   __syncthreads();
@@ -159,7 +164,11 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
       pw_b = q.b;
       pw_i0 = q.i;
       const int i = pw_i0 + lane;
-      pw_lane = i < q.n ? v.tables[(size_t)q.b * v.max_pages + (q.tok0 + i * kChunk) / v.P] : 0;
+      const int pi = (q.tok0 + i * kChunk) / v.P;
+      const int old = Pool ? s_cow[q.b] : -1;  // of the tail page, which holds the new token
+      pw_lane = i >= q.n ? 0
+                : old >= 0 && pi == (s_len[q.b] - 1) / v.P ? old
+                                                           : v.tables[(size_t)q.b * v.max_pages + pi];
     }
     return __shfl_sync(0xffffffffu, pw_lane, q.i - pw_i0);
   };
@@ -202,12 +211,18 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
   float l_lane[NS];
   int L = 0;
   bool fresh = true;
+  uint4 nrow = make_uint4(0u, 0u, 0u, 0u);  // 16 bytes of the pair's new rows: lanes 0-15 K, 16-31 V
+  int npage = 0;                            // the page they go to
   const char* qbase = static_cast<const char*>(qptr);
 
   for (int x = x_begin, k = 0; x < x_end; ++x, ++k) {
     if (fresh) {
       // New (beam, head): load the G query rows for this lane's dims, pre-scaled.
-      L = v.seq_len[it.b];
+      L = Pool ? s_len[it.b] : v.seq_len[it.b];
+      if (Pool && it.n - it.i <= x_end - x) {  // this warp holds the pair's last chunk
+        nrow = (lane < 16 ? nw.k : nw.v)[((size_t)it.b * v.Hkv + it.h) * 16 + (lane & 15)];
+        npage = v.tables[(size_t)it.b * v.max_pages + (L - 1) / v.P];
+      }
 #pragma unroll
       for (int g = 0; g < G; ++g) {
         const char* qrow = qbase + ((size_t)(it.b * v.Hq + it.h * G + g) * D) * T::ES;
@@ -241,6 +256,29 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
     const unsigned char* Vs = Ks + T::SLAB_BYTES;
     const int tok0 = it.tok0 + it.i * kChunk;
     const bool partial = tok0 + kChunk > L;
+    if constexpr (Pool) {
+      const int kv = lane >> 4, piece = lane & 15;
+      unsigned char* slab = wsm + stage * T::STAGE_BYTES + kv * T::SLAB_BYTES;
+      if (it.i == it.n - 1) {
+        // The step's new token is the chunk's last valid one: its row goes into the landed stage
+        // and into the pool.
+        reinterpret_cast<uint4*>(slab + (L - 1 - tok0) * T::ROW_BYTES)[piece] = nrow;
+        if (npage >= 0 && npage < v.num_pages)
+          reinterpret_cast<uint4*>(v.kv + kv_elem_offset(v, layer, npage, kv, it.h, (L - 1) % v.P) * T::ES)[piece] = nrow;
+        else if (lane == 0)
+          set_status(v.ctl, GB_ERR_INVALID);
+        fence_proxy_async_smem();  // ordered before the copy that later refills this stage
+        __syncwarp();
+      }
+      if (s_cow[it.b] >= 0 && tok0 / v.P == (L - 1) / v.P) {
+        // A chunk of a tail page copied on write: its rows before the new one go to the new page.
+        const int page = v.tables[(size_t)it.b * v.max_pages + (L - 1) / v.P];
+        if (page >= 0 && page < v.num_pages)
+          for (int t = 0; t < min(kChunk, L - 1 - tok0); ++t)
+            reinterpret_cast<uint4*>(v.kv + kv_elem_offset(v, layer, page, kv, it.h, (tok0 + t) % v.P) * T::ES)[piece] =
+                reinterpret_cast<const uint4*>(slab + t * T::ROW_BYTES)[piece];
+      }
+    }
 
     // ---- scores: 4 tokens per row, G heads each --------------------------
     float acc[4 * G];
@@ -405,10 +443,43 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
           rec[G * D + G + g] = ((g / NS) == b0) ? lsum[g % NS] : lother[g % NS];
         }
       }
+      if (Pool) record_arrive(cnt, it.b * v.Hkv + it.h, lane);
       fresh = true;
     }
     if (x + 1 < x_end) iter_advance(it, s_n, s_start, v.Hkv, v.max_beams);
   }
+}
+
+// Caller-owned rows: the records are merged by k_combine.
+template <int DT, int G>
+__global__ void __launch_bounds__(kDecodeWarps * 32, 1)
+    k_decode(PoolView v, const void* __restrict__ qptr, float qscale, int W) {
+  pdl_wait();
+  pdl_launch_dependents();
+  decode_body<DT, G, false>(v, Counters{}, 0, qptr, NewRows{}, qscale, W);
+}
+
+// A layer-step of an fp32 pool (or a bf16 one too large for a tensor map) in one launch: append,
+// attention and the merge (combine.cuh; one CTA per SM, so every CTA is resident and the merge's
+// waits end).  With launches of its own for the append and the merge a step of 8 beams x 256 tokens
+// took 11.8 us, half of it between kernels.
+template <int DT, int G>
+__global__ void __launch_bounds__(kDecodeWarps * 32, 1)
+    k_decode_pool(PoolView v, int layer, const void* __restrict__ qptr, NewRows nw, float qscale,
+                  float* __restrict__ out) {
+  pdl_wait();
+  pdl_launch_dependents();
+  constexpr int D = KvTraits<DT>::D;
+  const int c = (int)blockIdx.x, nctas = (int)gridDim.x;
+  if (v.ctl[kCtlStepOk] == 0) {
+    zero_all_pairs<G, D>(v, c, nctas, out);
+    return;
+  }
+  const int set = counter_set(v, layer), W = nctas * kDecodeWarps;
+  const Counters cnt = counters(v, set);
+  zero_counters(v, set ^ 1, c, nctas);
+  decode_body<DT, G, true>(v, cnt, layer, qptr, nw, qscale, W);
+  combine_pairs<G, D>(v, cnt, 0, W, 0, false, c, nctas, out);
 }
 
 // The per-beam kernel on its own (the per-beam path, every beam reading its whole context):
@@ -437,16 +508,16 @@ __global__ void __launch_bounds__(kMmaWarps * 32, 1)
   combine_pairs<G>(v, cnt, mode, nctas * kMmaWarps, 0, false, c, nctas, out);
 }
 
-// Merge the partial records of each (beam, kv head) into out[b][h*G+g][:]: the split-KV
-// records of the warps that covered the beam's range (the log-sum-exp merge, base 2), after
-// the fp32 kernel k_decode (the bf16 kernels merge their records themselves, combine.cuh).
+// Merge the partial records of each (row, kv head) into out[b][h*G+g][:]: the split-KV
+// records of the warps that covered the row's range (the log-sum-exp merge, base 2), after
+// k_decode on caller-owned rows (the pools' kernels merge their records themselves, combine.cuh).
 // One CTA of 128 threads per (beam, kv head); thread t owns 4 consecutive output elements
 // of one query head g and folds all records in one pass, 8 records of loads in flight at a
 // time: M = running max of the records' m, acc = sum o * 2^(m - M), L = sum l * 2^(m - M),
 // rescaled when M rises.  Every thread of a warp reads the same (m, l) words (one head per
 // warp at D = 128, two at D = 64), so those loads are broadcasts; the o loads are float4
 // and coalesced.
-__global__ void __launch_bounds__(128) k_combine(PoolView v, int mode, int W, float* __restrict__ out) {
+__global__ void __launch_bounds__(128) k_combine(PoolView v, int W, float* __restrict__ out) {
   pdl_wait();
   pdl_launch_dependents();
   const int bh = blockIdx.x;
@@ -454,14 +525,14 @@ __global__ void __launch_bounds__(128) k_combine(PoolView v, int mode, int W, fl
   const int G = v.G, D = v.D, GD = G * D;
   float* ob = out + ((size_t)b * v.Hq + (size_t)h * G) * D;
   const bool ok = v.ctl[kCtlStepOk] != 0 && v.active[b] != 0;
-  const int n = ok ? plan_n(v, mode)[b] : 0;
+  const int n = ok ? plan_n(v, 0)[b] : 0;
   if (n == 0) {
     for (int e = threadIdx.x; e < GD; e += blockDim.x) ob[e] = 0.f;
     return;
   }
-  const int Tot = plan_off(v, mode)[v.max_beams];
+  const int Tot = plan_off(v, 0)[v.max_beams];
   const int c = Tot > 0 ? (Tot + W - 1) / W : 1;
-  const int off = plan_off(v, mode)[b] + h * n;
+  const int off = plan_off(v, 0)[b] + h * n;
   const int first = off / c, npb = n > 0 ? (off + n - 1) / c - first + 1 : 0;  // per-beam records
   const int R = npb;
   const float* prec = v.partials + (size_t)(first + bh) * v.record_floats;
@@ -529,7 +600,7 @@ static cudaError_t launch_decode_t(gb_pool* pool, int layer, const void* q, cons
   using S = DecodeSmem<DT, G>;
   const float qscale = scale * 1.4426950408889634f;  // log2(e): softmax in base 2
   cudaError_t e;
-  if (fuses_append(pool)) {
+  if (DT == GB_BF16 && pool->have_dtmap && pool->num_sms * kMmaWarps <= kMaxDecodeWarps) {
     // One launch: the new rows, the attention roles and the merge of their records.
     if (mode == 1) {
       e = launch_attention(pool, layer, q, k_new, v_new, scale, out, allow_local, s);  // grouped and per-beam roles (grouped.cu)
@@ -549,18 +620,14 @@ static cudaError_t launch_decode_t(gb_pool* pool, int layer, const void* q, cons
     return e;
   }
   if (mode == 1) return cudaErrorInvalidValue;  // a grouped pool always has the per-beam tensor maps
-  const int W = pool->decode_warps;  // one CTA of kDecodeWarps warps per SM
-  e = set_max_dynamic_smem(reinterpret_cast<const void*>(k_decode<DT, G>), S::TOTAL);
+  e = set_max_dynamic_smem(reinterpret_cast<const void*>(k_decode_pool<DT, G>), S::TOTAL);
   if (e != cudaSuccess) return e;
   prof_begin(pool, GB_PROF_DECODE, s);
-  e = launch_pdl(k_decode<DT, G>, W / kDecodeWarps, kDecodeWarps * 32, S::TOTAL, s, pool->view, layer, q, qscale,
-                 mode, W);
+  e = launch_pdl(k_decode_pool<DT, G>, pool->decode_warps / kDecodeWarps, kDecodeWarps * 32, S::TOTAL, s, pool->view,
+                 layer, q, NewRows{static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new)}, qscale, out);
   prof_end(pool, GB_PROF_DECODE, s);
-  pool->launches += 1;
-  if (e != cudaSuccess) return e;
   prof_end(pool, GB_PROF_ATTENTION, s);
-  prof_begin(pool, GB_PROF_COMBINE, s);
-  e = launch_pdl(k_combine, pool->view.max_beams * pool->view.Hkv, 128, 0, s, pool->view, mode, W, out);
+  prof_begin(pool, GB_PROF_COMBINE, s);  // an empty interval: the launch merges its records itself
   prof_end(pool, GB_PROF_COMBINE, s);
   pool->launches += 1;
   return e;
@@ -582,42 +649,30 @@ cudaError_t launch_wait_selftest(gb_pool* pool, cudaStream_t s) {
 // Split-KV decode + combine on an explicit view (plan mode 0, W warps), for callers
 // that supply their own tables and scratch instead of a pool.
 template <int DT, int G>
-static cudaError_t launch_view_t(const PoolView& v, int W, int layer, const void* q, float scale, float* out,
-                                 cudaStream_t s) {
+static cudaError_t launch_view_t(const PoolView& v, int W, const void* q, float scale, float* out, cudaStream_t s) {
   using S = DecodeSmem<DT, G>;
-  {
-    const cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(k_decode<DT, G>), S::TOTAL);
-    if (e != cudaSuccess) return e;
-  }
-  const float qscale = scale * 1.4426950408889634f;
-  k_decode<DT, G><<<W / kDecodeWarps, kDecodeWarps * 32, S::TOTAL, s>>>(v, layer, q, qscale, 0, W);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(k_decode<DT, G>), S::TOTAL);
   if (e != cudaSuccess) return e;
-  k_combine<<<v.max_beams * v.Hkv, 128, 0, s>>>(v, 0, W, out);
-  return cudaGetLastError();
+  e = launch_pdl(k_decode<DT, G>, W / kDecodeWarps, kDecodeWarps * 32, S::TOTAL, s, v, q, scale * 1.4426950408889634f, W);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k_combine, v.max_beams * v.Hkv, 128, 0, s, v, W, out);
 }
 
-cudaError_t launch_decode_view(const PoolView& v, int W, int layer, const void* q, float scale, float* out,
-                               cudaStream_t s) {
+cudaError_t launch_decode_view(const PoolView& v, int W, const void* q, float scale, float* out, cudaStream_t s) {
   if (v.dtype == GB_BF16) {
     switch (v.G) {
-      case 2: return launch_view_t<GB_BF16, 2>(v, W, layer, q, scale, out, s);
-      case 4: return launch_view_t<GB_BF16, 4>(v, W, layer, q, scale, out, s);
-      case 8: return launch_view_t<GB_BF16, 8>(v, W, layer, q, scale, out, s);
+      case 2: return launch_view_t<GB_BF16, 2>(v, W, q, scale, out, s);
+      case 4: return launch_view_t<GB_BF16, 4>(v, W, q, scale, out, s);
+      case 8: return launch_view_t<GB_BF16, 8>(v, W, q, scale, out, s);
     }
   } else {
     switch (v.G) {
-      case 2: return launch_view_t<GB_F32, 2>(v, W, layer, q, scale, out, s);
-      case 4: return launch_view_t<GB_F32, 4>(v, W, layer, q, scale, out, s);
-      case 8: return launch_view_t<GB_F32, 8>(v, W, layer, q, scale, out, s);
+      case 2: return launch_view_t<GB_F32, 2>(v, W, q, scale, out, s);
+      case 4: return launch_view_t<GB_F32, 4>(v, W, q, scale, out, s);
+      case 8: return launch_view_t<GB_F32, 8>(v, W, q, scale, out, s);
     }
   }
   return cudaErrorInvalidValue;
-}
-
-// bf16 pools with the per-beam tensor maps: the warp-MMA kernels, which append as they go.
-bool fuses_append(const gb_pool* pool) {
-  return pool->view.dtype == GB_BF16 && pool->have_dtmap && pool->num_sms * kMmaWarps <= kMaxDecodeWarps;
 }
 
 cudaError_t launch_decode(gb_pool* pool, int layer, const void* q, const void* k_new, const void* v_new, float scale,

@@ -331,15 +331,12 @@ cudaError_t set_max_dynamic_smem(const void* kernel, int bytes);
 
 // Kernel launchers implemented in the other translation units.
 // The attention of one layer-step on s, written to out: mode 0, the per-beam kernel; mode 1,
-// the attention kernel with the grouped and per-beam roles (launch_attention).  The bf16
-// kernels merge their records themselves; the fp32 kernel is followed by k_combine.
-// With k_new/v_new the launch also writes the step's new rows into the pool (fuses_append(pool));
-// without them k_append has written them before.
+// the attention kernel with the grouped and per-beam roles (launch_attention).  Every kernel
+// merges its records itself.
+// The launch also writes the step's new rows into the pool.
 cudaError_t launch_decode(gb_pool* pool, int layer, const void* q, const void* k_new, const void* v_new, float scale,
                           float* out, int mode, bool allow_local, cudaStream_t s);
-bool fuses_append(const gb_pool* pool);
-cudaError_t launch_decode_view(const PoolView& v, int W, int layer, const void* q, float scale, float* out,
-                               cudaStream_t s);
+cudaError_t launch_decode_view(const PoolView& v, int W, const void* q, float scale, float* out, cudaStream_t s);
 cudaError_t rebuild_segments(gb_pool* pool, cudaStream_t s);
 cudaError_t launch_attention(gb_pool* pool, int layer, const void* q, const void* k_new, const void* v_new, float scale,
                              float* out, bool allow_local, cudaStream_t s);

@@ -144,9 +144,8 @@ extern "C" gb_status gb_paged_decode_noalloc(const gb_paged_decode_args* a, gb_s
   v.record_floats = record_floats;
 
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  k_noalloc_plan<<<1, 1024, 0, s>>>(v);
-  if (cudaGetLastError() != cudaSuccess) return GB_ERR_CUDA;
-  if (launch_decode_view(v, W, 0, a->q, a->scale, a->out, s) != cudaSuccess) return GB_ERR_CUDA;
+  if (launch_pdl(k_noalloc_plan, 1, 1024, 0, s, v) != cudaSuccess) return GB_ERR_CUDA;
+  if (launch_decode_view(v, W, a->q, a->scale, a->out, s) != cudaSuccess) return GB_ERR_CUDA;
   return GB_OK;
 }
 

@@ -787,8 +787,7 @@ extern "C" gb_status gb_decode_attention(gb_pool* pool, int layer, const void* q
   if (!q_dev || !out_dev) return fail(pool, GB_ERR_INVALID, "decode: null pointer");
   if (flags < GB_PATH_AUTO || flags > GB_PATH_GROUPED) return fail(pool, GB_ERR_INVALID, "decode: bad flags");
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  const bool fused = fuses_append(pool);
-  gb_status st = append_layer(pool, layer, 1, k_new_dev, v_new_dev, fused, s);
+  gb_status st = append_layer(pool, layer, 1, k_new_dev, v_new_dev, true, s);
   if (st != GB_OK) return st;
   // Mode 1: shared-prefix segments go through the grouped tensor-core kernel and the
   // per-beam kernel reads only each beam's remainder; mode 0: every beam reads everything.
@@ -796,8 +795,8 @@ extern "C" gb_status gb_decode_attention(gb_pool* pool, int layer, const void* q
   // shares of the SMs (decode_ctas), or one after the other on every SM.
   const int mode = (flags == GB_PATH_PER_BEAM || !pool->view.grouped) ? 0 : 1;
   prof_begin(pool, GB_PROF_ATTENTION, s);
-  if (launch_decode(pool, layer, q_dev, fused ? k_new_dev : nullptr, fused ? v_new_dev : nullptr, scale, out_dev, mode,
-                    flags != GB_PATH_GROUPED, s) != cudaSuccess)
+  if (launch_decode(pool, layer, q_dev, k_new_dev, v_new_dev, scale, out_dev, mode, flags != GB_PATH_GROUPED, s) !=
+      cudaSuccess)
     return check_launch(pool, "decode");
   return check_launch(pool, "decode");
 }
