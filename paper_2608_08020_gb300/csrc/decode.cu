@@ -490,20 +490,23 @@ __global__ void __launch_bounds__(kMmaWarps * 32, 1)
     k_decode_mma(PoolView v, const __grid_constant__ CUtensorMap tm, const __grid_constant__ CUtensorMap tmh,
                  int layer, const __nv_bfloat16* __restrict__ q, NewRows nw, float qscale, int mode,
                  float* __restrict__ out) {
-  pdl_wait();
-  pdl_launch_dependents();
+  const bool early = layer > 0;
+  enter(!early);
   const int c = (int)blockIdx.x, nctas = (int)gridDim.x;
   if (v.ctl[kCtlStepOk] == 0) {
+    enter(early);
     zero_all_pairs<G>(v, c, nctas, out);
     return;
   }
   const int set = counter_set(v, layer);
-  const Counters cnt = counters(v, set);
-  zero_counters(v, set ^ 1, c, nctas);
   if (local_step_per_beam(v, nctas)) {
-    local_attention<G>(v, &tm, &tmh, layer, q, nw, qscale, c, nctas, out);
+    local_attention<G>(v, &tm, &tmh, layer, q, nw, qscale, c, nctas, out, early);
+    zero_counters(v, set ^ 1, c, nctas);
     return;
   }
+  enter(early);
+  const Counters cnt = counters(v, set);
+  zero_counters(v, set ^ 1, c, nctas);
   decode_mma_body<G>(v, cnt, &tm, &tmh, layer, q, nw, qscale, mode, c, nctas);
   combine_pairs<G>(v, cnt, mode, nctas * kMmaWarps, 0, false, c, nctas, out);
 }

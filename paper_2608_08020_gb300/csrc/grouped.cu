@@ -700,8 +700,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     k_attention(PoolView v, const __grid_constant__ CUtensorMap tmg, const __grid_constant__ CUtensorMap tmd,
                 const __grid_constant__ CUtensorMap tmdh, int layer, const __nv_bfloat16* __restrict__ q, NewRows nw,
                 float qscale, int w_oob, bool allow_local, float* __restrict__ out) {
-  pdl_wait();
-  pdl_launch_dependents();
+  const bool early = layer > 0;
+  enter(!early);
   // Grid of 2 S CTAs (S = SM count).  Large steps: CTAs [0, S) take the grouped role and
   // leave, CTAs [S, 2S) the per-beam role, each on an SM as a grouped CTA leaves it (CTAs
   // start in index order), and merge the records; a grouped CTA never waits, so every
@@ -710,16 +710,20 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   // without either role (local.cuh).
   const int S = (int)gridDim.x / 2, c = (int)blockIdx.x;
   if (v.ctl[kCtlStepOk] == 0) {
+    enter(early);
     zero_all_pairs<G>(v, c, 2 * S, out);
     return;
   }
   const int set = counter_set(v, layer);
-  const Counters cnt = counters(v, set);
-  zero_counters(v, set ^ 1, c, 2 * S);
   if (allow_local && local_step(v, S)) {
-    if (c < S) local_attention<G>(v, &tmd, &tmdh, layer, q, nw, qscale, c, S, out);
+    if (c >= S) return;
+    local_attention<G>(v, &tmd, &tmdh, layer, q, nw, qscale, c, S, out, early);
+    zero_counters(v, set ^ 1, c, S);
     return;
   }
+  enter(early);
+  const Counters cnt = counters(v, set);
+  zero_counters(v, set ^ 1, c, 2 * S);
   const int nd = decode_ctas(v, S), ng = nd < S ? S - nd : S;
   const bool split = nd < S;
   const int pb0 = split ? ng : S;  // first per-beam CTA

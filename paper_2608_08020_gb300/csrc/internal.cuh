@@ -194,6 +194,21 @@ __device__ __forceinline__ long long kv_elem_offset(const PoolView& v, int layer
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Small attention steps (local.cuh) of layers above 0 begin before the previous kernel has
+// completed: the step's plan, tables and every K/V row but the step's own were final when layer 0's
+// launch began (each kernel of the library lets its dependents go only after its own pdl_wait, so
+// all but the directly preceding kernel have completed by then, and no call between the layers of
+// a step changes them), so page ids and the first K/V loads go out while the kernel that makes q
+// and the new rows drains.  `early` threads wait here, before they read q, the new rows or the
+// counters, and before any global write.  (The same in the roles of large steps gained nothing:
+// the next launch's loads then compete with the tail of this one.)
+__device__ __forceinline__ void enter(bool early) {
+  if (early) {
+    pdl_wait();
+    pdl_launch_dependents();
+  }
+}
+
 __device__ __forceinline__ bool split_sms(const PoolView& v, long long td, long long tg) {
   const long long bytes = (td + tg) * 2 * v.D * v.esize;
   return td > 0 && tg > 0 && bytes < GB_SPLIT_BYTES_PER_SM * v.num_sms;

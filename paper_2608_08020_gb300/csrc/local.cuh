@@ -81,7 +81,8 @@ __device__ __forceinline__ void team_sync(int team, int threads) {
 template <int G>
 __device__ __forceinline__ void local_attention(const PoolView& v, const CUtensorMap* tm_p, const CUtensorMap* tmh_p,
                                                 int layer, const __nv_bfloat16* __restrict__ q, const NewRows& nw,
-                                                float qscale, int cta, int nctas, float* __restrict__ out) {
+                                                float qscale, int cta, int nctas, float* __restrict__ out,
+                                                bool early) {
   using S = DecodeMmaSmem;
   constexpr int HS = 132;  // floats per head of a record: 128 and a pad, so that the stores below
                            // (4 head pairs x 8 rows) fall on 32 banks
@@ -110,12 +111,15 @@ __device__ __forceinline__ void local_attention(const PoolView& v, const CUtenso
   int stage = 0;
   uint32_t parity = 0;
   bool alive = true;  // false once a wait ran out: no more loads, the pairs' outputs are zero
+  bool wait = early;  // the first pair's loads go out before the wait
 
   for (int p = cta + nctas * team; p < npairs; p += nctas * tpc) {
     const int b = p / v.Hkv, h = p - b * v.Hkv;
     const int n = plan_n(v, 0)[b], L = v.seq_len[b], old = v.cow_old[b];
     float* ob = out + ((size_t)b * v.Hq + (size_t)h * G) * 128;
     if (n == 0) {  // an inactive slot
+      enter(wait);
+      wait = false;
       if (wi == 0) zero_pair<G>(v, b, h, out);
       continue;
     }
@@ -148,6 +152,8 @@ __device__ __forceinline__ void local_attention(const PoolView& v, const CUtenso
     load_pages(i0);
     int ii = i0;  // next chunk to load
     for (int s = 0; s < kMmaStages && ii < i1 && alive; ++s, ++ii) issue(ii, (stage + s) % kMmaStages);
+    enter(wait);
+    wait = false;
     pair_begin<G>(st, v, q, b, h, r, c);
     if (i0 < i1 && i1 == n) {  // this warp holds the pair's last chunk
       nrow = (lane < 16 ? nw.k : nw.v)[(size_t)p * 16 + (lane & 15)];
@@ -250,6 +256,7 @@ __device__ __forceinline__ void local_attention(const PoolView& v, const CUtenso
     fence_proxy_async_smem();  // the records' memory is refilled by TMA for the next pair
     team_sync(team, w * 32);
   }
+  enter(wait);
 }
 
 }  // namespace gb

@@ -240,6 +240,9 @@ __global__ void __launch_bounds__(1024) k_step_begin(PoolView v, int n_tokens, c
   __shared__ int s_alloc[kMaxBeams];
   __shared__ int s_tail[kMaxBeams];
   __shared__ int s_act[kMaxBeams], s_cow[kMaxBeams];  // active slots, slots that copy their tail page
+  constexpr int kTailHashBits = 11, kTailHash = 1 << kTailHashBits;
+  static_assert(kTailHash >= 2 * kMaxBeams, "a probe always finds its page or a free entry");
+  __shared__ int s_hkey[kTailHash], s_hmax[kTailHash];
   __shared__ int s_ncow, s_len;
   __shared__ int s_tok[2];
   __shared__ int s_ctl[8];  // free pages, steps, and the segment totals of the step record
@@ -261,24 +264,36 @@ __global__ void __launch_bounds__(1024) k_step_begin(PoolView v, int n_tokens, c
     s_ctl[7] = v.ctl[kCtlTailShared];
   }
 
-  // Copy-on-write decision for a still-shared partial tail page: holders
-  // decide in slot order against the current refcount, so the i-th holder
-  // (1-based) copies iff i < refcnt.  Only after a seed or a fork can a partial tail page be
-  // shared; the first step after one resolves them all.
+  // Copy-on-write decision for a still-shared partial tail page: holders decide in slot order
+  // against the current refcount, so every holder but the highest slot copies.  Only after a seed
+  // or a fork can a partial tail page be shared; the first step after one resolves them all.  The
+  // highest holder of each page comes from a hash table in shared memory (a scan over the other
+  // slots' pages took up to 10 us for 256 slots).
   __syncthreads();
   const bool tails_shared = s_ctl[7] != 0;
   int tail = -1;
-  if (tails_shared && act && (L % v.P) != 0) tail = v.tables[(size_t)b * v.max_pages + L / v.P];
-  if (b < kMaxBeams) s_tail[b] = tail;
-  __syncthreads();
   bool cow = false;
-  if (tail >= 0) {
-    const int R = v.refcnt[tail];
-    if (R > 1) {
-      int i = 1;
-      for (int o = 0; o < b; ++o) i += (s_tail[o] == tail);
-      cow = i < R;
+  if (tails_shared) {
+    if (act && (L % v.P) != 0) tail = v.tables[(size_t)b * v.max_pages + L / v.P];
+    const int R = tail >= 0 ? v.refcnt[tail] : 0;
+    for (int i = b; i < kTailHash; i += blockDim.x) {
+      s_hkey[i] = -1;
+      s_hmax[i] = -1;
     }
+    s_tail[b] = tail;
+    __syncthreads();
+    int at = 0;
+    if (R > 1) {
+      at = (int)(((unsigned)tail * 2654435761u) >> (32 - kTailHashBits));
+      for (;;) {  // fewer pages than entries, so a probe ends
+        const int k = atomicCAS(&s_hkey[at], -1, tail);
+        if (k == -1 || k == tail) break;
+        at = (at + 1) & (kTailHash - 1);
+      }
+      atomicMax(&s_hmax[at], b);
+    }
+    __syncthreads();
+    cow = R > 1 && s_hmax[at] > b;
   }
   // Pages this slot needs over the whole step, and the table capacity check.
   int need_total = 0;
