@@ -64,12 +64,14 @@ __device__ __forceinline__ void unpack16(const uint4& u, float* f) {
 template <int DT, int G>
 struct DecodeSmem {
   using T = KvTraits<DT>;
+  static constexpr int WARPS = kDecodeWarps, STAGES = kDecodeStages;
   static constexpr int PBUF = kChunk * G * 4;
   // Rounded to 128 bytes so every warp's stages start 16-byte aligned (bulk-copy destinations).
-  static constexpr int WARP_BYTES = (kDecodeStages * T::STAGE_BYTES + PBUF + 8 * kDecodeStages + 127) / 128 * 128;
+  static constexpr int WARP_BYTES = (STAGES * T::STAGE_BYTES + PBUF + 8 * STAGES + 127) / 128 * 128;
   static_assert(WARP_BYTES % 128 == 0 && T::STAGE_BYTES % 16 == 0, "stage alignment");
   static constexpr int PLAN_BYTES = 5 * (kMaxBeams + 1) * 4;  // offsets, chunk counts, start tokens, lengths, copied-from pages
-  static constexpr int TOTAL = kDecodeWarps * WARP_BYTES + PLAN_BYTES;
+  static constexpr int TOTAL = WARPS * WARP_BYTES + PLAN_BYTES;
+  static_assert(TOTAL <= 232448, "shared memory per block");
 };
 
 // The same, as DPC / 2 pairs of consecutive dims (operands of the paired fp32 FMA).
@@ -85,18 +87,11 @@ __device__ __forceinline__ void unpack16x2(const uint4& u, float2* f) {
   }
 }
 
-// The kernels' body (plan 0, W warps).  Pool: the step's new rows are appended on the way, as in
-// decode_mma_body, and every record is counted for the merge.
-template <int DT, int G, bool Pool>
-__device__ __forceinline__ void decode_body(const PoolView& v, const Counters& cnt, int layer,
-                                            const void* __restrict__ qptr, const NewRows& nw, float qscale, int W) {
-  using T = KvTraits<DT>;
-  using S = DecodeSmem<DT, G>;
-  constexpr int NS = G / 2;  // scores held per lane after the reduce-scatter
-  constexpr int D = T::D, DPC = T::DPC, DPL = T::DPL;
+// The plan (plan 0) in shared memory, and this warp's barriers.
+template <int DT, bool Pool, class S>
+__device__ __forceinline__ void decode_setup(const PoolView& v) {
   extern __shared__ __align__(128) unsigned char smem[];
-
-  int* s_off = reinterpret_cast<int*>(smem + kDecodeWarps * S::WARP_BYTES);
+  int* s_off = reinterpret_cast<int*>(smem + S::WARPS * S::WARP_BYTES);
   int* s_n = s_off + (kMaxBeams + 1);
   int* s_start = s_n + (kMaxBeams + 1);
   int* s_len = s_start + (kMaxBeams + 1);
@@ -115,29 +110,43 @@ __device__ __forceinline__ void decode_body(const PoolView& v, const Counters& c
       }
     }
   }
+  const int warp = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0) {
+    const uint32_t bar0 = smem_addr(smem + warp * S::WARP_BYTES + S::STAGES * KvTraits<DT>::STAGE_BYTES + S::PBUF);
+    for (int s = 0; s < S::STAGES; ++s) mbar_init(bar0 + 8 * s, 1);
+    fence_mbar_init();
+  }
   __syncthreads();
+}
+
+// The kernels' body: this warp's chunks [x_begin, x_end) of the flat list; w numbers the warp in the
+// records.  Pool: the step's new rows are appended on the way, as in decode_mma_body, and every
+// record is counted for the merge.  Local: the range lies in one pair and its record goes to `lrec`
+// in shared memory.  k counts the chunks consumed so far (stages and phases of the ring).  False
+// once a wait ran out.
+template <int DT, int G, bool Pool, bool Local, class S>
+__device__ __forceinline__ bool decode_range(const PoolView& v, const Counters& cnt, int layer,
+                                             const void* __restrict__ qptr, const NewRows& nw, float qscale, int w,
+                                             int x_begin, int x_end, int& k_io, float* lrec) {
+  using T = KvTraits<DT>;
+  constexpr int NS = G / 2;  // scores held per lane after the reduce-scatter
+  constexpr int D = T::D, DPC = T::DPC, DPL = T::DPL, kStages = S::STAGES;
+  extern __shared__ __align__(128) unsigned char smem[];
+  const int* s_off = reinterpret_cast<const int*>(smem + S::WARPS * S::WARP_BYTES);
+  const int* s_n = s_off + (kMaxBeams + 1);
+  const int* s_start = s_n + (kMaxBeams + 1);
+  const int* s_len = s_start + (kMaxBeams + 1);
+  const int* s_cow = s_len + (kMaxBeams + 1);
+  const int k0 = k_io;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = lane >> 3, j = lane & 7;
   const int b0 = lane & 1, b1 = (lane >> 1) & 1, b2 = (lane >> 2) & 1;
   const int my_t = 4 * (2 * b2 + b1) + row;  // token (within the chunk) of this lane's scores
   unsigned char* wsm = smem + warp * S::WARP_BYTES;
-  float* pbuf = reinterpret_cast<float*>(wsm + kDecodeStages * T::STAGE_BYTES);
+  float* pbuf = reinterpret_cast<float*>(wsm + kStages * T::STAGE_BYTES);
   const uint32_t stage0 = smem_addr(wsm);
-  const uint32_t bar0 = smem_addr(wsm + kDecodeStages * T::STAGE_BYTES + S::PBUF);
-
-  const int Tot = s_off[v.max_beams];
-  const int w = blockIdx.x * kDecodeWarps + warp;
-  const int c = (Tot + W - 1) / W;
-  const int x_begin = w * c;
-  const int x_end = min(Tot, x_begin + c);
-  if (x_begin >= x_end) return;
-
-  if (lane == 0) {
-    for (int s = 0; s < kDecodeStages; ++s) mbar_init(bar0 + 8 * s, 1);
-    fence_mbar_init();
-  }
-  __syncwarp();
+  const uint32_t bar0 = smem_addr(wsm + kStages * T::STAGE_BYTES + S::PBUF);
 
   // Locate the first chunk: the largest b with s_off[b] <= x_begin.
   ChunkIter it;
@@ -193,9 +202,9 @@ __device__ __forceinline__ void decode_body(const PoolView& v, const Counters& c
   ChunkIter ip = it;
   int ip_x = x_begin;
   int ip_page = load_page(ip);
-  for (int s = 0; s < kDecodeStages; ++s) {
+  for (int s = 0; s < kStages; ++s) {
     if (ip_x < x_end) {
-      issue(ip, ip_page, s);
+      issue(ip, ip_page, (k0 + s) % kStages);
       ++ip_x;
       if (ip_x < x_end) {
         iter_advance(ip, s_n, s_start, v.Hkv, v.max_beams);
@@ -215,7 +224,7 @@ __device__ __forceinline__ void decode_body(const PoolView& v, const Counters& c
   int npage = 0;                            // the page they go to
   const char* qbase = static_cast<const char*>(qptr);
 
-  for (int x = x_begin, k = 0; x < x_end; ++x, ++k) {
+  for (int x = x_begin, k = k0; x < x_end; ++x, ++k) {
     if (fresh) {
       // New (beam, head): load the G query rows for this lane's dims, pre-scaled.
       L = Pool ? s_len[it.b] : v.seq_len[it.b];
@@ -241,16 +250,16 @@ __device__ __forceinline__ void decode_body(const PoolView& v, const Counters& c
       for (int kk = 0; kk < NS; ++kk) l_lane[kk] = 0.f;
       fresh = false;
     }
-    const int stage = k % kDecodeStages;
-    const uint32_t parity = (k / kDecodeStages) & 1;
+    const int stage = k % kStages;
+    const uint32_t parity = (k / kStages) & 1;
     if (!mbar_wait_bounded(bar0 + 8 * stage, parity, kWaitLimitNs)) {
       if (lane == 0) set_status(v.ctl, GB_ERR_TIMEOUT);
       // Give copies still in flight a bounded chance to land before leaving.
-      for (int s = 0; s < kDecodeStages; ++s) {
+      for (int s = 0; s < kStages; ++s) {
         const int kk = k + s;
-        if (x + s < ip_x) mbar_wait_bounded(bar0 + 8 * (kk % kDecodeStages), (kk / kDecodeStages) & 1, kWaitLimitNs / 4);
+        if (x + s < ip_x) mbar_wait_bounded(bar0 + 8 * (kk % kStages), (kk / kStages) & 1, kWaitLimitNs / 4);
       }
-      return;
+      return false;
     }
     const unsigned char* Ks = wsm + stage * T::STAGE_BYTES;
     const unsigned char* Vs = Ks + T::SLAB_BYTES;
@@ -388,7 +397,7 @@ __device__ __forceinline__ void decode_body(const PoolView& v, const Counters& c
       }
     }
     __syncwarp();
-    // The stage is free again: refill it with the chunk kDecodeStages ahead.
+    // The stage is free again: refill it with the chunk kStages ahead.
     if (ip_x < x_end) {
       if (lane == 0) fence_proxy_async_smem();
       issue(ip, ip_page, stage);
@@ -422,12 +431,12 @@ __device__ __forceinline__ void decode_body(const PoolView& v, const Counters& c
       }
 #pragma unroll
       for (int kk = 0; kk < NS; ++kk) lother[kk] = __shfl_xor_sync(0xffffffffu, lsum[kk], 1);
-      float* rec = v.partials + (size_t)(w + it.b * v.Hkv + it.h) * v.record_floats;
+      float* rec = Local ? lrec : v.partials + (size_t)(w + it.b * v.Hkv + it.h) * v.record_floats;
       if (row == 0) {
 #pragma unroll
         for (int g = 0; g < G; ++g) {
           float* oa = rec + g * D + DPC * j;
-          float* ob = rec + g * D + D / 2 + DPC * j;
+          float* ob = oa + D / 2;
 #pragma unroll
           for (int e = 0; e < DC2; e += 2) {
             *reinterpret_cast<float4*>(oa + 2 * e) = make_float4(o[g][e].x, o[g][e].y, o[g][e + 1].x, o[g][e + 1].y);
@@ -443,43 +452,135 @@ __device__ __forceinline__ void decode_body(const PoolView& v, const Counters& c
           rec[G * D + G + g] = ((g / NS) == b0) ? lsum[g % NS] : lother[g % NS];
         }
       }
-      if (Pool) record_arrive(cnt, it.b * v.Hkv + it.h, lane);
+      if (Pool && !Local) record_arrive(cnt, it.b * v.Hkv + it.h, lane);
       fresh = true;
     }
     if (x + 1 < x_end) iter_advance(it, s_n, s_start, v.Hkv, v.max_beams);
   }
+  k_io = k0 + x_end - x_begin;
+  return true;
+}
+
+// An even share of all chunks per warp: warp `w` of W.
+template <int DT, int G, bool Pool, class S>
+__device__ __forceinline__ void decode_body(const PoolView& v, const Counters& cnt, int layer,
+                                            const void* __restrict__ qptr, const NewRows& nw, float qscale, int w, int W) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  const int Tot = reinterpret_cast<const int*>(smem + S::WARPS * S::WARP_BYTES)[v.max_beams];
+  const int c = (Tot + W - 1) / W, x_begin = w * c, x_end = min(Tot, x_begin + c);
+  int k = 0;
+  if (x_begin < x_end)
+    decode_range<DT, G, Pool, false, S>(v, cnt, layer, qptr, nw, qscale, w, x_begin, x_end, k, nullptr);
 }
 
 // Caller-owned rows: the records are merged by k_combine.
 template <int DT, int G>
 __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
-    k_decode(PoolView v, const void* __restrict__ qptr, float qscale, int W) {
+    k_decode(PoolView v, const void* __restrict__ qptr, float qscale) {
   pdl_wait();
   pdl_launch_dependents();
-  decode_body<DT, G, false>(v, Counters{}, 0, qptr, NewRows{}, qscale, W);
+  using S = DecodeSmem<DT, G>;
+  decode_setup<DT, false, S>(v);
+  decode_body<DT, G, false, S>(v, Counters{}, 0, qptr, NewRows{}, qscale, (int)blockIdx.x * kDecodeWarps + (int)(threadIdx.x >> 5),
+                               (int)gridDim.x * kDecodeWarps);
 }
 
 // A layer-step of an fp32 pool (or a bf16 one too large for a tensor map) in one launch: append,
-// attention and the merge (combine.cuh; one CTA per SM, so every CTA is resident and the merge's
-// waits end).  With launches of its own for the append and the merge a step of 8 beams x 256 tokens
-// took 11.8 us, half of it between kernels.
+// attention and the merge.  With launches of its own for the append and the merge a step of 8 beams
+// x 256 tokens took 11.8 us, half of it between kernels.  Small steps are merged inside each CTA: a
+// team of 1, 2, 4 or 8 warps takes a (beam, KV head) pair at a time (as in local.cuh).  Otherwise
+// every warp takes an even share of the chunks, and the records are merged through global memory
+// (combine.cuh; one CTA per SM, so every CTA is resident and the merge's waits end).
 template <int DT, int G>
 __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
     k_decode_pool(PoolView v, int layer, const void* __restrict__ qptr, NewRows nw, float qscale,
                   float* __restrict__ out) {
   pdl_wait();
   pdl_launch_dependents();
-  constexpr int D = KvTraits<DT>::D;
-  const int c = (int)blockIdx.x, nctas = (int)gridDim.x;
+  using S = DecodeSmem<DT, G>;
+  constexpr int D = KvTraits<DT>::D, GD = G * D;
+  const int cta = (int)blockIdx.x, nctas = (int)gridDim.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (v.ctl[kCtlStepOk] == 0) {
-    zero_all_pairs<G, D>(v, c, nctas, out);
+    zero_all_pairs<G, D>(v, cta, nctas, out);
     return;
   }
   const int set = counter_set(v, layer), W = nctas * kDecodeWarps;
   const Counters cnt = counters(v, set);
-  zero_counters(v, set ^ 1, c, nctas);
-  decode_body<DT, G, true>(v, cnt, layer, qptr, nw, qscale, W);
-  combine_pairs<G, D>(v, cnt, 0, W, 0, false, c, nctas, out);
+  zero_counters(v, set ^ 1, cta, nctas);
+  decode_setup<DT, true, S>(v);
+  extern __shared__ __align__(128) unsigned char smem[];
+  const int* s_off = reinterpret_cast<const int*>(smem + S::WARPS * S::WARP_BYTES);
+  const int* s_n = s_off + (kMaxBeams + 1);
+  const int Tot = s_off[v.max_beams], npairs = v.max_beams * v.Hkv;
+  // Rounds of pairs x (chunks per warp, about 2 us each, + a pair's start and merge) against an even
+  // share + the record, its count, the wait and the merge.
+  int tw = 0;
+  {
+    int best = (Tot + W - 1) / W + 4;
+    const int n = (Tot + npairs - 1) / npairs;
+    for (int w = 1; w <= kDecodeWarps; w *= 2) {
+      const int teams = nctas * (kDecodeWarps / w), cost = (npairs + teams - 1) / teams * ((n + w - 1) / w + 2);
+      if (cost < best) {
+        best = cost;
+        tw = w;
+      }
+    }
+  }
+  if (tw == 0) {
+    decode_body<DT, G, true, S>(v, cnt, layer, qptr, nw, qscale, cta * kDecodeWarps + warp, W);
+    combine_pairs<G, D>(v, cnt, 0, W, 0, false, cta, nctas, out);
+    return;
+  }
+  const int tpc = kDecodeWarps / tw, team = warp / tw, wi = warp - team * tw;
+  float* lrec = reinterpret_cast<float*>(smem + warp * S::WARP_BYTES);  // over the warp's idle stages
+  static_assert((GD + 2 * G) * 4 <= S::STAGES * KvTraits<DT>::STAGE_BYTES, "a record fits the warp's stages");
+  int k = 0;
+  bool alive = true;
+  for (int p = cta + nctas * team; p < npairs; p += nctas * tpc) {
+    const int b = p / v.Hkv, h = p - b * v.Hkv, n = s_n[b], o0 = s_off[b] + h * n;
+    if (n == 0) {
+      if (wi == 0) zero_pair<G, D>(v, b, h, out);
+      continue;
+    }
+    const int x0 = o0 + wi * n / tw, x1 = o0 + (wi + 1) * n / tw;
+    if (x0 < x1 && alive) alive = decode_range<DT, G, true, true, S>(v, cnt, layer, qptr, nw, qscale, 0, x0, x1, k, lrec);
+    if ((x0 >= x1 || !alive) && lane < G) {  // no chunks (m = -inf, l = 0), or a wait that ran out (l < 0)
+      lrec[GD + lane] = -INFINITY;
+      lrec[GD + G + lane] = alive ? 0.f : -1.f;
+    }
+    team_sync(team, tw * 32);
+    const float* recs = reinterpret_cast<const float*>(smem + (size_t)team * tw * S::WARP_BYTES);
+    constexpr int RS = S::WARP_BYTES / 4;
+    for (int e = wi * 32 + lane; e < GD / 4; e += tw * 32) {
+      const int g = 4 * e / D;
+      float M = -INFINITY;
+      bool good = true;
+      for (int i = 0; i < tw; ++i) {
+        M = fmaxf(M, recs[i * RS + GD + g]);
+        good = good && !(recs[i * RS + GD + G + g] < 0.f);
+      }
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+      float l = 0.f;
+      for (int i = 0; i < tw; ++i) {
+        const float m = recs[i * RS + GD + g];
+        if (m == -INFINITY) continue;
+        const float sc = exp2f(m - M);
+        const float4 y = *reinterpret_cast<const float4*>(recs + i * RS + 4 * e);
+        acc.x = fmaf(y.x, sc, acc.x);
+        acc.y = fmaf(y.y, sc, acc.y);
+        acc.z = fmaf(y.z, sc, acc.z);
+        acc.w = fmaf(y.w, sc, acc.w);
+        l = fmaf(recs[i * RS + GD + G + g], sc, l);
+      }
+      float* od = out + (size_t)p * GD + 4 * e;
+      od[0] = good ? acc.x / l : 0.f;
+      od[1] = good ? acc.y / l : 0.f;
+      od[2] = good ? acc.z / l : 0.f;
+      od[3] = good ? acc.w / l : 0.f;
+    }
+    fence_proxy_async_smem();  // the records' memory is refilled by bulk copies for the next pair
+    team_sync(team, tw * 32);
+  }
 }
 
 // The per-beam kernel on its own (the per-beam path, every beam reading its whole context):
@@ -656,7 +757,7 @@ static cudaError_t launch_view_t(const PoolView& v, int W, const void* q, float 
   using S = DecodeSmem<DT, G>;
   cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(k_decode<DT, G>), S::TOTAL);
   if (e != cudaSuccess) return e;
-  e = launch_pdl(k_decode<DT, G>, W / kDecodeWarps, kDecodeWarps * 32, S::TOTAL, s, v, q, scale * 1.4426950408889634f, W);
+  e = launch_pdl(k_decode<DT, G>, W / kDecodeWarps, kDecodeWarps * 32, S::TOTAL, s, v, q, scale * 1.4426950408889634f);
   if (e != cudaSuccess) return e;
   return launch_pdl(k_combine, v.max_beams * v.Hkv, 128, 0, s, v, W, out);
 }
