@@ -31,11 +31,11 @@ __device__ __forceinline__ void tma_tile(uint32_t dst, const CUtensorMap* tm, in
 
 __global__ void __launch_bounds__(128, 1)
     k_gemm_partials(const __grid_constant__ CUtensorMap tmh, const __grid_constant__ CUtensorMap tmw, int rows, int dh,
-               int H, float* __restrict__ zp, int* __restrict__ ctl) {
-  pdl_wait();
-  pdl_launch_dependents();
+               int H, float* __restrict__ zp, int* __restrict__ ctl, bool early_w) {
+  enter(!early_w);
   extern __shared__ __align__(1024) unsigned char sm[];
   if (smem_addr(sm) & 1023) {
+    enter(early_w);
     if (threadIdx.x == 0) set_status(ctl, GB_ERR_UNSUPPORTED);
     return;
   }
@@ -65,14 +65,23 @@ __global__ void __launch_bounds__(128, 1)
   bool ok = true;
   if (tid == 0) {
     constexpr uint32_t ID = idesc(kMT, kNT, false);
-    auto load = [&](int i) {
+    auto load_a = [&](int i) {
+      const uint32_t st = i % kMStages;
+      tma_tile(sbase + st * kMStage, &tmh, (kb0 + i) * kKB, mt * kMT, bar + kMBarFull + 8 * st);
+    };
+    auto load_b = [&](int i) {
       const uint32_t st = i % kMStages, full = bar + kMBarFull + 8 * st;
       mbar_arrive_expect_tx(full, kMStage);
-      const uint32_t a = sbase + st * kMStage;
-      tma_tile(a, &tmh, (kb0 + i) * kKB, mt * kMT, full);
-      tma_tile(a + kMT * kKB * 2, &tmw, (kb0 + i) * kKB, nt * kNT, full);
+      tma_tile(sbase + st * kMStage + kMT * kKB * 2, &tmw, (kb0 + i) * kKB, nt * kNT, full);
     };
-    for (int i = 0; i < nkb && i < kMStages; ++i) load(i);
+    auto load = [&](int i) {
+      load_b(i);
+      load_a(i);
+    };
+    // The first stages' weights may be loaded before the previous kernel has completed.
+    for (int i = 0; i < nkb && i < kMStages; ++i) load_b(i);
+    enter(early_w);
+    for (int i = 0; i < nkb && i < kMStages; ++i) load_a(i);
     for (int i = 0; i < nkb && ok; ++i) {
       const uint32_t st = i % kMStages;
       ok = mbar_wait_bounded(bar + kMBarFull + 8 * st, (i / kMStages) & 1, kWaitLimitNs);
@@ -91,6 +100,7 @@ __global__ void __launch_bounds__(128, 1)
     if (ok) mma_commit(bar + kMBarDone);
     if (!ok) set_status(ctl, GB_ERR_TIMEOUT);
   }
+  if (tid != 0) enter(early_w);
   __syncthreads();
   ok = __syncthreads_and(tid == 0 ? ok : 1);
   // The partial tile goes out through shared memory (the ring is idle once the MMAs are
@@ -162,7 +172,7 @@ int gemm_splits(int M, int N, int K, int num_sms, size_t max_floats) {
 }
 
 cudaError_t gemm_partials(const void* A, int M, const void* B, int N, int K, int splits, float* P, int* ctl,
-                          cudaStream_t s) {
+                          bool early_w, cudaStream_t s) {
   {
     const cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(k_gemm_partials), kMSmem);
     if (e != cudaSuccess) return e;
@@ -171,7 +181,7 @@ cudaError_t gemm_partials(const void* A, int M, const void* B, int N, int K, int
   CUtensorMap ta, tb;
   if (!encode_rows(&ta, A, M, K) || !encode_rows(&tb, B, N, K)) return cudaErrorInvalidValue;
   const int mtiles = (M + kMT - 1) / kMT, ntiles = (N + kNT - 1) / kNT;
-  return launch_pdl(k_gemm_partials, dim3(mtiles, ntiles, splits), 128, kMSmem, s, ta, tb, M, N, K, P, ctl);
+  return launch_pdl(k_gemm_partials, dim3(mtiles, ntiles, splits), 128, kMSmem, s, ta, tb, M, N, K, P, ctl, early_w);
 }
 
 }  // namespace gb

@@ -353,6 +353,7 @@ cudaError_t launch_decode(gb_pool* pool, int layer, const void* q, const void* k
                           float* out, int mode, bool allow_local, cudaStream_t s);
 cudaError_t launch_decode_view(const PoolView& v, int W, const void* q, float scale, float* out, cudaStream_t s);
 cudaError_t rebuild_segments(gb_pool* pool, cudaStream_t s);
+cudaError_t launch_forks(gb_pool* pool, const int32_t* parent_of, cudaStream_t s);
 cudaError_t launch_attention(gb_pool* pool, int layer, const void* q, const void* k_new, const void* v_new, float scale,
                              float* out, bool allow_local, cudaStream_t s);
 cudaError_t launch_wait_selftest(gb_pool* pool, cudaStream_t s);
@@ -361,9 +362,11 @@ cudaError_t launch_probe(gb_pool* pool, const void* hidden, int hidden_dtype, in
                          float bias, const uint8_t* mask, float* score_out, const float* scores_in,
                          cudaStream_t s);
 // Split-K bf16 GEMM on the tensor cores (gemm.cu): P[s][m][n] over k-range s of A[m][k] B[n][k].
+// early_w: B was not written by the kernel before this one in the stream, so its first loads need
+// not wait for that kernel.
 int gemm_splits(int M, int N, int K, int num_sms, size_t max_floats);
 cudaError_t gemm_partials(const void* A, int M, const void* B, int N, int K, int splits, float* P, int* ctl,
-                          cudaStream_t s);
+                          bool early_w, cudaStream_t s);
 cudaError_t launch_mlp(gb_pool* pool, const void* hidden, int H, const void* w1, const float* b1, const float* w2,
                        float b2, int dh, const uint8_t* mask, float* score_out, cudaStream_t s);
 cudaError_t launch_prune_branch(gb_pool* pool, int K, int fanout, int warmup, const uint8_t* elig,

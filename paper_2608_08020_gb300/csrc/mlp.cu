@@ -66,7 +66,7 @@ cudaError_t launch_mlp(gb_pool* pool, const void* hidden, int H, const void* w1,
   const int splits = gemm_splits(v.max_beams, dh, H, pool->num_sms, kMlpScratchFloats);
   if (splits == 0) return cudaErrorInvalidValue;
   prof_begin(pool, GB_PROF_PROBE, s);
-  cudaError_t e = gemm_partials(hidden, v.max_beams, w1, dh, H, splits, v.mlp_scratch, v.ctl, s);
+  cudaError_t e = gemm_partials(hidden, v.max_beams, w1, dh, H, splits, v.mlp_scratch, v.ctl, false, s);
   if (e != cudaSuccess) return e;
   e = launch_pdl(k_mlp_score, v.max_beams, kScoreThreads, 0, s, v, static_cast<const float*>(v.mlp_scratch), splits,
                  dh, b1, w2, b2, mask, score_out);

@@ -256,9 +256,9 @@ __global__ void __launch_bounds__(kRowThreads) k_head(const float* __restrict__ 
 // ---- products with their operand and epilogue in one launch -------------------------------------
 //
 // Grid (row tiles of mt = 32, 64 or 128 slots) x (64-column tiles).  A CTA of 256 threads builds its
-// rows' A operand in shared memory (128-byte swizzle, 512 of K at a time), loads its 64 rows of the
-// weights, multiplies (128 x 64 x 16 tcgen05.mma into tensor memory; the rows past mt are never
-// read) and finishes its tile.  At these sizes (64 slots, d = 512: 32 MFLOP and 0.5-2 MiB of weights
+// rows' A operand in shared memory (128-byte swizzle, pass_k of K at a time), loads its 64 rows of
+// the weights, multiplies (128 x 64 x 16 tcgen05.mma into tensor memory; the accumulator's rows past
+// mt, whatever the shared memory there gave them, are never read) and finishes its tile.  At these sizes (64 slots, d = 512: 32 MFLOP and 0.5-2 MiB of weights
 // a product) a product is latency: the chain of LayerNorm, GEMM with K-split partials in global
 // memory and epilogue was three launches of 6-9 us each.  So K is not split, the LayerNorm is
 // recomputed by every column tile (its rows come from L2), and the weights, which do not depend on
@@ -267,14 +267,18 @@ __global__ void __launch_bounds__(kRowThreads) k_head(const float* __restrict__ 
 enum AMode { kALn, kAF32, kABf16 };              // LayerNorm of fp32 rows; fp32 rows; bf16 rows
 enum EMode { kEQkv, kEResid, kESwiglu };         // RoPE and q/k/v in bf16; x += z; SwiGLU in bf16
 
-constexpr int kFThreads = 256, kFN = 64, kFK = 512;
-constexpr int kFA = 0, kFABlock = 128 * 128;               // 64 of K: 128 rows x 128 bytes
-constexpr int kFB = kFA + kFK / 64 * kFABlock, kFBBlock = kFN * 128;
-constexpr int kFCtl = kFB + kFK / 64 * kFBBlock;            // mbarrier, tensor-memory address
+constexpr int kFThreads = 256, kFN = 64;
+constexpr int kFK = 512;                                    // K a warp's registers hold of a row at a time
+constexpr int kFBBlock = kFN * 128;                         // 64 of K of the weights: 64 rows x 128 bytes
+constexpr int kFOperands = 192 * 1024;                      // A (mt rows x pass_k) and the weights (64 x pass_k)
+constexpr int kFCtl = kFOperands;                           // mbarrier, tensor-memory address
 constexpr int kFStat = kFCtl + 16;                          // float [2][128]: mean and 1/std of the rows
 constexpr int kFSmem = kFStat + 1024;
-constexpr int kFTile = kFN + 1;                             // epilogue tile [128][65] over the A operand
-static_assert(128 * kFTile * 4 <= kFB && kFSmem <= 232448 - 1024, "shared memory per block");
+constexpr int kFTile = kFN + 1;                             // epilogue tile [mt][65] over the A operand
+static_assert(kFSmem <= 232448 - 1024, "shared memory per block");
+// K per pass: what fits beside the weights, one pass up to 1024 for the 32-row tiles of small steps.
+__host__ __device__ constexpr int pass_k(int mt) { return mt == 32 ? 1024 : 512; }
+static_assert(32 * 1024 * 2 + kFN * 1024 * 2 <= kFOperands && 128 * 512 * 2 + kFN * 512 * 2 <= kFOperands, "operands");
 
 struct FusedArgs {
   const void* a;            // [M][K]
@@ -325,13 +329,17 @@ __global__ void __launch_bounds__(kFThreads, 1) k_fused_gemm(FusedArgs p) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(bar + 8), "r"(kFN));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
+  const int fk = pass_k(p.mt), a_block = p.mt * 128;  // A block: 64 of K, mt rows x 128 bytes
+  const uint32_t b_base = (uint32_t)(p.mt * fk * 2);
   auto load_b = [&](int k0) {
-    const int pc = min(kFK, p.K - k0) / 8;  // 16-byte pieces per row
-    for (int i = tid; i < kFN * pc; i += kFThreads) {
-      const int n = i / pc, c = i - n * pc;
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sbase + kFB + (c >> 3) * kFBBlock + swz(n, (c & 7) * 8)),
-                   "l"(p.w + (size_t)weight_row<E>(p, t, n) * p.K + k0 + 8 * c)
-                   : "memory");
+    const int pc = min(fk, p.K - k0) / 8;  // 16-byte pieces per row
+    for (int n = warp; n < kFN; n += kFThreads / 32) {  // a warp per row: 512 contiguous bytes at a time
+      const __nv_bfloat16* src = p.w + (size_t)weight_row<E>(p, t, n) * p.K + k0;
+      for (int c = lane; c < pc; c += 32)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sbase + b_base + (c >> 3) * kFBBlock +
+                                                                       swz(n, (c & 7) * 8)),
+                     "l"(src + 8 * c)
+                     : "memory");
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
@@ -373,13 +381,16 @@ __global__ void __launch_bounds__(kFThreads, 1) k_fused_gemm(FusedArgs p) {
   bool ok = true;
   int pass = 0;
   uint32_t tmem = 0;
-  for (int k0 = 0; k0 < p.K; k0 += kFK, ++pass) {
-    const int kw = min(kFK, p.K - k0);
+  for (int k0 = 0; k0 < p.K; k0 += fk, ++pass) {
+    const int kpass = min(fk, p.K - k0);
     if (pass > 0) {  // the previous pass's operands have been read
       ok = ok && mbar_wait_bounded(bar, (pass - 1) & 1, kWaitLimitNs);
       load_b(k0);
     }
-    // A: row r = warp + 8 j of the tile, four rows in flight per warp.
+    // A: row r = warp + 8 j of the tile, four rows in flight per warp, 512 of K at a time.
+    for (int h0 = 0; h0 < kpass; h0 += kFK) {
+    const int kw = min(kFK, kpass - h0), kh = k0 + h0;
+    unsigned char* sa = sm + (h0 >> 6) * a_block;
     if (A == kABf16) {
       const __nv_bfloat16* ab = static_cast<const __nv_bfloat16*>(p.a);
       for (int r0 = warp; r0 < p.mt; r0 += kFThreads / 32 * 4) {
@@ -391,7 +402,7 @@ __global__ void __launch_bounds__(kFThreads, 1) k_fused_gemm(FusedArgs p) {
 #pragma unroll
           for (int i = 0; i < kFK / 256; ++i) {
             const int c = 8 * lane + 256 * i;
-            v[u][i] = live && c < kw ? *reinterpret_cast<const uint4*>(ab + (size_t)(m0 + r) * p.K + k0 + c)
+            v[u][i] = live && c < kw ? *reinterpret_cast<const uint4*>(ab + (size_t)(m0 + r) * p.K + kh + c)
                                      : make_uint4(0u, 0u, 0u, 0u);
           }
         }
@@ -401,7 +412,7 @@ __global__ void __launch_bounds__(kFThreads, 1) k_fused_gemm(FusedArgs p) {
 #pragma unroll
           for (int i = 0; i < kFK / 256; ++i) {
             const int c = 8 * lane + 256 * i;
-            if (r < p.mt && c < kw) *reinterpret_cast<uint4*>(sm + kFA + (c >> 6) * kFABlock + swz(r, c & 63)) = v[u][i];
+            if (r < p.mt && c < kw) *reinterpret_cast<uint4*>(sa + (c >> 6) * a_block + swz(r, c & 63)) = v[u][i];
           }
         }
       }
@@ -411,8 +422,8 @@ __global__ void __launch_bounds__(kFThreads, 1) k_fused_gemm(FusedArgs p) {
 #pragma unroll
         for (int i = 0; i < kFK / 128; ++i) {
           const int c = 4 * lane + 128 * i;
-          gg[i] = c < kw ? *reinterpret_cast<const float4*>(p.g + k0 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-          bb[i] = c < kw ? *reinterpret_cast<const float4*>(p.b + k0 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+          gg[i] = c < kw ? *reinterpret_cast<const float4*>(p.g + kh + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+          bb[i] = c < kw ? *reinterpret_cast<const float4*>(p.b + kh + c) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
       }
       for (int r0 = warp; r0 < p.mt; r0 += kFThreads / 32 * 4) {
@@ -424,47 +435,68 @@ __global__ void __launch_bounds__(kFThreads, 1) k_fused_gemm(FusedArgs p) {
 #pragma unroll
           for (int i = 0; i < kFK / 128; ++i) {
             const int c = 4 * lane + 128 * i;
-            v[u][i] = live && c < kw ? *reinterpret_cast<const float4*>(af + (size_t)(m0 + r) * p.K + k0 + c)
+            v[u][i] = live && c < kw ? *reinterpret_cast<const float4*>(af + (size_t)(m0 + r) * p.K + kh + c)
                                      : make_float4(0.f, 0.f, 0.f, 0.f);
           }
+        }
+        // The four rows' statistics together: their shuffles are independent chains.
+        float mu[4] = {0.f, 0.f, 0.f, 0.f}, rs[4] = {1.f, 1.f, 1.f, 1.f};
+        if (A == kALn && p.K <= kFK) {
+          float s[4], q[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            s[u] = 0.f;
+#pragma unroll
+            for (int i = 0; i < kFK / 128; ++i) s[u] += (v[u][i].x + v[u][i].y) + (v[u][i].z + v[u][i].w);
+          }
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) s[u] += __shfl_xor_sync(0xffffffffu, s[u], o);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            mu[u] = s[u] / (float)p.K;
+#pragma unroll
+            for (int i = 0; i < kFK / 128; ++i)
+              if (4 * lane + 128 * i < kw) {
+                q[u] = fmaf(v[u][i].x - mu[u], v[u][i].x - mu[u], q[u]);
+                q[u] = fmaf(v[u][i].y - mu[u], v[u][i].y - mu[u], q[u]);
+                q[u] = fmaf(v[u][i].z - mu[u], v[u][i].z - mu[u], q[u]);
+                q[u] = fmaf(v[u][i].w - mu[u], v[u][i].w - mu[u], q[u]);
+              }
+          }
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) q[u] += __shfl_xor_sync(0xffffffffu, q[u], o);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) rs[u] = 1.0f / sqrtf(q[u] / (float)p.K + kLnEps);
+        } else if (A == kALn) {
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (live_row(r0 + kFThreads / 32 * u)) {
+              mu[u] = s_mu[r0 + kFThreads / 32 * u];
+              rs[u] = s_rs[r0 + kFThreads / 32 * u];
+            }
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           const int r = r0 + kFThreads / 32 * u;
-          if (r >= p.mt) break;
-          float mu = 0.f, rs = 1.f;
-          if (A == kALn && p.K <= kFK) {
-            float s = 0.f, q = 0.f;
-#pragma unroll
-            for (int i = 0; i < kFK / 128; ++i) s += (v[u][i].x + v[u][i].y) + (v[u][i].z + v[u][i].w);
-            mu = warp_sum(s) / (float)p.K;
-#pragma unroll
-            for (int i = 0; i < kFK / 128; ++i)
-              if (4 * lane + 128 * i < kw) {
-                q = fmaf(v[u][i].x - mu, v[u][i].x - mu, q);
-                q = fmaf(v[u][i].y - mu, v[u][i].y - mu, q);
-                q = fmaf(v[u][i].z - mu, v[u][i].z - mu, q);
-                q = fmaf(v[u][i].w - mu, v[u][i].w - mu, q);
-              }
-            rs = 1.0f / sqrtf(warp_sum(q) / (float)p.K + kLnEps);
-          } else if (A == kALn && live_row(r)) {
-            mu = s_mu[r];
-            rs = s_rs[r];
-          }
 #pragma unroll
           for (int i = 0; i < kFK / 128; ++i) {
             const int c = 4 * lane + 128 * i;
-            if (c >= kw) continue;
             float4 y = v[u][i];
             if (A == kALn)
-              y = make_float4((y.x - mu) * rs * gg[i].x + bb[i].x, (y.y - mu) * rs * gg[i].y + bb[i].y,
-                              (y.z - mu) * rs * gg[i].z + bb[i].z, (y.w - mu) * rs * gg[i].w + bb[i].w);
+              y = make_float4((y.x - mu[u]) * rs[u] * gg[i].x + bb[i].x, (y.y - mu[u]) * rs[u] * gg[i].y + bb[i].y,
+                              (y.z - mu[u]) * rs[u] * gg[i].z + bb[i].z, (y.w - mu[u]) * rs[u] * gg[i].w + bb[i].w);
             const __nv_bfloat162 lo = __floats2bfloat162_rn(y.x, y.y), hi = __floats2bfloat162_rn(y.z, y.w);
-            *reinterpret_cast<uint2*>(sm + kFA + (c >> 6) * kFABlock + swz(r, c & 63)) =
-                make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+            if (r < p.mt && c < kw)
+              *reinterpret_cast<uint2*>(sa + (c >> 6) * a_block + swz(r, c & 63)) =
+                  make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
           }
         }
       }
+    }
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     fence_proxy_async_smem();
@@ -474,18 +506,18 @@ __global__ void __launch_bounds__(kFThreads, 1) k_fused_gemm(FusedArgs p) {
     tmem = *reinterpret_cast<volatile uint32_t*>(sm + kFCtl + 8);
     if (tid == 0 && ok) {
       constexpr uint32_t ID = idesc(128, kFN, false);
-      for (int kb = 0; kb < kw / 64; ++kb)
+      for (int kb = 0; kb < kpass / 64; ++kb)
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
-          mma(tmem, sdesc(sbase + kFA + kb * kFABlock + kk * 32, 16, 1024),
-              sdesc(sbase + kFB + kb * kFBBlock + kk * 32, 16, 1024), ID, (pass > 0 || kb > 0 || kk > 0) ? 1u : 0u);
+          mma(tmem, sdesc(sbase + kb * a_block + kk * 32, 16, 1024),
+              sdesc(sbase + b_base + kb * kFBBlock + kk * 32, 16, 1024), ID, (pass > 0 || kb > 0 || kk > 0) ? 1u : 0u);
       mma_commit(bar);
     }
   }
   ok = ok && mbar_wait_bounded(bar, (pass - 1) & 1, kWaitLimitNs);
   ok = __syncthreads_and(ok) != 0;
   tc_fence_after();
-  float* tile = reinterpret_cast<float*>(sm + kFA);  // [mt][65]
+  float* tile = reinterpret_cast<float*>(sm);  // [mt][65]
   if (ok && warp < p.mt / 32) {
 #pragma unroll
     for (int c0 = 0; c0 < kFN; c0 += 32) {
@@ -580,7 +612,7 @@ struct Run {
   int gemm(const void* A, int M, const void* B, int N, int K) {
     const int splits = gemm_splits(M, N, K, pool->num_sms, L.part_floats);
     if (splits == 0) return 0;
-    if (gemm_partials(A, M, B, N, K, splits, part(), pool->view.ctl, st) != cudaSuccess) return 0;
+    if (gemm_partials(A, M, B, N, K, splits, part(), pool->view.ctl, true, st) != cudaSuccess) return 0;
     ++launches;
     return splits;
   }

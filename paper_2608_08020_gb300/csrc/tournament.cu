@@ -31,8 +31,8 @@
 //
 // Segment ids and member order follow atomics, but every output row of the grouped
 // kernel is computed independently of its position, so results do not depend on them.
-// Without a tournament (after seeding, a release or gb_fork_slots) the kernel runs phases
-// 2-4 only.  A barrier that waits too long records GB_ERR_TIMEOUT and the CTA returns.
+// gb_fork_slots runs the fork of phase 1 on the caller's parents; without either (after seeding or a
+// release) the kernel runs phases 2-4 only.  A barrier that waits too long records GB_ERR_TIMEOUT and the CTA returns.
 #include "internal.cuh"
 #include "ptx.cuh"
 
@@ -47,6 +47,7 @@ constexpr int kSegLenBuckets = 256;  // work units sorted by length in 128-token
 
 struct TourArgs {
   int prune;               // 1: run the tournament first
+  const int* parent_of;    // prune = 0: apply these forks (a tournament decided elsewhere) first, or nullptr
   int C, K, fanout, warmup;
   const uint8_t* elig;     // caller's eligibility mask or nullptr
   int* parent_out;
@@ -133,7 +134,8 @@ __global__ void __launch_bounds__(kTourThreads, 1) k_tournament(PoolView v, Tour
   const int tid = threadIdx.x;
   const int cap = v.max_beams;
   // The slot's state for the ranking, loaded first and together.
-  const bool in = a.prune && tid < cap;
+  const bool forks = a.prune || a.parent_of != nullptr;
+  const bool in = forks && tid < cap;
   const int act_w = in ? v.active[tid] : 0;
   const int gen_w = in ? v.gen[tid] : 0;
   const float mean_w = in ? v.mean[tid] : 0.f;
@@ -158,13 +160,15 @@ __global__ void __launch_bounds__(kTourThreads, 1) k_tournament(PoolView v, Tour
   __syncthreads();
 
   // ---- 1. tournament ---------------------------------------------------------------------
-  if (a.prune) {
+  if (forks) {
     const bool act = act_w != 0;
     const bool elig = act && gen_w >= a.warmup && elig_w != 0;
     s_act[tid] = act;
     s_elig[tid] = elig;
     s_pruned[tid] = 0;
     childof[tid] = -1;
+    int nchild = 0, per = 1;
+    if (a.prune) {
     int N;
     const int pos = block_exclusive_scan(act ? 1 : 0, tmp, &N);
     s_keys[tid] = ~0ull;
@@ -205,7 +209,7 @@ __global__ void __launch_bounds__(kTourThreads, 1) k_tournament(PoolView v, Tour
     __syncthreads();
     // Routing (identical in every CTA).
     const int f1 = a.fanout - 1;
-    int nchild = 0, kase = 0;
+    int kase = 0;
     if (N > 0 && N < a.C) {
       // Case 1 (Eq. 2): the top min(C - N, |B|) eligible traces, one child each, into vacant slots.
       kase = 1;
@@ -236,12 +240,24 @@ __global__ void __launch_bounds__(kTourThreads, 1) k_tournament(PoolView v, Tour
       const int pp = block_exclusive_scan(pr ? 1 : 0, tmp, &np);
       if (pr) cslot[pp] = tid;
     }
+    // Parent j has children [j * per, min((j + 1) * per, nchild)): per = 1 in Case 1, f - 1 in Case 2.
+    per = kase == 2 ? f1 : 1;
+    } else {
+      // Every slot with a parent other than itself is a child of its own "parent j"; the parents
+      // survive (parent_of[p] = p), so their pages keep a reference throughout.
+      const int p = tid < cap ? a.parent_of[tid] : -1;
+      const bool child = p >= 0 && p < cap && p != tid;
+      if (p >= cap && blockIdx.x == 0) set_status(v.ctl, GB_ERR_INVALID);
+      const int k = block_exclusive_scan(child ? 1 : 0, tmp, &nchild);
+      if (child) {
+        cslot[k] = tid;
+        blist[k] = p;
+      }
+    }
     __syncthreads();
     if (tid < nchild) childof[cslot[tid]] = tid;
     if (tid == 0) s_nchild = nchild;
     __syncthreads();
-    // Parent j has children [j * per, min((j + 1) * per, nchild)): per = 1 in Case 1, f - 1 in Case 2.
-    const int per = kase == 2 ? f1 : 1;
     const int npar = (nchild + per - 1) / per;
     const unsigned lin0 = s_lin0;
 
@@ -342,7 +358,7 @@ __global__ void __launch_bounds__(kTourThreads, 1) k_tournament(PoolView v, Tour
     return;
   }
   if (!grid_sync(v, &s_fail)) return;
-  if (blockIdx.x == 0 && tid == 0 && a.prune) v.ctl[kCtlNextLineage] = (int)(s_lin0 + s_nchild);
+  if (blockIdx.x == 0 && tid == 0 && forks) v.ctl[kCtlNextLineage] = (int)(s_lin0 + s_nchild);
   if (tid == 0) s_gen = (unsigned long long)(unsigned)v.ctl[kCtlSegGen];
   __syncthreads();
   const unsigned long long gen = s_gen;
@@ -646,8 +662,13 @@ cudaError_t launch_prune_branch(gb_pool* pool, int K, int fanout, int warmup, co
 
 cudaError_t rebuild_segments(gb_pool* pool, cudaStream_t s) {
   if (!pool->view.grouped) return cudaSuccess;
+  return launch_forks(pool, nullptr, s);
+}
+
+// Apply parent_of's forks (nullptr: none) and rebuild the segments.
+cudaError_t launch_forks(gb_pool* pool, const int32_t* parent_of, cudaStream_t s) {
   TourArgs a{};
-  a.prune = 0;
+  a.parent_of = parent_of;
   pool->launches += 1;
   return launch_pdl(k_tournament, tournament_grid(pool), kTourThreads, 0, s, pool->view, a);
 }
