@@ -78,10 +78,13 @@ __global__ void __launch_bounds__(128, 1)
       load_b(i);
       load_a(i);
     };
-    // The first stages' weights may be loaded before the previous kernel has completed.
-    for (int i = 0; i < nkb && i < kMStages; ++i) load_b(i);
-    enter(early_w);
-    for (int i = 0; i < nkb && i < kMStages; ++i) load_a(i);
+    if (early_w) {  // the first stages' weights before the previous kernel has completed
+      for (int i = 0; i < nkb && i < kMStages; ++i) load_b(i);
+      enter(true);
+      for (int i = 0; i < nkb && i < kMStages; ++i) load_a(i);
+    } else {
+      for (int i = 0; i < nkb && i < kMStages; ++i) load(i);
+    }
     for (int i = 0; i < nkb && ok; ++i) {
       const uint32_t st = i % kMStages;
       ok = mbar_wait_bounded(bar + kMBarFull + 8 * st, (i / kMStages) & 1, kWaitLimitNs);

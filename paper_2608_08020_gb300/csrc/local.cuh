@@ -173,7 +173,7 @@ __device__ __forceinline__ void local_attention(const PoolView& v, const CUtenso
       unsigned char* vs = smem + (stage0 + stage * kMmaStageBytes - smem_addr(smem));
       const int tok0 = i * kChunk, nvalid = min(kChunk, L - tok0);
       if (i == n - 1) chunk_append(v, layer, h, L, nvalid, nrow, npage, vs, lane);
-      if (old >= 0 && tok0 / v.P == tail) chunk_copied(v, layer, b, h, L, tok0, vs, lane);
+      if (old >= 0 && tok0 >= tail * v.P) chunk_copied(v, layer, b, h, L, tok0, vs, lane);
       chunk_attend(st, stage0 + stage * kMmaStageBytes, koff, voff, nvalid, qscale, r);
       __syncwarp();
       if (ii < i1) {
