@@ -1,7 +1,7 @@
 // Split-K bf16 GEMM on tcgen05 for the scorers: P[s][m][n] = sum over the s-th k-range of
 // A[m][k] * B[n][k] (A [M][K] and B [N][K] bf16 row-major, fp32 partials).
 // Grid (M / 128) x (N / 128) x splits; one thread streams 128 x 64 tiles of A and B
-// through a 4-stage TMA ring (2D tensor maps, 128-byte swizzle, K-major) into
+// through a 6-stage TMA ring (2D tensor maps, 128-byte swizzle, K-major) into
 // 128 x 128 x 16 tcgen05.mma accumulating in tensor memory; the CTA writes its partial
 // tile (rows < M, columns < N).  Out-of-range rows and columns load as zeros.  Waits are
 // bounded; a timeout records GB_ERR_TIMEOUT in the caller's status word.
@@ -15,7 +15,7 @@ namespace gb {
 namespace {
 
 constexpr int kMT = 128, kNT = 128, kKB = 64;  // tile rows (slots), tile columns (d_h), k per stage
-constexpr int kMStages = 4;
+constexpr int kMStages = 6;  // most of a split's k-blocks in flight at once (7 for 512 slots, H 4096, d_h 512)
 constexpr int kMStage = 2 * kMT * kKB * 2;      // A and B tiles: 32 KiB
 constexpr int kMBar = kMStages * kMStage;
 constexpr int kMSmem = kMBar + 128;
@@ -106,32 +106,43 @@ __global__ void __launch_bounds__(128, 1)
   if (tid != 0) enter(early_w);
   __syncthreads();
   ok = __syncthreads_and(tid == 0 ? ok : 1);
-  // The partial tile goes out through shared memory (the ring is idle once the MMAs are
-  // done): thread r reads row r's 32 columns of a chunk from TMEM into a padded tile, then
-  // each warp stores whole rows, lanes over consecutive columns (rows < M, columns < N).
+  // The partial tile goes out through shared memory (the ring is idle once the MMAs are done):
+  // thread r writes row r of the accumulator (16-byte pieces, rows 528 bytes apart: no bank
+  // conflicts), then each warp stores whole rows, 512 contiguous bytes an instruction.  In four
+  // 32-column rounds with scalar stores and two barriers each, the tile took about a microsecond more.
   const int r = tid, lane = tid & 31;
-  float* stile = reinterpret_cast<float*>(sm);  // [128][33]
+  constexpr int TS = kNT + 4;
+  static_assert(kMT * TS * 4 <= kMBar, "the tile fits the ring");
+  float* stile = reinterpret_cast<float*>(sm);  // [128][132]
   float* base = zp + (size_t)ks * rows * dh;
   const bool done = ok && nkb > 0 && mbar_wait_bounded(bar + kMBarDone, 0, kWaitLimitNs);
   const bool have = __syncthreads_and(done);  // uniform: tcgen05.ld is warp-collective
   if (ok && nkb > 0 && !have && tid == 0) set_status(ctl, GB_ERR_TIMEOUT);
   if (have) tc_fence_after();
-#pragma unroll 1
-  for (int c0 = 0; c0 < kNT; c0 += 32) {
-    if (nt * kNT + c0 >= dh) break;
-    if (have) {
-      float z[32];
-      tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + c0, z);
 #pragma unroll
-      for (int i = 0; i < 32; ++i) stile[r * 33 + i] = z[i];
+  for (int c0 = 0; c0 < kNT; c0 += 32) {
+    float z[32];
+    if (have) {
+      tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + c0, z);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 32; ++i) z[i] = 0.f;
     }
-    __syncthreads();
-    const int col = nt * kNT + c0 + lane;
-    for (int rr = warp; rr < kMT; rr += 4) {
-      const int row = mt * kMT + rr;
-      if (row < rows && col < dh) base[(size_t)row * dh + col] = have ? stile[rr * 33 + lane] : 0.f;
-    }
-    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 32; i += 4)
+      *reinterpret_cast<float4*>(stile + r * TS + c0 + i) = make_float4(z[i], z[i + 1], z[i + 2], z[i + 3]);
+  }
+  __syncthreads();
+  const int nrow = min(kMT, rows - mt * kMT), col = nt * kNT + 4 * lane;
+  if ((dh & 3) == 0) {  // rows of whole 16-byte pieces (the partial buffers are 256-byte aligned)
+    if (col < dh)
+      for (int rr = warp; rr < nrow; rr += 4)
+        *reinterpret_cast<float4*>(base + (size_t)(mt * kMT + rr) * dh + col) =
+            *reinterpret_cast<const float4*>(stile + rr * TS + 4 * lane);
+  } else {
+    for (int rr = warp; rr < nrow; rr += 4)
+      for (int c = lane; c < kNT && nt * kNT + c < dh; c += 32)
+        base[(size_t)(mt * kMT + rr) * dh + nt * kNT + c] = stile[rr * TS + c];
   }
   tc_fence_before();
   __syncthreads();
