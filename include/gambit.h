@@ -358,8 +358,8 @@ gb_status gb_pool_launch_count(gb_pool* pool, uint64_t* count);
  * GB_ERR_TIMEOUT.  gb_paged_decode_noalloc_status() reads that status word.
  *
  * The scratch array is shared by every call on a device and keeps the last call's
- * contents; each call rewrites all of it that it reads, and clears its own status
- * word first.  Calls whose GPU work overlaps (different streams, or host threads issuing
+ * contents; each call rewrites all of it that it reads, and its last launch
+ * publishes its status.  Calls whose GPU work overlaps (different streams, or host threads issuing
  * concurrently) race on it: keep them ordered, e.g. on one stream.
  * The first call on a device looks up the array's device address with
  * cudaGetSymbolAddress (with that device current); that first call should come

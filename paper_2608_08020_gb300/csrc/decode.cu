@@ -1,7 +1,8 @@
 // Split-KV flash-decode over the paged pool (per-beam path) and the LSE combine.
-// Two per-beam kernels share the work decomposition and the record format below:
-// k_decode_mma (bf16 pools with 128-dim heads; warp-level MMAs, further down) and
-// k_decode (fp32 pools, and callers' own pages without a tensor map; paired fp32 FMAs).
+// Three per-beam kernels share the work decomposition and the record format below:
+// k_decode_mma (bf16 pools with 128-dim heads; warp-level MMAs, further down),
+// k_decode_pool (other pools) and k_decode (callers' own pages without a tensor map),
+// both with paired fp32 FMAs (decode_range).
 //
 // Work decomposition: the per-beam work of a step is the flat list of
 // (beam, kv-head, 16-token chunk) units, ordered beam-major.  Every warp of a
@@ -9,10 +10,11 @@
 // balanced to within one chunk whatever the beams' lengths.  A warp streams
 // its chunks through a private ring of shared-memory stages filled by TMA.
 // When its range leaves a (beam, head) it writes an unnormalised partial
-// (m, l, o) for the G query heads of that KV head; the combine kernel merges
-// the partials of each (beam, head) with the standard log-sum-exp rule.
+// (m, l, o) for the G query heads of that KV head; the partials of each
+// (beam, head) are merged with the standard log-sum-exp rule: in the launch itself for a pool
+// (combine.cuh, or a team's shared memory on small steps), by k_combine for callers' rows.
 //
-// k_decode fills a stage with two 1D bulk copies (one 4 KiB K slab and one
+// decode_range fills a stage with two 1D bulk copies (one 4 KiB K slab and one
 // 4 KiB V slab per chunk, both contiguous in a page).  Its lane layout inside
 // a warp: 4 token rows x 8 lanes.  Lane j of row r owns
 // two 16-byte pieces of every token row (bytes [16j, 16j+16) and
@@ -87,8 +89,21 @@ __device__ __forceinline__ void unpack16x2(const uint4& u, float2* f) {
   }
 }
 
-// The plan (plan 0) in shared memory, and this warp's barriers.
-template <int DT, bool Pool, class S>
+// This warp's barriers.
+template <int DT, class S>
+__device__ __forceinline__ void decode_barriers() {
+  extern __shared__ __align__(128) unsigned char smem[];
+  if ((threadIdx.x & 31) == 0) {
+    const uint32_t bar0 =
+        smem_addr(smem + (threadIdx.x >> 5) * S::WARP_BYTES + S::STAGES * KvTraits<DT>::STAGE_BYTES + S::PBUF);
+    for (int s = 0; s < S::STAGES; ++s) mbar_init(bar0 + 8 * s, 1);
+    fence_mbar_init();
+  }
+  __syncwarp();
+}
+
+// The plan (plan 0) of a pool's step in shared memory, and the barriers.
+template <int DT, class S>
 __device__ __forceinline__ void decode_setup(const PoolView& v) {
   extern __shared__ __align__(128) unsigned char smem[];
   int* s_off = reinterpret_cast<int*>(smem + S::WARPS * S::WARP_BYTES);
@@ -104,18 +119,11 @@ __device__ __forceinline__ void decode_setup(const PoolView& v) {
       s_off[i] = off[i];
       s_n[i] = i < v.max_beams ? nn[i] : 0;
       s_start[i] = i < v.max_beams ? st[i] : 0;
-      if (Pool) {
-        s_len[i] = i < v.max_beams ? v.seq_len[i] : 0;
-        s_cow[i] = i < v.max_beams ? v.cow_old[i] : -1;
-      }
+      s_len[i] = i < v.max_beams ? v.seq_len[i] : 0;
+      s_cow[i] = i < v.max_beams ? v.cow_old[i] : -1;
     }
   }
-  const int warp = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0) {
-    const uint32_t bar0 = smem_addr(smem + warp * S::WARP_BYTES + S::STAGES * KvTraits<DT>::STAGE_BYTES + S::PBUF);
-    for (int s = 0; s < S::STAGES; ++s) mbar_init(bar0 + 8 * s, 1);
-    fence_mbar_init();
-  }
+  decode_barriers<DT, S>();
   __syncthreads();
 }
 
@@ -473,6 +481,57 @@ __device__ __forceinline__ void decode_body(const PoolView& v, const Counters& c
     decode_range<DT, G, Pool, false, S>(v, cnt, layer, qptr, nw, qscale, w, x_begin, x_end, k, nullptr);
 }
 
+// Work plan of caller-owned rows, made by every CTA for itself in shared memory: every row with
+// seq_len > 0 is read whole.  A row whose length is negative or longer than its table (max_pages x P
+// tokens) is not read at all: its output is zero and the call's status records GB_ERR_INVALID.
+// CTA 0 leaves the plan in global memory for k_combine.
+template <class S>
+__device__ __forceinline__ void rows_plan(const PoolView& v) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  int* s_off = reinterpret_cast<int*>(smem + S::WARPS * S::WARP_BYTES);
+  int* s_n = s_off + (kMaxBeams + 1);
+  int* s_start = s_n + (kMaxBeams + 1);
+  int* tmp = s_start + 2 * (kMaxBeams + 1);  // the pool form's last array: 33 words of the scan
+  constexpr int kMaxPer = kMaxBeams / (kDecodeWarps * 32);
+  static_assert(kMaxBeams % (kDecodeWarps * 32) == 0, "rows per thread");
+  const int nb = v.max_beams, per = (nb + (int)blockDim.x - 1) / (int)blockDim.x, r0 = (int)threadIdx.x * per;
+  int n[kMaxPer], sum = 0;
+#pragma unroll
+  for (int i = 0; i < kMaxPer; ++i) {
+    n[i] = 0;
+    if (i < per && r0 + i < nb) {
+      const int L = v.seq_len[r0 + i];
+      if (L < 0 || (long long)L > (long long)v.max_pages * v.P)
+        set_status(v.ctl, GB_ERR_INVALID);
+      else
+        n[i] = (L + kChunk - 1) / kChunk;
+    }
+    sum += n[i] * v.Hkv;
+  }
+  int total;
+  int off = block_exclusive_scan(sum, tmp, &total);
+#pragma unroll
+  for (int i = 0; i < kMaxPer; ++i) {
+    if (i < per && r0 + i < nb) {
+      s_off[r0 + i] = off;
+      s_n[r0 + i] = n[i];
+      s_start[r0 + i] = 0;
+    }
+    off += n[i] * v.Hkv;
+  }
+  if (threadIdx.x == 0) {
+    s_off[nb] = total;
+    s_n[nb] = 0;
+    s_start[nb] = 0;
+  }
+  __syncthreads();
+  if (blockIdx.x == 0)
+    for (int i = threadIdx.x; i <= nb; i += blockDim.x) {
+      plan_off(v, 0)[i] = s_off[i];
+      plan_n(v, 0)[i] = s_n[i];
+    }
+}
+
 // Caller-owned rows: the records are merged by k_combine.
 template <int DT, int G>
 __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
@@ -480,7 +539,8 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
   pdl_wait();
   pdl_launch_dependents();
   using S = DecodeSmem<DT, G>;
-  decode_setup<DT, false, S>(v);
+  rows_plan<S>(v);
+  decode_barriers<DT, S>();
   decode_body<DT, G, false, S>(v, Counters{}, 0, qptr, NewRows{}, qscale, (int)blockIdx.x * kDecodeWarps + (int)(threadIdx.x >> 5),
                                (int)gridDim.x * kDecodeWarps);
 }
@@ -507,7 +567,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
   const int set = counter_set(v, layer), W = nctas * kDecodeWarps;
   const Counters cnt = counters(v, set);
   zero_counters(v, set ^ 1, cta, nctas);
-  decode_setup<DT, true, S>(v);
+  decode_setup<DT, S>(v);
   extern __shared__ __align__(128) unsigned char smem[];
   const int* s_off = reinterpret_cast<const int*>(smem + S::WARPS * S::WARP_BYTES);
   const int* s_n = s_off + (kMaxBeams + 1);
@@ -628,8 +688,11 @@ __global__ void __launch_bounds__(128) k_combine(PoolView v, int W, float* __res
   const int b = bh / v.Hkv, h = bh % v.Hkv;
   const int G = v.G, D = v.D, GD = G * D;
   float* ob = out + ((size_t)b * v.Hq + (size_t)h * G) * D;
-  const bool ok = v.ctl[kCtlStepOk] != 0 && v.active[b] != 0;
-  const int n = ok ? plan_n(v, 0)[b] : 0;
+  if (bh == 0 && threadIdx.x == 0) {  // the call's status: published, and clear for the next call
+    v.ctl[kRowsStatus] = v.ctl[kCtlStatus];
+    v.ctl[kCtlStatus] = GB_OK;
+  }
+  const int n = plan_n(v, 0)[b];
   if (n == 0) {
     for (int e = threadIdx.x; e < GD; e += blockDim.x) ob[e] = 0.f;
     return;

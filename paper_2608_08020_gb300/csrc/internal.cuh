@@ -55,6 +55,10 @@ enum Ctl : int {
 
 // Words of a counter set.
 enum CounterWord : int {
+// Control words of a call on caller-owned rows: its kernels record errors in kCtlStatus, the last one
+// publishes that in kRowsStatus and clears it, so that no launch has to clear it first.
+constexpr int kRowsStatus = 2;
+
   kCntGrpNext = 0,   // next grouped work unit to hand out
   kCntGrpDone = 1,   // grouped-role CTAs finished
   kCntPairNext = 2,  // next (beam, KV head) pair to merge

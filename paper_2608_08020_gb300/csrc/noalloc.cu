@@ -44,49 +44,18 @@ cudaError_t scratch_address(int device, void** out) {
 size_t round256(size_t x) { return (x + 255) & ~size_t(255); }
 
 struct ScratchLayout {
-  size_t ctl, active, plan, partials, total;
+  size_t ctl, flags, plan, partials, total;
 };
 
 ScratchLayout scratch_layout(int beams, int Hkv, int W, int record_floats) {
   ScratchLayout s{};
   size_t o = 0;
   s.ctl = o;      o = round256(o + kCtlWords * sizeof(int));
-  s.active = o;   o = round256(o + (size_t)beams * sizeof(int));
+  s.flags = o;    o = round256(o + (size_t)beams * sizeof(int));  // counted in the documented size; not used
   s.plan = o;     o = round256(o + 3 * (size_t)(beams + 1) * sizeof(int));
   s.partials = o; o = round256(o + (size_t)(W + beams * Hkv) * record_floats * sizeof(float));
   s.total = o;
   return s;
-}
-
-// Work plan for caller-owned rows (one thread per row): every row with seq_len > 0 is
-// read whole.  A row whose length is negative or longer than its table
-// (max_pages_per_beam x page_size tokens) is not read at all: its output is zero and the
-// call's status records GB_ERR_INVALID.  The status word, the one scratch value that must
-// start at zero, is cleared first.
-__global__ void __launch_bounds__(1024) k_noalloc_plan(PoolView v) {
-  pdl_wait();
-  pdl_launch_dependents();
-  __shared__ int tmp[33];
-  const int b = threadIdx.x;
-  if (b == 0) v.ctl[kCtlStatus] = GB_OK;
-  __syncthreads();
-  const int L = b < v.max_beams ? v.seq_len[b] : 0;
-  const bool bad = b < v.max_beams && (L < 0 || (long long)L > (long long)v.max_pages * v.P);
-  if (bad) set_status(v.ctl, GB_ERR_INVALID);
-  const bool act = L > 0 && !bad;
-  const int n = act ? (L + kChunk - 1) / kChunk : 0;
-  int total;
-  const int off = block_exclusive_scan(n * v.Hkv, tmp, &total);
-  if (b < v.max_beams) {
-    v.active[b] = act ? 1 : 0;
-    plan_off(v, 0)[b] = off;
-    plan_n(v, 0)[b] = n;
-    plan_start(v, 0)[b] = 0;
-  }
-  if (b == 0) {
-    plan_off(v, 0)[v.max_beams] = total;
-    v.ctl[kCtlStepOk] = 1;
-  }
 }
 
 }  // namespace
@@ -138,13 +107,11 @@ extern "C" gb_status gb_paged_decode_noalloc(const gb_paged_decode_args* a, gb_s
   v.tables = const_cast<int*>(a->tables);
   v.seq_len = const_cast<int*>(a->seq_len);
   v.ctl = reinterpret_cast<int*>(sc + L.ctl);
-  v.active = reinterpret_cast<int*>(sc + L.active);
   v.plan = reinterpret_cast<int*>(sc + L.plan);
   v.partials = reinterpret_cast<float*>(sc + L.partials);
   v.record_floats = record_floats;
 
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if (launch_pdl(k_noalloc_plan, 1, 1024, 0, s, v) != cudaSuccess) return GB_ERR_CUDA;
   if (launch_decode_view(v, W, a->q, a->scale, a->out, s) != cudaSuccess) return GB_ERR_CUDA;
   return GB_OK;
 }
@@ -155,10 +122,10 @@ extern "C" gb_status gb_paged_decode_noalloc_status(int* device_status, gb_strea
   if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= kMaxDevices) return GB_ERR_CUDA;
   void* base = nullptr;
   if (scratch_address(device, &base) != cudaSuccess) return GB_ERR_CUDA;
-  // The status word is the first word of the scratch array (ScratchLayout::ctl = 0).
+  // The control words come first in the scratch array (ScratchLayout::ctl = 0).
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   int v = GB_OK;
-  if (cudaMemcpyAsync(&v, static_cast<const int*>(base) + kCtlStatus, sizeof(int), cudaMemcpyDeviceToHost, s) !=
+  if (cudaMemcpyAsync(&v, static_cast<const int*>(base) + kRowsStatus, sizeof(int), cudaMemcpyDeviceToHost, s) !=
           cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return GB_ERR_CUDA;
