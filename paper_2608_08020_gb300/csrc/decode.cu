@@ -564,7 +564,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
     zero_all_pairs<G, D>(v, cta, nctas, out);
     return;
   }
-  const int set = counter_set(v, layer), W = nctas * kDecodeWarps;
+  const int set = counter_set(v, layer, v.ctl[kCtlSteps]), W = nctas * kDecodeWarps;
   const Counters cnt = counters(v, set);
   zero_counters(v, set ^ 1, cta, nctas);
   decode_setup<DT, S>(v);
@@ -654,14 +654,15 @@ __global__ void __launch_bounds__(kMmaWarps * 32, 1)
   const bool early = layer > 0;
   enter(!early);
   const int c = (int)blockIdx.x, nctas = (int)gridDim.x;
-  if (v.ctl[kCtlStepOk] == 0) {
+  const int step_ok = v.ctl[kCtlStepOk], steps = v.ctl[kCtlSteps], team = v.ctl[kCtlTeamPerBeam];
+  if (step_ok == 0) {
     enter(early);
     zero_all_pairs<G>(v, c, nctas, out);
     return;
   }
-  const int set = counter_set(v, layer);
-  if (local_step_per_beam(v, nctas)) {
-    local_attention<G>(v, &tm, &tmh, layer, q, nw, qscale, c, nctas, out, early);
+  const int set = counter_set(v, layer, steps);
+  if (team > 0) {
+    local_attention<G>(v, &tm, &tmh, layer, q, nw, qscale, team, c, nctas, out, early);
     zero_counters(v, set ^ 1, c, nctas);
     return;
   }

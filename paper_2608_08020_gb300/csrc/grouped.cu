@@ -709,15 +709,18 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   // all S resident at once, all S merging; the rest leave at once.  The smallest steps run
   // without either role (local.cuh).
   const int S = (int)gridDim.x / 2, c = (int)blockIdx.x;
-  if (v.ctl[kCtlStepOk] == 0) {
+  // One round trip for the three words: a second is 0.6 us of a small layer-step, twice (the CTAs from
+  // S on start when the first ones have left).
+  const int step_ok = v.ctl[kCtlStepOk], steps = v.ctl[kCtlSteps], team = v.ctl[kCtlTeam];
+  if (step_ok == 0) {
     enter(early);
     zero_all_pairs<G>(v, c, 2 * S, out);
     return;
   }
-  const int set = counter_set(v, layer);
-  if (allow_local && local_step(v, S)) {
+  const int set = counter_set(v, layer, steps);
+  if (allow_local && team > 0) {
     if (c >= S) return;
-    local_attention<G>(v, &tmd, &tmdh, layer, q, nw, qscale, c, S, out, early);
+    local_attention<G>(v, &tmd, &tmdh, layer, q, nw, qscale, team, c, S, out, early);
     zero_counters(v, set ^ 1, c, S);
     return;
   }

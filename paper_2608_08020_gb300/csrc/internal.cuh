@@ -44,6 +44,8 @@ enum Ctl : int {
   kCtlSegTileTok = 11, // sum over segments of (128-row tiles) x tokens
   kCtlSteps = 12,      // steps opened so far (index into the step-stats ring)
   kCtlSegSplit = 13,   // tokens per grouped work unit (segments are split along tokens)
+  kCtlTeam = 14,       // warps per team of the local form this step takes on the default path, 0: the roles
+  kCtlTeamPerBeam = 15,  // the same on the per-beam path
   kCtlSegTok = 16,     // sum over segments of their tokens (the shared tokens the grouped path reads once)
   kCtlBarCount = 17,   // grid-barrier arrivals of the tournament kernel (only grows)
   kCtlSegGen = 19,     // segment rebuilds so far (stamps the per-page claim words)
@@ -53,12 +55,12 @@ enum Ctl : int {
   kCtlWords = 32
 };
 
-// Words of a counter set.
-enum CounterWord : int {
 // Control words of a call on caller-owned rows: its kernels record errors in kCtlStatus, the last one
 // publishes that in kRowsStatus and clears it, so that no launch has to clear it first.
 constexpr int kRowsStatus = 2;
 
+// Words of a counter set.
+enum CounterWord : int {
   kCntGrpNext = 0,   // next grouped work unit to hand out
   kCntGrpDone = 1,   // grouped-role CTAs finished
   kCntPairNext = 2,  // next (beam, KV head) pair to merge
@@ -153,8 +155,8 @@ struct Counters {
 __device__ __forceinline__ Counters counters(const PoolView& v, int set) {
   return {v.ctl + kCtlCounters + kCntWords * set, v.pair_cnt + (size_t)set * v.max_beams * v.Hkv};
 }
-__device__ __forceinline__ int counter_set(const PoolView& v, int layer) {
-  return (v.ctl[kCtlSteps] * v.layers + layer) & 1;
+__device__ __forceinline__ int counter_set(const PoolView& v, int layer, int steps) {  // steps: v.ctl[kCtlSteps]
+  return (steps * v.layers + layer) & 1;
 }
 // Zero set `set`, spread over the grid (`cta` of CTAs of this size).
 __device__ __forceinline__ void zero_counters(const PoolView& v, int set, int cta, int nctas) {
@@ -165,7 +167,7 @@ __device__ __forceinline__ void zero_counters(const PoolView& v, int set, int ct
 }
 
 #ifndef GB_DECODE_WEIGHT
-#define GB_DECODE_WEIGHT 45  // relative cost of a per-beam token against a grouped tile token (percent)
+#define GB_DECODE_WEIGHT 56  // relative cost of a per-beam token against a grouped tile token (percent)
 #endif
 
 #ifndef GB_SPLIT_BYTES_PER_SM
@@ -177,8 +179,13 @@ __device__ __forceinline__ void zero_counters(const PoolView& v, int set, int ct
 // latency-bound and run side by side, each on its own share of the CTAs (one per SM): the
 // per-beam role takes decode_ctas(v, grid) of them, in proportion to its (16-token chunk x
 // KV head) tokens against the grouped role's (128-row tile x token) work per KV head, and
-// the grouped role the rest.  Otherwise every CTA runs the grouped role and then the
-// per-beam role.  The kernel and the combine compute the same split from the step's plan.
+// the grouped role the rest.  Otherwise the per-beam CTAs follow the grouped ones onto the SMs
+// they leave.  The roles and the merge compute the same split from the step's plan.
+// A grouped unit costs about 256 tokens beside its own (its queries, its record).  Two CTAs more than
+// the share, rounded up: where the tails are short the share is 7-15 CTAs and one too few costs 5% of
+// the step.  Per layer-step (us), with weight 45, no unit term and the share rounded / now: 74 / 62
+// (64 beams x 4090, tails 0.13 of the grouped tokens), 231 / 183 (198 x 8190, 0.11), 189 / 178
+// (90 x 9000, 0.56), 113 / 114 (250 x 7000, 1.05), 116 / 117 (120 x 12000, G = 8, 0.74).
 __device__ __forceinline__ int decode_ctas(const PoolView& v, int grid);
 
 // Element offset of row `row` of the K (kv=0) or V (kv=1) slab of (layer, page, head).
@@ -221,9 +228,10 @@ __device__ __forceinline__ int decode_ctas(const PoolView& v, int grid) {
   const long long td = (long long)plan_off(v, 1)[v.max_beams] * kChunk;  // tokens x KV heads
   const long long tg = (long long)v.ctl[kCtlSegTileTok] * v.Hkv;
   if (!split_sms(v, td, tg)) return grid;
-  const long long wd = td * GB_DECODE_WEIGHT, wg = tg * 100;
-  const long long n = (wd * grid + (wd + wg) / 2) / (wd + wg);
-  return (int)(n < 1 ? 1 : (n > grid - 1 ? grid - 1 : n));
+  const long long wd = td * GB_DECODE_WEIGHT, wg = (tg + 256ll * v.ctl[kCtlSegTiles] * v.Hkv) * 100;
+  long long n = (wd * grid + wd + wg - 1) / (wd + wg);
+  if (2 * n < grid) n += 2;
+  return (int)(n > grid - 1 ? grid - 1 : n);
 }
 
 __device__ __forceinline__ void set_status(int* ctl, int code) {

@@ -6,83 +6,25 @@
 // w = 1, 2, 3, 4, 6 or 12 warps of one CTA takes a (beam, KV head) pair at a time, splits the beam's
 // whole context (shared pages included: they come from L2) into w runs of chunks, and merges the
 // warps' softmax states through shared memory: no records, no counters, no waits between CTAs.
-// The arithmetic of a chunk is the per-beam role's (decode_mma.cuh).
+// The arithmetic of a chunk is the per-beam role's (decode_mma.cuh).  Which steps take this form is
+// in step_form.cuh.
 #pragma once
 #include "decode_mma.cuh"
 
 namespace gb {
 
-#ifndef GB_LOCAL_SCALE
-#define GB_LOCAL_SCALE 1  // for sweeps of the rule below
-#endif
-
-// Whether local_attention on `nctas` CTAs beats the two roles.  It takes about 8 us + 1.0 us per
-// chunk and warp; the roles take 35-40 us at least with their merge, the time of their bytes above
-// that, and about 3 us per grouped unit and SM.  Measured per layer-step, local / roles (us):
-// 3.5 chunks per warp 11.5 / 28 (32 beams x 400), 17.7: 25.6 / 40 (64 x 1000), 26: 34 / 40
-// (64 x 1500), 28.5: 41 / 60 (13 x 8000, G = 8); from there on it depends on what sharing saves:
-// 35: 43 / 45.5 and 47 / 53.5 with 2-2.6 times the roles' reads, 40: 46 / 50 (2.9 times), 53: 68 / 64
-// (2.4 times), 56: 62 / 53 (4.8 times), 70: 72 / 45 (prompt of 3500 of 4000 tokens); and many small
-// segments cost the grouped role more: 56: 68 / 87 (9.5 units per SM), 74 / 158 (18 units).
-__device__ __forceinline__ bool local_step(const PoolView& v, int nctas) {
-  const long long all = plan_off(v, 0)[v.max_beams];  // (beam, head, chunk) units of the whole contexts
-  const long long roles = plan_off(v, 1)[v.max_beams] + (long long)v.ctl[kCtlSegTileTok] * v.Hkv / kChunk;
-  const long long units = (long long)v.ctl[kCtlSegTiles] * v.Hkv - 3 * nctas;  // grouped units above 3 per SM
-  const long long w = (long long)kMmaWarps * nctas;
-  return all <= GB_LOCAL_SCALE * (w * (all <= 3 * roles ? 44 : 28) + (units > 0 ? 4 * kMmaWarps * units : 0));
-}
-
-// Warps per team: the number that minimises rounds of pairs x (chunks per warp + what a pair
-// costs beside its chunks: page ids, query rows and the first load, then the merge of a team).
-// *cost gets that, in the time of a chunk.
-__device__ __forceinline__ int local_team(int npairs, int chunks_per_pair, int nctas, int* cost_out) {
-  const int ws[6] = {1, 2, 3, 4, 6, 12};
-  int best = 1, best_cost = 0x7fffffff;
-#pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    const int w = ws[i], teams = nctas * (kMmaWarps / w);
-    const int cost = (npairs + teams - 1) / teams * ((chunks_per_pair + w - 1) / w + 3 + (w > 1 ? 1 : 0));
-    if (cost < best_cost) {
-      best = w;
-      best_cost = cost;
-    }
-  }
-  *cost_out = best_cost;
-  return best;
-}
-static_assert(kMmaWarps == 12, "team sizes divide the CTA's warps");
-
-// The same for the per-beam path, whose other form splits the whole contexts evenly over all warps
-// of the GPU.  Where beams share pages, siblings of neighbouring teams read them at about the same
-// time here, and from L2: 79 against 117 us per layer-step for 64 beams x 4000 tokens, 188 / 326
-// (193 x 2962), 101 / 160 (40 x 8000, whose pairs fill 73% of the teams' rounds), 370 / 448
-// (256 x 4000), 265 / 256-303 (152 x 4000).  So a tree whose beams share a third of their contexts
-// takes this form unless uneven rounds cost it more than 1.6 times; one that shares little has
-// nothing to gain but an even split.
-__device__ __forceinline__ bool local_step_per_beam(const PoolView& v, int nctas) {
-  const long long all = plan_off(v, 0)[v.max_beams], w = kMmaWarps * nctas;
-  if (all <= GB_LOCAL_SCALE * 44 * w) return true;
-  if (!v.grouped || v.ctl[kCtlSegCount] == 0) return false;
-  const long long unshared = plan_off(v, 1)[v.max_beams] + (long long)v.ctl[kCtlSegTok] * v.Hkv / kChunk;
-  if (2 * all < 3 * unshared) return false;
-  const int npairs = v.max_beams * v.Hkv;
-  int cost;
-  local_team(npairs, (int)((all + npairs - 1) / npairs), nctas, &cost);
-  return 5ll * cost <= 8 * ((all + w - 1) / w + 6);
-}
-
 __device__ __forceinline__ void team_sync(int team, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(threads) : "memory");
 }
 
-// All pairs of the pool, CTA `cta` of `nctas`; kMmaWarps * 32 threads.  Shared memory: the warps'
+// All pairs of the pool by teams of w warps, CTA `cta` of `nctas`; kMmaWarps * 32 threads.  Shared memory: the warps'
 // stages and barriers as in decode_mma_body; a warp's record for its team's merge lies over its
 // own stages, which are idle by then.
 template <int G>
 __device__ __forceinline__ void local_attention(const PoolView& v, const CUtensorMap* tm_p, const CUtensorMap* tmh_p,
                                                 int layer, const __nv_bfloat16* __restrict__ q, const NewRows& nw,
-                                                float qscale, int cta, int nctas, float* __restrict__ out,
-                                                bool early) {
+                                                float qscale, int w, int cta, int nctas,
+                                                float* __restrict__ out, bool early) {
   using S = DecodeMmaSmem;
   constexpr int HS = 132;  // floats per head of a record: 128 and a pad, so that the stores below
                            // (4 head pairs x 8 rows) fall on 32 banks
@@ -95,8 +37,6 @@ __device__ __forceinline__ void local_attention(const PoolView& v, const CUtenso
   static_assert((G * HS + 2 * G) * 4 <= kMmaStages * kMmaStageBytes, "a record fits the warp's stages");
 
   const int npairs = v.max_beams * v.Hkv;
-  int cost;
-  const int w = local_team(npairs, (plan_off(v, 0)[v.max_beams] + npairs - 1) / npairs, nctas, &cost);
   const int tpc = kMmaWarps / w, team = warp / w, wi = warp - team * w;
 
   if (lane == 0) {

@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "internal.cuh"
+#include "step_form.cuh"
 
 namespace gb {
 
@@ -254,6 +255,7 @@ __global__ void __launch_bounds__(1024) k_step_begin(PoolView v, int n_tokens, c
   if (b == 0) {
     s_ncow = 0;
     s_len = 0;
+    s_tok[0] = s_tok[1] = 0;
     s_ctl[0] = v.ctl[kCtlFree];
     s_ctl[1] = v.ctl[kCtlSteps];
     s_ctl[2] = v.ctl[kCtlSegRowTok];
@@ -414,11 +416,15 @@ __global__ void __launch_bounds__(1024) k_step_begin(PoolView v, int n_tokens, c
   }
   // Decode plans: mode 0 reads every token per beam; mode 1 skips the prefix
   // covered by grouped shared-prefix segments.
+  int chunks[2];
+#pragma unroll
   for (int mode = 0; mode < 2; ++mode) {
     int start = 0;
     if (mode == 1 && act) start = cover * v.P;
     if (start > Lnew) start = Lnew;
     const int n = act ? (Lnew - start + kChunk - 1) / kChunk : 0;
+    const int toks = __reduce_add_sync(0xffffffffu, act ? Lnew - start : 0);
+    if ((b & 31) == 0) atomicAdd(&s_tok[mode], toks);  // read after the scan's barriers
     int total;
     const int off = block_exclusive_scan(n * v.Hkv, tmp, &total);
     if (b < v.max_beams) {
@@ -427,10 +433,10 @@ __global__ void __launch_bounds__(1024) k_step_begin(PoolView v, int n_tokens, c
       plan_start(v, mode)[b] = start;
     }
     if (b == 0) plan_off(v, mode)[v.max_beams] = total;
-    int tok_total;
-    block_exclusive_scan(act ? Lnew - start : 0, tmp, &tok_total);
-    if (b == 0) s_tok[mode] = tok_total;
+    chunks[mode] = total;
   }
+  if (b < 32 && v.dtype == GB_BF16 && v.D == 128)
+    choose_forms(v, chunks[0], chunks[1], nact, s_ctl[3], s_ctl[5], s_ctl[4], s_ctl[6]);
   if (b == 0) {
     // Work of this step: tokens each path reads per KV head, and the segment work of the
     // grouped path (valid until the next rebuild).
