@@ -12,9 +12,10 @@
 //   x   += W_o a;   u = LN2(x);   x += W_2 (SiLU(W_1 u) * W_3 u)  (Eq. 5)
 //   y_t  = sigmoid(w_out . LN(x) + b_out)                        (Eq. 6)
 // Every product runs on tcgen05 (bf16 operands, fp32 accumulation).  W_in, whose K is the
-// generator's hidden size, is the split-K GEMM of gemm.cu; the others are k_fused_gemm, which
-// builds its A operand itself (LayerNorm of the residual stream, or the attention output rounded
-// to bf16) and finishes the product (RoPE, residual add, SwiGLU) in the same launch.  The residual
+// generator's hidden size, is the split-K GEMM of gemm.cu; the others are, up to d_model 512,
+// k_fused_gemm, which builds its A operand itself (LayerNorm of the residual stream, or the
+// attention output rounded to bf16) and finishes the product (RoPE, residual add, SwiGLU) in the
+// same launch, and above that the split-K GEMM and an epilogue (split_products).  The residual
 // stream x is fp32; the operands of the products (LayerNorm outputs, q/k/v, attention outputs,
 // SwiGLU outputs) are rounded to bf16.
 //
@@ -264,7 +265,7 @@ __global__ void __launch_bounds__(kRowThreads) k_head(const float* __restrict__ 
 // recomputed by every column tile (its rows come from L2), and the weights, which do not depend on
 // the previous launch, are loaded before waiting for it.  mt is the smallest that keeps the grid
 // within the SMs: fewer rows per CTA shorten its own chain.
-enum AMode { kALn, kAF32, kABf16 };              // LayerNorm of fp32 rows; fp32 rows; bf16 rows
+enum AMode { kALn, kAF32, kABf16 };              // LayerNorm of fp32 rows (K <= kFK); fp32 rows; bf16 rows
 enum EMode { kEQkv, kEResid, kESwiglu };         // RoPE and q/k/v in bf16; x += z; SwiGLU in bf16
 
 constexpr int kFThreads = 256, kFN = 64;
@@ -272,8 +273,7 @@ constexpr int kFK = 512;                                    // K a warp's regist
 constexpr int kFBBlock = kFN * 128;                         // 64 of K of the weights: 64 rows x 128 bytes
 constexpr int kFOperands = 192 * 1024;                      // A (mt rows x pass_k) and the weights (64 x pass_k)
 constexpr int kFCtl = kFOperands;                           // mbarrier, tensor-memory address
-constexpr int kFStat = kFCtl + 16;                          // float [2][128]: mean and 1/std of the rows
-constexpr int kFSmem = kFStat + 1024;
+constexpr int kFSmem = kFCtl + 16;
 constexpr int kFTile = kFN + 1;                             // epilogue tile [mt][65] over the A operand
 static_assert(kFSmem <= 232448 - 1024, "shared memory per block");
 // K per pass: what fits beside the weights, one pass up to 1024 for the 32-row tiles of small steps.
@@ -315,8 +315,6 @@ __global__ void __launch_bounds__(kFThreads, 1) k_fused_gemm(FusedArgs p) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int m0 = blockIdx.x * p.mt, t = blockIdx.y;
   const uint32_t sbase = smem_addr(sm), bar = sbase + kFCtl;
-  float* s_mu = reinterpret_cast<float*>(sm + kFStat);
-  float* s_rs = s_mu + 128;
   if (sbase & 1023) {
     if (tid == 0) set_status(p.ctl, GB_ERR_UNSUPPORTED);
     return;
@@ -349,35 +347,6 @@ __global__ void __launch_bounds__(kFThreads, 1) k_fused_gemm(FusedArgs p) {
 
   const float* af = static_cast<const float*>(p.a);
   auto live_row = [&](int r) { return r < p.mt && m0 + r < p.M && row_live(p.active, m0 + r); };
-  // LayerNorm statistics of rows longer than one pass: the mean, then the centred squares.
-  if (A == kALn && p.K > kFK) {
-    for (int r = warp; r < p.mt; r += kFThreads / 32) {
-      if (!live_row(r)) continue;
-      const float4* row = reinterpret_cast<const float4*>(af + (size_t)(m0 + r) * p.K);
-      float s = 0.f, v = 0.f;
-#pragma unroll 4
-      for (int i = lane; i < p.K / 4; i += 32) {
-        const float4 y = row[i];
-        s += (y.x + y.y) + (y.z + y.w);
-      }
-      const float mu = warp_sum(s) / (float)p.K;
-#pragma unroll 4
-      for (int i = lane; i < p.K / 4; i += 32) {
-        const float4 y = row[i];
-        v = fmaf(y.x - mu, y.x - mu, v);
-        v = fmaf(y.y - mu, y.y - mu, v);
-        v = fmaf(y.z - mu, y.z - mu, v);
-        v = fmaf(y.w - mu, y.w - mu, v);
-      }
-      const float rs = 1.0f / sqrtf(warp_sum(v) / (float)p.K + kLnEps);
-      if (lane == 0) {
-        s_mu[r] = mu;
-        s_rs[r] = rs;
-      }
-    }
-    __syncwarp();  // a row's statistics are read by the warp that wrote them
-  }
-
   bool ok = true;
   int pass = 0;
   uint32_t tmem = 0;
@@ -441,7 +410,7 @@ __global__ void __launch_bounds__(kFThreads, 1) k_fused_gemm(FusedArgs p) {
         }
         // The four rows' statistics together: their shuffles are independent chains.
         float mu[4] = {0.f, 0.f, 0.f, 0.f}, rs[4] = {1.f, 1.f, 1.f, 1.f};
-        if (A == kALn && p.K <= kFK) {
+        if (A == kALn) {
           float s[4], q[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
@@ -471,13 +440,6 @@ __global__ void __launch_bounds__(kFThreads, 1) k_fused_gemm(FusedArgs p) {
             for (int u = 0; u < 4; ++u) q[u] += __shfl_xor_sync(0xffffffffu, q[u], o);
 #pragma unroll
           for (int u = 0; u < 4; ++u) rs[u] = 1.0f / sqrtf(q[u] / (float)p.K + kLnEps);
-        } else if (A == kALn) {
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-            if (live_row(r0 + kFThreads / 32 * u)) {
-              mu[u] = s_mu[r0 + kFThreads / 32 * u];
-              rs[u] = s_rs[r0 + kFThreads / 32 * u];
-            }
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
@@ -590,6 +552,151 @@ __global__ void k_first_position_attention(const __nv_bfloat16* __restrict__ vn,
   for (int j = threadIdx.x; j < Hq * kHd; j += blockDim.x) att[j] = __bfloat162float(vn[(j / kHd / G) * kHd + j % kHd]);
 }
 
+// ---- products with K-split partials (split_products) ----------------------------------------------
+//
+// d_model above 512: a product is k_gemm_partials (gemm.cu) and an epilogue that sums its partials,
+// one CTA per row, four columns per thread (16-byte loads, the splits in flight together).
+
+// Columns n .. n + 3 of row m, the splits in order.
+__device__ __forceinline__ float4 sum_partials(const float* __restrict__ P, int splits, int M, int N, int m, int n) {
+  float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+  for (int k = 0; k < splits; ++k) {
+    const float4 y = *reinterpret_cast<const float4*>(P + ((size_t)k * M + m) * N + n);
+    z = make_float4(z.x + y.x, z.y + y.y, z.z + y.z, z.w + y.w);
+  }
+  return z;
+}
+
+__device__ __forceinline__ void store_bf16x4(__nv_bfloat16* d, float a, float b, float c, float e) {
+  __nv_bfloat162 p[2] = {__floats2bfloat162_rn(a, b), __floats2bfloat162_rn(c, e)};
+  *reinterpret_cast<uint2*>(d) = *reinterpret_cast<const uint2*>(p);
+}
+
+enum RowMode { kGeluLn = 0, kResidLn = 1, kResid = 2 };
+
+// Epilogue of a d-wide product: x = GELU(z) (kGeluLn) or x += z, then u = LN(x) in bf16 (not kResid,
+// which the head follows).  Inactive rows: u = 0.
+template <int Mode>
+__global__ void __launch_bounds__(kRowThreads) k_row_epilogue(const float* __restrict__ P, int splits, int M, int d,
+                                                              float* __restrict__ x, const float* __restrict__ g,
+                                                              const float* __restrict__ b, const int* __restrict__ active,
+                                                              __nv_bfloat16* __restrict__ u) {
+  pdl_wait();
+  pdl_launch_dependents();
+  extern __shared__ float row[];
+  __shared__ float red[33];
+  const int m = blockIdx.x, n4 = d / 4;
+  __nv_bfloat16* um = u + (size_t)m * d;
+  if (!row_live(active, m)) {
+    if (Mode != kResid)
+      for (int i = threadIdx.x; i < n4; i += blockDim.x) store_bf16x4(um + 4 * i, 0.f, 0.f, 0.f, 0.f);
+    return;
+  }
+  float4* xm = reinterpret_cast<float4*>(x + (size_t)m * d);
+  float4* row4 = reinterpret_cast<float4*>(row);
+  float s = 0.f;
+  for (int i = threadIdx.x; i < n4; i += blockDim.x) {
+    float4 z = sum_partials(P, splits, M, d, m, 4 * i);
+    if (Mode == kGeluLn) {
+      z.x = 0.5f * z.x * (1.0f + erff(z.x * 0.70710678118654752f));
+      z.y = 0.5f * z.y * (1.0f + erff(z.y * 0.70710678118654752f));
+      z.z = 0.5f * z.z * (1.0f + erff(z.z * 0.70710678118654752f));
+      z.w = 0.5f * z.w * (1.0f + erff(z.w * 0.70710678118654752f));
+    } else {
+      const float4 y = xm[i];
+      z = make_float4(y.x + z.x, y.y + z.y, y.z + z.z, y.w + z.w);
+    }
+    xm[i] = z;
+    row4[i] = z;
+    s += (z.x + z.y) + (z.z + z.w);
+  }
+  if (Mode == kResid) return;
+  const float mu = block_sum(s, red) / (float)d;
+  float v = 0.f;
+  for (int i = threadIdx.x; i < n4; i += blockDim.x) {  // the elements this thread wrote
+    const float4 y = row4[i];
+    v = fmaf(y.x - mu, y.x - mu, v);
+    v = fmaf(y.y - mu, y.y - mu, v);
+    v = fmaf(y.z - mu, y.z - mu, v);
+    v = fmaf(y.w - mu, y.w - mu, v);
+  }
+  const float r = 1.0f / sqrtf(block_sum(v, red) / (float)d + kLnEps);
+  for (int i = threadIdx.x; i < n4; i += blockDim.x) {
+    const float4 y = row4[i], gg = reinterpret_cast<const float4*>(g)[i], bb = reinterpret_cast<const float4*>(b)[i];
+    store_bf16x4(um + 4 * i, (y.x - mu) * r * gg.x + bb.x, (y.y - mu) * r * gg.y + bb.y, (y.z - mu) * r * gg.z + bb.z,
+                 (y.w - mu) * r * gg.w + bb.w);
+  }
+}
+
+// Epilogue of the q/k/v product: the (i, i + 64) pairs of every q and k head are rotated by
+// pos * 10000^(-i/64) with pos = pos_of[m] + pos_shift (0 without pos_of).
+__global__ void __launch_bounds__(kRowThreads) k_qkv_epilogue(const float* __restrict__ P, int splits, int M, int Hq,
+                                                              int Hkv, const int* __restrict__ pos_of, int pos_shift,
+                                                              const int* __restrict__ active,
+                                                              __nv_bfloat16* __restrict__ q,
+                                                              __nv_bfloat16* __restrict__ kn,
+                                                              __nv_bfloat16* __restrict__ vn) {
+  pdl_wait();
+  pdl_launch_dependents();
+  const int m = blockIdx.x, N = (Hq + 2 * Hkv) * kHd;
+  const bool live = row_live(active, m);
+  const float pos = pos_of && live ? (float)(pos_of[m] + pos_shift) : 0.f;
+  constexpr int kQuads = kHd / 8;  // groups of four pairs per head
+  for (int j = threadIdx.x; j < (Hq + Hkv) * kQuads; j += blockDim.x) {
+    const int head = j / kQuads, i = 4 * (j % kQuads);
+    float a[4] = {0.f, 0.f, 0.f, 0.f}, c[4] = {0.f, 0.f, 0.f, 0.f};
+    if (live) {
+      const float4 y1 = sum_partials(P, splits, M, N, m, head * kHd + i);
+      const float4 y2 = sum_partials(P, splits, M, N, m, head * kHd + i + kHd / 2);
+      const float x1[4] = {y1.x, y1.y, y1.z, y1.w}, x2[4] = {y2.x, y2.y, y2.z, y2.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        float sn, cs;
+        sincosf(pos * powf(10000.0f, -(float)(i + e) / (float)(kHd / 2)), &sn, &cs);
+        a[e] = x1[e] * cs - x2[e] * sn;
+        c[e] = x1[e] * sn + x2[e] * cs;
+      }
+    }
+    __nv_bfloat16* dst = head < Hq ? q + ((size_t)m * Hq + head) * kHd : kn + ((size_t)m * Hkv + head - Hq) * kHd;
+    store_bf16x4(dst + i, a[0], a[1], a[2], a[3]);
+    store_bf16x4(dst + i + kHd / 2, c[0], c[1], c[2], c[3]);
+  }
+  for (int j = 4 * threadIdx.x; j < Hkv * kHd; j += 4 * blockDim.x) {
+    const float4 z = live ? sum_partials(P, splits, M, N, m, (Hq + Hkv) * kHd + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+    store_bf16x4(vn + (size_t)m * Hkv * kHd + j, z.x, z.y, z.z, z.w);
+  }
+}
+
+// SwiGLU epilogue: u[m][n] = SiLU(z[m][n]) * z[m][F + n] in bf16 (z = W_13 u, F wide halves).
+__global__ void __launch_bounds__(kRowThreads) k_swiglu_epilogue(const float* __restrict__ P, int splits, int M, int F,
+                                                                 const int* __restrict__ active,
+                                                                 __nv_bfloat16* __restrict__ u) {
+  pdl_wait();
+  pdl_launch_dependents();
+  const int m = blockIdx.x;
+  const bool live = row_live(active, m);
+  auto act = [](float g1, float g3) { return g1 / (1.0f + expf(-g1)) * g3; };
+  for (int n = 4 * threadIdx.x; n < F; n += 4 * blockDim.x) {
+    float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (live) {
+      const float4 g1 = sum_partials(P, splits, M, 2 * F, m, n), g3 = sum_partials(P, splits, M, 2 * F, m, F + n);
+      y = make_float4(act(g1.x, g3.x), act(g1.y, g3.y), act(g1.z, g3.z), act(g1.w, g3.w));
+    }
+    store_bf16x4(u + (size_t)m * F + n, y.x, y.y, y.z, y.w);
+  }
+}
+
+// Attention outputs (fp32) to the bf16 operand of W_o.
+__global__ void __launch_bounds__(kRowThreads) k_to_bf16(const float* __restrict__ a, int n4, __nv_bfloat16* __restrict__ u) {
+  pdl_wait();
+  pdl_launch_dependents();
+  const int i = blockIdx.x * kRowThreads + threadIdx.x;
+  if (i >= n4) return;
+  const float4 y = reinterpret_cast<const float4*>(a)[i];
+  store_bf16x4(u + 4 * (size_t)i, y.x, y.y, y.z, y.w);
+}
+
 struct Run {
   gb_pool* pool;
   Dims s;
@@ -628,6 +735,56 @@ struct Run {
     return launch_pdl(k_fused_gemm<A, E>, dim3((p.M + p.mt - 1) / p.mt, tiles), kFThreads, kFSmem, st, p) == cudaSuccess;
   }
 
+  template <int Mode>
+  void rows(int splits, int M, const float* g, const float* b, const int* active) {
+    launch_pdl(k_row_epilogue<Mode>, M, kRowThreads, s.d * sizeof(float), st, static_cast<const float*>(part()), splits,
+               M, s.d, x(), g, b, active, u());
+    ++launches;
+  }
+
+  // How a layer's products run: above d_model 512 a fused product's CTAs would each normalise rows of
+  // several passes (and W_2's K runs with it).
+  bool split_products() const { return s.d > kFK; }
+
+  bool layer_split(int l, int M, bool step, const int* active, __nv_bfloat16* q, __nv_bfloat16* kn, __nv_bfloat16* vn,
+                   float* att) {
+    const float* P = part();
+    int sp = gemm(u(), M, wt<__nv_bfloat16>(layer_tensor(l, kWqkv)), s.Nqkv, s.d);
+    if (!sp) return false;
+    launch_pdl(k_qkv_epilogue, M, kRowThreads, 0, st, P, sp, M, s.Hq, s.Hkv,
+               step ? static_cast<const int*>(pool->view.seq_len) : nullptr, l > 0 ? -1 : 0, active, q, kn, vn);
+    ++launches;
+    if (!step && l + 1 == s.L) return true;  // the seed needs only each layer's k and v
+    if (!attend(l, step, q, kn, vn, att)) return false;
+    const int n4 = M * (s.d / 4);
+    launch_pdl(k_to_bf16, (n4 + kRowThreads - 1) / kRowThreads, kRowThreads, 0, st, static_cast<const float*>(att), n4, u());
+    ++launches;
+    sp = gemm(u(), M, wt<__nv_bfloat16>(layer_tensor(l, kWo)), s.d, s.d);
+    if (!sp) return false;
+    rows<kResidLn>(sp, M, wt<float>(layer_tensor(l, kLn2G)), wt<float>(layer_tensor(l, kLn2B)), active);
+    sp = gemm(u(), M, wt<__nv_bfloat16>(layer_tensor(l, kW13)), 2 * s.F, s.d);
+    if (!sp) return false;
+    launch_pdl(k_swiglu_epilogue, M, kRowThreads, 0, st, P, sp, M, s.F, active, u());
+    ++launches;
+    sp = gemm(u(), M, wt<__nv_bfloat16>(layer_tensor(l, kW2)), s.d, s.F);
+    if (!sp) return false;
+    if (l + 1 < s.L)
+      rows<kResidLn>(sp, M, wt<float>(layer_tensor(l + 1, kLn1G)), wt<float>(layer_tensor(l + 1, kLn1B)), active);
+    else
+      rows<kResid>(sp, M, nullptr, nullptr, active);
+    return true;
+  }
+
+  // Attention of layer l over each trace's history, or of the first position alone.
+  bool attend(int l, bool step, __nv_bfloat16* q, __nv_bfloat16* kn, __nv_bfloat16* vn, float* att) {
+    if (step)
+      return gb_decode_attention(pool, l, q, kn, vn, 0.08838834764831845f, att, GB_PATH_AUTO,
+                                 reinterpret_cast<gb_stream_t>(st)) == GB_OK;
+    launch_pdl(k_first_position_attention, 1, kRowThreads, 0, st, static_cast<const __nv_bfloat16*>(vn), s.Hq, s.G, att);
+    ++launches;
+    return true;
+  }
+
   // The layer stack on M rows.  step = true: rows are the step pool's slots, attention
   // runs over each trace's cached history (and appends to it); RoPE positions are the
   // slots' sequence lengths.  step = false: one row at position 0 (the seed), whose
@@ -645,6 +802,10 @@ struct Run {
                           (step ? 0 : (size_t)l * s.Hkv * kHd);
       __nv_bfloat16* vn = reinterpret_cast<__nv_bfloat16*>(ws + (step ? L.vn : L.seedv)) +
                           (step ? 0 : (size_t)l * s.Hkv * kHd);
+      if (split_products()) {
+        if (!layer_split(l, M, step, active, q, kn, vn, att)) return false;
+        continue;
+      }
       // q, k, v = RoPE(W_qkv LN1(x)).  Layer 0 opens the step pool's step, which advances every
       // length by one: the new position is seq_len before layer 0 and seq_len - 1 after it.
       FusedArgs p = base;
@@ -662,15 +823,7 @@ struct Run {
       p.pos_shift = l > 0 ? -1 : 0;
       if (!fused<kALn, kEQkv>(p, s.Nqkv / kFN)) return false;
       if (!step && l + 1 == s.L) break;  // the seed needs only each layer's k and v
-      if (step) {
-        if (gb_decode_attention(pool, l, q, kn, vn, 0.08838834764831845f, att, GB_PATH_AUTO,
-                                reinterpret_cast<gb_stream_t>(st)) != GB_OK)
-          return false;
-      } else {
-        launch_pdl(k_first_position_attention, 1, kRowThreads, 0, st, static_cast<const __nv_bfloat16*>(vn), s.Hq, s.G,
-                   att);
-        ++launches;
-      }
+      if (!attend(l, step, q, kn, vn, att)) return false;
       p = base;  // x += W_o a
       p.a = att;
       p.w = wt<__nv_bfloat16>(layer_tensor(l, kWo));
@@ -707,6 +860,10 @@ struct Run {
     ++launches;
     const int sp = gemm(u(), M, wt<__nv_bfloat16>(2), s.d, s.H);
     if (!sp) return false;
+    if (split_products()) {  // with LN1 of layer 0
+      rows<kGeluLn>(sp, M, wt<float>(layer_tensor(0, kLn1G)), wt<float>(layer_tensor(0, kLn1B)), active);
+      return true;
+    }
     const int n4 = M * (s.d / 4);
     launch_pdl(k_gelu_epilogue, (n4 + kRowThreads - 1) / kRowThreads, kRowThreads, 0, st,
                static_cast<const float*>(part()), sp, n4, x());
