@@ -140,9 +140,12 @@ __global__ void __launch_bounds__(128, 1)
         *reinterpret_cast<float4*>(base + (size_t)(mt * kMT + rr) * dh + col) =
             *reinterpret_cast<const float4*>(stile + rr * TS + 4 * lane);
   } else {
+    const int ncol = min(kNT, dh - nt * kNT);
+#pragma unroll 4
     for (int rr = warp; rr < nrow; rr += 4)
-      for (int c = lane; c < kNT && nt * kNT + c < dh; c += 32)
-        base[(size_t)(mt * kMT + rr) * dh + nt * kNT + c] = stile[rr * TS + c];
+#pragma unroll
+      for (int c = lane; c < kNT; c += 32)
+        if (c < ncol) base[(size_t)(mt * kMT + rr) * dh + nt * kNT + c] = stile[rr * TS + c];
   }
   tc_fence_before();
   __syncthreads();

@@ -23,7 +23,9 @@ namespace {
 // One CTA per slot: thread t sums the K-split partials of columns 4t .. 4t + 3, ... (16-byte loads,
 // several splits in flight; single columns where d_h is not a multiple of 4), applies b1 and relu,
 // weights by w2; the block reduces in a fixed order.
-constexpr int kScoreThreads = 128;
+// Widths that are not a multiple of 4 use all of them, a column each: 132 slots of width 786 take 11.9 us
+// (14.5 before the GEMM's six stages and unrolled stores; 17.6 with 128 threads and rolled stores).
+constexpr int kScoreThreads = 256;  // at most
 
 __global__ void __launch_bounds__(kScoreThreads) k_mlp_score(PoolView v, const float* __restrict__ zp, int splits,
                                                              int dh, const float* __restrict__ b1,
@@ -40,7 +42,7 @@ __global__ void __launch_bounds__(kScoreThreads) k_mlp_score(PoolView v, const f
   }
   float acc = 0.f;
   if ((dh & 3) == 0) {  // four columns per thread, 16-byte loads
-    for (int n = 4 * tid; n < dh; n += 4 * kScoreThreads) {
+    for (int n = 4 * tid; n < dh; n += 4 * (int)blockDim.x) {
       float4 z = make_float4(b1[n], b1[n + 1], b1[n + 2], b1[n + 3]);
 #pragma unroll 8
       for (int k = 0; k < splits; ++k) {
@@ -53,7 +55,7 @@ __global__ void __launch_bounds__(kScoreThreads) k_mlp_score(PoolView v, const f
       acc = fmaf(fmaxf(z.w, 0.f), w2[n + 3], acc);
     }
   } else {
-    for (int n = tid; n < dh; n += kScoreThreads) {
+    for (int n = tid; n < dh; n += (int)blockDim.x) {
       float z = b1[n];
 #pragma unroll 8
       for (int k = 0; k < splits; ++k) z += zp[((size_t)k * v.max_beams + b) * dh + n];
@@ -66,7 +68,7 @@ __global__ void __launch_bounds__(kScoreThreads) k_mlp_score(PoolView v, const f
   __syncthreads();
   if (tid == 0) {
     float y = 0.f;
-    for (int w = 0; w < kScoreThreads / 32; ++w) y += red[w];
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) y += red[w];
     const float x = 1.0f / (1.0f + expf(-(y + b2)));
     if (score_out) score_out[b] = x;
     if (mask == nullptr || mask[b] != 0) {
@@ -88,8 +90,8 @@ cudaError_t launch_mlp(gb_pool* pool, const void* hidden, int H, const void* w1,
   prof_begin(pool, GB_PROF_PROBE, s);
   cudaError_t e = gemm_partials(hidden, v.max_beams, w1, dh, H, splits, v.mlp_scratch, v.ctl, false, s);
   if (e != cudaSuccess) return e;
-  e = launch_pdl(k_mlp_score, v.max_beams, kScoreThreads, 0, s, v, static_cast<const float*>(v.mlp_scratch), splits,
-                 dh, b1, w2, b2, mask, score_out);
+  e = launch_pdl(k_mlp_score, v.max_beams, (dh & 3) == 0 ? kScoreThreads / 2 : kScoreThreads, 0, s, v,
+                 static_cast<const float*>(v.mlp_scratch), splits, dh, b1, w2, b2, mask, score_out);
   if (e != cudaSuccess) return e;
   prof_end(pool, GB_PROF_PROBE, s);
   pool->launches += 2;
