@@ -741,7 +741,7 @@ def run_ours(args) -> None:
             "plan": statistics.mean(profs[i]["plan"][0].elapsed_time(profs[i]["plan"][1]) for i in pl) * 1e3,
             "append": statistics.mean(a.elapsed_time(b) for i in pl for a, b in profs[i]["app"]) * 1e3,
             "attention": statistics.mean(dec_ms) * 1e3,
-            # the bf16 kernels merge their records in the same launch; the fp32 one is followed by k_combine
+            # every pool's attention launch appends and merges itself: these events bracket no launch
             "combine": (statistics.mean(a.elapsed_time(b) for i in pl for a, b in profs[i]["comb"]) * 1e3
                         if not (wl.kv_dtype == "bf16" and D == 128) else None),
         }
