@@ -387,14 +387,14 @@ __device__ __forceinline__ void decode_mma_body(const PoolView& v, const Counter
   bool fresh = true;
   uint4 nrow = make_uint4(0u, 0u, 0u, 0u);  // 16 bytes of the pair's new rows: lanes 0-15 K, 16-31 V
   int npage = 0;                            // the page they go to
-  int tail0 = 0x7fffffff;                   // first token of a tail page copied on write, if the beam has one
+  int special = 0;  // first token of the pair's chunks that are appended to or copied: one test per chunk
 
   int stage = 0;
   uint32_t parity = 0;
   for (int x = x_begin, k = 0; x < x_end; ++x, ++k) {
     if (fresh) {
       L = s_len[it.b];
-      tail0 = s_cow[it.b] >= 0 ? (L - 1) / v.P * v.P : 0x7fffffff;
+      special = s_cow[it.b] >= 0 ? (L - 1) / v.P * v.P : it.tok0 + (it.n - 1) * kChunk;
       if (it.n - it.i <= x_end - x) {  // this warp holds the pair's last chunk
         nrow = (lane < 16 ? nw.k : nw.v)[((size_t)it.b * v.Hkv + it.h) * 16 + (lane & 15)];
         npage = v.tables[(size_t)it.b * v.max_pages + (L - 1) / v.P];
@@ -413,9 +413,11 @@ __device__ __forceinline__ void decode_mma_body(const PoolView& v, const Counter
     const uint32_t sb = stage0 + stage * kMmaStageBytes;
     const int tok0 = it.tok0 + it.i * kChunk;
     const int nvalid = min(kChunk, L - tok0);  // >= 1: a chunk starts before the beam's length
-    unsigned char* vs = smem + (sb - smem_addr(smem));
-    if (it.i == it.n - 1) chunk_append(v, layer, it.h, L, nvalid, nrow, npage, vs, lane);
-    if (tok0 >= tail0) chunk_copied(v, layer, it.b, it.h, L, tok0, vs, lane);
+    if (tok0 >= special) {
+      unsigned char* vs = smem + (sb - smem_addr(smem));
+      if (it.i == it.n - 1) chunk_append(v, layer, it.h, L, nvalid, nrow, npage, vs, lane);
+      if (s_cow[it.b] >= 0) chunk_copied(v, layer, it.b, it.h, L, tok0, vs, lane);
+    }
     chunk_attend(st, sb, koff, voff, nvalid, qscale, r);
     __syncwarp();
     if (ip_x < x_end) {

@@ -66,6 +66,7 @@ __device__ __forceinline__ void local_attention(const PoolView& v, const CUtenso
     const int i0 = wi * n / w, i1 = (wi + 1) * n / w;
     const int* tb = v.tables + (size_t)b * v.max_pages;
     const int tail = (L - 1) / v.P;
+    const int special = old >= 0 ? tail * v.P / kChunk : n - 1;  // first chunk that is appended to or copied
     PairState st;
     uint4 nrow = make_uint4(0u, 0u, 0u, 0u);
     int npage = 0, pw = 0, pages = 0;
@@ -110,10 +111,12 @@ __device__ __forceinline__ void local_attention(const PoolView& v, const CUtenso
         alive = false;
         break;
       }
-      unsigned char* vs = smem + (stage0 + stage * kMmaStageBytes - smem_addr(smem));
       const int tok0 = i * kChunk, nvalid = min(kChunk, L - tok0);
-      if (i == n - 1) chunk_append(v, layer, h, L, nvalid, nrow, npage, vs, lane);
-      if (old >= 0 && tok0 >= tail * v.P) chunk_copied(v, layer, b, h, L, tok0, vs, lane);
+      if (i >= special) {
+        unsigned char* vs = smem + (stage0 + stage * kMmaStageBytes - smem_addr(smem));
+        if (i == n - 1) chunk_append(v, layer, h, L, nvalid, nrow, npage, vs, lane);
+        if (old >= 0) chunk_copied(v, layer, b, h, L, tok0, vs, lane);
+      }
       chunk_attend(st, stage0 + stage * kMmaStageBytes, koff, voff, nvalid, qscale, r);
       __syncwarp();
       if (ii < i1) {

@@ -435,7 +435,8 @@ __global__ void __launch_bounds__(1024) k_step_begin(PoolView v, int n_tokens, c
     if (b == 0) plan_off(v, mode)[v.max_beams] = total;
     chunks[mode] = total;
   }
-  if (b < 32 && v.dtype == GB_BF16 && v.D == 128)
+  // The last warp, while the first writes the step's record.
+  if (b >> 5 == (int)(blockDim.x >> 5) - 1 && v.dtype == GB_BF16 && v.D == 128)
     choose_forms(v, chunks[0], chunks[1], nact, s_ctl[3], s_ctl[5], s_ctl[4], s_ctl[6]);
   if (b == 0) {
     // Work of this step: tokens each path reads per KV head, and the segment work of the
