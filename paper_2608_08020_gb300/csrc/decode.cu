@@ -469,13 +469,14 @@ __device__ __forceinline__ bool decode_range(const PoolView& v, const Counters& 
   return true;
 }
 
-// An even share of all chunks per warp: warp `w` of W.
+// Share w of all chunks, c per warp.
 template <int DT, int G, bool Pool, class S>
 __device__ __forceinline__ void decode_body(const PoolView& v, const Counters& cnt, int layer,
-                                            const void* __restrict__ qptr, const NewRows& nw, float qscale, int w, int W) {
+                                            const void* __restrict__ qptr, const NewRows& nw, float qscale, int w, int c) {
   extern __shared__ __align__(128) unsigned char smem[];
   const int Tot = reinterpret_cast<const int*>(smem + S::WARPS * S::WARP_BYTES)[v.max_beams];
-  const int c = (Tot + W - 1) / W, x_begin = w * c, x_end = min(Tot, x_begin + c);
+  const long long x0 = (long long)w * c;
+  const int x_begin = (int)min(x0, (long long)Tot), x_end = (int)min(x0 + c, (long long)Tot);
   int k = 0;
   if (x_begin < x_end)
     decode_range<DT, G, Pool, false, S>(v, cnt, layer, qptr, nw, qscale, w, x_begin, x_end, k, nullptr);
@@ -484,18 +485,20 @@ __device__ __forceinline__ void decode_body(const PoolView& v, const Counters& c
 // Work plan of caller-owned rows, made by every CTA for itself in shared memory: every row with
 // seq_len > 0 is read whole.  A row whose length is negative or longer than its table (max_pages x P
 // tokens) is not read at all: its output is zero and the call's status records GB_ERR_INVALID.
-// CTA 0 leaves the plan in global memory for k_combine.
+// CTA 0 leaves the plan in global memory for k_combine.  Returns the chunks per warp: an even share of
+// W warps, but for few rows more, since a row's records are merged in batches of eight by one CTA, a
+// batch taking about as long as a chunk: c + n / (9 c) is least at sqrt(n / 9) for the longest row.
 template <class S>
-__device__ __forceinline__ void rows_plan(const PoolView& v) {
+__device__ __forceinline__ int rows_plan(const PoolView& v, int W) {
   extern __shared__ __align__(128) unsigned char smem[];
   int* s_off = reinterpret_cast<int*>(smem + S::WARPS * S::WARP_BYTES);
   int* s_n = s_off + (kMaxBeams + 1);
   int* s_start = s_n + (kMaxBeams + 1);
-  int* tmp = s_start + 2 * (kMaxBeams + 1);  // the pool form's last array: 33 words of the scan
+  int* tmp = s_start + 2 * (kMaxBeams + 1);  // the pool form's last array: 33 words of the scan, one for the maximum
   constexpr int kMaxPer = kMaxBeams / (kDecodeWarps * 32);
   static_assert(kMaxBeams % (kDecodeWarps * 32) == 0, "rows per thread");
   const int nb = v.max_beams, per = (nb + (int)blockDim.x - 1) / (int)blockDim.x, r0 = (int)threadIdx.x * per;
-  int n[kMaxPer], sum = 0;
+  int n[kMaxPer], sum = 0, longest = 0;
 #pragma unroll
   for (int i = 0; i < kMaxPer; ++i) {
     n[i] = 0;
@@ -507,9 +510,12 @@ __device__ __forceinline__ void rows_plan(const PoolView& v) {
         n[i] = (L + kChunk - 1) / kChunk;
     }
     sum += n[i] * v.Hkv;
+    longest = max(longest, n[i]);
   }
+  if (threadIdx.x == 0) tmp[33] = 0;
   int total;
   int off = block_exclusive_scan(sum, tmp, &total);
+  atomicMax(&tmp[33], longest);
 #pragma unroll
   for (int i = 0; i < kMaxPer; ++i) {
     if (i < per && r0 + i < nb) {
@@ -525,11 +531,15 @@ __device__ __forceinline__ void rows_plan(const PoolView& v) {
     s_start[nb] = 0;
   }
   __syncthreads();
-  if (blockIdx.x == 0)
+  const int c = max(max((total + W - 1) / W, 1), (int)(sqrtf((float)tmp[33] / 9.f) + 0.5f));
+  if (blockIdx.x == 0) {
     for (int i = threadIdx.x; i <= nb; i += blockDim.x) {
       plan_off(v, 0)[i] = s_off[i];
       plan_n(v, 0)[i] = s_n[i];
     }
+    if (threadIdx.x == 0) v.ctl[kRowsShare] = c;
+  }
+  return c;
 }
 
 // Caller-owned rows: the records are merged by k_combine.
@@ -539,10 +549,10 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
   pdl_wait();
   pdl_launch_dependents();
   using S = DecodeSmem<DT, G>;
-  rows_plan<S>(v);
+  const int c = rows_plan<S>(v, (int)gridDim.x * kDecodeWarps);
   decode_barriers<DT, S>();
-  decode_body<DT, G, false, S>(v, Counters{}, 0, qptr, NewRows{}, qscale, (int)blockIdx.x * kDecodeWarps + (int)(threadIdx.x >> 5),
-                               (int)gridDim.x * kDecodeWarps);
+  decode_body<DT, G, false, S>(v, Counters{}, 0, qptr, NewRows{}, qscale,
+                               (int)blockIdx.x * kDecodeWarps + (int)(threadIdx.x >> 5), c);
 }
 
 // A layer-step of an fp32 pool (or a bf16 one too large for a tensor map) in one launch: append,
@@ -587,7 +597,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
     }
   }
   if (tw == 0) {
-    decode_body<DT, G, true, S>(v, cnt, layer, qptr, nw, qscale, cta * kDecodeWarps + warp, W);
+    decode_body<DT, G, true, S>(v, cnt, layer, qptr, nw, qscale, cta * kDecodeWarps + warp, (Tot + W - 1) / W);
     combine_pairs<G, D>(v, cnt, 0, W, 0, false, cta, nctas, out);
     return;
   }
@@ -682,7 +692,7 @@ __global__ void __launch_bounds__(kMmaWarps * 32, 1)
 // rescaled when M rises.  Every thread of a warp reads the same (m, l) words (one head per
 // warp at D = 128, two at D = 64), so those loads are broadcasts; the o loads are float4
 // and coalesced.
-__global__ void __launch_bounds__(128) k_combine(PoolView v, int W, float* __restrict__ out) {
+__global__ void __launch_bounds__(128) k_combine(PoolView v, float* __restrict__ out) {
   pdl_wait();
   pdl_launch_dependents();
   const int bh = blockIdx.x;
@@ -698,8 +708,7 @@ __global__ void __launch_bounds__(128) k_combine(PoolView v, int W, float* __res
     for (int e = threadIdx.x; e < GD; e += blockDim.x) ob[e] = 0.f;
     return;
   }
-  const int Tot = plan_off(v, 0)[v.max_beams];
-  const int c = Tot > 0 ? (Tot + W - 1) / W : 1;
+  const int c = v.ctl[kRowsShare];
   const int off = plan_off(v, 0)[b] + h * n;
   const int first = off / c, npb = n > 0 ? (off + n - 1) / c - first + 1 : 0;  // per-beam records
   const int R = npb;
@@ -823,7 +832,7 @@ static cudaError_t launch_view_t(const PoolView& v, int W, const void* q, float 
   if (e != cudaSuccess) return e;
   e = launch_pdl(k_decode<DT, G>, W / kDecodeWarps, kDecodeWarps * 32, S::TOTAL, s, v, q, scale * 1.4426950408889634f);
   if (e != cudaSuccess) return e;
-  return launch_pdl(k_combine, v.max_beams * v.Hkv, 128, 0, s, v, W, out);
+  return launch_pdl(k_combine, v.max_beams * v.Hkv, 128, 0, s, v, out);
 }
 
 cudaError_t launch_decode_view(const PoolView& v, int W, const void* q, float scale, float* out, cudaStream_t s) {

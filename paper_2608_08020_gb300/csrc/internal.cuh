@@ -58,6 +58,7 @@ enum Ctl : int {
 // Control words of a call on caller-owned rows: its kernels record errors in kCtlStatus, the last one
 // publishes that in kRowsStatus and clears it, so that no launch has to clear it first.
 constexpr int kRowsStatus = 2;
+constexpr int kRowsShare = 3;  // chunks per warp of the call
 
 // Words of a counter set.
 enum CounterWord : int {
