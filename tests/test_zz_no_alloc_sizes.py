@@ -1,6 +1,6 @@
-"""gb_paged_decode_noalloc over both ways it splits its work (teams of warps inside a CTA, and even
-shares with records merged by the last arrival), each call twice and different sizes interleaved, so
-that a call finds the counters and records another size left.
+"""gb_paged_decode_noalloc over the shares its warps take (one chunk, longer ones for few long rows,
+even shares), each call twice and different sizes interleaved, so that a call finds the plan and the
+records another size left.
 
 fp32 and bf16 pages, probabilities in fp32: 1e-5 of the output's scale (fp32 sums), against fp64."""
 import math
@@ -14,8 +14,8 @@ CASES = [  # dtype, G, Hkv, P, row lengths
     ("bf16", 4, 1, 16, [1]),                          # one pair, one chunk
     ("f32", 2, 2, 32, [15, 16, 17, 0, 33]),           # chunk edges, an empty row
     ("bf16", 8, 2, 64, [700, 1, 256, 129]),           # a few ragged rows
-    ("f32", 4, 8, 16, [5000, 3]),                     # one long row: many records of a pair
-    ("bf16", 2, 8, 16, list(range(1, 301))),          # 2400 pairs: a team takes several
+    ("f32", 4, 8, 16, [5000, 3]),                     # one long row: many records of a pair, longer shares
+    ("bf16", 2, 8, 16, list(range(1, 301))),          # 2400 pairs: a warp takes several
     ("bf16", 4, 8, 32, [3000, 4096, 1, 2500] * 12),   # even shares
     ("f32", 8, 4, 64, [900 + 7 * i for i in range(90)]),
 ]
