@@ -13,7 +13,8 @@
 //      keys, shuffles for the strides inside a warp) and derives the same routing; the
 //      parents are spread over the CTAs, and each forks its children's block tables:
 //      a page that c of the parent's children newly hold gets one +c, each child drops
-//      the references of its old table, and the children's per-slot state is written.
+//      the references of its old table, and the children's per-slot state is written once
+//      every CTA has read the state before the round.
 //      Why no page is freed too early: a page held by a surviving beam keeps that
 //      reference for the whole round (survivors are never pruned), so only pages held by
 //      pruned beams alone can reach zero, and no child takes such a page.
@@ -64,30 +65,32 @@ __device__ __forceinline__ unsigned rank_key(float m) {
   return ~asc;
 }
 
-// Grid-wide barrier over a grid whose CTAs are all resident.  The arrival counter only ever
-// grows: barrier n of a grid of G CTAs is passed once it reaches the next multiple of G above
-// a CTA's own arrival, so the last arrival releases everyone with no reset (the count is a
-// multiple of G between launches, which every launch of this kernel on the pool keeps).
+// Grid-wide barrier over a grid whose CTAs are all resident, in two halves (called by thread 0).
+// The arrival counter only ever grows: barrier n of a grid of G CTAs is passed once it reaches the
+// next multiple of G above a CTA's own arrival, so the last arrival releases everyone with no reset
+// (the count is a multiple of G between launches, which every launch of this kernel on the pool
+// keeps).  grid_arrive returns the count to wait for; a CTA waits for it before it arrives again.
+__device__ unsigned grid_arrive(const PoolView& v) {
+  fence_acq_rel_gpu();  // this CTA's accesses before its arrival
+  const unsigned G = gridDim.x;
+  const unsigned old = atomicAdd(reinterpret_cast<unsigned*>(v.ctl + kCtlBarCount), 1u);
+  return (old / G + 1) * G;
+}
+__device__ void grid_wait(const PoolView& v, unsigned target, int* s_fail) {
+  volatile unsigned* cnt = reinterpret_cast<volatile unsigned*>(v.ctl + kCtlBarCount);
+  const uint64_t t0 = globaltimer_ns();
+  for (unsigned it = 1; (int)(*cnt - target) < 0; ++it) {
+    if ((it & 63) == 0 && globaltimer_ns() - t0 > kWaitLimitNs) {
+      set_status(v.ctl, GB_ERR_TIMEOUT);
+      *s_fail = 1;
+      break;
+    }
+  }
+  fence_acq_rel_gpu();  // the other CTAs' accesses after the barrier
+}
 __device__ bool grid_sync(const PoolView& v, int* s_fail) {
   __syncthreads();
-  if (threadIdx.x == 0 && *s_fail == 0) {
-    fence_acq_rel_gpu();  // this CTA's writes before its arrival
-    const unsigned G = gridDim.x;
-    const unsigned old = atomicAdd(reinterpret_cast<unsigned*>(v.ctl + kCtlBarCount), 1u);
-    const unsigned target = (old / G + 1) * G;
-    volatile unsigned* cnt = reinterpret_cast<volatile unsigned*>(v.ctl + kCtlBarCount);
-    if (old + 1 != target) {
-      const uint64_t t0 = globaltimer_ns();
-      for (unsigned it = 1; (int)(*cnt - target) < 0; ++it) {
-        if ((it & 63) == 0 && globaltimer_ns() - t0 > kWaitLimitNs) {
-          set_status(v.ctl, GB_ERR_TIMEOUT);
-          *s_fail = 1;
-          break;
-        }
-      }
-    }
-    fence_acq_rel_gpu();  // the other CTAs' writes after the barrier
-  }
+  if (threadIdx.x == 0 && *s_fail == 0) grid_wait(v, grid_arrive(v), s_fail);
   __syncthreads();
   return *s_fail == 0;
 }
@@ -108,6 +111,16 @@ __device__ __forceinline__ int group_exclusive_scan(int x, int tpb, int* tmp, in
   return pre - base;
 }
 
+// Slot s becomes a child of slot p (its table is done).
+__device__ __forceinline__ void write_child(const PoolView& v, int s, int p, unsigned lineage) {
+  v.seq_len[s] = v.seq_len[p];
+  v.mean[s] = v.mean[p];
+  v.nsteps[s] = v.nsteps[p];
+  v.gen[s] = 0;
+  v.active[s] = 1;
+  v.lineage[s] = lineage;
+}
+
 __global__ void __launch_bounds__(kTourThreads, 1) k_tournament(PoolView v, TourArgs a) {
   pdl_wait();
   __shared__ unsigned long long s_keys[kMaxBeams];
@@ -119,8 +132,8 @@ __global__ void __launch_bounds__(kTourThreads, 1) k_tournament(PoolView v, Tour
   __shared__ unsigned char s_act[kMaxBeams], s_elig[kMaxBeams], s_pruned[kMaxBeams];
   __shared__ int s_pref[kTourThreads];
   __shared__ int tmp[33];
-  __shared__ int s_fail, s_nchild;
-  __shared__ unsigned s_lin0;
+  __shared__ int s_fail, s_nchild, s_per;
+  __shared__ unsigned s_lin0, s_snap;  // s_snap: the arrival count once every CTA has its snapshot (grouped pools)
   __shared__ unsigned long long s_gen;
   // phase 2 (per group of threads: up to 32 groups)
   __shared__ int s_low[32], s_cap[32], s_nst[32], s_carry_g[32];
@@ -159,6 +172,15 @@ __global__ void __launch_bounds__(kTourThreads, 1) k_tournament(PoolView v, Tour
   }
   __syncthreads();
 
+  // parent_of, pruned flags, lineage ids after the round.
+  auto outputs = [&] {
+    if (tid >= cap) return;
+    const int k = childof[tid];
+    if (a.parent_out) a.parent_out[tid] = k >= 0 ? blist[k / s_per] : (s_act[tid] ? tid : -1);
+    if (a.pruned_out) a.pruned_out[tid] = s_pruned[tid];
+    if (a.lineage_out) a.lineage_out[tid] = k >= 0 ? s_lin0 + k : v.lineage[tid];
+  };
+
   // ---- 1. tournament ---------------------------------------------------------------------
   if (forks) {
     const bool act = act_w != 0;
@@ -175,6 +197,8 @@ __global__ void __launch_bounds__(kTourThreads, 1) k_tournament(PoolView v, Tour
     __syncthreads();
     if (act) s_keys[pos] = ((unsigned long long)rank_key(mean_w) << 32) | (unsigned)tid;
     __syncthreads();
+    // This CTA has read every slot's state: from here on others may change it.
+    if (v.grouped && tid == 0) s_snap = grid_arrive(v);
     // Rank (ascending keys; the slot in the low word makes them distinct): each warp sorts its
     // 32 keys in registers (bitonic, by shuffles), then a key's rank is its position in its
     // warp's list plus, for every other list, the number of keys there below it (a binary
@@ -256,20 +280,16 @@ __global__ void __launch_bounds__(kTourThreads, 1) k_tournament(PoolView v, Tour
     }
     __syncthreads();
     if (tid < nchild) childof[cslot[tid]] = tid;
-    if (tid == 0) s_nchild = nchild;
+    if (tid == 0) {
+      s_nchild = nchild;
+      s_per = per;
+    }
     __syncthreads();
     const int npar = (nchild + per - 1) / per;
     const unsigned lin0 = s_lin0;
 
     // Children share their parents' partial tail pages until the next step's planner copies them.
     if (blockIdx.x == 0 && tid == 0 && nchild > 0) v.ctl[kCtlTailShared] = 1;
-    // Outputs (CTA 0): parent_of, pruned flags, lineage ids after the round.
-    if (blockIdx.x == 0 && tid < cap) {
-      const int k = childof[tid];
-      if (a.parent_out) a.parent_out[tid] = k >= 0 ? blist[k / per] : (s_act[tid] ? tid : -1);
-      if (a.pruned_out) a.pruned_out[tid] = s_pruned[tid];
-      if (a.lineage_out) a.lineage_out[tid] = k >= 0 ? lin0 + k : v.lineage[tid];
-    }
     // Fork: this CTA's parents, each by its own group of threads (ppc parents at a time).  For
     // table index i of parent p, each child c either already holds page tp[i] (nothing
     // changes) or drops its old page and takes tp[i]; the new references of one parent's page
@@ -323,18 +343,18 @@ __global__ void __launch_bounds__(kTourThreads, 1) k_tournament(PoolView v, Tour
         if (add > 0) atomicAdd(&v.refcnt[nw], add);
       }
     }
-    __syncthreads();  // every thread has read the children's old lengths
-    // The children's per-slot state, for the parents this CTA forked.
-    for (int c = tid; c < nchild; c += blockDim.x) {
-      const int j = c / per;
-      if (j % (int)gridDim.x != (int)blockIdx.x) continue;
-      const int sl = cslot[c], p = blist[j];
-      v.seq_len[sl] = v.seq_len[p];
-      v.mean[sl] = v.mean[p];
-      v.nsteps[sl] = v.nsteps[p];
-      v.gen[sl] = 0;
-      v.active[sl] = 1;
-      v.lineage[sl] = lin0 + c;
+    // The outputs, and the children's per-slot state for the parents this CTA forked, once every CTA
+    // has read the state before the round (and the caller's mask, which an output may overwrite): a CTA
+    // that started late and read a mix of old and new would route differently from the others.
+    // (Forks decided elsewhere are routed by the caller's array alone, and a CTA uses only its own
+    // children's state.)  A pool without segments writes them at the end.
+    if (v.grouped) {
+      if (a.prune && tid == 0) grid_wait(v, s_snap, &s_fail);
+      __syncthreads();  // also: every thread has read the children's old lengths
+      if (s_fail) return;
+      if (blockIdx.x == 0) outputs();
+      for (int c = tid; c < nchild; c += blockDim.x)
+        if (c / per % (int)gridDim.x == (int)blockIdx.x) write_child(v, cslot[c], blist[c / per], lin0 + c);
     }
     __syncthreads();
     if (tid == 0 && s_freed > 0) {
@@ -343,16 +363,24 @@ __global__ void __launch_bounds__(kTourThreads, 1) k_tournament(PoolView v, Tour
     }
   }
   if (!v.grouped) {
-    // No grouped path: no segments to rebuild.  The lineage counter moves on once every CTA
-    // has read it, which without a barrier the last CTA to finish guarantees.
+    // No grouped path: no segments to rebuild.  The last CTA to finish, by when every CTA has read
+    // the state before the round, writes all children's state and moves the lineage counter on; no
+    // CTA waits for another.
     __shared__ int s_last;
     __threadfence();
     __syncthreads();
-    if (tid == 0) s_last = atomicAdd(&v.ctl[kCtlDone], 1) == (int)gridDim.x - 1;
+    if (tid == 0) {
+      s_last = atomicAdd(&v.ctl[kCtlDone], 1) == (int)gridDim.x - 1;
+      fence_acq_rel_gpu();
+    }
     __syncthreads();
-    if (s_last && tid == 0) {
-      v.ctl[kCtlNextLineage] = (int)(s_lin0 + s_nchild);
-      v.ctl[kCtlDone] = 0;
+    if (s_last) {
+      outputs();
+      if (tid < s_nchild) write_child(v, cslot[tid], blist[tid / s_per], s_lin0 + tid);
+      if (tid == 0) {
+        v.ctl[kCtlNextLineage] = (int)(s_lin0 + s_nchild);
+        v.ctl[kCtlDone] = 0;
+      }
     }
     pdl_launch_dependents();
     return;
