@@ -123,15 +123,17 @@ struct PairState {
   float m0, m1, l0, l1;
 };
 
-// Start pair (b, h): its query rows, an empty softmax.
-template <int G>
+// Start pair (b, h): its query rows, an empty softmax.  Split (chunk_attend): columns G .. 2G - 1 repeat
+// the heads.
+template <int G, bool Split = false>
 __device__ __forceinline__ void pair_begin(PairState& st, const PoolView& v, const __nv_bfloat16* __restrict__ q, int b,
                                            int h, int r, int c) {
-  const uint32_t* qrow = reinterpret_cast<const uint32_t*>(q + ((size_t)b * v.Hq + h * G + r) * 128);
+  const uint32_t* qrow = reinterpret_cast<const uint32_t*>(q + ((size_t)b * v.Hq + h * G + (Split ? r % G : r)) * 128);
+  const bool used = r < (Split ? 2 * G : G);
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
-    st.qf[j][0] = r < G ? qrow[8 * j + c] : 0u;
-    st.qf[j][1] = r < G ? qrow[8 * j + 4 + c] : 0u;
+    st.qf[j][0] = used ? qrow[8 * j + c] : 0u;
+    st.qf[j][1] = used ? qrow[8 * j + 4 + c] : 0u;
   }
 #pragma unroll
   for (int mt = 0; mt < 8; ++mt) st.o[mt][0] = st.o[mt][1] = st.o[mt][2] = st.o[mt][3] = 0.f;
@@ -152,9 +154,19 @@ __device__ __forceinline__ void ldsm_offsets(uint32_t (&koff)[4], uint32_t (&vof
   }
 }
 
+// The two bf16 terms of a pair of fp32 values: hi + lo is within 2^-17 of each.
+__device__ __forceinline__ void split_bf16x2(float a, float b, uint32_t& hi, uint32_t& lo) {
+  hi = pack_bf16x2(a, b);
+  lo = pack_bf16x2(a - __uint_as_float(hi << 16), b - __uint_as_float(hi & 0xffff0000u));
+}
+
 // One landed 16-token chunk (stage address sb, its first nvalid >= 1 tokens) into the pair's state.
+// Split: each probability goes into P.V as two bf16 terms instead of one rounding to bf16.  G <= 4: the
+// second terms take the columns that the heads leave free, whose queries repeat the heads' (pair_begin), so
+// every lane still finds its probabilities in its own scores, and pair_finish adds the columns up.
+template <int G, bool Split>
 __device__ __forceinline__ void chunk_attend(PairState& st, uint32_t sb, const uint32_t (&koff)[4],
-                                             const uint32_t (&voff)[4], int nvalid, float qscale, int r) {
+                                             const uint32_t (&voff)[4], int nvalid, float qscale, int r, int c) {
   // ---- S^T = K . Q^T (kMmaChains independent accumulator chains) -----------
   float sacc[kMmaChains][4];
 #pragma unroll
@@ -205,14 +217,49 @@ __device__ __forceinline__ void chunk_attend(PairState& st, uint32_t sb, const u
   const float p2 = ex2_approx(sc[2] - st.m0), p3 = ex2_approx(sc[3] - st.m1);
   st.l0 += p0 + p2;
   st.l1 += p1 + p3;
-  const uint32_t pb0 = movmatrix_t(pack_bf16x2(p0, p1));  // P^T fragments: tokens 2c (+1), head r
-  const uint32_t pb1 = movmatrix_t(pack_bf16x2(p2, p3));  // tokens 8 + 2c (+1)
+  uint32_t h0, h1, e0 = 0u, e1 = 0u;  // first and second terms
+  if (Split) {
+    split_bf16x2(p0, p1, h0, e0);
+    split_bf16x2(p2, p3, h1, e1);
+    if (G < 8 && 2 * c >= G) {
+      h0 = e0;
+      h1 = e1;
+    }
+  } else {
+    h0 = pack_bf16x2(p0, p1);
+    h1 = pack_bf16x2(p2, p3);
+  }
+  const uint32_t pb0 = movmatrix_t(h0);  // P^T fragments: tokens 2c (+1), head r
+  const uint32_t pb1 = movmatrix_t(h1);  // tokens 8 + 2c (+1)
+  uint32_t pe0 = 0u, pe1 = 0u;
+  if (Split && G == 8) {
+    pe0 = movmatrix_t(e0);
+    pe1 = movmatrix_t(e1);
+  }
   // ---- O^T += V^T . P^T ------------------------------------------------------
 #pragma unroll
   for (int mt = 0; mt < 8; ++mt) {
     uint32_t a0, a1, a2, a3;
     ldsm_x4_t(sb + voff[mt & 3] + (mt >> 2) * 1024, a0, a1, a2, a3);
     mma_bf16(st.o[mt], a0, a1, a2, a3, pb0, pb1);
+    if (Split && G == 8) mma_bf16(st.o[mt], a0, a1, a2, a3, pe0, pe1);
+  }
+}
+
+// After a pair's last chunk: add the second terms' columns to the heads' (Split, G <= 4) and this lane's
+// shares of the sums.
+template <int G, bool Split>
+__device__ __forceinline__ void pair_finish(PairState& st) {
+  if (Split && G < 8) {
+#pragma unroll
+    for (int mt = 0; mt < 8; ++mt)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) st.o[mt][e] += __shfl_down_sync(0xffffffffu, st.o[mt][e], G / 2);
+  }
+#pragma unroll
+  for (int sh = 4; sh < 32; sh <<= 1) {
+    st.l0 += __shfl_xor_sync(0xffffffffu, st.l0, sh);
+    st.l1 += __shfl_xor_sync(0xffffffffu, st.l1, sh);
   }
 }
 
@@ -418,7 +465,7 @@ __device__ __forceinline__ void decode_mma_body(const PoolView& v, const Counter
       if (it.i == it.n - 1) chunk_append(v, layer, it.h, L, nvalid, nrow, npage, vs, lane);
       if (s_cow[it.b] >= 0) chunk_copied(v, layer, it.b, it.h, L, tok0, vs, lane);
     }
-    chunk_attend(st, sb, koff, voff, nvalid, qscale, r);
+    chunk_attend<G, false>(st, sb, koff, voff, nvalid, qscale, r, c);
     __syncwarp();
     if (ip_x < x_end) {
       if (lane == 0) fence_proxy_async_smem();
@@ -435,11 +482,7 @@ __device__ __forceinline__ void decode_mma_body(const PoolView& v, const Counter
     }
     const bool last_of_bh = (it.i == it.n - 1) || (x + 1 == x_end);
     if (last_of_bh) {
-#pragma unroll
-      for (int sh = 4; sh < 32; sh <<= 1) {
-        st.l0 += __shfl_xor_sync(0xffffffffu, st.l0, sh);
-        st.l1 += __shfl_xor_sync(0xffffffffu, st.l1, sh);
-      }
+      pair_finish<G, false>(st);
       float* rec = v.partials + (size_t)(w + it.b * v.Hkv + it.h) * v.record_floats;
       if (2 * c < G) {
         float* o0 = rec + (2 * c) * D + r;

@@ -6,8 +6,10 @@
 // w = 1, 2, 3, 4, 6 or 12 warps of one CTA takes a (beam, KV head) pair at a time, splits the beam's
 // whole context (shared pages included: they come from L2) into w runs of chunks, and merges the
 // warps' softmax states through shared memory: no records, no counters, no waits between CTAs.
-// The arithmetic of a chunk is the per-beam role's (decode_mma.cuh).  Which steps take this form is
-// in step_form.cuh.
+// The arithmetic of a chunk is the per-beam role's (decode_mma.cuh), but for the probabilities, which
+// enter P.V as two bf16 terms: a run of a few chunks rounded to one against its first chunk's maximum is up
+// to 20% less exact than the roles, whose tiles hold 128 tokens and whose runs are other ones.  Which
+// steps take this form is in step_form.cuh.
 #pragma once
 #include "decode_mma.cuh"
 
@@ -95,7 +97,7 @@ __device__ __forceinline__ void local_attention(const PoolView& v, const CUtenso
     for (int s = 0; s < kMmaStages && ii < i1 && alive; ++s, ++ii) issue(ii, (stage + s) % kMmaStages);
     enter(wait);
     wait = false;
-    pair_begin<G>(st, v, q, b, h, r, c);
+    pair_begin<G, true>(st, v, q, b, h, r, c);
     if (i0 < i1 && i1 == n) {  // this warp holds the pair's last chunk
       nrow = (lane < 16 ? nw.k : nw.v)[(size_t)p * 16 + (lane & 15)];
       npage = tb[tail];
@@ -117,7 +119,7 @@ __device__ __forceinline__ void local_attention(const PoolView& v, const CUtenso
         if (i == n - 1) chunk_append(v, layer, h, L, nvalid, nrow, npage, vs, lane);
         if (old >= 0) chunk_copied(v, layer, b, h, L, tok0, vs, lane);
       }
-      chunk_attend(st, stage0 + stage * kMmaStageBytes, koff, voff, nvalid, qscale, r);
+      chunk_attend<G, true>(st, stage0 + stage * kMmaStageBytes, koff, voff, nvalid, qscale, r, c);
       __syncwarp();
       if (ii < i1) {
         if (lane == 0) fence_proxy_async_smem();
@@ -128,11 +130,7 @@ __device__ __forceinline__ void local_attention(const PoolView& v, const CUtenso
         parity ^= 1u;
       }
     }
-#pragma unroll
-    for (int sh = 4; sh < 32; sh <<= 1) {
-      st.l0 += __shfl_xor_sync(0xffffffffu, st.l0, sh);
-      st.l1 += __shfl_xor_sync(0xffffffffu, st.l1, sh);
-    }
+    pair_finish<G, true>(st);
     if (w == 1) {
       if (2 * c < G) {
         float* o0 = ob + 2 * c * 128 + r;
