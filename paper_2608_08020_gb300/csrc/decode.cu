@@ -572,11 +572,12 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
   using S = DecodeSmem<DT, G>;
   constexpr int D = KvTraits<DT>::D, GD = G * D;
   const int cta = (int)blockIdx.x, nctas = (int)gridDim.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (v.ctl[kCtlStepOk] == 0) {
+  const int step_ok = v.ctl[kCtlStepOk], steps = v.ctl[kCtlSteps], nact = v.ctl[kCtlActive];  // one round trip
+  if (step_ok == 0) {
     zero_all_pairs<G, D>(v, cta, nctas, out);
     return;
   }
-  const int set = counter_set(v, layer, v.ctl[kCtlSteps]), W = nctas * kDecodeWarps;
+  const int set = counter_set(v, layer, steps), W = nctas * kDecodeWarps;
   const Counters cnt = counters(v, set);
   zero_counters(v, set ^ 1, cta, nctas);
   decode_setup<DT, S>(v);
@@ -584,20 +585,21 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
   const int* s_off = reinterpret_cast<const int*>(smem + S::WARPS * S::WARP_BYTES);
   const int* s_n = s_off + (kMaxBeams + 1);
   const int Tot = s_off[v.max_beams], npairs = v.max_beams * v.Hkv;
-  // Rounds of pairs x (chunks per warp, about 2 us each, + a pair's start and merge) against an even
-  // share + the record, its count, the wait and the merge.
+  // Rounds of active pairs (a vacant slot's takes no time) x (chunks per warp, about 2 us each, + a pair's
+  // start and merge) against an even share + the record, its count, the wait and the merge.
   int tw = 0;
   {
     int best = (Tot + W - 1) / W + 4;
-    const int n = (Tot + npairs - 1) / npairs;
+    const int pairs = max(nact, 1) * v.Hkv, n = (Tot + pairs - 1) / pairs;
     for (int w = 1; w <= kDecodeWarps; w *= 2) {
-      const int teams = nctas * (kDecodeWarps / w), cost = (npairs + teams - 1) / teams * ((n + w - 1) / w + 2);
+      const int teams = nctas * (kDecodeWarps / w), cost = (pairs + teams - 1) / teams * ((n + w - 1) / w + 2);
       if (cost < best) {
         best = cost;
         tw = w;
       }
     }
   }
+  if (cta == 0 && threadIdx.x == 0) v.ctl[kCtlTeam] = tw;
   if (tw == 0) {
     decode_body<DT, G, true, S>(v, cnt, layer, qptr, nw, qscale, cta * kDecodeWarps + warp, (Tot + W - 1) / W);
     combine_pairs<G, D>(v, cnt, 0, W, 0, false, cta, nctas, out);

@@ -45,9 +45,11 @@ enum Ctl : int {
   kCtlSteps = 12,      // steps opened so far (index into the step-stats ring)
   kCtlSegSplit = 13,   // tokens per grouped work unit (segments are split along tokens)
   kCtlTeam = 14,       // warps per team of the local form this step takes on the default path, 0: the roles
+                       // (an fp32 pool: of the last layer-step's team form, 0: the even split)
   kCtlTeamPerBeam = 15,  // the same on the per-beam path
   kCtlSegTok = 16,     // sum over segments of their tokens (the shared tokens the grouped path reads once)
   kCtlBarCount = 17,   // grid-barrier arrivals of the tournament kernel (only grows)
+  kCtlActive = 18,     // active slots of the open step
   kCtlSegGen = 19,     // segment rebuilds so far (stamps the per-page claim words)
   kCtlSegAlloc = 20,   // words 20-21: (segments << 32 | member slots) handed out by the running rebuild
   kCtlTailShared = 22, // 1 when a partial tail page may be shared (set by seed and forks, cleared by the planner)

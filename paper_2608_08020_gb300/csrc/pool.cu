@@ -454,6 +454,7 @@ __global__ void __launch_bounds__(1024) k_step_begin(PoolView v, int n_tokens, c
     e[8] = v.grouped ? s_ctl[6] : 0;
     e[9] = nact;
     v.ctl[kCtlSteps] = step + 1;
+    v.ctl[kCtlActive] = nact;
   }
   if (b == 0) {
     if (tails_shared) v.ctl[kCtlTailShared] = 0;
