@@ -144,9 +144,10 @@ gb_status gb_pool_seed(gb_pool* pool, int n_beams, int prompt_len, const void* k
  * Launches: one attention launch that also appends the new rows and merges
  * the split and shared-prefix partial results into out_dev; layer 0 adds the
  * step's planner first.  The
- * attention launch's CTAs wait (bounded) on each other's partial results, so
- * they must all get an SM within the wait limit (2 s): nothing else should
- * hold the GPU's SMs for that long meanwhile.
+ * attention launch's CTAs wait (bounded) on each other's partial results where
+ * the pool is bf16 and the step is not a small one, so they must all get an SM
+ * within the wait limit (2 s): nothing else should hold the GPU's SMs for that
+ * long meanwhile.  An fp32 pool's CTAs never wait on one another.
  * Errors: GB_ERR_STATE for a layer out of order; out of pages is reported in
  * the device status and makes the whole step a no-op; a wait that runs out
  * records GB_ERR_TIMEOUT and zeroes the outputs it could not complete.

@@ -1,5 +1,6 @@
 // The log-sum-exp merge of a layer-step's partial attention records, run at the end of the
-// attention launch itself (k_attention, k_decode_mma) rather than as a launch of its own.
+// attention launch itself rather than as a launch of its own: with bounded waits (k_attention,
+// k_decode_mma), as described here, or without any (k_decode_pool, merge_completed below).
 //
 // Each (beam b, KV head h) pair has R = nseg + npb records: on the grouped path, nseg records
 // of the beam's shared-prefix segments, and npb split-KV records of the per-beam warps whose
@@ -182,9 +183,10 @@ __device__ __forceinline__ void zero_all_pairs(const PoolView& v, int cta, int n
 // that start at different times) and fold a pair's segment records before they wait for its
 // split-KV records; otherwise merging CTA `cta` of `nctas` takes the pairs
 // p = cta + nctas * (warp + k * warps per CTA) and waits for all of a pair's records at once.
-template <int G, int D = 128>
+template <int G>
 __device__ __forceinline__ void combine_pairs(const PoolView& v, const Counters& cnt, int mode, int W, int ng,
                                               bool claim, int cta, int nctas, float* __restrict__ out) {
+  constexpr int D = 128;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int npairs = v.max_beams * v.Hkv;
   const int* off = plan_off(v, mode);
@@ -207,7 +209,7 @@ __device__ __forceinline__ void combine_pairs(const PoolView& v, const Counters&
     const int first = o0 / c;
     const int npb = n > 0 ? (o0 + n - 1) / c - first + 1 : 0;
     if (npb + nseg == 0) {
-      zero_pair<G, D>(v, b, h, out);
+      zero_pair<G>(v, b, h, out);
       continue;
     }
     const float* grec = v.grec + ((size_t)b * kMaxSegRecords * v.Hkv + h) * rf;  // [b][record][Hkv]
@@ -233,6 +235,62 @@ __device__ __forceinline__ void combine_pairs(const PoolView& v, const Counters&
       if (lane == 0) set_status(v.ctl, GB_ERR_TIMEOUT);  // kept if already set
       zero_pair<G, D>(v, b, h, out);
     }
+  }
+}
+
+// The merge of a launch whose warps each took chunks [w c, w c + c) of the Tot chunks of the flat list
+// (s_off, s_n: its offsets and chunks per beam), run by every warp after its own: no warp waits.  A
+// warp counts itself at the first and the last pair of its range (release: fence, then the add), and the
+// one that completes a pair's count merges the pair; the pairs between those two are its own.  `good`:
+// the warp wrote all of its records; a pair that misses one gets zeros (the count's high half).
+template <int G, int D>
+__device__ __forceinline__ void merge_completed(const PoolView& v, const Counters& cnt, const int* s_off,
+                                                const int* s_n, int Tot, int c, int w, bool good,
+                                                float* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  const int x0 = (int)min((long long)w * c, (long long)Tot), x1 = min(x0 + c, Tot);
+  if (x0 >= x1) return;
+  const int x = lane == 0 ? x0 : x1 - 1;
+  int lo = 0, hi = v.max_beams;  // invariant: s_off[lo] <= x < s_off[hi]
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (s_off[mid] <= x) lo = mid; else hi = mid;
+  }
+  auto records = [&](int b, int h, int* first) {
+    const int n = s_n[b], o = s_off[b] + h * n;
+    *first = o / c;
+    return (o + n - 1) / c - *first + 1;
+  };
+  int h = (x - s_off[lo]) / s_n[lo], first;
+  const int p = lo * v.Hkv + h, need = records(lo, h, &first);
+  const int p0 = __shfl_sync(0xffffffffu, p, 0), p1 = __shfl_sync(0xffffffffu, p, 1);
+  fence_acq_rel_gpu();  // this warp's records before its counts
+  __syncwarp();
+  int seen = 0;
+  if (lane == 0 || (lane == 1 && p1 != p0)) seen = atomicAdd(&cnt.pair[p], good ? 1 : 0x10001);
+  const bool last = (seen & 0xffff) == need - 1, bad = !good || (seen >> 16) != 0;
+  const unsigned m_last = __ballot_sync(0xffffffffu, last), m_bad = __ballot_sync(0xffffffffu, bad);
+  fence_acq_rel_gpu();  // the other warps' records after their counts
+  int b = __shfl_sync(0xffffffffu, lo, 0);
+  h = p0 - b * v.Hkv;
+  for (int q = p0; q <= p1; ++q, ++h) {
+    if (h == v.Hkv) {
+      h = 0;
+      ++b;
+    }
+    if (s_n[b] == 0) continue;
+    const int l = q == p0 ? 0 : 1;  // the lane that counted this pair, at either end of the range
+    const bool own = q != p0 && q != p1;
+    if (!own && !((m_last >> l) & 1u)) continue;
+    if (own ? !good : ((m_bad >> l) & 1u) != 0) {
+      zero_pair<G, D>(v, b, h, out);
+      continue;
+    }
+    const int npb = records(b, h, &first);
+    MergeState<G, D> st;
+    merge_init(st);
+    merge_fold(st, v.partials + (size_t)(first + q) * v.record_floats, (size_t)v.record_floats, npb);
+    merge_write(v, st, b, h, out);
   }
 }
 

@@ -129,12 +129,11 @@ __device__ __forceinline__ void decode_setup(const PoolView& v) {
 
 // The kernels' body: this warp's chunks [x_begin, x_end) of the flat list; w numbers the warp in the
 // records.  Pool: the step's new rows are appended on the way, as in decode_mma_body, and every
-// record is counted for the merge.  Local: the range lies in one pair and its record goes to `lrec`
+// record is read back by the merge.  Local: the range lies in one pair and its record goes to `lrec`
 // in shared memory.  k counts the chunks consumed so far (stages and phases of the ring).  False
 // once a wait ran out.
 template <int DT, int G, bool Pool, bool Local, class S>
-__device__ __forceinline__ bool decode_range(const PoolView& v, const Counters& cnt, int layer,
-                                             const void* __restrict__ qptr, const NewRows& nw, float qscale, int w,
+__device__ __forceinline__ bool decode_range(const PoolView& v, int layer, const void* __restrict__ qptr, const NewRows& nw, float qscale, int w,
                                              int x_begin, int x_end, int& k_io, float* lrec) {
   using T = KvTraits<DT>;
   constexpr int NS = G / 2;  // scores held per lane after the reduce-scatter
@@ -460,7 +459,6 @@ __device__ __forceinline__ bool decode_range(const PoolView& v, const Counters& 
           rec[G * D + G + g] = ((g / NS) == b0) ? lsum[g % NS] : lother[g % NS];
         }
       }
-      if (Pool && !Local) record_arrive(cnt, it.b * v.Hkv + it.h, lane);
       fresh = true;
     }
     if (x + 1 < x_end) iter_advance(it, s_n, s_start, v.Hkv, v.max_beams);
@@ -469,17 +467,16 @@ __device__ __forceinline__ bool decode_range(const PoolView& v, const Counters& 
   return true;
 }
 
-// Share w of all chunks, c per warp.
+// Share w of all chunks, c per warp.  False once a wait ran out.
 template <int DT, int G, bool Pool, class S>
-__device__ __forceinline__ void decode_body(const PoolView& v, const Counters& cnt, int layer,
-                                            const void* __restrict__ qptr, const NewRows& nw, float qscale, int w, int c) {
+__device__ __forceinline__ bool decode_body(const PoolView& v, int layer, const void* __restrict__ qptr, const NewRows& nw, float qscale, int w, int c) {
   extern __shared__ __align__(128) unsigned char smem[];
   const int Tot = reinterpret_cast<const int*>(smem + S::WARPS * S::WARP_BYTES)[v.max_beams];
   const long long x0 = (long long)w * c;
   const int x_begin = (int)min(x0, (long long)Tot), x_end = (int)min(x0 + c, (long long)Tot);
   int k = 0;
-  if (x_begin < x_end)
-    decode_range<DT, G, Pool, false, S>(v, cnt, layer, qptr, nw, qscale, w, x_begin, x_end, k, nullptr);
+  return x_begin >= x_end ||
+         decode_range<DT, G, Pool, false, S>(v, layer, qptr, nw, qscale, w, x_begin, x_end, k, nullptr);
 }
 
 // Work plan of caller-owned rows, made by every CTA for itself in shared memory: every row with
@@ -553,7 +550,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
   using S = DecodeSmem<DT, G>;
   const int c = rows_plan<S>(v, (int)gridDim.x * kDecodeWarps);
   decode_barriers<DT, S>();
-  decode_body<DT, G, false, S>(v, Counters{}, 0, qptr, NewRows{}, qscale,
+  decode_body<DT, G, false, S>(v, 0, qptr, NewRows{}, qscale,
                                (int)blockIdx.x * kDecodeWarps + (int)(threadIdx.x >> 5), c);
 }
 
@@ -561,8 +558,9 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
 // attention and the merge.  With launches of its own for the append and the merge a step of 8 beams
 // x 256 tokens took 11.8 us, half of it between kernels.  Small steps are merged inside each CTA: a
 // team of 1, 2, 4 or 8 warps takes a (beam, KV head) pair at a time (as in local.cuh).  Otherwise
-// every warp takes an even share of the chunks, and the records are merged through global memory
-// (combine.cuh; one CTA per SM, so every CTA is resident and the merge's waits end).
+// every warp takes an even share of the chunks, and the warp that completes a pair's records merges
+// them through global memory (merge_completed): no CTA waits for another, so the launch needs no
+// residency.
 template <int DT, int G>
 __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
     k_decode_pool(PoolView v, int layer, const void* __restrict__ qptr, NewRows nw, float qscale,
@@ -601,8 +599,11 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
   }
   if (cta == 0 && threadIdx.x == 0) v.ctl[kCtlTeam] = tw;
   if (tw == 0) {
-    decode_body<DT, G, true, S>(v, cnt, layer, qptr, nw, qscale, cta * kDecodeWarps + warp, (Tot + W - 1) / W);
-    combine_pairs<G, D>(v, cnt, 0, W, 0, false, cta, nctas, out);
+    const int c = (Tot + W - 1) / W, w = cta * kDecodeWarps + warp;
+    const bool good = decode_body<DT, G, true, S>(v, layer, qptr, nw, qscale, w, c);
+    merge_completed<G, D>(v, cnt, s_off, s_n, Tot, c, w, good, out);
+    for (int p = w; p < npairs; p += W)  // vacant slots
+      if (s_n[p / v.Hkv] == 0) zero_pair<G, D>(v, p / v.Hkv, p % v.Hkv, out);
     return;
   }
   const int tpc = kDecodeWarps / tw, team = warp / tw, wi = warp - team * tw;
@@ -617,7 +618,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
       continue;
     }
     const int x0 = o0 + wi * n / tw, x1 = o0 + (wi + 1) * n / tw;
-    if (x0 < x1 && alive) alive = decode_range<DT, G, true, true, S>(v, cnt, layer, qptr, nw, qscale, 0, x0, x1, k, lrec);
+    if (x0 < x1 && alive) alive = decode_range<DT, G, true, true, S>(v, layer, qptr, nw, qscale, 0, x0, x1, k, lrec);
     if ((x0 >= x1 || !alive) && lane < G) {  // no chunks (m = -inf, l = 0), or a wait that ran out (l < 0)
       lrec[GD + lane] = -INFINITY;
       lrec[GD + G + lane] = alive ? 0.f : -1.f;
