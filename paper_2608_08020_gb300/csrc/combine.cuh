@@ -238,15 +238,56 @@ __device__ __forceinline__ void combine_pairs(const PoolView& v, const Counters&
   }
 }
 
+// Merge w records in shared memory, `stride` floats apart, into ob[g][:]: out = sum o 2^(m - M) /
+// sum l 2^(m - M), threads t of nt.  A record holds head g's D values at g HS, its m at G HS + g and its l
+// at G HS + G + g; one without tokens has m = -inf and l = 0, and one whose warp's wait ran out has
+// l < 0 (its heads' outputs are zero).
+template <int G, int D, int HS>
+__device__ __forceinline__ void merge_team(const float* recs, int stride, int w, int t, int nt, float* __restrict__ ob) {
+  for (int e = t; e < G * D / 4; e += nt) {
+    const int g = 4 * e / D, d = 4 * e % D;
+    float M = -INFINITY;
+    bool good = true;
+    for (int k = 0; k < w; ++k) {
+      M = fmaxf(M, recs[k * stride + G * HS + g]);
+      good = good && !(recs[k * stride + G * HS + G + g] < 0.f);
+    }
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    float l = 0.f;
+    for (int k = 0; k < w; ++k) {
+      const float m = recs[k * stride + G * HS + g];
+      if (m == -INFINITY) continue;
+      const float sc = exp2f(m - M);
+      const float4 x = *reinterpret_cast<const float4*>(recs + k * stride + g * HS + d);
+      acc.x = fmaf(x.x, sc, acc.x);
+      acc.y = fmaf(x.y, sc, acc.y);
+      acc.z = fmaf(x.z, sc, acc.z);
+      acc.w = fmaf(x.w, sc, acc.w);
+      l = fmaf(recs[k * stride + G * HS + G + g], sc, l);
+    }
+    float* od = ob + 4 * e;
+    od[0] = good ? acc.x / l : 0.f;
+    od[1] = good ? acc.y / l : 0.f;
+    od[2] = good ? acc.z / l : 0.f;
+    od[3] = good ? acc.w / l : 0.f;
+  }
+}
+
+// A pair of more records than this (two batches of merge_fold's loads) is merged by the whole CTA of the
+// warp that completes it, see merge_long.
+template <int G, int D>
+constexpr int kMergeAlone = 2 * (MergeState<G, D>::N >= 8 ? 1 : 16 / MergeState<G, D>::N);
+
 // The merge of a launch whose warps each took chunks [w c, w c + c) of the Tot chunks of the flat list
 // (s_off, s_n: its offsets and chunks per beam), run by every warp after its own: no warp waits.  A
 // warp counts itself at the first and the last pair of its range (release: fence, then the add), and the
 // one that completes a pair's count merges the pair; the pairs between those two are its own.  `good`:
-// the warp wrote all of its records; a pair that misses one gets zeros (the count's high half).
+// the warp wrote all of its records; a pair that misses one gets zeros (the count's high half).  Pairs
+// of many records are left in p_long (room for two a warp), counted in *n_long, for merge_long.
 template <int G, int D>
 __device__ __forceinline__ void merge_completed(const PoolView& v, const Counters& cnt, const int* s_off,
-                                                const int* s_n, int Tot, int c, int w, bool good,
-                                                float* __restrict__ out) {
+                                                const int* s_n, int Tot, int c, int w, bool good, int* n_long,
+                                                int* p_long, float* __restrict__ out) {
   const int lane = threadIdx.x & 31;
   const int x0 = (int)min((long long)w * c, (long long)Tot), x1 = min(x0 + c, Tot);
   if (x0 >= x1) return;
@@ -287,10 +328,46 @@ __device__ __forceinline__ void merge_completed(const PoolView& v, const Counter
       continue;
     }
     const int npb = records(b, h, &first);
+    if (npb > kMergeAlone<G, D>) {
+      if (lane == 0) p_long[atomicAdd(n_long, 1)] = q;
+      continue;
+    }
     MergeState<G, D> st;
     merge_init(st);
     merge_fold(st, v.partials + (size_t)(first + q) * v.record_floats, (size_t)v.record_floats, npb);
     merge_write(v, st, b, h, out);
+  }
+}
+
+// The pairs with many records, by the whole CTA (called by all of its threads after a barrier): each warp
+// folds every Warps-th record, and the warps' states are merged through shared memory (recs, a record every
+// `stride` floats).  With one warp folding them all, a step of one beam x 4000 tokens with 8 heads per KV
+// head spent 60 of its 75 us here.
+template <int G, int D, int Warps>
+__device__ __forceinline__ void merge_long(const PoolView& v, const int* s_off, const int* s_n, int c, int n_long,
+                                           const int* p_long, float* recs, int stride, float* __restrict__ out) {
+  constexpr int GD = G * D;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int i = 0; i < n_long; ++i) {
+    const int q = p_long[i], b = q / v.Hkv, h = q - b * v.Hkv, n = s_n[b], o = s_off[b] + h * n;
+    const int first = o / c, npb = (o + n - 1) / c - first + 1;
+    MergeState<G, D> st;
+    merge_init(st);
+    merge_fold(st, v.partials + (size_t)(first + q + warp) * v.record_floats, (size_t)Warps * v.record_floats,
+               npb > warp ? (npb - warp + Warps - 1) / Warps : 0);
+    float* rec = recs + warp * stride;
+#pragma unroll
+    for (int g = 0; g < MergeState<G, D>::N; ++g) {
+      const int e = 4 * (lane + 32 * g);
+      *reinterpret_cast<float4*>(rec + e) = st.acc[g];
+      if (e % D == 0) {
+        rec[GD + e / D] = st.M[g];
+        rec[GD + G + e / D] = st.L[g];
+      }
+    }
+    __syncthreads();
+    merge_team<G, D, D>(recs, stride, Warps, (int)threadIdx.x, Warps * 32, out + (size_t)q * GD);
+    __syncthreads();
   }
 }
 

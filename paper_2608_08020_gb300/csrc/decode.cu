@@ -129,11 +129,12 @@ __device__ __forceinline__ void decode_setup(const PoolView& v) {
 
 // The kernels' body: this warp's chunks [x_begin, x_end) of the flat list; w numbers the warp in the
 // records.  Pool: the step's new rows are appended on the way, as in decode_mma_body, and every
-// record is read back by the merge.  Local: the range lies in one pair and its record goes to `lrec`
-// in shared memory.  k counts the chunks consumed so far (stages and phases of the ring).  False
-// once a wait ran out.
-template <int DT, int G, bool Pool, bool Local, class S>
-__device__ __forceinline__ bool decode_range(const PoolView& v, int layer, const void* __restrict__ qptr, const NewRows& nw, float qscale, int w,
+// record is read back by the merge.  lrec: the range lies in one pair and its record goes there (shared
+// memory) instead of to the partials.  k counts the chunks consumed so far (stages and phases of the
+// ring).  False once a wait ran out.
+template <int DT, int G, bool Pool, class S>
+__device__ __forceinline__ bool decode_range(const PoolView& v, int layer, const void* __restrict__ qptr,
+                                             const NewRows& nw, float qscale, int w,
                                              int x_begin, int x_end, int& k_io, float* lrec) {
   using T = KvTraits<DT>;
   constexpr int NS = G / 2;  // scores held per lane after the reduce-scatter
@@ -438,7 +439,7 @@ __device__ __forceinline__ bool decode_range(const PoolView& v, int layer, const
       }
 #pragma unroll
       for (int kk = 0; kk < NS; ++kk) lother[kk] = __shfl_xor_sync(0xffffffffu, lsum[kk], 1);
-      float* rec = Local ? lrec : v.partials + (size_t)(w + it.b * v.Hkv + it.h) * v.record_floats;
+      float* rec = lrec != nullptr ? lrec : v.partials + (size_t)(w + it.b * v.Hkv + it.h) * v.record_floats;
       if (row == 0) {
 #pragma unroll
         for (int g = 0; g < G; ++g) {
@@ -467,16 +468,15 @@ __device__ __forceinline__ bool decode_range(const PoolView& v, int layer, const
   return true;
 }
 
-// Share w of all chunks, c per warp.  False once a wait ran out.
-template <int DT, int G, bool Pool, class S>
-__device__ __forceinline__ bool decode_body(const PoolView& v, int layer, const void* __restrict__ qptr, const NewRows& nw, float qscale, int w, int c) {
+// Share w of all chunks of caller-owned rows, c per warp.
+template <int DT, int G, class S>
+__device__ __forceinline__ void decode_body(const PoolView& v, const void* __restrict__ qptr, float qscale, int w, int c) {
   extern __shared__ __align__(128) unsigned char smem[];
   const int Tot = reinterpret_cast<const int*>(smem + S::WARPS * S::WARP_BYTES)[v.max_beams];
   const long long x0 = (long long)w * c;
   const int x_begin = (int)min(x0, (long long)Tot), x_end = (int)min(x0 + c, (long long)Tot);
   int k = 0;
-  return x_begin >= x_end ||
-         decode_range<DT, G, Pool, false, S>(v, layer, qptr, nw, qscale, w, x_begin, x_end, k, nullptr);
+  if (x_begin < x_end) decode_range<DT, G, false, S>(v, 0, qptr, NewRows{}, qscale, w, x_begin, x_end, k, nullptr);
 }
 
 // Work plan of caller-owned rows, made by every CTA for itself in shared memory: every row with
@@ -550,8 +550,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
   using S = DecodeSmem<DT, G>;
   const int c = rows_plan<S>(v, (int)gridDim.x * kDecodeWarps);
   decode_barriers<DT, S>();
-  decode_body<DT, G, false, S>(v, 0, qptr, NewRows{}, qscale,
-                               (int)blockIdx.x * kDecodeWarps + (int)(threadIdx.x >> 5), c);
+  decode_body<DT, G, S>(v, qptr, qscale, (int)blockIdx.x * kDecodeWarps + (int)(threadIdx.x >> 5), c);
 }
 
 // A layer-step of an fp32 pool (or a bf16 one too large for a tensor map) in one launch: append,
@@ -583,11 +582,15 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
   const int* s_off = reinterpret_cast<const int*>(smem + S::WARPS * S::WARP_BYTES);
   const int* s_n = s_off + (kMaxBeams + 1);
   const int Tot = s_off[v.max_beams], npairs = v.max_beams * v.Hkv;
-  // Rounds of active pairs (a vacant slot's takes no time) x (chunks per warp, about 2 us each, + a pair's
-  // start and merge) against an even share + the record, its count, the wait and the merge.
+  // Rounds of active pairs (a vacant slot's takes no time) x (chunks per warp + a pair's start and merge)
+  // against an even share + the record, its count and the merge, in the time of a chunk (1.0-1.4 us in a
+  // team, 1.6-1.9 in an even share).  Over 312 trees of 1 to 128 beams, 1 to 8 KV heads, 40 to 3000 tokens and G
+  // = 2 to 8 with every form forced, this choice takes 0.6% more than the best one on average and 18% at
+  // worst; with + 4 for the even share 1.2% and 26%.  Even / team of 8 / of 4, G = 4, us: 10.4 / 9.6 / 12.3 (1
+  // beam x 8 heads x 300), 30.4 / 33.9 / 28.2 (32 x 8 x 1000), 12.4 / 17.7 / 23.2 (4 x 8 x 1000).
   int tw = 0;
   {
-    int best = (Tot + W - 1) / W + 4;
+    int best = (Tot + W - 1) / W + 5;
     const int pairs = max(nact, 1) * v.Hkv, n = (Tot + pairs - 1) / pairs;
     for (int w = 1; w <= kDecodeWarps; w *= 2) {
       const int teams = nctas * (kDecodeWarps / w), cost = (pairs + teams - 1) / teams * ((n + w - 1) / w + 2);
@@ -598,64 +601,50 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
     }
   }
   if (cta == 0 && threadIdx.x == 0) v.ctl[kCtlTeam] = tw;
-  if (tw == 0) {
-    const int c = (Tot + W - 1) / W, w = cta * kDecodeWarps + warp;
-    const bool good = decode_body<DT, G, true, S>(v, layer, qptr, nw, qscale, w, c);
-    merge_completed<G, D>(v, cnt, s_off, s_n, Tot, c, w, good, out);
-    for (int p = w; p < npairs; p += W)  // vacant slots
-      if (s_n[p / v.Hkv] == 0) zero_pair<G, D>(v, p / v.Hkv, p % v.Hkv, out);
-    return;
-  }
-  const int tpc = kDecodeWarps / tw, team = warp / tw, wi = warp - team * tw;
+  // One loop and one decode_range for both: an even share is a range of its own, a pair a range of each
+  // warp of its team.
+  const int c = (Tot + W - 1) / W, wall = cta * kDecodeWarps + warp;
+  const int tpc = tw > 0 ? kDecodeWarps / tw : 1, team = tw > 0 ? warp / tw : 0, wi = warp - team * tw;
   float* lrec = reinterpret_cast<float*>(smem + warp * S::WARP_BYTES);  // over the warp's idle stages
   static_assert((GD + 2 * G) * 4 <= S::STAGES * KvTraits<DT>::STAGE_BYTES, "a record fits the warp's stages");
   int k = 0;
   bool alive = true;
-  for (int p = cta + nctas * team; p < npairs; p += nctas * tpc) {
-    const int b = p / v.Hkv, h = p - b * v.Hkv, n = s_n[b], o0 = s_off[b] + h * n;
-    if (n == 0) {
-      if (wi == 0) zero_pair<G, D>(v, b, h, out);
-      continue;
+  for (int p = cta + nctas * team; tw == 0 || p < npairs; p += nctas * tpc) {
+    int x0, x1;
+    if (tw == 0) {
+      x0 = (int)min((long long)wall * c, (long long)Tot);
+      x1 = min(x0 + c, Tot);
+    } else {
+      const int b = p / v.Hkv, h = p - b * v.Hkv, n = s_n[b], o0 = s_off[b] + h * n;
+      if (n == 0) {
+        if (wi == 0) zero_pair<G, D>(v, b, h, out);
+        continue;
+      }
+      x0 = o0 + wi * n / tw;
+      x1 = o0 + (wi + 1) * n / tw;
     }
-    const int x0 = o0 + wi * n / tw, x1 = o0 + (wi + 1) * n / tw;
-    if (x0 < x1 && alive) alive = decode_range<DT, G, true, true, S>(v, layer, qptr, nw, qscale, 0, x0, x1, k, lrec);
+    if (x0 < x1 && alive)
+      alive = decode_range<DT, G, true, S>(v, layer, qptr, nw, qscale, wall, x0, x1, k, tw > 0 ? lrec : nullptr);
+    if (tw == 0) break;
     if ((x0 >= x1 || !alive) && lane < G) {  // no chunks (m = -inf, l = 0), or a wait that ran out (l < 0)
       lrec[GD + lane] = -INFINITY;
       lrec[GD + G + lane] = alive ? 0.f : -1.f;
     }
     team_sync(team, tw * 32);
-    const float* recs = reinterpret_cast<const float*>(smem + (size_t)team * tw * S::WARP_BYTES);
-    constexpr int RS = S::WARP_BYTES / 4;
-    for (int e = wi * 32 + lane; e < GD / 4; e += tw * 32) {
-      const int g = 4 * e / D;
-      float M = -INFINITY;
-      bool good = true;
-      for (int i = 0; i < tw; ++i) {
-        M = fmaxf(M, recs[i * RS + GD + g]);
-        good = good && !(recs[i * RS + GD + G + g] < 0.f);
-      }
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-      float l = 0.f;
-      for (int i = 0; i < tw; ++i) {
-        const float m = recs[i * RS + GD + g];
-        if (m == -INFINITY) continue;
-        const float sc = exp2f(m - M);
-        const float4 y = *reinterpret_cast<const float4*>(recs + i * RS + 4 * e);
-        acc.x = fmaf(y.x, sc, acc.x);
-        acc.y = fmaf(y.y, sc, acc.y);
-        acc.z = fmaf(y.z, sc, acc.z);
-        acc.w = fmaf(y.w, sc, acc.w);
-        l = fmaf(recs[i * RS + GD + G + g], sc, l);
-      }
-      float* od = out + (size_t)p * GD + 4 * e;
-      od[0] = good ? acc.x / l : 0.f;
-      od[1] = good ? acc.y / l : 0.f;
-      od[2] = good ? acc.z / l : 0.f;
-      od[3] = good ? acc.w / l : 0.f;
-    }
+    merge_team<G, D, D>(reinterpret_cast<const float*>(smem + (size_t)team * tw * S::WARP_BYTES), S::WARP_BYTES / 4, tw,
+                        wi * 32 + lane, tw * 32, out + (size_t)p * GD);
     fence_proxy_async_smem();  // the records' memory is refilled by bulk copies for the next pair
     team_sync(team, tw * 32);
   }
+  if (tw > 0) return;
+  __shared__ int n_long, p_long[2 * kDecodeWarps];
+  if (threadIdx.x == 0) n_long = 0;
+  __syncthreads();
+  merge_completed<G, D>(v, cnt, s_off, s_n, Tot, c, wall, alive, &n_long, p_long, out);
+  for (int p = wall; p < npairs; p += W)  // vacant slots
+    if (s_n[p / v.Hkv] == 0) zero_pair<G, D>(v, p / v.Hkv, p % v.Hkv, out);
+  __syncthreads();
+  merge_long<G, D, kDecodeWarps>(v, s_off, s_n, c, n_long, p_long, reinterpret_cast<float*>(smem), S::WARP_BYTES / 4, out);
 }
 
 // The per-beam kernel on its own (the per-beam path, every beam reading its whole context):

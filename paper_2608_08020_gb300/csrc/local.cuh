@@ -144,8 +144,7 @@ __device__ __forceinline__ void local_attention(const PoolView& v, const CUtenso
       }
       continue;
     }
-    // The warp's record, then the team's merge: out = sum o 2^(m - M) / sum l 2^(m - M).  A warp
-    // without chunks has m = -inf and l = 0; one whose wait ran out marks its record with l < 0.
+    // The warp's record, then the team's merge (merge_team).
     __syncwarp();
     float* rec = reinterpret_cast<float*>(smem + warp * kMmaStages * kMmaStageBytes);
     if (2 * c < G) {
@@ -165,35 +164,8 @@ __device__ __forceinline__ void local_attention(const PoolView& v, const CUtenso
       }
     }
     team_sync(team, w * 32);
-    const float* recs = reinterpret_cast<const float*>(smem + team * w * kMmaStages * kMmaStageBytes);
-    constexpr int RS = kMmaStages * kMmaStageBytes / 4;  // floats from one warp's record to the next
-    for (int e = wi * 32 + lane; e < G * 32; e += w * 32) {
-      const int g = e >> 5, d = 4 * (e & 31);
-      float M = -INFINITY;
-      bool good = true;
-      for (int k = 0; k < w; ++k) {
-        M = fmaxf(M, recs[k * RS + G * HS + g]);
-        good = good && !(recs[k * RS + G * HS + G + g] < 0.f);
-      }
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-      float l = 0.f;
-      for (int k = 0; k < w; ++k) {
-        const float m = recs[k * RS + G * HS + g];
-        if (m == -INFINITY) continue;
-        const float sc = exp2f(m - M);
-        const float4 x = *reinterpret_cast<const float4*>(recs + k * RS + g * HS + d);
-        acc.x = fmaf(x.x, sc, acc.x);
-        acc.y = fmaf(x.y, sc, acc.y);
-        acc.z = fmaf(x.z, sc, acc.z);
-        acc.w = fmaf(x.w, sc, acc.w);
-        l = fmaf(recs[k * RS + G * HS + G + g], sc, l);
-      }
-      float* od = ob + g * 128 + d;
-      od[0] = good ? acc.x / l : 0.f;
-      od[1] = good ? acc.y / l : 0.f;
-      od[2] = good ? acc.z / l : 0.f;
-      od[3] = good ? acc.w / l : 0.f;
-    }
+    merge_team<G, 128, HS>(reinterpret_cast<const float*>(smem + team * w * kMmaStages * kMmaStageBytes),
+                           kMmaStages * kMmaStageBytes / 4, w, wi * 32 + lane, w * 32, ob);
     fence_proxy_async_smem();  // the records' memory is refilled by TMA for the next pair
     team_sync(team, w * 32);
   }
