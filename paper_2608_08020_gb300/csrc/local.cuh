@@ -59,10 +59,20 @@ __device__ __forceinline__ void local_attention(const PoolView& v, const CUtenso
     const int b = p / v.Hkv, h = p - b * v.Hkv;
     const int n = plan_n(v, 0)[b], L = v.seq_len[b], old = v.cow_old[b];
     float* ob = out + ((size_t)b * v.Hq + (size_t)h * G) * 128;
-    if (n == 0) {  // an inactive slot
+    if (n == 0) {
+      // Vacant slots: the run of them among the team's next 32 pairs at once, shared out among its warps
+      // (1024 slots, 8 of them active: a round trip for each was 15 us of a layer-step's 24).
       enter(wait);
       wait = false;
-      if (wi == 0) zero_pair<G>(v, b, h, out);
+      const int pl = p + lane * nctas * tpc;
+      const bool end = pl >= npairs || plan_n(v, 0)[pl / v.Hkv] != 0;
+      const unsigned ends = __ballot_sync(0xffffffffu, end);
+      const int run = ends != 0 ? __ffs(ends) - 1 : 32;  // >= 1: this one
+      for (int i = wi; i < run; i += w) {
+        const int z = p + i * nctas * tpc;
+        zero_pair<G>(v, z / v.Hkv, z % v.Hkv, out);
+      }
+      p += (run - 1) * nctas * tpc;
       continue;
     }
     const int i0 = wi * n / w, i1 = (wi + 1) * n / w;
