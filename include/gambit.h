@@ -140,7 +140,8 @@ gb_status gb_pool_seed(gb_pool* pool, int n_beams, int prompt_len, const void* k
  *   k_new_dev, v_new_dev: [max_beams][Hkv][D] in kv_dtype
  *   out_dev:    [max_beams][Hq][D] fp32 (rows of inactive slots are zero)
  *   flags:      GB_PATH_AUTO / GB_PATH_PER_BEAM / GB_PATH_GROUPED
- * Rows of inactive slots in the inputs are ignored.
+ * Rows of inactive slots in the inputs are ignored.  out_dev may overlap k_new_dev and
+ * v_new_dev (the rows are then copied first).
  * Launches: one attention launch that also appends the new rows and merges
  * the split and shared-prefix partial results into out_dev; layer 0 adds the
  * step's planner first.  The

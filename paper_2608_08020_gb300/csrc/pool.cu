@@ -20,6 +20,11 @@ namespace gb {
 
 static size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
+// One layer-step's new K (or V) rows.
+static size_t new_rows_bytes(const gb_pool_config& c) {
+  return (size_t)c.max_beams * c.num_kv_heads * c.head_dim * (c.kv_dtype == GB_BF16 ? 2 : 4);
+}
+
 MetaLayout meta_layout(const gb_pool_config& c) {
   MetaLayout m{};
   const size_t B = (size_t)c.max_beams;
@@ -65,7 +70,8 @@ MetaLayout meta_layout(const gb_pool_config& c) {
   m.seg_hist = take(2 * 256 * sizeof(int));
   m.pair_cnt = take(2 * B * c.num_kv_heads * sizeof(int));
   m.stats = take((size_t)kStatsRing * kStatsWords * sizeof(int));
-  m.mlp_scratch = take((size_t)kMlpScratchFloats * sizeof(float));
+  // Also holds a step's new K and V rows where the caller's output overlaps them.
+  m.mlp_scratch = take(std::max((size_t)kMlpScratchFloats * sizeof(float), 2 * new_rows_bytes(c)));
   m.total = o;
   return m;
 }
@@ -803,6 +809,11 @@ extern "C" gb_status gb_append_kv(gb_pool* pool, int layer, int n_tokens, const 
   return append_layer(pool, layer, n_tokens, k_dev, v_dev, false, reinterpret_cast<cudaStream_t>(stream));
 }
 
+static bool overlap(const void* a, size_t an, const void* b, size_t bn) {
+  const char *x = static_cast<const char*>(a), *y = static_cast<const char*>(b);
+  return x < y + bn && y < x + an;
+}
+
 extern "C" gb_status gb_decode_attention(gb_pool* pool, int layer, const void* q_dev,
                                          const void* k_new_dev, const void* v_new_dev, float scale,
                                          float* out_dev, int flags, gb_stream_t stream) {
@@ -812,6 +823,17 @@ extern "C" gb_status gb_decode_attention(gb_pool* pool, int layer, const void* q
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   gb_status st = append_layer(pool, layer, 1, k_new_dev, v_new_dev, true, s);
   if (st != GB_OK) return st;
+  // The launch writes a pair's output while other pairs' new rows are still to be read.
+  const size_t rows = new_rows_bytes(pool->cfg);
+  const size_t outb = (size_t)pool->cfg.max_beams * pool->cfg.num_q_heads * pool->cfg.head_dim * sizeof(float);
+  if (overlap(out_dev, outb, k_new_dev, rows) || overlap(out_dev, outb, v_new_dev, rows)) {
+    char* copy = reinterpret_cast<char*>(pool->view.mlp_scratch);
+    if (cudaMemcpyAsync(copy, k_new_dev, rows, cudaMemcpyDeviceToDevice, s) != cudaSuccess ||
+        cudaMemcpyAsync(copy + rows, v_new_dev, rows, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
+      return check_launch(pool, "new rows");
+    k_new_dev = copy;
+    v_new_dev = copy + rows;
+  }
   // Mode 1: shared-prefix segments go through the grouped tensor-core kernel and the
   // per-beam kernel reads only each beam's remainder; mode 0: every beam reads everything.
   // In mode 1 one attention kernel runs both: the grouped and the per-beam roles on their
