@@ -133,7 +133,7 @@ __device__ __forceinline__ void decode_setup(const PoolView& v) {
 // memory) instead of to the partials.  k counts the chunks consumed so far (stages and phases of the
 // ring).  False once a wait ran out.
 template <int DT, int G, bool Pool, class S>
-__device__ __forceinline__ bool decode_range(const PoolView& v, int layer, const void* __restrict__ qptr,
+__device__ __forceinline__ bool decode_range(const PoolView& v, int layer, const void* qptr,
                                              const NewRows& nw, float qscale, int w,
                                              int x_begin, int x_end, int& k_io, float* lrec) {
   using T = KvTraits<DT>;
@@ -470,7 +470,7 @@ __device__ __forceinline__ bool decode_range(const PoolView& v, int layer, const
 
 // Share w of all chunks of caller-owned rows, c per warp.
 template <int DT, int G, class S>
-__device__ __forceinline__ void decode_body(const PoolView& v, const void* __restrict__ qptr, float qscale, int w, int c) {
+__device__ __forceinline__ void decode_body(const PoolView& v, const void* qptr, float qscale, int w, int c) {
   extern __shared__ __align__(128) unsigned char smem[];
   const int Tot = reinterpret_cast<const int*>(smem + S::WARPS * S::WARP_BYTES)[v.max_beams];
   const long long x0 = (long long)w * c;
@@ -544,7 +544,7 @@ __device__ __forceinline__ int rows_plan(const PoolView& v, int W) {
 // Caller-owned rows: the records are merged by k_combine.
 template <int DT, int G>
 __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
-    k_decode(PoolView v, const void* __restrict__ qptr, float qscale) {
+    k_decode(PoolView v, const void* qptr, float qscale) {
   pdl_wait();
   pdl_launch_dependents();
   using S = DecodeSmem<DT, G>;
@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
 // residency.
 template <int DT, int G>
 __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
-    k_decode_pool(PoolView v, int layer, const void* __restrict__ qptr, NewRows nw, float qscale,
+    k_decode_pool(PoolView v, int layer, const void* qptr, NewRows nw, float qscale,
                   float* __restrict__ out) {
   pdl_wait();
   pdl_launch_dependents();
@@ -653,7 +653,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
 template <int G>
 __global__ void __launch_bounds__(kMmaWarps * 32, 1)
     k_decode_mma(PoolView v, const __grid_constant__ CUtensorMap tm, const __grid_constant__ CUtensorMap tmh,
-                 int layer, const __nv_bfloat16* __restrict__ q, NewRows nw, float qscale, int mode,
+                 int layer, const __nv_bfloat16* q, NewRows nw, float qscale, int mode,
                  float* __restrict__ out) {
   const bool early = layer > 0;
   enter(!early);

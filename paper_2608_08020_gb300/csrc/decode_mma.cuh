@@ -126,7 +126,7 @@ struct PairState {
 // Start pair (b, h): its query rows, an empty softmax.  Split (chunk_attend): columns G .. 2G - 1 repeat
 // the heads.
 template <int G, bool Split = false>
-__device__ __forceinline__ void pair_begin(PairState& st, const PoolView& v, const __nv_bfloat16* __restrict__ q, int b,
+__device__ __forceinline__ void pair_begin(PairState& st, const PoolView& v, const __nv_bfloat16* q, int b,
                                            int h, int r, int c) {
   const uint32_t* qrow = reinterpret_cast<const uint32_t*>(q + ((size_t)b * v.Hq + h * G + (Split ? r % G : r)) * 128);
   const bool used = r < (Split ? 2 * G : G);
@@ -316,7 +316,7 @@ struct NewRows {
 template <int G>
 __device__ __forceinline__ void decode_mma_body(const PoolView& v, const Counters& cnt, const CUtensorMap* tm_p,
                                                 const CUtensorMap* tmh_p, int layer,
-                                                const __nv_bfloat16* __restrict__ q, const NewRows& nw, float qscale,
+                                                const __nv_bfloat16* q, const NewRows& nw, float qscale,
                                                 int mode, int cta, int nctas) {
   using S = DecodeMmaSmem;
   constexpr int D = 128;

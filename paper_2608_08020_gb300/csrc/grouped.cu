@@ -161,7 +161,7 @@ __device__ __forceinline__ Unit load_unit(const PoolView& v, long long u) {
 // barriers.
 template <int G>
 __device__ __forceinline__ void grouped_body(const PoolView& v, const Counters& cnt, const CUtensorMap* tm_p, int layer,
-                                             const __nv_bfloat16* __restrict__ q, float qscale, int w_oob, int ng) {
+                                             const __nv_bfloat16* q, float qscale, int w_oob, int ng) {
   extern __shared__ __align__(1024) unsigned char sm[];
   const long long units = (long long)v.ctl[kCtlSegTiles] * v.Hkv;
   if (units == 0) return;
@@ -698,7 +698,7 @@ constexpr int kAttnSmem = kSmem > DecodeMmaSmem::TOTAL ? kSmem : DecodeMmaSmem::
 template <int G>
 __global__ void __launch_bounds__(kAttnThreads, 1)
     k_attention(PoolView v, const __grid_constant__ CUtensorMap tmg, const __grid_constant__ CUtensorMap tmd,
-                const __grid_constant__ CUtensorMap tmdh, int layer, const __nv_bfloat16* __restrict__ q, NewRows nw,
+                const __grid_constant__ CUtensorMap tmdh, int layer, const __nv_bfloat16* q, NewRows nw,
                 float qscale, int w_oob, bool allow_local, float* __restrict__ out) {
   const bool early = layer > 0;
   enter(!early);

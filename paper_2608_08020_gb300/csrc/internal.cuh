@@ -198,13 +198,23 @@ __device__ __forceinline__ long long kv_elem_offset(const PoolView& v, int layer
          (long long)row * v.D;
 }
 
-// Programmatic dependent launch.  Every kernel of the library begins with pdl_wait(),
-// before any global memory access: launched normally it returns at once; launched with
+// Programmatic dependent launch.  Every kernel of the library calls pdl_wait() before any global
+// memory access but those named here: launched normally it returns at once; launched with
 // programmatic stream serialization (launch_pdl) the kernel may be scheduled while the
 // previous kernel in the stream is still running, and pdl_wait() blocks until that
 // kernel has completed and its writes are visible - the same ordering as a plain launch,
 // without the gap between the two kernels.  pdl_launch_dependents() lets the next
-// kernel be scheduled as soon as every CTA of this one has started.
+// kernel be scheduled as soon as every CTA of this one has called it or left; each kernel calls it
+// only after its own pdl_wait, so all but the directly preceding kernel have completed when one starts.
+// Before the wait, three kernels read what the directly preceding kernel cannot have written:
+//   - k_attention and k_decode_mma of layers above 0: the step's control words, and in the small-step
+//     form its plan, tables and first K/V chunks (enter, below);
+//   - k_fused_gemm: its rows of the weights;
+//   - k_gemm_partials with early_w: its first weight tiles (the scorer's, whose preceding kernel is one
+//     of the scorer's).
+// What a preceding kernel of the library writes (q, partial sums, activity) is read through pointers
+// without __restrict__: const __restrict__ data may be read as constant for the kernel's whole life,
+// which here begins before those writes.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -215,7 +225,9 @@ __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepc
 // a step changes them), so page ids and the first K/V loads go out while the kernel that makes q
 // and the new rows drains.  `early` threads wait here, before they read q, the new rows or the
 // counters, and before any global write.  (The same in the roles of large steps gained nothing:
-// the next launch's loads then compete with the tail of this one.)
+// the next launch's loads then compete with the tail of this one.)  How early depends on the kernel:
+// k_decode_mma is one CTA per SM; of k_attention's 2 x SM CTAs the second half has nothing to do in the
+// small-step form but must get an SM to say so, so the next launch begins as the first half leaves.
 __device__ __forceinline__ void enter(bool early) {
   if (early) {
     pdl_wait();

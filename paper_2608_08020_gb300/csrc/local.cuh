@@ -24,7 +24,7 @@ __device__ __forceinline__ void team_sync(int team, int threads) {
 // own stages, which are idle by then.
 template <int G>
 __device__ __forceinline__ void local_attention(const PoolView& v, const CUtensorMap* tm_p, const CUtensorMap* tmh_p,
-                                                int layer, const __nv_bfloat16* __restrict__ q, const NewRows& nw,
+                                                int layer, const __nv_bfloat16* q, const NewRows& nw,
                                                 float qscale, int w, int cta, int nctas,
                                                 float* __restrict__ out, bool early) {
   using S = DecodeMmaSmem;

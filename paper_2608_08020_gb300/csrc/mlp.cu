@@ -27,7 +27,7 @@ namespace {
 // (14.5 before the GEMM's six stages and unrolled stores; 17.6 with 128 threads and rolled stores).
 constexpr int kScoreThreads = 256;  // at most
 
-__global__ void __launch_bounds__(kScoreThreads) k_mlp_score(PoolView v, const float* __restrict__ zp, int splits,
+__global__ void __launch_bounds__(kScoreThreads) k_mlp_score(PoolView v, const float* zp, int splits,
                                                              int dh, const float* __restrict__ b1,
                                                              const float* __restrict__ w2, float b2,
                                                              const uint8_t* __restrict__ mask,

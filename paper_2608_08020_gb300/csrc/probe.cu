@@ -49,7 +49,7 @@ template <int HT>
 __global__ void __launch_bounds__(kProbeThreads) k_probe(PoolView v, const void* __restrict__ hidden, int H,
                                                          const float* __restrict__ w, float bias,
                                                          const uint8_t* __restrict__ mask, float* __restrict__ score_out,
-                                                         const float* __restrict__ scores_in) {
+                                                         const float* scores_in) {
   pdl_wait();
   pdl_launch_dependents();
   __shared__ float s_part[kProbeThreads / 32];

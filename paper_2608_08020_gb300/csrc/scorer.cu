@@ -151,7 +151,7 @@ __device__ __forceinline__ bool row_live(const int* active, int m) { return acti
 // rows give zeros.  16-byte loads and stores (8 values); the row is staged in shared memory.
 __global__ void __launch_bounds__(kRowThreads) k_ln_in(const __nv_bfloat16* __restrict__ h, int H,
                                                        const float* __restrict__ g, const float* __restrict__ b,
-                                                       const int* __restrict__ active,
+                                                       const int* active,
                                                        __nv_bfloat16* __restrict__ u) {
   pdl_wait();
   pdl_launch_dependents();
@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(kRowThreads) k_ln_in(const __nv_bfloat16* __re
 }
 
 // x = GELU(z) of Eq. 4 (exact, erf), z = the sum of the product's K-split partials.
-__global__ void __launch_bounds__(kRowThreads) k_gelu_epilogue(const float* __restrict__ P, int splits, int n4,
+__global__ void __launch_bounds__(kRowThreads) k_gelu_epilogue(const float* P, int splits, int n4,
                                                                float* __restrict__ x) {
   pdl_wait();
   pdl_launch_dependents();
@@ -218,10 +218,10 @@ __device__ __forceinline__ float warp_sum(float v) {
 }
 
 // Output head (Eq. 6), one warp per row: score = sigmoid(w_out . LN(x) + b_out); 0 for inactive rows.
-__global__ void __launch_bounds__(kRowThreads) k_head(const float* __restrict__ x, int M, int d,
+__global__ void __launch_bounds__(kRowThreads) k_head(const float* x, int M, int d,
                                                       const float* __restrict__ g, const float* __restrict__ b,
                                                       const float* __restrict__ w_out, const float* __restrict__ b_out,
-                                                      const int* __restrict__ active, float* __restrict__ score) {
+                                                      const int* active, float* __restrict__ score) {
   pdl_wait();
   pdl_launch_dependents();
   const int m = blockIdx.x * (kRowThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -545,7 +545,7 @@ __global__ void __launch_bounds__(kFThreads, 1) k_fused_gemm(FusedArgs p) {
 
 // Attention of the first position alone (the seed row): softmax over one key is 1, so
 // query head h returns the value of KV head h / G.
-__global__ void k_first_position_attention(const __nv_bfloat16* __restrict__ vn, int Hq, int G,
+__global__ void k_first_position_attention(const __nv_bfloat16* vn, int Hq, int G,
                                            float* __restrict__ att) {
   pdl_wait();
   pdl_launch_dependents();
@@ -558,7 +558,7 @@ __global__ void k_first_position_attention(const __nv_bfloat16* __restrict__ vn,
 // one CTA per row, four columns per thread (16-byte loads, the splits in flight together).
 
 // Columns n .. n + 3 of row m, the splits in order.
-__device__ __forceinline__ float4 sum_partials(const float* __restrict__ P, int splits, int M, int N, int m, int n) {
+__device__ __forceinline__ float4 sum_partials(const float* P, int splits, int M, int N, int m, int n) {
   float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
   for (int k = 0; k < splits; ++k) {
@@ -578,9 +578,9 @@ enum RowMode { kGeluLn = 0, kResidLn = 1, kResid = 2 };
 // Epilogue of a d-wide product: x = GELU(z) (kGeluLn) or x += z, then u = LN(x) in bf16 (not kResid,
 // which the head follows).  Inactive rows: u = 0.
 template <int Mode>
-__global__ void __launch_bounds__(kRowThreads) k_row_epilogue(const float* __restrict__ P, int splits, int M, int d,
+__global__ void __launch_bounds__(kRowThreads) k_row_epilogue(const float* P, int splits, int M, int d,
                                                               float* __restrict__ x, const float* __restrict__ g,
-                                                              const float* __restrict__ b, const int* __restrict__ active,
+                                                              const float* __restrict__ b, const int* active,
                                                               __nv_bfloat16* __restrict__ u) {
   pdl_wait();
   pdl_launch_dependents();
@@ -631,9 +631,9 @@ __global__ void __launch_bounds__(kRowThreads) k_row_epilogue(const float* __res
 
 // Epilogue of the q/k/v product: the (i, i + 64) pairs of every q and k head are rotated by
 // pos * 10000^(-i/64) with pos = pos_of[m] + pos_shift (0 without pos_of).
-__global__ void __launch_bounds__(kRowThreads) k_qkv_epilogue(const float* __restrict__ P, int splits, int M, int Hq,
-                                                              int Hkv, const int* __restrict__ pos_of, int pos_shift,
-                                                              const int* __restrict__ active,
+__global__ void __launch_bounds__(kRowThreads) k_qkv_epilogue(const float* P, int splits, int M, int Hq,
+                                                              int Hkv, const int* pos_of, int pos_shift,
+                                                              const int* active,
                                                               __nv_bfloat16* __restrict__ q,
                                                               __nv_bfloat16* __restrict__ kn,
                                                               __nv_bfloat16* __restrict__ vn) {
@@ -669,8 +669,8 @@ __global__ void __launch_bounds__(kRowThreads) k_qkv_epilogue(const float* __res
 }
 
 // SwiGLU epilogue: u[m][n] = SiLU(z[m][n]) * z[m][F + n] in bf16 (z = W_13 u, F wide halves).
-__global__ void __launch_bounds__(kRowThreads) k_swiglu_epilogue(const float* __restrict__ P, int splits, int M, int F,
-                                                                 const int* __restrict__ active,
+__global__ void __launch_bounds__(kRowThreads) k_swiglu_epilogue(const float* P, int splits, int M, int F,
+                                                                 const int* active,
                                                                  __nv_bfloat16* __restrict__ u) {
   pdl_wait();
   pdl_launch_dependents();
@@ -688,7 +688,7 @@ __global__ void __launch_bounds__(kRowThreads) k_swiglu_epilogue(const float* __
 }
 
 // Attention outputs (fp32) to the bf16 operand of W_o.
-__global__ void __launch_bounds__(kRowThreads) k_to_bf16(const float* __restrict__ a, int n4, __nv_bfloat16* __restrict__ u) {
+__global__ void __launch_bounds__(kRowThreads) k_to_bf16(const float* a, int n4, __nv_bfloat16* __restrict__ u) {
   pdl_wait();
   pdl_launch_dependents();
   const int i = blockIdx.x * kRowThreads + threadIdx.x;
