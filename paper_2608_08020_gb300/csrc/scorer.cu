@@ -735,11 +735,21 @@ struct Run {
     return launch_pdl(k_fused_gemm<A, E>, dim3((p.M + p.mt - 1) / p.mt, tiles), kFThreads, kFSmem, st, p) == cudaSuccess;
   }
 
+  // A row of `floats` in dynamic shared memory beside the kernel's static words (red) may pass the 48 KiB
+  // that a launch gets without asking.
+  template <class K>
+  static bool row_smem(K* kernel, int floats) {
+    return floats * sizeof(float) + 256 <= 48 * 1024 ||
+           set_max_dynamic_smem(reinterpret_cast<const void*>(kernel), 48 * 1024) == cudaSuccess;
+  }
+
   template <int Mode>
-  void rows(int splits, int M, const float* g, const float* b, const int* active) {
+  bool rows(int splits, int M, const float* g, const float* b, const int* active) {
+    if (!row_smem(k_row_epilogue<Mode>, s.d)) return false;
     launch_pdl(k_row_epilogue<Mode>, M, kRowThreads, s.d * sizeof(float), st, static_cast<const float*>(part()), splits,
                M, s.d, x(), g, b, active, u());
     ++launches;
+    return true;
   }
 
   // How a layer's products run: above d_model 512 a fused product's CTAs would each normalise rows of
@@ -761,7 +771,7 @@ struct Run {
     ++launches;
     sp = gemm(u(), M, wt<__nv_bfloat16>(layer_tensor(l, kWo)), s.d, s.d);
     if (!sp) return false;
-    rows<kResidLn>(sp, M, wt<float>(layer_tensor(l, kLn2G)), wt<float>(layer_tensor(l, kLn2B)), active);
+    if (!rows<kResidLn>(sp, M, wt<float>(layer_tensor(l, kLn2G)), wt<float>(layer_tensor(l, kLn2B)), active)) return false;
     sp = gemm(u(), M, wt<__nv_bfloat16>(layer_tensor(l, kW13)), 2 * s.F, s.d);
     if (!sp) return false;
     launch_pdl(k_swiglu_epilogue, M, kRowThreads, 0, st, P, sp, M, s.F, active, u());
@@ -769,10 +779,8 @@ struct Run {
     sp = gemm(u(), M, wt<__nv_bfloat16>(layer_tensor(l, kW2)), s.d, s.F);
     if (!sp) return false;
     if (l + 1 < s.L)
-      rows<kResidLn>(sp, M, wt<float>(layer_tensor(l + 1, kLn1G)), wt<float>(layer_tensor(l + 1, kLn1B)), active);
-    else
-      rows<kResid>(sp, M, nullptr, nullptr, active);
-    return true;
+      return rows<kResidLn>(sp, M, wt<float>(layer_tensor(l + 1, kLn1G)), wt<float>(layer_tensor(l + 1, kLn1B)), active);
+    return rows<kResid>(sp, M, nullptr, nullptr, active);
   }
 
   // Attention of layer l over each trace's history, or of the first position alone.
@@ -855,15 +863,14 @@ struct Run {
 
   // Eq. 4 on M rows of h.
   bool input(const void* h, int M, const int* active) {
+    if (!row_smem(k_ln_in, s.H)) return false;
     launch_pdl(k_ln_in, M, kRowThreads, s.H * sizeof(float), st, reinterpret_cast<const __nv_bfloat16*>(h), s.H,
                wt<float>(0), wt<float>(1), active, u());
     ++launches;
     const int sp = gemm(u(), M, wt<__nv_bfloat16>(2), s.d, s.H);
     if (!sp) return false;
-    if (split_products()) {  // with LN1 of layer 0
-      rows<kGeluLn>(sp, M, wt<float>(layer_tensor(0, kLn1G)), wt<float>(layer_tensor(0, kLn1B)), active);
-      return true;
-    }
+    if (split_products())  // with LN1 of layer 0
+      return rows<kGeluLn>(sp, M, wt<float>(layer_tensor(0, kLn1G)), wt<float>(layer_tensor(0, kLn1B)), active);
     const int n4 = M * (s.d / 4);
     launch_pdl(k_gelu_epilogue, (n4 + kRowThreads - 1) / kRowThreads, kRowThreads, 0, st,
                static_cast<const float*>(part()), sp, n4, x());
