@@ -85,7 +85,8 @@ __global__ void __launch_bounds__(128, 1)
     } else {
       for (int i = 0; i < nkb && i < kMStages; ++i) load(i);
     }
-    for (int i = 0; i < nkb && ok; ++i) {
+    int i = 0;
+    for (; i < nkb; ++i) {
       const uint32_t st = i % kMStages;
       ok = mbar_wait_bounded(bar + kMBarFull + 8 * st, (i / kMStages) & 1, kWaitLimitNs);
       if (!ok) break;
@@ -97,11 +98,17 @@ __global__ void __launch_bounds__(128, 1)
       mma_commit(bar + kMBarEmpty + 8 * st);
       if (i + kMStages < nkb) {  // refill this stage once its MMAs have read it
         ok = mbar_wait_bounded(bar + kMBarEmpty + 8 * st, (i / kMStages) & 1, kWaitLimitNs);
-        if (ok) load(i + kMStages);
+        if (!ok) break;
+        load(i + kMStages);
       }
     }
-    if (ok) mma_commit(bar + kMBarDone);
-    if (!ok) set_status(ctl, GB_ERR_TIMEOUT);
+    if (ok) {
+      mma_commit(bar + kMBarDone);
+    } else {
+      set_status(ctl, GB_ERR_TIMEOUT);
+      for (int j = i; j < nkb && j < i + kMStages; ++j)  // a bounded chance for the copies in flight
+        mbar_wait_bounded(bar + kMBarFull + 8 * (j % kMStages), (j / kMStages) & 1, kWaitLimitNs / 4);
+    }
   }
   if (tid != 0) enter(early_w);
   __syncthreads();
