@@ -325,8 +325,8 @@ __global__ void __launch_bounds__(1024) k_step_begin(PoolView v, int n_tokens, c
 
   // The sequential rule takes the lowest free page at every need, token by token and slots
   // ascending; nothing is freed in between, so the r-th need of the step gets the r-th lowest free
-  // page.  Beams of one length (every state the calls build: all advance together and a child takes
-  // its parent's length) need their pages at the same tokens, so need r is copy r of the first
+  // page.  Beams of one length (all advance together and a child takes its parent's length; only a
+  // child of a released slot starts at 0) need their pages at the same tokens, so need r is copy r of the first
   // ncow, then page j = (r - ncow) / nact of active slot (r - ncow) % nact, and one pass over the
   // bitmap places them all.  (A pass per token with its block barriers took 88 us for 256 beams x
   // 199 tokens.)  Other states take the sequential form below.

@@ -1,6 +1,6 @@
 """The work plan that gb_paged_decode_noalloc's kernel makes for itself: one to four rows per thread,
-rows that cannot be read (their output zero, the status of that call only), merged in the CTAs and
-by the second launch.  Tolerance as in test_zz_no_alloc_sizes (fp32 sums against fp64)."""
+rows that cannot be read (their output zero, the status of that call only), and the
+merge of the rest by the second launch.  Tolerance as in test_zz_no_alloc_sizes (fp32 sums against fp64)."""
 import numpy as np
 import pytest
 
