@@ -358,107 +358,107 @@ __global__ void __launch_bounds__(kFThreads, 1) k_fused_gemm(FusedArgs p) {
     }
     // A: row r = warp + 8 j of the tile, four rows in flight per warp, 512 of K at a time.
     for (int h0 = 0; h0 < kpass; h0 += kFK) {
-    const int kw = min(kFK, kpass - h0), kh = k0 + h0;
-    unsigned char* sa = sm + (h0 >> 6) * a_block;
-    if (A == kABf16) {
-      const __nv_bfloat16* ab = static_cast<const __nv_bfloat16*>(p.a);
-      for (int r0 = warp; r0 < p.mt; r0 += kFThreads / 32 * 4) {
-        uint4 v[4][kFK / 256];
+      const int kw = min(kFK, kpass - h0), kh = k0 + h0;
+      unsigned char* sa = sm + (h0 >> 6) * a_block;
+      if (A == kABf16) {
+        const __nv_bfloat16* ab = static_cast<const __nv_bfloat16*>(p.a);
+        for (int r0 = warp; r0 < p.mt; r0 += kFThreads / 32 * 4) {
+          uint4 v[4][kFK / 256];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int r = r0 + kFThreads / 32 * u;
-          const bool live = live_row(r);
+          for (int u = 0; u < 4; ++u) {
+            const int r = r0 + kFThreads / 32 * u;
+            const bool live = live_row(r);
 #pragma unroll
-          for (int i = 0; i < kFK / 256; ++i) {
-            const int c = 8 * lane + 256 * i;
-            v[u][i] = live && c < kw ? *reinterpret_cast<const uint4*>(ab + (size_t)(m0 + r) * p.K + kh + c)
-                                     : make_uint4(0u, 0u, 0u, 0u);
+            for (int i = 0; i < kFK / 256; ++i) {
+              const int c = 8 * lane + 256 * i;
+              v[u][i] = live && c < kw ? *reinterpret_cast<const uint4*>(ab + (size_t)(m0 + r) * p.K + kh + c)
+                                       : make_uint4(0u, 0u, 0u, 0u);
+            }
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int r = r0 + kFThreads / 32 * u;
+#pragma unroll
+            for (int i = 0; i < kFK / 256; ++i) {
+              const int c = 8 * lane + 256 * i;
+              if (r < p.mt && c < kw) *reinterpret_cast<uint4*>(sa + (c >> 6) * a_block + swz(r, c & 63)) = v[u][i];
+            }
           }
         }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int r = r0 + kFThreads / 32 * u;
-#pragma unroll
-          for (int i = 0; i < kFK / 256; ++i) {
-            const int c = 8 * lane + 256 * i;
-            if (r < p.mt && c < kw) *reinterpret_cast<uint4*>(sa + (c >> 6) * a_block + swz(r, c & 63)) = v[u][i];
-          }
-        }
-      }
-    } else {
-      float4 gg[kFK / 128], bb[kFK / 128];
-      if (A == kALn) {
-#pragma unroll
-        for (int i = 0; i < kFK / 128; ++i) {
-          const int c = 4 * lane + 128 * i;
-          gg[i] = c < kw ? *reinterpret_cast<const float4*>(p.g + kh + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-          bb[i] = c < kw ? *reinterpret_cast<const float4*>(p.b + kh + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-      }
-      for (int r0 = warp; r0 < p.mt; r0 += kFThreads / 32 * 4) {
-        float4 v[4][kFK / 128];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int r = r0 + kFThreads / 32 * u;
-          const bool live = live_row(r);
-#pragma unroll
-          for (int i = 0; i < kFK / 128; ++i) {
-            const int c = 4 * lane + 128 * i;
-            v[u][i] = live && c < kw ? *reinterpret_cast<const float4*>(af + (size_t)(m0 + r) * p.K + kh + c)
-                                     : make_float4(0.f, 0.f, 0.f, 0.f);
-          }
-        }
-        // The four rows' statistics together: their shuffles are independent chains.
-        float mu[4] = {0.f, 0.f, 0.f, 0.f}, rs[4] = {1.f, 1.f, 1.f, 1.f};
+      } else {
+        float4 gg[kFK / 128], bb[kFK / 128];
         if (A == kALn) {
-          float s[4], q[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            s[u] = 0.f;
-#pragma unroll
-            for (int i = 0; i < kFK / 128; ++i) s[u] += (v[u][i].x + v[u][i].y) + (v[u][i].z + v[u][i].w);
-          }
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int u = 0; u < 4; ++u) s[u] += __shfl_xor_sync(0xffffffffu, s[u], o);
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            mu[u] = s[u] / (float)p.K;
-#pragma unroll
-            for (int i = 0; i < kFK / 128; ++i)
-              if (4 * lane + 128 * i < kw) {
-                q[u] = fmaf(v[u][i].x - mu[u], v[u][i].x - mu[u], q[u]);
-                q[u] = fmaf(v[u][i].y - mu[u], v[u][i].y - mu[u], q[u]);
-                q[u] = fmaf(v[u][i].z - mu[u], v[u][i].z - mu[u], q[u]);
-                q[u] = fmaf(v[u][i].w - mu[u], v[u][i].w - mu[u], q[u]);
-              }
-          }
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int u = 0; u < 4; ++u) q[u] += __shfl_xor_sync(0xffffffffu, q[u], o);
-#pragma unroll
-          for (int u = 0; u < 4; ++u) rs[u] = 1.0f / sqrtf(q[u] / (float)p.K + kLnEps);
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int r = r0 + kFThreads / 32 * u;
 #pragma unroll
           for (int i = 0; i < kFK / 128; ++i) {
             const int c = 4 * lane + 128 * i;
-            float4 y = v[u][i];
-            if (A == kALn)
-              y = make_float4((y.x - mu[u]) * rs[u] * gg[i].x + bb[i].x, (y.y - mu[u]) * rs[u] * gg[i].y + bb[i].y,
-                              (y.z - mu[u]) * rs[u] * gg[i].z + bb[i].z, (y.w - mu[u]) * rs[u] * gg[i].w + bb[i].w);
-            const __nv_bfloat162 lo = __floats2bfloat162_rn(y.x, y.y), hi = __floats2bfloat162_rn(y.z, y.w);
-            if (r < p.mt && c < kw)
-              *reinterpret_cast<uint2*>(sa + (c >> 6) * a_block + swz(r, c & 63)) =
-                  make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+            gg[i] = c < kw ? *reinterpret_cast<const float4*>(p.g + kh + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+            bb[i] = c < kw ? *reinterpret_cast<const float4*>(p.b + kh + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+          }
+        }
+        for (int r0 = warp; r0 < p.mt; r0 += kFThreads / 32 * 4) {
+          float4 v[4][kFK / 128];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int r = r0 + kFThreads / 32 * u;
+            const bool live = live_row(r);
+#pragma unroll
+            for (int i = 0; i < kFK / 128; ++i) {
+              const int c = 4 * lane + 128 * i;
+              v[u][i] = live && c < kw ? *reinterpret_cast<const float4*>(af + (size_t)(m0 + r) * p.K + kh + c)
+                                       : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+          }
+          // The four rows' statistics together: their shuffles are independent chains.
+          float mu[4] = {0.f, 0.f, 0.f, 0.f}, rs[4] = {1.f, 1.f, 1.f, 1.f};
+          if (A == kALn) {
+            float s[4], q[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              s[u] = 0.f;
+#pragma unroll
+              for (int i = 0; i < kFK / 128; ++i) s[u] += (v[u][i].x + v[u][i].y) + (v[u][i].z + v[u][i].w);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+              for (int u = 0; u < 4; ++u) s[u] += __shfl_xor_sync(0xffffffffu, s[u], o);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              mu[u] = s[u] / (float)p.K;
+#pragma unroll
+              for (int i = 0; i < kFK / 128; ++i)
+                if (4 * lane + 128 * i < kw) {
+                  q[u] = fmaf(v[u][i].x - mu[u], v[u][i].x - mu[u], q[u]);
+                  q[u] = fmaf(v[u][i].y - mu[u], v[u][i].y - mu[u], q[u]);
+                  q[u] = fmaf(v[u][i].z - mu[u], v[u][i].z - mu[u], q[u]);
+                  q[u] = fmaf(v[u][i].w - mu[u], v[u][i].w - mu[u], q[u]);
+                }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+              for (int u = 0; u < 4; ++u) q[u] += __shfl_xor_sync(0xffffffffu, q[u], o);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) rs[u] = 1.0f / sqrtf(q[u] / (float)p.K + kLnEps);
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int r = r0 + kFThreads / 32 * u;
+#pragma unroll
+            for (int i = 0; i < kFK / 128; ++i) {
+              const int c = 4 * lane + 128 * i;
+              float4 y = v[u][i];
+              if (A == kALn)
+                y = make_float4((y.x - mu[u]) * rs[u] * gg[i].x + bb[i].x, (y.y - mu[u]) * rs[u] * gg[i].y + bb[i].y,
+                                (y.z - mu[u]) * rs[u] * gg[i].z + bb[i].z, (y.w - mu[u]) * rs[u] * gg[i].w + bb[i].w);
+              const __nv_bfloat162 lo = __floats2bfloat162_rn(y.x, y.y), hi = __floats2bfloat162_rn(y.z, y.w);
+              if (r < p.mt && c < kw)
+                *reinterpret_cast<uint2*>(sa + (c >> 6) * a_block + swz(r, c & 63)) =
+                    make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+            }
           }
         }
       }
-    }
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     fence_proxy_async_smem();

@@ -191,81 +191,81 @@ __global__ void __launch_bounds__(kTourThreads, 1) k_tournament(PoolView v, Tour
     childof[tid] = -1;
     int nchild = 0, per = 1;
     if (a.prune) {
-    int N;
-    const int pos = block_exclusive_scan(act ? 1 : 0, tmp, &N);
-    s_keys[tid] = ~0ull;
-    __syncthreads();
-    if (act) s_keys[pos] = ((unsigned long long)rank_key(mean_w) << 32) | (unsigned)tid;
-    __syncthreads();
-    // This CTA has read every slot's state: from here on others may change it.
-    if (v.grouped && tid == 0) s_snap = grid_arrive(v);
-    // Rank (ascending keys; the slot in the low word makes them distinct): each warp sorts its
-    // 32 keys in registers (bitonic, by shuffles), then a key's rank is its position in its
-    // warp's list plus, for every other list, the number of keys there below it (a binary
-    // search over 32 sorted keys; four lists at a time).
-    const int nl = (N + 31) >> 5, lane = tid & 31, wl = tid >> 5;
-    if (wl < nl) {
-      unsigned long long my = s_keys[tid];  // ~0 past the N keys
-      for (int k = 2; k <= 32; k <<= 1)
-        for (int j = k >> 1; j > 0; j >>= 1) {
-          const unsigned long long other = __shfl_xor_sync(0xffffffffu, my, j);
-          const bool asc = (lane & k) == 0, lower = (lane & j) == 0;
-          my = (asc == lower) ? (my < other ? my : other) : (my > other ? my : other);
-        }
-      s_keys[tid] = my;
-      asm volatile("bar.sync 1, %0;" ::"r"(nl * 32) : "memory");
-      if (my != ~0ull) {
-        int rank = lane;
-        for (int l0 = 0; l0 < nl; l0 += 4) {
-          int pos[4] = {0, 0, 0, 0};
+      int N;
+      const int pos = block_exclusive_scan(act ? 1 : 0, tmp, &N);
+      s_keys[tid] = ~0ull;
+      __syncthreads();
+      if (act) s_keys[pos] = ((unsigned long long)rank_key(mean_w) << 32) | (unsigned)tid;
+      __syncthreads();
+      // This CTA has read every slot's state: from here on others may change it.
+      if (v.grouped && tid == 0) s_snap = grid_arrive(v);
+      // Rank (ascending keys; the slot in the low word makes them distinct): each warp sorts its
+      // 32 keys in registers (bitonic, by shuffles), then a key's rank is its position in its
+      // warp's list plus, for every other list, the number of keys there below it (a binary
+      // search over 32 sorted keys; four lists at a time).
+      const int nl = (N + 31) >> 5, lane = tid & 31, wl = tid >> 5;
+      if (wl < nl) {
+        unsigned long long my = s_keys[tid];  // ~0 past the N keys
+        for (int k = 2; k <= 32; k <<= 1)
+          for (int j = k >> 1; j > 0; j >>= 1) {
+            const unsigned long long other = __shfl_xor_sync(0xffffffffu, my, j);
+            const bool asc = (lane & k) == 0, lower = (lane & j) == 0;
+            my = (asc == lower) ? (my < other ? my : other) : (my > other ? my : other);
+          }
+        s_keys[tid] = my;
+        asm volatile("bar.sync 1, %0;" ::"r"(nl * 32) : "memory");
+        if (my != ~0ull) {
+          int rank = lane;
+          for (int l0 = 0; l0 < nl; l0 += 4) {
+            int pos[4] = {0, 0, 0, 0};
 #pragma unroll
-          for (int st = 16; st > 0; st >>= 1)
+            for (int st = 16; st > 0; st >>= 1)
+#pragma unroll
+              for (int u = 0; u < 4; ++u)
+                if (l0 + u < nl && s_keys[32 * (l0 + u) + pos[u] + st - 1] < my) pos[u] += st;
 #pragma unroll
             for (int u = 0; u < 4; ++u)
-              if (l0 + u < nl && s_keys[32 * (l0 + u) + pos[u] + st - 1] < my) pos[u] += st;
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-            if (l0 + u < nl && l0 + u != wl) rank += pos[u] + (s_keys[32 * (l0 + u) + pos[u]] < my ? 1 : 0);
+              if (l0 + u < nl && l0 + u != wl) rank += pos[u] + (s_keys[32 * (l0 + u) + pos[u]] < my ? 1 : 0);
+          }
+          ord[rank] = (int)(my & 0xffffffffu);
         }
-        ord[rank] = (int)(my & 0xffffffffu);
       }
-    }
-    __syncthreads();
-    // Routing (identical in every CTA).
-    const int f1 = a.fanout - 1;
-    int kase = 0;
-    if (N > 0 && N < a.C) {
-      // Case 1 (Eq. 2): the top min(C - N, |B|) eligible traces, one child each, into vacant slots.
-      kase = 1;
-      const bool f = tid < N && s_elig[ord[tid]];
-      int nb;
-      const int pb = block_exclusive_scan(f ? 1 : 0, tmp, &nb);
-      if (f) blist[pb] = ord[tid];
-      nchild = min(a.C - N, nb);
-      const bool vac = tid < cap && !act;
-      int nv;
-      const int pv = block_exclusive_scan(vac ? 1 : 0, tmp, &nv);
-      if (vac && pv < nchild) cslot[pv] = tid;
-    } else if (N > 0) {
-      // Case 2 (Eq. 3, fan-out f; N = C): prune the bottom K_eff, branch the top eligible survivors.
-      kase = 2;
-      const int Kc = a.K < 0 ? 0 : (a.K > N ? N : a.K);
-      const int nsurv = N - Kc;
-      const bool f = tid < nsurv && s_elig[ord[tid]];
-      int nb;
-      const int pb = block_exclusive_scan(f ? 1 : 0, tmp, &nb);
-      if (f) blist[pb] = ord[tid];
-      const long long cap_children = (long long)f1 * nb;
-      nchild = (int)(Kc < cap_children ? Kc : cap_children);
-      if (tid >= N - nchild && tid < N) s_pruned[ord[tid]] = 1;
       __syncthreads();
-      const bool pr = tid < cap && s_pruned[tid];
-      int np;
-      const int pp = block_exclusive_scan(pr ? 1 : 0, tmp, &np);
-      if (pr) cslot[pp] = tid;
-    }
-    // Parent j has children [j * per, min((j + 1) * per, nchild)): per = 1 in Case 1, f - 1 in Case 2.
-    per = kase == 2 ? f1 : 1;
+      // Routing (identical in every CTA).
+      const int f1 = a.fanout - 1;
+      int kase = 0;
+      if (N > 0 && N < a.C) {
+        // Case 1 (Eq. 2): the top min(C - N, |B|) eligible traces, one child each, into vacant slots.
+        kase = 1;
+        const bool f = tid < N && s_elig[ord[tid]];
+        int nb;
+        const int pb = block_exclusive_scan(f ? 1 : 0, tmp, &nb);
+        if (f) blist[pb] = ord[tid];
+        nchild = min(a.C - N, nb);
+        const bool vac = tid < cap && !act;
+        int nv;
+        const int pv = block_exclusive_scan(vac ? 1 : 0, tmp, &nv);
+        if (vac && pv < nchild) cslot[pv] = tid;
+      } else if (N > 0) {
+        // Case 2 (Eq. 3, fan-out f; N = C): prune the bottom K_eff, branch the top eligible survivors.
+        kase = 2;
+        const int Kc = a.K < 0 ? 0 : (a.K > N ? N : a.K);
+        const int nsurv = N - Kc;
+        const bool f = tid < nsurv && s_elig[ord[tid]];
+        int nb;
+        const int pb = block_exclusive_scan(f ? 1 : 0, tmp, &nb);
+        if (f) blist[pb] = ord[tid];
+        const long long cap_children = (long long)f1 * nb;
+        nchild = (int)(Kc < cap_children ? Kc : cap_children);
+        if (tid >= N - nchild && tid < N) s_pruned[ord[tid]] = 1;
+        __syncthreads();
+        const bool pr = tid < cap && s_pruned[tid];
+        int np;
+        const int pp = block_exclusive_scan(pr ? 1 : 0, tmp, &np);
+        if (pr) cslot[pp] = tid;
+      }
+      // Parent j has children [j * per, min((j + 1) * per, nchild)): per = 1 in Case 1, f - 1 in Case 2.
+      per = kase == 2 ? f1 : 1;
     } else {
       // Every slot with a parent other than itself is a child of its own "parent j"; the parents
       // survive (parent_of[p] = p), so their pages keep a reference throughout.
