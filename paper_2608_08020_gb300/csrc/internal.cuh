@@ -186,9 +186,13 @@ __device__ __forceinline__ void zero_counters(const PoolView& v, int set, int ct
 // they leave.  The roles and the merge compute the same split from the step's plan.
 // A grouped unit costs about 256 tokens beside its own (its queries, its record).  Two CTAs more than
 // the share, rounded up: where the tails are short the share is 7-15 CTAs and one too few costs 5% of
-// the step.  Per layer-step (us), with weight 45, no unit term and the share rounded / now: 74 / 62
-// (64 beams x 4090, tails 0.13 of the grouped tokens), 231 / 183 (198 x 8190, 0.11), 189 / 178
-// (90 x 9000, 0.56), 113 / 114 (250 x 7000, 1.05), 116 / 117 (120 x 12000, G = 8, 0.74).
+// the step.  Per layer-step (us), with weight 45, no unit term and the share rounded / now, for trees
+// named by beams x tokens, prompt, tokens between rounds (and the per-beam tokens over the grouped
+// ones): 98.5 / 61.2 (64 x 4090, 1000, 512; 0.04), 282 / 193 (198 x 8190, 1000, 512; 0.04), 229 / 182
+// (198 x 7800, 512, 512; 0.11), 188 / 178 (90 x 9000, 2000, 1200, G = 8; 0.51), 215 / 206 (128 x 6100, 200,
+// 1000; 0.63), 104 / 101 (300 x 3000, 50, 200, G = 2; 0.78).  No difference where the tails are a fair
+// share: 69.3 / 68.9 (64 x 3900, 512, 512; 0.34), 114.5 / 114.4 (250 x 7000, 100, 700; 0.92), 117.5 / 117.4
+// (120 x 12000, 1000, 2000, G = 8; 0.68).
 __device__ __forceinline__ int decode_ctas(const PoolView& v, int grid);
 
 // Element offset of row `row` of the K (kv=0) or V (kv=1) slab of (layer, page, head).

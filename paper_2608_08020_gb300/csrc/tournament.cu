@@ -160,6 +160,8 @@ __global__ void __launch_bounds__(kTourThreads, 1) k_tournament(PoolView v, Tour
     s_freed = 0;
     s_minword = 0x7fffffff;
     s_lin0 = (unsigned)v.ctl[kCtlNextLineage];
+    // The first barrier's count: this CTA has not arrived, so no more than the others' arrivals are in it.
+    s_snap = (*reinterpret_cast<volatile unsigned*>(v.ctl + kCtlBarCount) / gridDim.x + 1) * gridDim.x;
   }
   if (blockIdx.x == 0 && tid < 2 * kSegLenBuckets) v.seg_hist[tid] = 0;
   if (blockIdx.x == 0 && tid == 0) {
@@ -197,8 +199,12 @@ __global__ void __launch_bounds__(kTourThreads, 1) k_tournament(PoolView v, Tour
       __syncthreads();
       if (act) s_keys[pos] = ((unsigned long long)rank_key(mean_w) << 32) | (unsigned)tid;
       __syncthreads();
-      // This CTA has read every slot's state: from here on others may change it.
-      if (v.grouped && tid == 0) s_snap = grid_arrive(v);
+      // This CTA has read every slot's state: from here on others may change it.  Its arrival at the first
+      // barrier, from a thread that has no key to rank unless the pool is nearly full.
+      if (v.grouped && tid == kTourThreads - 1) {
+        fence_acq_rel_gpu();
+        atomicAdd(reinterpret_cast<unsigned*>(v.ctl + kCtlBarCount), 1u);
+      }
       // Rank (ascending keys; the slot in the low word makes them distinct): each warp sorts its
       // 32 keys in registers (bitonic, by shuffles), then a key's rank is its position in its
       // warp's list plus, for every other list, the number of keys there below it (a binary
