@@ -154,10 +154,13 @@ __device__ __forceinline__ void ldsm_offsets(uint32_t (&koff)[4], uint32_t (&vof
   }
 }
 
-// The two bf16 terms of a pair of fp32 values: hi + lo is within 2^-17 of each.
+// The two bf16 terms of a pair of probabilities: hi + lo is within 2^-16 of each.  Cut off rather than
+// rounded, so that both terms of a positive value are positive (an exact one gets 2^-20 of itself): an
+// infinite V then stays infinite, where a zero or negative second term would make it NaN.
 __device__ __forceinline__ void split_bf16x2(float a, float b, uint32_t& hi, uint32_t& lo) {
-  hi = pack_bf16x2(a, b);
-  lo = pack_bf16x2(a - __uint_as_float(hi << 16), b - __uint_as_float(hi & 0xffff0000u));
+  const float ah = __uint_as_float(__float_as_uint(a) & 0xffff0000u), bh = __uint_as_float(__float_as_uint(b) & 0xffff0000u);
+  hi = __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
+  lo = pack_bf16x2(fmaxf(a - ah, ah * 0x1p-20f), fmaxf(b - bh, bh * 0x1p-20f));
 }
 
 // One landed 16-token chunk (stage address sb, its first nvalid >= 1 tokens) into the pair's state.
