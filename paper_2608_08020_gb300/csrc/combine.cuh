@@ -291,12 +291,15 @@ __device__ __forceinline__ void merge_completed(const PoolView& v, const Counter
   const int lane = threadIdx.x & 31;
   const int x0 = (int)min((long long)w * c, (long long)Tot), x1 = min(x0 + c, Tot);
   if (x0 >= x1) return;
-  const int x = lane == 0 ? x0 : x1 - 1;
-  int lo = 0, hi = v.max_beams;  // invariant: s_off[lo] <= x < s_off[hi]
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (s_off[mid] <= x) lo = mid; else hi = mid;
-  }
+  auto beam_of = [&](int x) {  // the beam of chunk x
+    int lo = 0, hi = v.max_beams;  // invariant: s_off[lo] <= x < s_off[hi]
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (s_off[mid] <= x) lo = mid; else hi = mid;
+    }
+    return lo;
+  };
+  const int x = lane == 0 ? x0 : x1 - 1, lo = beam_of(x);
   auto records = [&](int b, int h, int* first) {
     const int n = s_n[b], o = s_off[b] + h * n;
     *first = o / c;
@@ -315,11 +318,11 @@ __device__ __forceinline__ void merge_completed(const PoolView& v, const Counter
   int b = __shfl_sync(0xffffffffu, lo, 0);
   h = p0 - b * v.Hkv;
   for (int q = p0; q <= p1; ++q, ++h) {
-    if (h == v.Hkv) {
+    if (h == v.Hkv) {  // on to the next beam that has chunks
+      b = beam_of(s_off[b + 1]);
       h = 0;
-      ++b;
+      q = b * v.Hkv;
     }
-    if (s_n[b] == 0) continue;
     const int l = q == p0 ? 0 : 1;  // the lane that counted this pair, at either end of the range
     const bool own = q != p0 && q != p1;
     if (!own && !((m_last >> l) & 1u)) continue;
